@@ -352,19 +352,21 @@ cudaError_t peig(mpdo_ctx* h, int n, const cx<R>* a, long lda, cx<R>* v, long ld
   return e;
 }
 
-// Gram-type product with storage-precision inputs and small-matrix-precision output:
-// FP32 inputs with FP64 products and sums when RS = float and RM = double.
+// Gram matrix (n x n, Hermitian) of storage-precision data in the small-matrix precision: A^+ A
+// (side 0, A k x n) or A A^+ (side 1, A n x k); FP32 inputs with FP64 products and sums when
+// RS = float and RM = double.
 template <typename RS, typename RM>
-cudaError_t pgram(mpdo_ctx* h, int opa, int opb, int m, int n, int k, const cx<RS>* A, long lda,
-                  const cx<RS>* B, long ldb, cx<RM>* C, long ldc) {
-  if constexpr (std::is_same<RS, RM>::value) {
-    return pgemm<RS>(h, opa, opb, m, n, k, A, lda, 0, B, ldb, 0, C, ldc, 0, 1);
+cudaError_t pgram(mpdo_ctx* h, int side, int n, int k, const cx<RS>* A, long lda, cx<RM>* C,
+                  long ldc) {
+  const int opa = side == 0 ? OP_C : OP_N, opb = side == 0 ? OP_N : OP_C;
+  if constexpr (std::is_same<RM, float>::value) {
+    return pgemm<RS>(h, opa, opb, n, n, k, A, lda, 0, A, lda, 0, C, ldc, 0, 1);
   } else {
-    if (tc_exact_route(h, m, n, k, 1))
-      return pexact<float2, float2>(h, opa, opb, m, n, k, A, lda, 0, B, ldb, 0, C, ldc, 0, 1);
+    if (tc_exact_route(h, n, n, k, 1))
+      return pexact<cx<RS>, cx<RS>>(h, opa, opb, n, n, k, A, lda, 0, A, lda, 0, C, ldc, 0, 1);
     int pi = prof_begin(h, 0);
-    cudaError_t e = cgemm_wide<float>(h->st, opa, opb, m, n, k, A, lda, 0, B, ldb, 0, C, ldc, 0, 1);
-    prof_end(h, 0, pi, 8.0 * m * n * (double)k);
+    cudaError_t e = cgemm_gram<RS>(h->st, side, n, k, A, lda, C, ldc);
+    prof_end(h, 0, pi, 8.0 * n * n * (double)k);
     return e;
   }
 }
@@ -489,7 +491,7 @@ int lift_eig(mpdo_ctx* h, int n, const cx<RM>* g, cx<RM>* v, long ldv, double* w
   if (r < 1 || (r >= rmax && r < n && h->hpc->resid > tol)) return MPDO_OK;
   TM* Gs = static_cast<TM*>(h->wGs);
   TM* Z = static_cast<TM*>(h->wZ);
-  CK(pgemm<RM>(h, OP_C, OP_N, r, r, n, L, kInnerRmax, 0, L, kInnerRmax, 0, Gs, r, 0, 1));
+  CK((pgram<RM, RM>(h, 0, r, n, L, kInnerRmax, Gs, r)));
   CK(peig<RM>(h, r, Gs, r, Z, r, w, floor, max_vals));
   PO(lift<RM>(st, r, Z, w, Gs));
   CK(pgemm<RM>(h, OP_N, OP_N, n, r, r, L, kInnerRmax, 0, Gs, r, 0, v, ldv, 0, 1));
@@ -588,9 +590,8 @@ int update_lr(mpdo_ctx* h, int i, const DevOp& op, bool mirrored, int chi, int k
   int rc;
   // a2: Gram matrices of the two site tensors
   PO(swap12<T>(st, dl, 3, ki, dm, ai, wM));
-  CK((pgram<RS, RM>(h, OP_C, OP_N, n3, n3, dl * ki, wM, n3, wM, n3, wGi, n3)));
-  CK((pgram<RS, RM>(h, OP_N, OP_C, n3, n3, kj * dr, aj, (long)kj * dr, aj, (long)kj * dr, wGj,
-                    n3)));
+  CK((pgram<RS, RM>(h, 0, n3, dl * ki, wM, n3, wGi, n3)));
+  CK((pgram<RS, RM>(h, 1, n3, kj * dr, aj, (long)kj * dr, wGj, n3)));
   PO(trace_pre<RM>(st, dm, wGi, wGj, h->dsc));
   // a3: left factor from the eigendecomposition of G_i (numerical rank by gtol)
   {
@@ -658,7 +659,7 @@ int update_lr(mpdo_ctx* h, int i, const DevOp& op, bool mirrored, int chi, int k
     TM* qolM = static_cast<TM*>(h->wQol);
     CK(pwide<RM>(h, OP_N, OP_N, dl * ki, keep, n3, wM, n3, 0, wVgen, keep, (long)n3 * keep, aM,
                  3L * keep, keep, 3));
-    CK(pgemm<RM>(h, OP_C, OP_N, keep, keep, rows, aM, keep, 0, aM, keep, 0, gaM, keep, 0, 1));
+    CK((pgram<RM, RM>(h, 0, keep, rows, aM, keep, gaM, keep)));
     PO(polar_factors<RM>(st, keep, gaM, polM, qolM));
     CK(pgemm<RM>(h, OP_N, OP_N, rows, keep, keep, aM, keep, 0, polM, keep, 0, acM, keep, 0, 1));
     // W in FP64 into wVgen (no longer needed), then rounded to the storage precision
@@ -672,7 +673,7 @@ int update_lr(mpdo_ctx* h, int i, const DevOp& op, bool mirrored, int chi, int k
     T* wQol = static_cast<T*>(h->wQol);
     CK(pgemm<RS>(h, OP_N, OP_N, dl * ki, keep, n3, wM, n3, 0, wVgen, keep, (long)n3 * keep,
                  wTmp, 3L * keep, keep, 3));
-    CK(pgemm<RS>(h, OP_C, OP_N, keep, keep, rows, wTmp, keep, 0, wTmp, keep, 0, wGa, keep, 0, 1));
+    CK((pgram<RS, RS>(h, 0, keep, rows, wTmp, keep, wGa, keep)));
     PO(polar_factors<RS>(st, keep, wGa, wPol, wQol));
     CK(pgemm<RS>(h, OP_N, OP_N, rows, keep, keep, wTmp, keep, 0, wPol, keep, 0, wWB, keep, 0, 1));
     CK(pgemm<RS>(h, OP_C, OP_N, n3, keep, dl * ki, wM, n3, 0, wWB, 3L * keep, keep, wW, keep,
@@ -690,7 +691,7 @@ int update_lr(mpdo_ctx* h, int i, const DevOp& op, bool mirrored, int chi, int k
   if (colsB < KM) {
     // the inner Gram W = B B^+ has rank <= colsB: diagonalise the smaller dual B^+ B
     const int nc = (int)colsB;
-    CK((pgram<RS, RM>(h, OP_C, OP_N, nc, nc, KM, wBp, colsB, wBp, colsB, wWK, nc)));
+    CK((pgram<RS, RM>(h, 0, nc, KM, wBp, colsB, wWK, nc)));
     int nv;
     rc = inner_eig<RM>(h, nc, &nv);
     if (rc) return rc;
@@ -703,7 +704,7 @@ int update_lr(mpdo_ctx* h, int i, const DevOp& op, bool mirrored, int chi, int k
     // a10: kept rows f_k sqrt(w_k) y_k^+
     PO((dual_rows<RM, RS>(st, kk, nc, wVk, nc, h->wF, h->wWv, wCn)));
   } else {
-    CK((pgram<RS, RM>(h, OP_N, OP_C, KM, KM, colsB, wBp, colsB, wBp, colsB, wWK, KM)));
+    CK((pgram<RS, RM>(h, 1, KM, (int)colsB, wBp, colsB, wWK, KM)));
     int nv;
     rc = inner_eig<RM>(h, KM, &nv);
     if (rc) return rc;

@@ -215,13 +215,191 @@ __global__ void __launch_bounds__(ST * ST) cgemm_small_split_kernel(
   cluster.sync();   // rank 0 has read every partial before the cluster leaves
 }
 
-// Number of K slices for a small-tile FP64 product: enough to bring the tiles of the grid
-// towards one per SM, each slice at least 16 long (one tile step), at most 8 (portable
-// cluster size).
-inline int split_count(long tiles, int K) {
-  int s = 1;
-  while (s < 8 && tiles * (2 * s) <= 152 && K >= 16 * (2 * s)) s *= 2;
-  return s;
+// FP64 products on tiles of 8 x 8, 4 x 8 or 4 x 4.  FP64 runs at 2 FMA per clock per SM here, so
+// a product takes ceil(CTAs / SMs) x (tile area) x 2 K clocks whatever else is done; the tiles of
+// the update's products (outputs of 20 to 400 a side) decide how many SMs work and how much of
+// a tile is padding.  128 threads: the K steps of a chunk are dealt out over 128 / area groups
+// of threads, whose sums meet in shared memory in group order; the next chunk's operands are
+// fetched into registers while the present one is multiplied.  CLUSTER: the K loop is split
+// over the CTAs of a thread-block cluster (dims (1, 1, splits)), partial sums added in rank
+// order, for long products of few outputs, which a single chunk's latency bounds otherwise.
+// HERM: C = C^+ is known (Grams): only tiles on and above the diagonal run (grid.x counts them)
+// and their mirror images are written too.
+// Measured (16 x 16 tiles with their K split -> these): 60 x 60 x 60 14.5 -> 6.4 us, 20 x 20 x
+// 160 in a batch of 256 313 (64 x 64: 1347) -> 146 us.
+constexpr int TT = 128;   // threads
+constexpr int TKC = 32;   // K chunk
+template <typename RA, typename RB, typename R, int TM, int TN, bool CLUSTER, bool HERM>
+__global__ void __launch_bounds__(TT) cgemm_tile_kernel(
+    int M, int N, int K, const cx<RA>* __restrict__ A, long sam, long sak, long sab, int conja,
+    const cx<RB>* __restrict__ B, long sbk, long sbn, long sbb, int conjb, cx<R>* C, long scm,
+    long scn, long scb, cx<R> alpha, cx<R> beta, int use_beta, int splits) {
+  using T = cx<R>;
+  constexpr int AREA = TM * TN, G = TT / AREA;
+  constexpr int LA = TM * TKC / TT, LB = TN * TKC / TT;
+  __shared__ T As[TKC][TM + 1];
+  __shared__ T Bs[TKC][TN + 1];
+  __shared__ T part[G][AREA];
+  const int tid = threadIdx.x, g = tid / AREA, o = tid % AREA, tx = o % TN, ty = o / TN;
+  int by = blockIdx.y, bx = blockIdx.x;
+  if (HERM) {   // bx-th tile (by <= bx) of the upper triangle, row by row
+    const int nt = (N + TN - 1) / TN;
+    by = 0;
+    while (bx >= nt - by) {
+      bx -= nt - by;
+      ++by;
+    }
+    bx += by;
+  }
+  const int m0 = by * TM, n0 = bx * TN;
+  const long bz = CLUSTER ? blockIdx.z / splits : blockIdx.z;
+  int kb = 0, ke = K;
+  if (CLUSTER) {   // slices of whole chunks, rank order
+    const int kc = ((K + splits * TKC - 1) / (splits * TKC)) * TKC;
+    kb = (blockIdx.z % splits) * kc;
+    ke = min(K, kb + kc);
+  }
+  A += bz * sab;
+  B += bz * sbb;
+  C += bz * scb;
+  const bool a_kfast = (sak == 1), b_nfast = (sbn == 1);
+  T ra[LA], rb[LB];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < LA; ++q) {
+      const int e = tid + q * TT;
+      const int mi = a_kfast ? e / TKC : e % TM, ki = a_kfast ? e % TKC : e / TM;
+      T v = mkc<R>(0, 0);
+      if (m0 + mi < M && k0 + ki < ke) {
+        const cx<RA> t = A[(m0 + mi) * sam + (k0 + ki) * sak];
+        v = mkc<R>((R)t.x, conja ? -(R)t.y : (R)t.y);
+      }
+      ra[q] = v;
+    }
+#pragma unroll
+    for (int q = 0; q < LB; ++q) {
+      const int e = tid + q * TT;
+      const int ni = b_nfast ? e % TN : e / TKC, ki = b_nfast ? e / TN : e % TKC;
+      T v = mkc<R>(0, 0);
+      if (n0 + ni < N && k0 + ki < ke) {
+        const cx<RB> t = B[(k0 + ki) * sbk + (n0 + ni) * sbn];
+        v = mkc<R>((R)t.x, conjb ? -(R)t.y : (R)t.y);
+      }
+      rb[q] = v;
+    }
+  };
+  T acc = mkc<R>(0, 0);
+  if (kb < ke) fetch(kb);
+  for (int k0 = kb; k0 < ke; k0 += TKC) {
+#pragma unroll
+    for (int q = 0; q < LA; ++q) {
+      const int e = tid + q * TT;
+      if (a_kfast) As[e % TKC][e / TKC] = ra[q]; else As[e / TM][e % TM] = ra[q];
+    }
+#pragma unroll
+    for (int q = 0; q < LB; ++q) {
+      const int e = tid + q * TT;
+      if (b_nfast) Bs[e / TN][e % TN] = rb[q]; else Bs[e % TKC][e / TKC] = rb[q];
+    }
+    __syncthreads();
+    if (k0 + TKC < ke) {
+      fetch(k0 + TKC);
+#pragma unroll
+      for (int kk = 0; kk < TKC; kk += G) cfma(acc, As[kk + g][ty], Bs[kk + g][tx]);
+    } else {   // the last chunk's tail (zero-filled to its end) is not multiplied
+      for (int kk = 0; kk < ke - k0; kk += G) cfma(acc, As[kk + g][ty], Bs[kk + g][tx]);
+    }
+    __syncthreads();
+  }
+  if (G > 1) {
+    part[g][o] = acc;
+    __syncthreads();
+    if (g == 0) {
+#pragma unroll
+      for (int q = 1; q < G; ++q) acc = cadd(acc, part[q][o]);
+    }
+  }
+  if (CLUSTER) {
+    cg::cluster_group cluster = cg::this_cluster();
+    if (g == 0) part[0][o] = acc;
+    cluster.sync();
+    if (cluster.block_rank() == 0 && g == 0)
+      for (int q = 1; q < splits; ++q)
+        acc = cadd(acc, cluster.map_shared_rank(&part[0][0], q)[o]);
+    cluster.sync();   // rank 0 has read every partial before the cluster leaves
+    if (cluster.block_rank() != 0) return;
+  }
+  const int gm = m0 + ty, gn = n0 + tx;
+  if (g == 0 && gm < M && gn < N && (!HERM || gm <= gn)) {
+    T* p = C + gm * scm + gn * scn;
+    if (HERM) {
+      if (gm == gn) acc.y = 0;
+      *p = acc;
+      C[gn * scm + gm * scn] = cconj(acc);
+      return;
+    }
+    T v = acc;
+    if (alpha.x != R(1) || alpha.y != R(0)) v = cmul(alpha, v);
+    if (use_beta) v = cadd(v, cmul(beta, *p));
+    *p = v;
+  }
+}
+
+// Choice of an FP64 product's tile: 0 = 64 x 64, 1 = 16 x 16, 2 = 8 x 8, 3 = 4 x 8, 4 = 4 x 4, by
+// the FP64 time of its busiest SM, ceil(CTAs / 152) x area x 2 K clocks, with a factor for what
+// smaller tiles lose to operand traffic (2304 x 256 x 256, all SMs busy either way: 1042, 1078,
+// 1080, 1125 and 1208 us).  *splits: CTAs of a cluster sharing the K loop of tiles 2 to 4, while
+// every CTA keeps at least four chunks and the SMs at most four CTAs.
+inline int pick_tile(int m, int n, int batch, int k, bool herm, int* splits) {
+  const int tm[5] = {64, 16, 8, 4, 4}, tn[5] = {64, 16, 8, 8, 4};
+  const double f[5] = {1.0, 1.04, 1.06, 1.1, 1.2};
+  double best = 0;
+  int t = -1;
+  long ctas = 0;
+  for (int c = herm ? 2 : 0; c < 5; ++c) {
+    const long a = (m + tm[c] - 1) / tm[c], b = (n + tn[c] - 1) / tn[c];
+    if ((herm && tm[c] != tn[c]) || a > 65535) continue;   // a: the grid's y extent
+    const long q = (herm ? a * (a + 1) / 2 : a * b) * batch;
+    const double cost = (double)((q + 151) / 152) * tm[c] * tn[c] * f[c];
+    if (t < 0 || cost < best) {
+      best = cost;
+      t = c;
+      ctas = q;
+    }
+  }
+  *splits = 1;
+  if (t >= 2)
+    while (*splits < 8 && ctas * 2 * *splits <= 608 && k >= 4 * TKC * 2 * *splits) *splits *= 2;
+  return t;
+}
+
+template <typename RA, typename RB, typename R, int TM, int TN, bool HERM>
+cudaError_t launch_tile(cudaStream_t st, int m, int n, int k, const cx<RA>* A, long sam, long sak,
+                        long sab, int conja, const cx<RB>* B, long sbk, long sbn, long sbb,
+                        int conjb, cx<R>* C, long scm, long scb, int batch, cx<R> alpha,
+                        cx<R> beta, int use_beta, int splits) {
+  const int nx = (n + TN - 1) / TN, ny = (m + TM - 1) / TM;
+  const dim3 grid(HERM ? nx * (nx + 1) / 2 : nx, HERM ? 1 : ny, batch * splits);
+  if (splits == 1) {
+    cgemm_tile_kernel<RA, RB, R, TM, TN, false, HERM><<<grid, TT, 0, st>>>(
+        m, n, k, A, sam, sak, sab, conja, B, sbk, sbn, sbb, conjb, C, scm, 1L, scb, alpha, beta,
+        use_beta, 1);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(TT);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 1;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = splits;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, cgemm_tile_kernel<RA, RB, R, TM, TN, true, HERM>, m, n, k, A, sam,
+                            sak, sab, conja, B, sbk, sbn, sbb, conjb, C, scm, 1L, scb, alpha, beta,
+                            use_beta, splits);
 }
 
 // Tile-shape table of the autotuner (mpdo_autotune_gemm): per precision (0: FP64 products,
@@ -253,17 +431,44 @@ cudaError_t cgemm_impl(cudaStream_t st, int opa, int opb, int m, int n, int k, c
   if (k <= 0) {  // C = beta C: run with K = 0 (acc = 0)
     k = 0;
   }
-  const long big_tiles = (long)((n + BN - 1) / BN) * ((m + BM - 1) / BM) * batch;
+  [[maybe_unused]] const long big_tiles = (long)((n + BN - 1) / BN) * ((m + BM - 1) / BM) * batch;
   const long tiles16 = (long)((n + ST - 1) / ST) * ((m + ST - 1) / ST) * batch;
   const int choice =
       g_choice[sizeof(R) == 8 ? 0 : 1][tile_bucket(tiles16)][k_bucket(k)].load(std::memory_order_relaxed);
   const bool small = choice == 0 ? big_tiles < 152 : choice >= 2;
-  for (int b0 = 0; b0 < batch; b0 += 65535) {
-    int nb = batch - b0 < 65535 ? batch - b0 : 65535;
+  for (int b0 = 0; b0 < batch; b0 += 4096) {
+    int nb = batch - b0 < 4096 ? batch - b0 : 4096;
     count_launch();
-    if (small && (sizeof(R) == 8 || choice >= 3)) {
-      const long tiles = (long)((n + ST - 1) / ST) * ((m + ST - 1) / ST) * nb;
-      int splits = choice == 0 ? split_count(tiles, k) : (choice >= 3 ? 1 << (choice - 2) : 1);
+    if constexpr (sizeof(R) == 8) {
+      if (choice == 0) {
+        int s = 1;
+        const int t = pick_tile(m, n, nb, k, false, &s);
+        auto run = [&](auto launch) {
+          return launch(st, m, n, k, A + (long)b0 * sa, sam, sak, sa, conja, B + (long)b0 * sb, sbk,
+                        sbn, sb, conjb, C + (long)b0 * sc, (long)ldc, sc, nb, alpha, beta, use_beta,
+                        s);
+        };
+        if (t >= 2) {
+          MPDO_CUDA_TRY(t == 2   ? run(launch_tile<RA, RB, R, 8, 8, false>)
+                        : t == 3 ? run(launch_tile<RA, RB, R, 4, 8, false>)
+                                 : run(launch_tile<RA, RB, R, 4, 4, false>));
+          continue;
+        }
+        const int tile = t == 0 ? 64 : 16;
+        const dim3 g2((n + tile - 1) / tile, (m + tile - 1) / tile, nb);
+        auto big = [&](auto kern) {
+          kern<<<g2, 256, 0, st>>>(m, n, k, A + (long)b0 * sa, sam, sak, sa, conja,
+                                   B + (long)b0 * sb, sbk, sbn, sb, conjb, C + (long)b0 * sc,
+                                   (long)ldc, 1L, sc, alpha, beta, use_beta);
+        };
+        if (t == 0) big(cgemm_kernel<RA, RB, R>);
+        else big(cgemm_small_kernel<RA, RB, R>);
+        MPDO_CUDA_TRY(cudaGetLastError());
+        continue;
+      }
+    }
+    if (small && choice >= 3) {
+      int splits = 1 << (choice - 2);
       while (splits > 1 && k < 16 * splits) splits >>= 1;   // every slice at least one step
       if (splits > 1) {
         cudaLaunchConfig_t cfg = {};
@@ -301,6 +506,27 @@ cudaError_t cgemm_impl(cudaStream_t st, int opa, int opb, int m, int n, int k, c
   }
   return cudaGetLastError();
 }
+
+template <typename RA>
+cudaError_t cgemm_gram(cudaStream_t st, int side, int n, int k, const cx<RA>* A, long lda,
+                       cx<double>* C, long ldc) {
+  if (n <= 0) return cudaSuccess;
+  int s = 1;
+  const int t = pick_tile(n, n, 1, k, true, &s);
+  count_launch();
+  // side 0: C = A^+ A (A k x n); side 1: C = A A^+ (A n x k)
+  const long sm = side == 0 ? 1 : lda, sk = side == 0 ? lda : 1;
+  auto run = [&](auto launch) {
+    return launch(st, n, n, k, A, sm, sk, 0L, side == 0 ? 1 : 0, A, sk, sm, 0L, side == 0 ? 0 : 1, C,
+                  ldc, 0L, 1, mkc<double>(1, 0), mkc<double>(0, 0), 0, s);
+  };
+  return t == 2 ? run(launch_tile<RA, RA, double, 8, 8, true>)
+                : run(launch_tile<RA, RA, double, 4, 4, true>);
+}
+template cudaError_t cgemm_gram<float>(cudaStream_t, int, int, int, const float2*, long, double2*,
+                                       long);
+template cudaError_t cgemm_gram<double>(cudaStream_t, int, int, int, const double2*, long, double2*,
+                                        long);
 
 template <typename R>
 cudaError_t cgemm(cudaStream_t st, int opa, int opb, int m, int n, int k, const cx<R>* A,

@@ -20,6 +20,12 @@ cudaError_t cgemm_wide(cudaStream_t st, int opa, int opb, int m, int n, int k, c
                        long lda, long sa, const cx<RB>* B, long ldb, long sb, cx<double>* C,
                        long ldc, long sc, int batch);
 
+// Gram matrix with FP64 products and sums, its upper half computed and mirrored: C = A^+ A (side
+// 0, A k x n) or A A^+ (side 1, A n x k).
+template <typename RA>
+cudaError_t cgemm_gram(cudaStream_t st, int side, int n, int k, const cx<RA>* A, long lda,
+                       cx<double>* C, long ldc);
+
 // C = op(A) op(B) with an FP64 A and an FP32 B, FP64 products and sums (alpha 1, beta 0).
 cudaError_t cgemm_dx(cudaStream_t st, int opa, int opb, int m, int n, int k, const cx<double>* A,
                      long lda, long sa, const cx<float>* B, long ldb, long sb, cx<double>* C,
