@@ -475,7 +475,7 @@ def run_ours(args):
     g.profile(0)
     names = {0: "complex GEMMs (cgemm_kernel, cgemm_small_kernel, FP64-product cgemm_wide; "
                 "tc_gemm_kernel for the tensor-core forms)",
-             1: "eigensolvers (pchol_kernel, osj_kernel, jacobi_smem_kernel / jacobi_coop_kernel "
+             1: "eigensolvers (pchol_kernel, jacobi_graded_kernel, jacobi_smem_kernel / jacobi_coop_kernel "
                 "FP32 sweeps, FP64 refinement sg_refine_kernel, level_out_kernel)",
              2: "other kernels (selection, PPT, phi, layout)"}
 

@@ -412,6 +412,15 @@ int mpdo_kernel_cgemm(int prec, int opa, int opb, int m, int n, int k, const voi
  * pipeline wait gave up. */
 int mpdo_kernel_heig(int prec, int n, void* a, void* v, double* w, int* sweeps, void* stream);
 
+/* Largest n of the graded solver, which the update runs on L^+ L of pivoted Cholesky factors. */
+#define MPDO_HEIG_GRADED_NMAX 168
+/* Eigenpairs of a graded Hermitian PSD matrix a (complex128, n x n row-major, device; A = D C D
+ * with C of unit diagonal and moderate condition): eigenvalues, descending, into w (device
+ * double[n]) and eigenvectors into the columns of v, each pair resolved relative to its own
+ * size (FP32 sweeps with a relative threshold, two FP64 refinement passes).  n in
+ * 1..MPDO_HEIG_GRADED_NMAX.  Allocates its scratch and synchronises the stream. */
+int mpdo_kernel_heig_graded(int n, const void* a, void* v, double* w, void* stream);
+
 /* Tensor-core GEMMs (tcgen05.mma, TMEM accumulators, TMA-fed shared-memory pipeline) on
  * which the contractions of the two-site update run in the split-precision modes (Sec.
  * III.A: contracting the site tensors and the gate, Fig. 6a; the Gram products of the

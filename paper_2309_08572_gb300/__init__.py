@@ -144,6 +144,7 @@ def _load():
         "mpdo_kernel_cgemm": (I, [I, I, I, I, I, I, VP, C.c_long, C.c_long, VP, C.c_long,
                                   C.c_long, VP, C.c_long, C.c_long, I, VP]),
         "mpdo_kernel_heig": (I, [I, I, VP, VP, P(D), P(I), VP]),
+        "mpdo_kernel_heig_graded": (I, [I, VP, VP, P(D), VP]),
         "mpdo_heig_noalloc": (I, [I, I, VP, VP, P(D), P(I), VP]),
         "mpdo_tc_gemm_launches": (C.c_longlong, []),
         "mpdo_kernel_tcgemm_exact": (I, [I, I, I, I, I, VP, C.c_long, C.c_long, VP, C.c_long,
@@ -639,6 +640,17 @@ def kernel_heig(prec: int, n: int, a, v, w, stream=None) -> int:
                                 C.cast(C.c_void_p(w.data_ptr()), C.POINTER(C.c_double)),
                                 C.byref(sweeps), st))
     return sweeps.value
+
+
+HEIG_GRADED_NMAX = 168
+
+
+def kernel_heig_graded(n: int, a, v, w, stream=None):
+    """Eigenpairs of the graded PSD device matrix a (n x n complex128, n <= 168) -> w (desc), v."""
+    st = _current_stream() if stream is None else C.c_void_p(stream)
+    _check(LIB.mpdo_kernel_heig_graded(n, C.c_void_p(a.data_ptr()), C.c_void_p(v.data_ptr()),
+                                       C.cast(C.c_void_p(w.data_ptr()), C.POINTER(C.c_double)),
+                                       st))
 
 
 HEIG_NOALLOC_NMAX = 192

@@ -116,8 +116,8 @@ struct mpdo_ctx {
   // circuits, whose spinning host threads would otherwise take every core.
   cudaEvent_t bev = nullptr;
   bool block_sync = false;
-  // inner eigenproblem through a pivoted Cholesky (see inner_eig)
-  void *wL = nullptr, *wGs = nullptr, *wZ = nullptr, *wLg = nullptr;
+  // eigenproblems through a pivoted Cholesky factor (see lift_eig)
+  void *wGs = nullptr, *wZ = nullptr, *wLg = nullptr;
   struct PcOut { int r; int pad; double resid; };
   PcOut* dpc = nullptr;
   PcOut* hpc = nullptr;       // pinned
@@ -320,11 +320,7 @@ cudaError_t pgemm(mpdo_ctx* h, int opa, int opb, int m, int n, int k, const cx<R
   return e;
 }
 // floor: eigenpairs below floor * lambda_max need not be resolved (used by the mixed mode).
-// kMixedEigMax: largest factor rank taken through the lifted route (the factor buffer holds
-// 128 columns); the mixed solver itself serves any n up to the handle's capacity (one-CTA
-// FP32 sweeps up to n = 118, the cooperative FP32 block Jacobi above, FP64 refinement).
 // max_vals > 0: only that many leading pairs are needed (the rest come back as zeros).
-constexpr int kMixedEigMax = 118;
 template <typename R>
 cudaError_t peig(mpdo_ctx* h, int n, const cx<R>* a, long lda, cx<R>* v, long ldv, double* w,
                  double floor, int max_vals = 0) {
@@ -385,13 +381,12 @@ cudaError_t pwide(mpdo_ctx* h, int opa, int opb, int m, int n, int k, const cx<f
   return e;
 }
 
-// a8: eigenpairs of the inner Gram W (nin x nin, in wWK).  Small problems: all of them by
-// Jacobi.  Larger ones: only the leading part matters (at most k_max are kept; the total
-// weight comes from tr W and the PPT's |w|^2 from the eigenvalues, where the tail below the
-// factor's tolerance is negligible), so W ~ L L^+ by a pivoted Cholesky stopping at
-// kInnerTol64 (FP64 mode) or kInnerTol (FP32 factor) of tr W, and the eigenpairs of W are
-// lifted from those of the r x r matrix L^+ L: u_c = L z_c / sqrt(s_c).  A factor that
-// reaches kInnerRmax columns above the tolerance falls back to the full solve.
+// a8: eigenpairs of the inner Gram W (nin x nin, in wWK).  Only the leading part matters (at
+// most k_max are kept; the total weight comes from tr W and the PPT's |w|^2 from ||W||_F), so
+// W ~ L L^+ by a pivoted Cholesky factor stopping at kInnerTol64 (FP64 form), kInnerTolMixed
+// (mixed form) or kInnerTol (FP32 factor) of tr W, and the eigenpairs of W are lifted from
+// those of the r x r matrix L^+ L: u_c = L z_c / sqrt(s_c).  A factor that reaches its column
+// cap above the tolerance falls back to the full solve.
 // Eigenvectors go to wVk (row stride nin); returns their count.
 constexpr int kInnerDirect = 32;
 
@@ -405,76 +400,22 @@ inline double pc_tol(const mpdo_ctx* h, double cut) {
 constexpr double kInnerTol = 1e-7;
 constexpr double kInnerTol64 = 1e-14;
 constexpr double kInnerTolMixed = 1e-10;
-constexpr int kInnerRmax = 128;
-
-// Eigenpairs of the PSD Gram g (n x n, Gram precision RM) through its pivoted Cholesky
-// factor g ~ L L^+ (stopping at tol * tr g) and one-sided Jacobi on L: eigenvectors to
-// v (row stride ldv), eigenvalues to w, descending (FP64 factor and rotations for FP64
-// Grams, FP32 for FP32 Grams).
-// *nvals = r on success (columns r..n-1 of v and w[r..n) zeroed when zero_tail), 0 when
-// the factor does not fit (rank above the shared-memory cap) and the caller must solve
-// otherwise.  One host synchronisation (the rank).
-template <typename RM>
-int pc_eig(mpdo_ctx* h, int n, const cx<RM>* g, cx<RM>* v, long ldv, double* w, double tol,
-           bool zero_tail, int* nvals) {
-  cudaStream_t st = h->st;
-  *nvals = 0;
-  if (n < 1 || n > 1024) return MPDO_OK;
-  const size_t rbytes = std::is_same<RM, double>::value ? 16 : 8;
-  int rcap = (int)std::min<size_t>(128, kOsjMaxSmem / (rbytes * (size_t)n));
-  rcap -= rcap & 1;
-  const int rmax = std::min(n, rcap);
-  if (rmax < 1) return MPDO_OK;
-  int pi = prof_begin(h, 1);
-  if constexpr (std::is_same<RM, double>::value) {
-    CK(pchol<double>(st, n, g, rmax, tol, static_cast<double2*>(h->wLg), kInnerRmax,
-                     &h->dpc->r, &h->dpc->resid));
-  } else {
-    CK(pchol<float>(st, n, g, rmax, tol, static_cast<float2*>(h->wLg), kInnerRmax, &h->dpc->r,
-                    &h->dpc->resid));
-  }
-  CK(cudaMemcpyAsync(h->hpc, h->dpc, sizeof(mpdo_ctx::PcOut), cudaMemcpyDeviceToHost, st));
-  CK(sync_stream(h));
-  const int r = h->hpc->r;
-  if (r < 1 || (r >= rmax && r < n && h->hpc->resid > tol)) {
-    prof_end(h, 1, pi, 0.0);
-    prof_drain(h);
-    return MPDO_OK;
-  }
-  int* cnt = eigw<RM>(h).counters;
-  if constexpr (std::is_same<RM, double>::value) {
-    const double2* L = static_cast<const double2*>(h->wLg);
-    CK((osj<double, double, double>(st, n, r, L, kInnerRmax, v, (int)ldv, w, cnt, 0)));
-  } else {
-    const float2* L = static_cast<const float2*>(h->wLg);
-    CK((osj<float, float, float>(st, n, r, L, kInnerRmax, v, (int)ldv, w, cnt, 0)));
-  }
-  if (zero_tail && r < n) {
-    CK(cudaMemset2DAsync(v + r, ldv * sizeof(cx<RM>), 0, (n - r) * sizeof(cx<RM>), n, st));
-    CK(cudaMemsetAsync(w + r, 0, (n - r) * sizeof(double), st));
-  }
-  // executed flops: per rotation 3 dot products and 2 column updates of n complex entries
-  // (8 real flops each); the rotation count is read back with the profile
-  if (pi >= 0 && h->prof_slot < h->prof_nslots) {
-    int slot = h->prof_slot++;
-    CK(cudaMemcpyAsync(&h->prof_counts[slot], cnt + 3, sizeof(int), cudaMemcpyDeviceToHost, st));
-    prof_end(h, 1, pi, 0.0, slot, 8.0 * 5 * (double)n);
-  } else {
-    prof_end(h, 1, pi, 0.0);
-  }
-  *nvals = r;
-  return MPDO_OK;
-}
+constexpr int kInnerRmax = kGradedMax;   // columns of a factor (FP64)
+constexpr int kInnerRmaxF32 = 128;         // and of the FP32 factor
 
 // Eigenpairs of the PSD Gram g (n x n) through a pivoted Cholesky factor g ~ L L^+
 // (stopping at tol * tr g, at most rmax columns; FP64 factor for FP64 Grams, FP32 for
-// FP32 Grams) and the eigenpairs of the r x r matrix L^+ L (solved down to floor of its
-// largest), lifted as u = L z / sqrt(s): eigenvectors to v (row stride ldv), eigenvalues
-// to w, descending.  *nvals = r, or 0 when the factor needs more than rmax columns (the
-// caller solves the full problem).  zero_tail: columns r..n-1 of v and w[r..n) zeroed.
+// FP32 Grams) and the eigenpairs of the r x r matrix L^+ L, lifted as u = L z / sqrt(s):
+// eigenvectors to v (row stride ldv), eigenvalues to w, descending.  *nvals = r, or 0 when
+// the factor needs more than rmax columns (the caller solves the full problem).  zero_tail:
+// columns r..n-1 of v and w[r..n) zeroed.
+// FP64 Grams: L's columns fall off by decades, so L^+ L is graded and one graded solve
+// (heig_graded) resolves all of its pairs.  The levels of the mixed solver that it replaced took
+// 5 rounds of ~9 launches for such a matrix, and the FP64 form's one-sided Jacobi sweeps on L
+// 3.6 ms on one SM (n = 180, r = 40).
 template <typename RM>
 int lift_eig(mpdo_ctx* h, int n, const cx<RM>* g, cx<RM>* v, long ldv, double* w, double tol,
-             int rmax, double floor, bool zero_tail, int* nvals, int max_vals = 0) {
+             int rmax, bool zero_tail, int* nvals) {
   using TM = cx<RM>;
   cudaStream_t st = h->st;
   *nvals = 0;
@@ -492,7 +433,14 @@ int lift_eig(mpdo_ctx* h, int n, const cx<RM>* g, cx<RM>* v, long ldv, double* w
   TM* Gs = static_cast<TM*>(h->wGs);
   TM* Z = static_cast<TM*>(h->wZ);
   CK((pgram<RM, RM>(h, 0, r, n, L, kInnerRmax, Gs, r)));
-  CK(peig<RM>(h, r, Gs, r, Z, r, w, floor, max_vals));
+  if constexpr (std::is_same<RM, double>::value) {
+    int pe = prof_begin(h, 1);
+    double fl = 0.0;
+    CK(heig_graded(st, r, Gs, r, Z, r, w, h->mixw, &fl));
+    prof_end(h, 1, pe, fl);
+  } else {
+    CK(peig<RM>(h, r, Gs, r, Z, r, w, 0.0));
+  }
   PO(lift<RM>(st, r, Z, w, Gs));
   CK(pgemm<RM>(h, OP_N, OP_N, n, r, r, L, kInnerRmax, 0, Gs, r, 0, v, ldv, 0, 1));
   if (zero_tail && r < n) {
@@ -507,34 +455,21 @@ template <typename RM>
 int inner_eig(mpdo_ctx* h, int nin, int* nvals) {
   cx<RM>* W = static_cast<cx<RM>*>(h->wWK);
   cx<RM>* V = static_cast<cx<RM>*>(h->wVk);
-  int rc;
-  if (h->dbl) {
-    // FP64 mode: factor + one-sided Jacobi when the rank fits; the Kraus tail below the
-    // tolerance is negligible for the cut and the PPT sums
-    int nv = 0;
-    rc = pc_eig<RM>(h, nin, W, V, nin, h->wWv, kInnerTol64, false, &nv);
-    if (rc) return rc;
-    if (nv > 0) {
-      *nvals = nv;
-      return MPDO_OK;
-    }
-  }
-  if (nin <= kInnerDirect) {
+  const bool fp64 = std::is_same<RM, double>::value;
+  if (!fp64 && nin <= kInnerDirect) {
     CK(peig<RM>(h, nin, W, nin, V, nin, h->wWv, 1e-10));
     *nvals = nin;
     return MPDO_OK;
   }
-  // FP64 and mixed modes: FP64 factor (down to 1e-14 resp. 1e-10 of the trace); C64: FP32
-  // factor down to its floor.  (An FP32 factor of the FP64 Gram in mixed mode resolved the
-  // kept Kraus directions only to ~1e-7 of the largest weight, which moved energies by
-  // up to 1e-5 where two weights at the cut were close.)  Mixed: L^+ L stays within the
-  // mixed solver's size.
-  const double tol = h->dbl ? kInnerTol64 : h->mixed ? kInnerTolMixed : kInnerTol;
+  // FP64 Grams: FP64 factor; C64: FP32 factor down to its floor.  (An FP32 factor of the FP64
+  // Gram in mixed mode resolved the kept Kraus directions only to ~1e-7 of the largest weight,
+  // which moved energies by up to 1e-5 where two weights at the cut were close.)
+  const double tol = (h->dbl || (fp64 && nin <= kInnerDirect)) ? kInnerTol64
+                     : h->mixed                                ? kInnerTolMixed
+                                                               : kInnerTol;
   int nv = 0;
-  // at most k_max pairs are kept (the PPT's sum of squares comes from ||W||_F), so the
-  // solver may stop once k_max + 1 leading pairs are resolved
-  rc = lift_eig<RM>(h, nin, W, V, nin, h->wWv, tol, h->mixed ? kMixedEigMax : kInnerRmax, 1e-10,
-                    false, &nv, h->kmax + 1);
+  int rc = lift_eig<RM>(h, nin, W, V, nin, h->wWv, tol, fp64 ? kInnerRmax : kInnerRmaxF32, false,
+                        &nv);
   if (rc) return rc;
   if (nv == 0) {
     // at most k_max pairs are kept; the PPT's sum of squares comes from ||W||_F
@@ -596,17 +531,11 @@ int update_lr(mpdo_ctx* h, int i, const DevOp& op, bool mirrored, int chi, int k
   // a3: left factor from the eigendecomposition of G_i (numerical rank by gtol)
   {
     int nv = 0;
-    // FP64 mode: FP64 factor + one-sided Jacobi.  Mixed: FP64 factor and the mixed solver
-    // on L^+ L (rank r instead of 3D; rotating an FP32 copy of the factor instead loses the
-    // small eigenvalues: its rounding is relative to whole columns, not to eigen-
-    // directions), the factor route on larger ranks.  C64: the FP32 Jacobi solver.
-    if (h->mixed) {
-      rc = lift_eig<RM>(h, n3, wGi, wVg, n3, h->wSig, pc_tol(h, h->gtol), kMixedEigMax,
-                        0.1 * h->gtol, true, &nv);
-      if (rc) return rc;
-    }
-    if (nv == 0 && (h->dbl || (h->mixed && n3 > h->mixw.n_cap))) {
-      rc = pc_eig<RM>(h, n3, wGi, wVg, n3, h->wSig, pc_tol(h, h->gtol), true, &nv);
+    // FP64 Grams: FP64 factor and the graded solver on L^+ L (rank r instead of 3D; rotating
+    // an FP32 copy of the factor instead loses the small eigenvalues: its rounding is relative
+    // to whole columns, not to eigendirections).  C64: the FP32 Jacobi solver.
+    if (h->eltm == 16) {
+      rc = lift_eig<RM>(h, n3, wGi, wVg, n3, h->wSig, pc_tol(h, h->gtol), kInnerRmax, true, &nv);
       if (rc) return rc;
     }
     if (nv == 0) CK(peig<RM>(h, n3, wGi, n3, wVg, n3, h->wSig, 0.1 * h->gtol));
@@ -621,13 +550,8 @@ int update_lr(mpdo_ctx* h, int i, const DevOp& op, bool mirrored, int chi, int k
   // a6: bond eigenpairs and cut
   {
     int nv = 0;
-    if (h->mixed) {
-      rc = lift_eig<RM>(h, n9, wH, wU, n9, h->wLam, pc_tol(h, h->htol), kMixedEigMax,
-                        0.1 * h->htol, true, &nv, chi + 1);
-      if (rc) return rc;
-    }
-    if (nv == 0 && (h->dbl || (h->mixed && n9 > h->mixw.n_cap))) {
-      rc = pc_eig<RM>(h, n9, wH, wU, n9, h->wLam, pc_tol(h, h->htol), true, &nv);
+    if (h->eltm == 16) {
+      rc = lift_eig<RM>(h, n9, wH, wU, n9, h->wLam, pc_tol(h, h->htol), kInnerRmax, true, &nv);
       if (rc) return rc;
     }
     // at most chi pairs are kept: the (chi+1)-th decides nothing more (the discarded weight
@@ -1448,7 +1372,6 @@ int mpdo_create(const mpdo_config* cfg, const double* init_site_vec, mpdo_t* out
   if (em == 16) eig_work_bind<double>(h->eig64, h->eigmem, ncap);
   else eig_work_bind<float>(h->eig32, h->eigmem, ncap);
   if ((rc = alloc_dev(hp, &h->wLg, (size_t)std::max(n9, KM) * kInnerRmax * em)) ||
-      (rc = alloc_dev(hp, &h->wL, (size_t)KM * kInnerRmax * em)) ||
       (rc = B(&h->wGs, (size_t)kInnerRmax * kInnerRmax)) ||
       (rc = B(&h->wZ, (size_t)kInnerRmax * kInnerRmax)) ||
       (rc = alloc_dev(hp, (void**)&h->dpc, sizeof(mpdo_ctx::PcOut))))
@@ -1462,10 +1385,11 @@ int mpdo_create(const mpdo_config* cfg, const double* init_site_vec, mpdo_t* out
     cudaGetLastError();
     return fail(nullptr, MPDO_ERR_OOM, "pinned host allocation");
   }
-  if (h->mixed) {
+  if (em == 16) {
     // the mixed solver serves every Gram of the update (bond H up to 9 chi, inner W up to
-    // m_max k_max), so its workspace is sized for the largest
-    const int mcap = ncap;
+    // m_max k_max), so its workspace is sized for the largest; the FP64 form takes only its
+    // graded solver
+    const int mcap = h->mixed ? ncap : std::min(ncap, kGradedMax);
     if ((rc = alloc_dev(hp, &h->mixmem, mix_work_bytes(mcap)))) return rc;
     mix_work_bind(h->mixw, h->mixmem, mcap);
     // MPDO_NO_GRAPHS=1: launch the mixed eigensolver's levels directly (no CUDA graphs)
@@ -1921,6 +1845,30 @@ int mpdo_kernel_heig(int prec, int n, void* a, void* v, double* w, int* sweeps, 
   cudaFree(mem);
   if (e != cudaSuccess) return fail(nullptr, MPDO_ERR_CUDA, cudaGetErrorString(e));
   if (sweeps) *sweeps = sw;
+  return MPDO_OK;
+}
+
+int mpdo_kernel_heig_graded(int n, const void* a, void* v, double* w, void* stream) {
+  static_assert(MPDO_HEIG_GRADED_NMAX == kGradedMax, "header and solver agree");
+  if (n < 1 || n > kGradedMax || !a || !v || !w)
+    return fail(nullptr, MPDO_ERR_ARG, "bad heig_graded arguments");
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  void* mm = nullptr;
+  if (cudaMalloc(&mm, mix_work_bytes(n)) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(nullptr, MPDO_ERR_OOM, "heig_graded work");
+  }
+  MixWork mw;
+  mix_work_bind(mw, mm, n);
+  // the solver's CTA ticket starts at zero
+  cudaError_t e = cudaMemsetAsync(mm, 0, mix_work_bytes(n), st);
+  if (e == cudaSuccess)
+    e = heig_graded(st, n, (const double2*)a, n, (double2*)v, n, w, mw);
+  cudaError_t es = cudaStreamSynchronize(st);
+  mix_work_release(mw);
+  cudaFree(mm);
+  if (e == cudaSuccess) e = es;
+  if (e != cudaSuccess) return fail(nullptr, MPDO_ERR_CUDA, cudaGetErrorString(e));
   return MPDO_OK;
 }
 

@@ -246,7 +246,7 @@ __device__ void ritz_cluster(int m, const double2* SG, int c0, int c, double* la
   }
   __syncthreads();
   // B = P Q with its columns sorted, into Ps (P is read before the barrier below)
-  double2 bv[(kRitzMax * kRitzMax + 255) / 256];
+  double2 bv[(kRitzMax * kRitzMax + 127) / 128];   // blockDim.x >= 128
   int nb = 0;
   for (int e = tid; e < c * c; e += nt, ++nb) {
     const int a = e / c, b = e % c;
@@ -268,7 +268,7 @@ __device__ void ritz_cluster(int m, const double2* SG, int c0, int c, double* la
       continue;
     }
     double2 x[kRitzMax];
-    for (int k = 0; k < c; ++k) x[k] = row[k];
+    for (int k = 0; k < c; ++k) x[k] = __ldcg(&row[k]);   // maybe another CTA's
     for (int b = 0; b < c; ++b) {
       double2 acc = make_double2(0.0, 0.0);
       for (int k = 0; k < c; ++k) cfma(acc, x[k], Ps[k][b]);
@@ -505,6 +505,121 @@ __global__ void __launch_bounds__(RT * RT) refine_kernel(int m, int n, const dou
     refine_step<false>(m, n, SG, level0, level, floor, rot, lam, scan, IE, cid, emax, sepg);
 }
 
+// ---- graded matrices (heig_graded): one refinement pass.
+//
+// For a graded matrix (see heig_graded_f32) the mixing of a pair is measured relative to its
+// sizes: with lam_i > lam_j the FP32 sweeps leave S_ij ~ delta sqrt(lam_i lam_j) and G_ij ~
+// delta sqrt(lam_j / lam_i), so the correction E is graded as well and a pair is separated when
+// |S_ij - lam G_ij| sqrt(lam_i / lam_j) < emax |lam_i - lam_j| and its relative gap exceeds the
+// rounding of the products (100 m eps_64).  No pair is left to another level.
+//
+// The step is bound by FP64: a pair costs two dot products of length m and one division.  So
+// one CTA takes a 4 x 4 block of pairs above the diagonal, forms its S, G and the diagonal
+// entries it needs (48 dot products on 96 threads, halves of the sum over k) and writes its
+// part of I + E: 120 CTAs at m = 60, where a 16 x 16 tiling would use 30 SMs and leave the
+// elementwise step to one.  In the final pass the last CTA to finish (a ticket; nobody waits)
+// settles runs of unseparated neighbours by Rayleigh-Ritz, 16 at a time.
+constexpr int GT = 4;
+constexpr int kSgeThreads = 128;
+__global__ void __launch_bounds__(kSgeThreads) sge_kernel(int m, const double2* __restrict__ TZ,
+                                                          double2* SG, int final_pass,
+                                                          double emax, double* lam, double2* IE,
+                                                          unsigned char* sep, unsigned int* ticket) {
+  extern __shared__ double2 sge_col[];   // [k][16]: Z_I, Z_J, T_I, T_J
+  __shared__ double2 part[48];
+  __shared__ double2 val[48];            // S, G (16 each), then S_ii, G_ii, S_jj, G_jj (4 each)
+  __shared__ int s_last;
+  const int tid = threadIdx.x;
+  const long ld = 2L * m;
+  const int nt = (m + GT - 1) / GT;
+  // block pair (I <= J) of this CTA
+  int I = 0, rem = blockIdx.x;
+  while (rem >= nt - I) {
+    rem -= nt - I;
+    ++I;
+  }
+  const int J = I + rem, i0 = I * GT, j0 = J * GT;
+  for (int e = tid; e < 16 * m; e += kSgeThreads) {
+    const int k = e >> 4, c = e & 15;
+    const int col = (c & 4 ? j0 : i0) + (c & 3);
+    double2 v = make_double2(0.0, 0.0);
+    if (col < m) v = TZ[k * ld + (c < 8 ? m : 0) + col];
+    sge_col[e] = v;
+  }
+  __syncthreads();
+  if (tid < 96) {
+    const int d = tid % 48, hf = tid / 48;
+    int xa, ya;
+    if (d < 32) {
+      xa = (d >> 2) & 3;
+      ya = (d < 16 ? 12 : 4) + (d & 3);
+    } else {
+      const int q = d - 32, c = q & 3;   // S_ii, G_ii, S_jj, G_jj
+      xa = (q < 8 ? 0 : 4) + c;
+      ya = xa + ((q & 4) ? 0 : 8);
+    }
+    double2 acc = make_double2(0.0, 0.0);
+    for (int k = hf; k < m; k += 2) cfma(acc, cconj(sge_col[16 * k + xa]), sge_col[16 * k + ya]);
+    (hf ? part : val)[d] = acc;
+  }
+  __syncthreads();
+  if (tid < 48) val[tid] = cadd(val[tid], part[tid]);
+  __syncthreads();
+  if (tid < 16) {
+    const int a = tid >> 2, b = tid & 3, i = i0 + a, j = j0 + b;
+    const double gi = val[36 + a].x, gj = val[44 + b].x;
+    const double li = gi > 0 ? val[32 + a].x / gi : 0.0, lj = gj > 0 ? val[40 + b].x / gj : 0.0;
+    const double2 s = val[tid], g = val[16 + tid];
+    if (i == j && i < m) {
+      lam[i] = li;
+      IE[(long)i * m + i] = make_double2(1.0 + 0.5 * (1.0 - gi), 0.0);
+      SG[i * ld + i] = s;
+      SG[i * ld + m + i] = g;
+    } else if (i < j && j < m) {
+      SG[i * ld + j] = s;
+      SG[i * ld + m + j] = g;
+      SG[j * ld + i] = cconj(s);
+      SG[j * ld + m + i] = cconj(g);
+      const double d = lj - li, mx = fmax(fabs(li), fabs(lj)), mn = fmin(li, lj);
+      const double2 nij = make_double2(s.x - lj * g.x, s.y - lj * g.y);
+      const double2 nji = make_double2(s.x - li * g.x, -(s.y - li * g.y));
+      const double lim = emax * emax * d * d * mn;
+      const bool newton = mn > 0.0 && fabs(d) > 100.0 * m * 1.1e-16 * mx &&
+                          cabs2(nij) * mx < lim && cabs2(nji) * mx < lim;
+      if (newton) {
+        const double r = 1.0 / d;
+        IE[(long)i * m + j] = cscale(nij, r);
+        IE[(long)j * m + i] = cscale(nji, -r);
+      } else {
+        IE[(long)i * m + j] = cscale(g, -0.5);
+        IE[(long)j * m + i] = cscale(cconj(g), -0.5);
+      }
+      if (j == i + 1) sep[i] = newton;
+    }
+  }
+  if (!final_pass) return;
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (tid == 0) *ticket = 0u;
+  unsigned char* flags = reinterpret_cast<unsigned char*>(sge_col);
+  int open = 0;
+  for (int i = tid; i + 1 < m; i += kSgeThreads) {
+    flags[i] = __ldcg(&sep[i]);
+    open |= !flags[i];
+  }
+  if (!__syncthreads_or(open)) return;
+  for (int i = 0; i + 1 < m;) {
+    int j = i;
+    while (j + 1 < m && !flags[j] && j - i + 1 < kRitzMax) ++j;   // run [i, j]
+    if (j > i) ritz_cluster(m, SG, i, j - i + 1, lam, IE);
+    i = j + 1;
+  }
+}
+
 // K slices of a small FP64 product: enough to bring the CTAs towards one per SM, each
 // slice at least 16 long (one tile step), at most 8 (portable cluster size).
 inline int split_count(long tiles, int K) {
@@ -654,7 +769,7 @@ void mix_work_release(MixWork& w) {
 size_t mix_work_bytes(int n_cap) {
   size_t sq = (size_t)n_cap * n_cap;
   return 8 * sq * sizeof(double2) + 2 * sq * sizeof(float2) + 6 * (size_t)n_cap * 8 +
-         eig_work_bytes<float>(n_cap) + 12 * 256;
+         eig_work_bytes<float>(n_cap) + graded_log_bytes(std::min(n_cap, kGradedMax)) + 13 * 256;
 }
 
 void mix_work_bind(MixWork& w, void* base, int n_cap) {
@@ -679,6 +794,7 @@ void mix_work_bind(MixWork& w, void* base, int n_cap) {
   w.ticket = reinterpret_cast<unsigned int*>(take(64));
   w.cid = reinterpret_cast<int*>(take((size_t)n_cap * sizeof(int)));
   w.sepf = reinterpret_cast<unsigned char*>(take((size_t)n_cap));
+  w.glog = take(graded_log_bytes(std::min(n_cap, kGradedMax)));
   eig_work_bind<float>(w.ew, take(eig_work_bytes<float>(n_cap)), n_cap);
 }
 
@@ -888,6 +1004,54 @@ cudaError_t heig_mixed(cudaStream_t st, int n, const double2* a, long lda, doubl
   }
   if (levels_out) *levels_out = level + 1;
   if (flops_out) *flops_out = flops;
+  return cudaSuccess;
+}
+
+// Eigenpairs of a graded FP64 Hermitian PSD matrix a (n x n, n <= kGradedMax; L^+ L of a pivoted
+// Cholesky factor), every one resolved relative to its own size: FP32 sweeps with a relative
+// threshold, then two FP64 refinement passes (file comment of sge_kernel).  One solve takes the
+// place of the levels of heig_mixed and of FP64 sweeps, whose time went into a chain of small
+// launches per two decades of the spectrum (mixed form) or into one SM's FP64 pipe (FP64 form).
+cudaError_t heig_graded(cudaStream_t st, int n, const double2* a, long lda, double2* z, long ldz,
+                        double* w, MixWork& wk, double* flops_out) {
+  if (n <= 0) return cudaSuccess;
+  if (n > kGradedMax || n > wk.n_cap) return cudaErrorInvalidValue;
+  const long l2 = 2L * n;
+  double2 *cur = wk.tz, *nxt = wk.tz2;
+  // FP64 on the CUDA cores whatever the size: the slice products carry each entry to 2^-48 of
+  // its row's largest, which is not enough for the small entries of a graded row
+  auto mul = [&](const double2* x, long ldx, long sx, const double2* y, long ldy, double2* c,
+                 long ldc, long sc, int batch) {
+    return cgemm<double>(st, OP_N, OP_N, n, n, n, x, ldx, sx, y, ldy, 0, c, ldc, sc, batch,
+                         make_double2(1, 0), make_double2(0, 0));
+  };
+  MPDO_CUDA_TRY(heig_graded_f32(st, n, a, lda, cur + n, l2, wk.glog, nullptr));
+  MPDO_CUDA_TRY(mul(a, lda, 0, cur + n, l2, cur, l2, 0, 1));
+  const int nt = (n + GT - 1) / GT, grid = nt * (nt + 1) / 2;
+  const size_t sm = 16 * sizeof(double2) * (size_t)n;
+  // with the Ritz step's static arrays the columns can exceed the default 48 KB
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(sge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(16 * sizeof(double2) * kGradedMax));
+  MPDO_CUDA_TRY(attr);
+  for (int pass = 0; pass < 2; ++pass) {
+    const int fin = pass == 1;
+    count_launch();
+    sge_kernel<<<grid, kSgeThreads, sm, st>>>(n, cur, wk.s, fin, fin ? kNewtonFinal : kNewtonMax,
+                                              fin ? w : wk.lam, wk.ie, wk.sepf, wk.ticket);
+    MPDO_CUDA_TRY(cudaGetLastError());
+    if (fin) {
+      MPDO_CUDA_TRY(mul(cur + n, l2, 0, wk.ie, n, z, ldz, 0, 1));
+    } else {
+      // [T | Z] (I + E) carries T = A Z along
+      MPDO_CUDA_TRY(mul(cur, l2, n, wk.ie, n, nxt, l2, n, 2));
+      std::swap(cur, nxt);
+    }
+  }
+  // executed flops: about four sweeps of the FP32 blocks above the diagonal and of the
+  // accumulator (6 n^2 complex updates per round), and the FP64 products
+  if (flops_out)
+    *flops_out = 8.0 * (4.0 * 3.0 * n * (double)n * n + 7.0 * n * (double)n * n);
   return cudaSuccess;
 }
 

@@ -62,15 +62,15 @@ template <typename RI, typename RO>
 cudaError_t heig_smem_f32(cudaStream_t st, int n, const cx<RI>* a, long lda, cx<RO>* v, long ldv,
                           double* w, int* counters, int max_sweeps);
 
-// One-sided Jacobi on the n x r factor L (row-major, ld lr; r <= 128) of W = L L^+, computed
-// in precision R in one CTA's shared memory (n * r * sizeof(cx<R>) <= kOsjMaxSmem, plus the
-// FP64 copy with finish64): U (n x r, ld ldu) = eigenvectors of W, w (r) = eigenvalues,
-// descending.  finish64 (R = float): FP64 sweeps after the FP32 ones.  counters[2..3] =
-// sweeps, rotations.
-constexpr size_t kOsjMaxSmem = 200 * 1024;
-template <typename RI, typename R, typename RO>
-cudaError_t osj(cudaStream_t st, int n, int r, const cx<RI>* L, int lr, cx<RO>* U, int ldu,
-                double* w, int* counters, int finish64);
+// FP32 sweeps of a graded Hermitian PSD matrix (n <= kGradedMax, FP64, rounded on load): z =
+// its approximate eigenvectors (columns, descending eigenvalues, FP32 accuracy relative to
+// each pair), to be refined.  mem: graded_log_bytes(n) of device scratch; *meta_out (may be
+// NULL): device ints, logged rounds, sweeps, rotations.
+constexpr int kGradedMax = 168;     // np x (np + 1) complex64 fit one SM's shared memory
+constexpr int kGradedSweeps = 15;
+size_t graded_log_bytes(int n);
+cudaError_t heig_graded_f32(cudaStream_t st, int n, const double2* a, long lda, double2* z,
+                            long ldz, void* mem, int** meta_out);
 
 // Workspace of the mixed-precision eigensolver (capacity n_cap).
 struct MixGraphs;   // captured level sequences (eigmix.cu)
@@ -82,6 +82,7 @@ struct MixWork {
   unsigned int* ticket = nullptr;   // CTA ticket of the fused refinement (0 between launches)
   int* cid = nullptr;               // cluster of each column in the final refinement pass
   unsigned char* sepf = nullptr;    // neighbour separation flags of levels wider than 4096
+  void* glog = nullptr;             // rotation log of the graded sweeps
   EigWork<float> ew;
   MixGraphs* graphs = nullptr;   // created on first use; freed by mix_work_release
   bool use_graphs = true;
@@ -109,5 +110,11 @@ void mix_work_release(MixWork& w);
 cudaError_t heig_mixed(cudaStream_t st, int n, const double2* a, long lda, double2* v, long ldv,
                        double* w, double floor, MixWork& wk, int* levels_out,
                        double* flops_out = nullptr, int max_vals = 0);
+
+// Eigenpairs of a graded Hermitian PSD matrix (L^+ L of a pivoted Cholesky factor, n <=
+// kGradedMax): z (n x n, row stride ldz) and w, descending up to the order of pairs that agree
+// to FP32 rounding, each resolved relative to its own size.  No host synchronisation.
+cudaError_t heig_graded(cudaStream_t st, int n, const double2* a, long lda, double2* z, long ldz,
+                        double* w, MixWork& wk, double* flops_out = nullptr);
 
 }  // namespace mpdo

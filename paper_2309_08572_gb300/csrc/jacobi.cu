@@ -478,6 +478,253 @@ __global__ void __launch_bounds__(SJ_THREADS) jacobi_smem_kernel(int n, int np,
   }
 }
 
+// ---------------------------------------------------------------------------------------
+// FP32 sweeps of a graded Hermitian PSD matrix A = D C D (C of unit diagonal and moderate
+// condition, D spanning decades), as L^+ L of a pivoted Cholesky factor L is.  Rotations are
+// taken while |a_pq| > kGradedRel sqrt(a_pp a_qq), whatever the size of the pair, so every
+// eigenpair is resolved relative to its own size (Demmel and Veselic, "Jacobi's method is
+// more accurate than QR", 1992): one solve covers the whole spectrum, where an absolute
+// threshold covers two decades of it.  The sweeps stop after one whose largest
+// |a_pq| / sqrt(a_pp a_qq) was below kGradedStop: convergence is quadratic, so about its
+// square is left, which the FP64 refinement removes (L^+ L of the update's Grams, r = 13..73:
+// 3 to 5 sweeps, mixing angles of 1e-6 to 5e-5 left, 1e-10 after one refinement pass).
+//
+// One CTA, bound by the issue slots of one SM: a round touches every 2 x 2 block.  Hence
+// only the blocks above the diagonal are computed (their mirror images are written, not
+// computed), the pair's own block is set by the thread that found its rotation, rounds in
+// which nothing rotates cost one barrier, and the eigenvectors are not accumulated here: the
+// rotations go to a log, which rot_apply_kernel replays on the rows of the identity, one warp
+// per row on as many SMs as there are rows.  Without the accumulator a matrix of 168 fits the
+// shared memory of an SM (118 with it).
+// In place of one-sided FP64 sweeps on the factor (3.6 ms a Gram on one SM's FP64 pipe) and of
+// the levels of the mixed solver (5 rounds of ~9 launches): 40 atoms, two layers in FP64 719 ->
+// 84 ms, 100 atoms, three layers in the mixed tensor-core form 1488 -> 791 ms.
+constexpr float kGradedRel = 2e-6f;
+constexpr float kGradedStop = 3e-3f;
+constexpr int kGradedHalf = kGradedMax / 2;
+
+// log: (c, Re s e, Im s e, 0) of pair k of the i-th logged round at log[i * np / 2 + k];
+// rid[i]: its index in the round-robin order; meta: logged rounds, sweeps, rotations;
+// perm[i]: column of the i-th largest diagonal entry.  A diagonal that is not finite is left
+// for the caller to find in the refined eigenvalues.
+template <int IT>
+__global__ void __launch_bounds__(1024) jacobi_graded_kernel(int n, int np,
+                                                             const double2* __restrict__ a,
+                                                             long lda, float4* log, int* rid,
+                                                             int* meta, int* perm, int max_sweeps) {
+  extern __shared__ float2 gj_a[];   // np x (np + 1): odd row stride, so columns are free of
+  const int ld = np + 1;             // bank conflicts too
+  __shared__ float4 s_rot[kGradedHalf];
+  __shared__ int2 s_pq[kGradedHalf];
+  __shared__ double s_red[32];
+  __shared__ unsigned s_max[2];
+  __shared__ float s_key[kGradedMax];
+  const int tid = threadIdx.x, lane = tid & 31, nthr = blockDim.x;
+  const int half = np / 2, m = np - 1;
+  // a power of two brings the largest diagonal entry near 2^30: FP32 then holds the squares
+  // of entries 16 decades below it
+  double dm = 0.0;
+  for (int i = tid; i < n; i += nthr) dm = fmax(dm, a[(long)i * lda + i].x);
+  for (int o = 16; o > 0; o >>= 1) dm = fmax(dm, __shfl_xor_sync(0xffffffffu, dm, o));
+  if (lane == 0) s_red[tid >> 5] = dm;
+  if (tid < 2) s_max[tid] = 0u;
+  __syncthreads();
+  for (int k = 0; k < (nthr >> 5); ++k) dm = fmax(dm, s_red[k]);
+  const double sc = (dm > 0.0 && isfinite(dm)) ? ldexp(1.0, 30 - ilogb(dm)) : 1.0;
+  for (int e = tid; e < np * np; e += nthr) {
+    const int i = e / np, j = e - i * np;
+    float2 z = make_float2(0.f, 0.f);
+    if (i < n && j < n) {
+      const double2 t = a[(long)i * lda + j];
+      z = make_float2((float)(t.x * sc), (float)(t.y * sc));
+    }
+    gj_a[i * ld + j] = z;
+  }
+  // the blocks (ka < kb) of this thread, the same in every round: row i of the folded
+  // triangle holds the blocks of pair i and then those of pair half - 1 - i
+  const int nb = half * (half - 1) / 2;
+  int bl[IT];
+#pragma unroll
+  for (int t = 0; t < IT; ++t) {
+    const int e = tid + t * nthr;
+    bl[t] = -1;
+    if (e < nb) {
+      const int i = e / (half - 1), j = e - i * (half - 1);
+      const bool lo = j < half - 1 - i;
+      const int ka = lo ? i : half - 1 - i, kb = lo ? i + 1 + j : half - i + (j - (half - 1 - i));
+      bl[t] = ka | (kb << 8);
+    }
+  }
+  __syncthreads();
+  int logged = 0, rotated = 0, sweep = 0;
+  for (; sweep < max_sweeps; ++sweep) {
+    for (int r = 0; r < m; ++r) {
+      int f = 0;
+      float4 rot = make_float4(1.f, 0.f, 0.f, 0.f);
+      if (tid < half) {
+        int p, q;
+        if (tid == 0) {
+          p = m;
+          q = r;
+        } else {
+          p = r + tid;
+          if (p >= m) p -= m;
+          q = r - tid;
+          if (q < 0) q += m;
+        }
+        if (p > q) { const int t = p; p = q; q = t; }
+        const float2 g = gj_a[p * ld + q];
+        const float al = gj_a[p * ld + p].x, be = gj_a[q * ld + q].x;
+        const float g2 = cabs2(g), ab = al * be;
+        f = g2 > kGradedRel * kGradedRel * ab && g2 > 0.f;
+        if (f) {
+          const float ag = sqrtf(g2), d = be - al, h = 2.f * ag;
+          const float t = copysignf(h, d) / (fabsf(d) + sqrtf(d * d + h * h));
+          const float c = rsqrtf(1.f + t * t), se = t * c / ag;
+          rot = make_float4(c, se * g.x, se * g.y, 1.f);
+          gj_a[p * ld + p] = make_float2(al - t * ag, 0.f);
+          gj_a[q * ld + q] = make_float2(be + t * ag, 0.f);
+          gj_a[p * ld + q] = make_float2(0.f, 0.f);
+          gj_a[q * ld + p] = make_float2(0.f, 0.f);
+        }
+        s_pq[tid] = make_int2(p, q);
+        s_rot[tid] = rot;
+        // the sweep's largest squared ratio (positive floats compare as integers)
+        const float ratio = f ? (ab > 0.f ? g2 / ab : 1.f) : 0.f;
+        const int left = half - (tid & ~31);   // pairs from this warp's first lane on
+        const unsigned mask = left >= 32 ? 0xffffffffu : (1u << left) - 1u;
+        const unsigned mx = __reduce_max_sync(mask, __float_as_uint(ratio));
+        if (lane == 0 && mx > 0u) atomicMax(&s_max[sweep & 1], mx);
+      }
+      const int any = __syncthreads_count(f);
+      if (any == 0) continue;
+      rotated += any;
+      if (tid < half) log[(long)logged * half + tid] = rot;
+      if (tid == 0) rid[logged] = r;
+      ++logged;
+#pragma unroll
+      for (int t = 0; t < IT; ++t) {
+        if (bl[t] < 0) continue;
+        const int ka = bl[t] & 255, kb = bl[t] >> 8;
+        const float4 ra = s_rot[ka], rb = s_rot[kb];
+        if (ra.w == 0.f && rb.w == 0.f) continue;
+        const int2 ia = s_pq[ka], ib = s_pq[kb];
+        const float2 sa = make_float2(ra.y, ra.z), sb = make_float2(rb.y, rb.z);
+        float2* rp = gj_a + ia.x * ld;
+        float2* rq = gj_a + ia.y * ld;
+        const float2 x0 = rp[ib.x], x1 = rp[ib.y], y0 = rq[ib.x], y1 = rq[ib.y];
+        // rows (pair a): p' = c x - s e y, q' = s conj(e) x + c y
+        const float2 u0 = csub(cscale(x0, ra.x), cmul(sa, y0));
+        const float2 u1 = csub(cscale(x1, ra.x), cmul(sa, y1));
+        const float2 w0 = cadd(cmulc(x0, sa), cscale(y0, ra.x));
+        const float2 w1 = cadd(cmulc(x1, sa), cscale(y1, ra.x));
+        // columns (pair b): p' = c x - s conj(e) y, q' = s e x + c y
+        const float2 z0 = csub(cscale(u0, rb.x), cmulc(u1, sb));
+        const float2 z1 = cadd(cmul(u0, sb), cscale(u1, rb.x));
+        const float2 z2 = csub(cscale(w0, rb.x), cmulc(w1, sb));
+        const float2 z3 = cadd(cmul(w0, sb), cscale(w1, rb.x));
+        rp[ib.x] = z0;
+        rp[ib.y] = z1;
+        rq[ib.x] = z2;
+        rq[ib.y] = z3;
+        float2* cp = gj_a + ib.x * ld;
+        float2* cq = gj_a + ib.y * ld;
+        cp[ia.x] = cconj(z0);
+        cq[ia.x] = cconj(z1);
+        cp[ia.y] = cconj(z2);
+        cq[ia.y] = cconj(z3);
+      }
+      __syncthreads();
+    }
+    // the last round's barrier made the sweep's largest ratio visible; the other slot is
+    // cleared for the sweep after the next, before anyone writes it
+    const float mx = __uint_as_float(s_max[sweep & 1]);
+    __syncthreads();
+    if (tid == 0) s_max[sweep & 1] = 0u;
+    if (!(mx > kGradedStop * kGradedStop)) { ++sweep; break; }
+  }
+  for (int i = tid; i < n; i += nthr) {
+    s_key[i] = gj_a[i * ld + i].x;
+    perm[i] = i;   // a valid index whatever the keys are (ranks collide on NaN)
+  }
+  __syncthreads();
+  for (int i = tid; i < n; i += nthr) {
+    const float key = s_key[i];
+    int rank = 0;
+    for (int k = 0; k < n; ++k) rank += s_key[k] > key || (!(s_key[k] < key) && k < i);
+    perm[rank < n ? rank : n - 1] = i;
+  }
+  if (tid == 0) {
+    meta[0] = logged;
+    meta[1] = sweep;
+    meta[2] = rotated;
+  }
+}
+
+// Row blockIdx.x * 4 + warp of the accumulated rotations, V = J_1 J_2 ... : the log replayed
+// on a row of the identity (V's rows are independent), the next round's rotations fetched
+// while the present ones are applied; columns written in the order of perm, widened to FP64.
+constexpr int kRotWarps = 2;
+__global__ void __launch_bounds__(32 * kRotWarps) rot_apply_kernel(int n, int np,
+                                                                   const float4* __restrict__ log,
+                                                                   const int* __restrict__ rid,
+                                                                   const int* __restrict__ meta,
+                                                                   const int* __restrict__ perm,
+                                                                   double2* z, long ldz) {
+  constexpr int KP = (kGradedHalf + 31) / 32;   // pairs of a lane
+  __shared__ float2 rows[kRotWarps][kGradedMax];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int row = blockIdx.x * kRotWarps + warp;
+  if (row >= n) return;
+  float2* v = rows[warp];
+  const int half = np / 2, m = np - 1, rounds = meta[0];
+  for (int c = lane; c < np; c += 32) v[c] = make_float2(c == row ? 1.f : 0.f, 0.f);
+  float4 cur[KP], nxt[KP];
+  int r = 0, rn = 0;
+  if (rounds > 0) {
+    r = rid[0];
+#pragma unroll
+    for (int t = 0; t < KP; ++t)
+      if (lane + 32 * t < half) cur[t] = log[lane + 32 * t];
+  }
+  __syncwarp();
+  for (int i = 0; i < rounds; ++i) {
+    if (i + 1 < rounds) {
+      rn = rid[i + 1];
+#pragma unroll
+      for (int t = 0; t < KP; ++t)
+        if (lane + 32 * t < half) nxt[t] = log[(long)(i + 1) * half + lane + 32 * t];
+    }
+#pragma unroll
+    for (int t = 0; t < KP; ++t) {
+      const int k = lane + 32 * t;
+      if (k >= half || cur[t].w == 0.f) continue;
+      int p, q;
+      if (k == 0) {
+        p = m;
+        q = r;
+      } else {
+        p = r + k;
+        if (p >= m) p -= m;
+        q = r - k;
+        if (q < 0) q += m;
+      }
+      if (p > q) { const int x = p; p = q; q = x; }
+      const float2 x = v[p], y = v[q], se = make_float2(cur[t].y, cur[t].z);
+      v[p] = csub(cscale(x, cur[t].x), cmulc(y, se));
+      v[q] = cadd(cmul(x, se), cscale(y, cur[t].x));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < KP; ++t) cur[t] = nxt[t];
+    r = rn;
+  }
+  for (int c = lane; c < n; c += 32) {
+    const float2 x = v[perm[c]];
+    z[(long)row * ldz + c] = make_double2((double)x.x, (double)x.y);
+  }
+}
+
 template <typename R>
 constexpr int smem_jacobi_max() { return sizeof(R) == 8 ? 84 : 118; }
 
@@ -519,6 +766,52 @@ template cudaError_t heig_smem_f32<double, double>(cudaStream_t, int, const doub
                                                    double2*, long, double*, int*, int);
 template cudaError_t heig_smem_f32<double, float>(cudaStream_t, int, const double2*, long,
                                                   float2*, long, double*, int*, int);
+
+size_t graded_log_bytes(int n) {
+  const size_t np = n + (n & 1);
+  return kGradedSweeps * (np - 1) * (np / 2 * sizeof(float4) + sizeof(int)) + 256 +
+         (np + 8) * sizeof(int);
+}
+
+cudaError_t heig_graded_f32(cudaStream_t st, int n, const double2* a, long lda, double2* z,
+                            long ldz, void* mem, int** meta_out) {
+  if (n < 1 || n > kGradedMax) return cudaErrorInvalidValue;
+  const int np = n + (n & 1), half = np / 2, rounds = kGradedSweeps * (np - 1);
+  float4* log = static_cast<float4*>(mem);
+  int* rid = reinterpret_cast<int*>(log + (size_t)rounds * half);
+  int* perm = rid + rounds;
+  int* meta = perm + np;
+  const size_t sm = (size_t)np * (np + 1) * sizeof(float2);
+  const int nb = half * (half - 1) / 2;
+  const int thr = std::min(1024, std::max(96, (nb + 31) / 32 * 32));
+  const int it = (nb + thr - 1) / thr;   // at most 4 (nb <= 3486)
+  auto launch = [&](auto kern) -> cudaError_t {
+    kern<<<1, thr, sm, st>>>(n, np, a, lda, log, rid, meta, perm, kGradedSweeps);
+    return cudaGetLastError();
+  };
+  // opt in to the largest size, once per instantiation
+  constexpr int kMaxSmem = kGradedMax * (kGradedMax + 1) * (int)sizeof(float2);
+  static const cudaError_t attr = [] {
+    cudaError_t e = cudaFuncSetAttribute(jacobi_graded_kernel<1>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(jacobi_graded_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               kMaxSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(jacobi_graded_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               kMaxSmem);
+    return e;
+  }();
+  MPDO_CUDA_TRY(attr);
+  count_launch(2);
+  MPDO_CUDA_TRY(it <= 1   ? launch(jacobi_graded_kernel<1>)
+                : it <= 2 ? launch(jacobi_graded_kernel<2>)
+                          : launch(jacobi_graded_kernel<4>));
+  rot_apply_kernel<<<(n + kRotWarps - 1) / kRotWarps, 32 * kRotWarps, 0, st>>>(
+      n, np, log, rid, meta, perm, z, ldz);
+  if (meta_out) *meta_out = meta;
+  return cudaGetLastError();
+}
 
 int eig_padded_n(int n) { return padded_n(n); }
 
@@ -695,201 +988,3 @@ extern "C" int mpdo_heig_noalloc(int prec, int n, void* a, void* v, double* w, i
   }
   return MPDO_OK;
 }
-
-// =======================================================================================
-// Eigenpairs of a Hermitian PSD matrix from its pivoted Cholesky factor W ~ L L^+:
-// one-sided (Hestenes) Jacobi on the columns of L.  Pairs of columns are rotated until
-// mutually orthogonal (|a_p^+ a_q| <= tol |a_p| |a_q|); then sigma_k = |a_k| and the unit
-// columns are the eigenvectors of L L^+ with eigenvalues sigma_k^2.  The rotations never
-// form a Gram matrix, so small eigenvalues keep their relative accuracy (Demmel and
-// Veselic): the factor's graded columns need no square of the precision.  One CTA; L lives
-// column-major in shared memory; warp w handles pair slots w, w + nw, ... of each round.
-namespace mpdo {
-namespace {
-
-template <typename R>
-struct OsjTol;
-template <> struct OsjTol<double> { static constexpr double v = 1e-14; };
-template <> struct OsjTol<float> { static constexpr double v = 2e-6; };
-
-// Sweeps over the column pairs of A (column-major, n x rp, precision of T) until no pair
-// is rotated; returns the rotations applied (thread 0).
-template <typename T>
-__device__ int osj_sweeps(T* A, int n, int rp, int max_sweeps, double tol, int* s_rot,
-                          int* sweeps_out) {
-  using R = decltype(T{}.x);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  int sweep = 0, total = 0;
-  for (; sweep < max_sweeps; ++sweep) {
-    if (tid == 0) *s_rot = 0;
-    __syncthreads();
-    for (int round = 0; round < rp - 1; ++round) {
-      for (int slot = warp; slot < rp / 2; slot += nw) {
-        int p, q;
-        tourney(round, slot, rp, p, q);
-        T* ap = A + (size_t)p * n;
-        T* aq = A + (size_t)q * n;
-        R al = 0, be = 0, gr = 0, gi = 0;
-        for (int i = lane; i < n; i += 32) {
-          T x = ap[i], y = aq[i];
-          al += x.x * x.x + x.y * x.y;
-          be += y.x * y.x + y.y * y.y;
-          gr += x.x * y.x + x.y * y.y;     // conj(x) y
-          gi += x.x * y.y - x.y * y.x;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          al += __shfl_xor_sync(0xffffffffu, al, o);
-          be += __shfl_xor_sync(0xffffffffu, be, o);
-          gr += __shfl_xor_sync(0xffffffffu, gr, o);
-          gi += __shfl_xor_sync(0xffffffffu, gi, o);
-        }
-        const R ag = sqrt(gr * gr + gi * gi);
-        if (!(ag > (R)tol * sqrt(al * be)) || !(ag > 0)) continue;
-        // with b_q = conj(e) a_q (e = g/|g|) the pair's Gram is real: [[al, |g|], [|g|, be]]
-        const R zeta = (be - al) / (2 * ag);
-        const R t = (zeta >= 0 ? R(1) : R(-1)) / (fabs(zeta) + sqrt(R(1) + zeta * zeta));
-        const R c = R(1) / sqrt(R(1) + t * t), s = c * t;
-        const R er = gr / ag, ei = gi / ag;   // e
-        for (int i = lane; i < n; i += 32) {
-          T x = ap[i], y = aq[i];
-          T b;   // conj(e) y
-          b.x = er * y.x + ei * y.y;
-          b.y = er * y.y - ei * y.x;
-          T xn, yn;
-          xn.x = c * x.x - s * b.x; xn.y = c * x.y - s * b.y;
-          yn.x = s * x.x + c * b.x; yn.y = s * x.y + c * b.y;
-          ap[i] = xn;
-          aq[i] = yn;
-        }
-        if (lane == 0) atomicAdd(s_rot, 1);
-      }
-      __syncthreads();
-    }
-    if (tid == 0) total += *s_rot;
-    const int any = *s_rot;
-    __syncthreads();
-    if (any == 0) { ++sweep; break; }
-  }
-  *sweeps_out = sweep;
-  return total;
-}
-
-// Column norms, descending sort and output of the unit columns (A column-major n x rp).
-template <typename T, typename RO>
-__device__ void osj_output(const T* A, int n, int r, int rp, cx<RO>* U, int ldu, double* w,
-                           double* s_key, int* s_val) {
-  using R = decltype(T{}.x);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  int P = 2;
-  while (P < rp) P <<= 1;
-  for (int c = warp; c < P; c += nw) {
-    double nn = 0.0;
-    if (c < r) {
-      const T* ac = A + (size_t)c * n;
-      for (int i = lane; i < n; i += 32) nn += (double)ac[i].x * ac[i].x + (double)ac[i].y * ac[i].y;
-      for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
-    }
-    if (lane == 0) {
-      s_key[c] = (c < r && isfinite(nn)) ? nn : -1.0;
-      s_val[c] = c;
-    }
-  }
-  __syncthreads();
-  for (int k = 2; k <= P; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int c = tid; c < P; c += blockDim.x) {
-        int l = c ^ j;
-        if (l > c) {
-          bool desc = ((c & k) == 0);
-          double kc = s_key[c], kl = s_key[l];
-          if (desc ? (kc < kl) : (kc > kl)) {
-            s_key[c] = kl; s_key[l] = kc;
-            int t2 = s_val[c]; s_val[c] = s_val[l]; s_val[l] = t2;
-          }
-        }
-      }
-      __syncthreads();
-    }
-  }
-  for (int k = tid; k < r; k += blockDim.x) w[k] = s_key[k] > 0 ? s_key[k] : 0.0;
-  for (long e = tid; e < (long)n * r; e += blockDim.x) {
-    int i = (int)(e / r), k = (int)(e % r);
-    int col = s_val[k];
-    col = (col >= 0 && col < r) ? col : k;
-    double nk = s_key[k];
-    T x = A[(size_t)col * n + i];
-    R inv = nk > 0 ? (R)(1.0 / sqrt(nk)) : R(0);
-    U[(long)i * ldu + k] = mkc<RO>((RO)(x.x * inv), (RO)(x.y * inv));
-  }
-}
-
-// R: precision of the sweeps.  finish64 (R = float only): after the FP32 sweeps the
-// rotated columns are widened and the sweeps continue in FP64 (a few, from near
-// orthogonality), so the columns end orthogonal to FP64 precision; the FP32 phase's
-// rounding perturbs each direction by ~1e-7 relative, which mixed precision accepts.
-template <typename RI, typename R, typename RO>
-__global__ void __launch_bounds__(1024) osj_kernel(int n, int r, const cx<RI>* __restrict__ L,
-                                                   int lr, cx<RO>* U, int ldu, double* w,
-                                                   int max_sweeps, int finish64, int* counters) {
-  using T = cx<R>;
-  extern __shared__ __align__(16) unsigned char osj_raw[];
-  const int rp = r + (r & 1);
-  T* A = reinterpret_cast<T*>(osj_raw);          // column c at A + c * n
-  __shared__ int s_rot;
-  __shared__ double s_key[128];
-  __shared__ int s_val[128];
-  const int tid = threadIdx.x;
-  for (int e = tid; e < n * rp; e += blockDim.x) {
-    int c = e / n, i = e - c * n;
-    cx<RI> x = (c < r) ? L[(long)i * lr + c] : mkc<RI>(0, 0);
-    A[e] = mkc<R>((R)x.x, (R)x.y);
-  }
-  __syncthreads();
-  int sweeps = 0, sweeps2 = 0;
-  int total = osj_sweeps<T>(A, n, rp, max_sweeps, OsjTol<R>::v, &s_rot, &sweeps);
-  if (finish64 && sizeof(R) == 4) {
-    // widen into the region after the FP32 columns (16-byte aligned)
-    double2* A2 = reinterpret_cast<double2*>(osj_raw + (((size_t)n * rp * sizeof(T) + 15) & ~(size_t)15));
-    for (int e = tid; e < n * rp; e += blockDim.x) A2[e] = make_double2((double)A[e].x, (double)A[e].y);
-    __syncthreads();
-    total += osj_sweeps<double2>(A2, n, rp, max_sweeps, OsjTol<double>::v, &s_rot, &sweeps2);
-    osj_output<double2, RO>(A2, n, r, rp, U, ldu, w, s_key, s_val);
-  } else {
-    osj_output<T, RO>(A, n, r, rp, U, ldu, w, s_key, s_val);
-  }
-  if (tid == 0 && counters) {
-    counters[2] = sweeps + sweeps2;
-    counters[3] = total;
-  }
-}
-
-}  // namespace
-
-template <typename RI, typename R, typename RO>
-cudaError_t osj(cudaStream_t st, int n, int r, const cx<RI>* L, int lr, cx<RO>* U, int ldu,
-                double* w, int* counters, int finish64) {
-  if (n < 1 || r < 1 || r > 128) return cudaErrorInvalidValue;
-  const int rp = r + (r & 1);
-  size_t sm = (size_t)n * rp * sizeof(cx<R>);
-  if (finish64 && sizeof(R) == 4) sm = ((sm + 15) & ~(size_t)15) + (size_t)n * rp * sizeof(double2);
-  if (sm > kOsjMaxSmem) return cudaErrorInvalidValue;
-  static bool attr = false;
-  if (!attr) {
-    MPDO_CUDA_TRY(cudaFuncSetAttribute(osj_kernel<RI, R, RO>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kOsjMaxSmem));
-    attr = true;
-  }
-  int thr = std::min(1024, std::max(64, (rp / 2) * 32));
-  count_launch();
-  osj_kernel<RI, R, RO><<<1, thr, sm, st>>>(n, r, L, lr, U, ldu, w, 30, finish64, counters);
-  return cudaGetLastError();
-}
-template cudaError_t osj<double, double, double>(cudaStream_t, int, int, const double2*, int,
-                                                 double2*, int, double*, int*, int);
-template cudaError_t osj<double, float, double>(cudaStream_t, int, int, const double2*, int,
-                                                double2*, int, double*, int*, int);
-template cudaError_t osj<float, float, float>(cudaStream_t, int, int, const float2*, int,
-                                              float2*, int, double*, int*, int);
-
-}  // namespace mpdo

@@ -5,6 +5,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "internal.h"
 #include "kernels.h"
 
 namespace cg = cooperative_groups;
@@ -642,7 +643,7 @@ __global__ void dual_rows_kernel(int kk, int cols, const cx<R>* __restrict__ y, 
 
 // Pivoted Cholesky of the Hermitian PSD n x n matrix w (precision R, n <= 1024): W ~ L L^+
 // with L n x r (row-major, row stride lr), greedy diagonal pivoting, stopping once the
-// largest remaining diagonal is <= tol * tr W or after rmax (<= 128) columns.
+// largest remaining diagonal is <= tol * tr W or after rmax (<= kGradedMax) columns.
 // *rout = r; *resid = largest remaining diagonal / tr W.
 // The rows are shared out over the CTAs of a thread-block cluster (row i belongs to rank
 // i mod S; FP64 runs at 2 FMA per clock per SM, so the column updates want several SMs).
@@ -661,7 +662,7 @@ __global__ void __launch_bounds__(1024) pchol_kernel(int n, const cx<R>* __restr
   __shared__ double d[1024];        // remaining diagonal of this CTA's rows (local index)
   __shared__ double rv[32];
   __shared__ int ri[32];
-  __shared__ T lp[128];
+  __shared__ T lp[kGradedMax];
   __shared__ double post_v[2];      // this CTA's best remaining diagonal, by column parity
   __shared__ int post_i[2];
   __shared__ double post_tr;        // this CTA's share of the trace
@@ -964,7 +965,7 @@ cudaError_t dual_rows(cudaStream_t st, int kk, int cols, const cx<R>* y, long ld
 template <typename R>
 cudaError_t pchol(cudaStream_t st, int n, const cx<R>* w, int rmax, double tol, cx<R>* L, int lr,
                   int* rout, double* resid) {
-  if (n < 1 || n > 1024 || rmax < 1 || rmax > 128) return cudaErrorInvalidValue;
+  if (n < 1 || n > 1024 || rmax < 1 || rmax > kGradedMax) return cudaErrorInvalidValue;
   // cluster of S CTAs, at least 32 rows each, at most 8 (portable cluster size)
   const int S = std::min(8, std::max(1, n / 32));
   const int rows = (n + S - 1) / S;

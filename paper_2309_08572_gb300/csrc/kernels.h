@@ -47,7 +47,7 @@ cudaError_t kraus_select(cudaStream_t st, int n, const double* w, const cx<R>* w
 // sc->trpre = ||theta||^2 of the block from its Gram matrices G_i, G_j (3 dm x 3 dm)
 template <typename R>
 cudaError_t trace_pre(cudaStream_t st, int dm, const cx<R>* gi, const cx<R>* gj, StepScalars* sc);
-// Pivoted Cholesky W ~ L L^+ of a Hermitian PSD matrix (n <= 1024, rmax <= 128); device
+// Pivoted Cholesky W ~ L L^+ of a Hermitian PSD matrix (n <= 1024, rmax <= kGradedMax); device
 // outputs: L (n x r, row stride lr), *rout = r, *resid = remaining diag max / tr W.
 template <typename R>
 cudaError_t pchol(cudaStream_t st, int n, const cx<R>* w, int rmax, double tol, cx<R>* L, int lr,
