@@ -578,9 +578,12 @@ __global__ void __launch_bounds__(1024) jacobi_graded_kernel(int n, int np,
         const float g2 = cabs2(g), ab = al * be;
         f = g2 > kGradedRel * kGradedRel * ab && g2 > 0.f;
         if (f) {
-          const float ag = sqrtf(g2), d = be - al, h = 2.f * ag;
-          const float t = copysignf(h, d) / (fabsf(d) + sqrtf(d * d + h * h));
-          const float c = rsqrtf(1.f + t * t), se = t * c / ag;
+          // approximate reciprocals and roots (a few ulp): their error is that of the
+          // accumulated rotations' rounding, which the refinement removes
+          const float rg = rsqrtf(g2), ag = g2 * rg, d = be - al, h = 2.f * ag;
+          const float s2 = d * d + h * h;
+          const float t = __fdividef(copysignf(h, d), fabsf(d) + s2 * rsqrtf(s2));
+          const float c = rsqrtf(fmaf(t, t, 1.f)), se = t * c * rg;
           rot = make_float4(c, se * g.x, se * g.y, 1.f);
           gj_a[p * ld + p] = make_float2(al - t * ag, 0.f);
           gj_a[q * ld + q] = make_float2(be + t * ag, 0.f);
@@ -590,7 +593,7 @@ __global__ void __launch_bounds__(1024) jacobi_graded_kernel(int n, int np,
         s_pq[tid] = make_int2(p, q);
         s_rot[tid] = rot;
         // the sweep's largest squared ratio (positive floats compare as integers)
-        const float ratio = f ? (ab > 0.f ? g2 / ab : 1.f) : 0.f;
+        const float ratio = f ? (ab > 0.f ? __fdividef(g2, ab) : 1.f) : 0.f;
         const int left = half - (tid & ~31);   // pairs from this warp's first lane on
         const unsigned mask = left >= 32 ? 0xffffffffu : (1u << left) - 1u;
         const unsigned mx = __reduce_max_sync(mask, __float_as_uint(ratio));
@@ -661,64 +664,75 @@ __global__ void __launch_bounds__(1024) jacobi_graded_kernel(int n, int np,
   }
 }
 
-// Row blockIdx.x * 4 + warp of the accumulated rotations, V = J_1 J_2 ... : the log replayed
-// on a row of the identity (V's rows are independent), the next round's rotations fetched
-// while the present ones are applied; columns written in the order of perm, widened to FP64.
-constexpr int kRotWarps = 2;
+// Rows of the accumulated rotations, V = J_1 J_2 ... : the log replayed on rows of the identity
+// (V's rows are independent), one warp per row, kRotWarps rows of a CTA sharing the log, which
+// comes into shared memory kRotChunk rounds at a time, the next chunk in flight while the
+// present one is applied.  Bound by the latency of a round (two columns read, rotated and
+// written back): 37 us at n = 60, where fetching each round's rotations one round ahead from L2
+// took 96 us.  Columns are written in the order of perm, widened to FP64.
+constexpr int kRotWarps = 4;
+constexpr int kRotChunk = 16;
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+template <int KP>   // pairs of a lane
 __global__ void __launch_bounds__(32 * kRotWarps) rot_apply_kernel(int n, int np,
                                                                    const float4* __restrict__ log,
                                                                    const int* __restrict__ rid,
                                                                    const int* __restrict__ meta,
                                                                    const int* __restrict__ perm,
                                                                    double2* z, long ldz) {
-  constexpr int KP = (kGradedHalf + 31) / 32;   // pairs of a lane
   __shared__ float2 rows[kRotWarps][kGradedMax];
+  __shared__ __align__(16) float4 buf[2][kRotChunk][32 * KP];
+  __shared__ int ids[2][kRotChunk];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int row = blockIdx.x * kRotWarps + warp;
-  if (row >= n) return;
+  const bool live = row < n;
   float2* v = rows[warp];
   const int half = np / 2, m = np - 1, rounds = meta[0];
   for (int c = lane; c < np; c += 32) v[c] = make_float2(c == row ? 1.f : 0.f, 0.f);
-  float4 cur[KP], nxt[KP];
-  int r = 0, rn = 0;
-  if (rounds > 0) {
-    r = rid[0];
-#pragma unroll
-    for (int t = 0; t < KP; ++t)
-      if (lane + 32 * t < half) cur[t] = log[lane + 32 * t];
-  }
-  __syncwarp();
-  for (int i = 0; i < rounds; ++i) {
-    if (i + 1 < rounds) {
-      rn = rid[i + 1];
-#pragma unroll
-      for (int t = 0; t < KP; ++t)
-        if (lane + 32 * t < half) nxt[t] = log[(long)(i + 1) * half + lane + 32 * t];
+  auto fetch = [&](int i0, int b) {
+    const int cnt = min(kRotChunk, rounds - i0);
+    for (int e = threadIdx.x; e < cnt * half; e += 32 * kRotWarps) {
+      const int i = e / half, k = e - i * half;
+      cp_async16(&buf[b][i][k], &log[(long)(i0 + i) * half + k]);
     }
+    if (threadIdx.x < cnt) ids[b][threadIdx.x] = rid[i0 + threadIdx.x];
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (rounds > 0) fetch(0, 0);
+  for (int i0 = 0, b = 0; i0 < rounds; i0 += kRotChunk, b ^= 1) {
+    if (i0 + kRotChunk < rounds) {
+      fetch(i0 + kRotChunk, b ^ 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    const int cnt = min(kRotChunk, rounds - i0);
+    for (int i = 0; live && i < cnt; ++i) {
+      const int r = ids[b][i];
 #pragma unroll
-    for (int t = 0; t < KP; ++t) {
-      const int k = lane + 32 * t;
-      if (k >= half || cur[t].w == 0.f) continue;
-      int p, q;
-      if (k == 0) {
-        p = m;
-        q = r;
-      } else {
-        p = r + k;
-        if (p >= m) p -= m;
-        q = r - k;
+      for (int t = 0; t < KP; ++t) {
+        const int k = lane + 32 * t;
+        if (k >= half) continue;
+        const float4 rot = buf[b][i][k];
+        int p = k == 0 ? m : r + k, q = k == 0 ? r : r - k;
+        if (k && p >= m) p -= m;
         if (q < 0) q += m;
+        if (p > q) { const int x = p; p = q; q = x; }
+        const float2 x = v[p], y = v[q], se = make_float2(rot.y, rot.z);
+        v[p] = csub(cscale(x, rot.x), cmulc(y, se));
+        v[q] = cadd(cmul(x, se), cscale(y, rot.x));
       }
-      if (p > q) { const int x = p; p = q; q = x; }
-      const float2 x = v[p], y = v[q], se = make_float2(cur[t].y, cur[t].z);
-      v[p] = csub(cscale(x, cur[t].x), cmulc(y, se));
-      v[q] = cadd(cmul(x, se), cscale(y, cur[t].x));
+      __syncwarp();
     }
-    __syncwarp();
-#pragma unroll
-    for (int t = 0; t < KP; ++t) cur[t] = nxt[t];
-    r = rn;
+    __syncthreads();   // the chunk is free for the fetch after the next
   }
+  if (!live) return;
   for (int c = lane; c < n; c += 32) {
     const float2 x = v[perm[c]];
     z[(long)row * ldz + c] = make_double2((double)x.x, (double)x.y);
@@ -807,8 +821,13 @@ cudaError_t heig_graded_f32(cudaStream_t st, int n, const double2* a, long lda, 
   MPDO_CUDA_TRY(it <= 1   ? launch(jacobi_graded_kernel<1>)
                 : it <= 2 ? launch(jacobi_graded_kernel<2>)
                           : launch(jacobi_graded_kernel<4>));
-  rot_apply_kernel<<<(n + kRotWarps - 1) / kRotWarps, 32 * kRotWarps, 0, st>>>(
-      n, np, log, rid, meta, perm, z, ldz);
+  auto apply = [&](auto kern) {
+    kern<<<(n + kRotWarps - 1) / kRotWarps, 32 * kRotWarps, 0, st>>>(n, np, log, rid, meta, perm, z,
+                                                                   ldz);
+  };
+  if (half <= 32) apply(rot_apply_kernel<1>);
+  else if (half <= 64) apply(rot_apply_kernel<2>);
+  else apply(rot_apply_kernel<3>);
   if (meta_out) *meta_out = meta;
   return cudaGetLastError();
 }
