@@ -645,124 +645,176 @@ __global__ void dual_rows_kernel(int kk, int cols, const cx<R>* __restrict__ y, 
 // with L n x r (row-major, row stride lr), greedy diagonal pivoting, stopping once the
 // largest remaining diagonal is <= tol * tr W or after rmax (<= kGradedMax) columns.
 // *rout = r; *resid = largest remaining diagonal / tr W.
-// The rows are shared out over the CTAs of a thread-block cluster (row i belongs to rank
-// i mod S; FP64 runs at 2 FMA per clock per SM, so the column updates want several SMs).
-// Per column, one cluster barrier: each CTA posts its best remaining diagonal in shared
-// memory (two slots, alternating by column, so a slot is rewritten only after every CTA
-// has passed the next barrier), then every CTA reads all posts through distributed shared
-// memory and takes the same pivot.  Sums and the pivot choice follow rank order, so the
+//
+// The columns depend on one another, so the factor is bound by the latency of a column: a
+// barrier or two and a chain of FP64 operations, at ~64 clocks each on this chip; beyond ~64 rows
+// its dot products also want the FP64 pipes (2 FMA per clock) of several SMs.  So the rows go to
+// the CTAs of a thread-block cluster of up to 16 (row i belongs to rank i mod S), or to one CTA
+// without any cluster barrier; four lanes to a row, each row's part of L -- and of W, where it
+// fits -- in its CTA's shared memory.  Per column: every CTA stores its best remaining diagonal
+// into all CTAs' shared memory, one cluster barrier, every warp takes the same pivot from its
+// own CTA's copies, the pivot's row comes from its owner's shared memory, and the lanes of a row
+// split its dot product while one further warp takes the pivot's square root; the remaining
+// diagonals follow from the unscaled column, beside its scaling.  Posts alternate between two
+// slots by column parity, so a slot is rewritten only after every CTA has passed the next
+// barrier; candidates are compared as integers (non-negative doubles order alike), which keeps
+// the FP64 pipe to the dot products.  Sums and the pivot choice follow a fixed order, so the
 // factor does not depend on scheduling.
-template <typename R>
-__global__ void __launch_bounds__(1024) pchol_kernel(int n, const cx<R>* __restrict__ w,
-                                                     int rmax, double tol, cx<R>* L, int lr,
-                                                     int* rout, double* resid) {
+constexpr int kPcLanes = 4;              // lanes of a row
+constexpr int kPcWarps = 8;              // row warps of a CTA, at most 64 rows
+constexpr int kPcCtas = 16;
+// largest key of the warp (bits of a non-negative double, or -1) and the smallest index with it
+__device__ __forceinline__ void warp_best(long long& key, int& idx) {
+  const int hi = (int)(key >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned lo = hi == mh ? (unsigned)key : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
+  const int x = hi == mh && lo == ml ? idx : 0x7fffffff;
+  idx = __reduce_min_sync(0xffffffffu, x);
+  key = ((long long)mh << 32) | ml;
+}
+template <typename R, bool CLUSTER>
+__global__ void __launch_bounds__(32 * (kPcWarps + 1)) pchol_kernel(
+    int n, const cx<R>* __restrict__ w, int rmax, double tol, cx<R>* L, int lr, int* rout,
+    double* resid, int* piv, int w_rows) {
   using T = cx<R>;
   cg::cluster_group cluster = cg::this_cluster();
-  const int S = (int)cluster.num_blocks(), c = (int)cluster.block_rank();
-  __shared__ double d[1024];        // remaining diagonal of this CTA's rows (local index)
-  __shared__ double rv[32];
-  __shared__ int ri[32];
+  const int S = CLUSTER ? (int)cluster.num_blocks() : 1, c = CLUSTER ? (int)cluster.block_rank() : 0;
+  auto barrier = [&]() {
+    if constexpr (CLUSTER) cluster.sync(); else __syncthreads();
+  };
+  // x of the CTA of that rank
+  auto remote = [&](auto* x, int rank) {
+    if constexpr (CLUSTER) return cluster.map_shared_rank(x, rank); else return x;
+  };
+  extern __shared__ __align__(16) unsigned char pc_raw[];
+  T* Ls = reinterpret_cast<T*>(pc_raw);          // own rows of L, stride rmax
+  const int nlm = (n + S - 1) / S;
+  T* Ws = Ls + (size_t)nlm * rmax;               // own rows of W, stride n (w_rows)
   __shared__ T lp[kGradedMax];
-  __shared__ double post_v[2];      // this CTA's best remaining diagonal, by column parity
-  __shared__ int post_i[2];
-  __shared__ double post_tr;        // this CTA's share of the trace
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-  const int nloc = (n - c + S - 1) / S;   // rows c, c + S, ...
-  double tp = 0.0;
-  for (int li = tid; li < nloc; li += blockDim.x) {
-    const int i = c + li * S;
-    double v = (double)w[(long)i * n + i].x;
-    d[li] = v > 0 ? v : 0.0;
-    tp += d[li];
+  __shared__ long long post_v[2][kPcCtas], s_v[2][kPcWarps];   // best remaining diagonals, as bits
+  __shared__ int post_i[2][kPcCtas], s_i[2][kPcWarps];
+  __shared__ double s_tr[kPcWarps], post_tr, s_inv, s_inv2, s_dp;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = (blockDim.x >> 5) - 1;
+  const int l4 = lane & (kPcLanes - 1), li = tid / kPcLanes, i = c + li * S;
+  const bool own = warp < nw && li < nlm && i < n;
+  if (w_rows)
+    for (int e = tid; e < nlm * n; e += blockDim.x) {
+      const int row = c + (e / n) * S;
+      if (row < n) Ws[e] = w[(long)row * n + e % n];
+    }
+  double d = 0.0;
+  if (own) {
+    d = (double)w[(long)i * n + i].x;
+    if (!(d > 0.0)) d = 0.0;
   }
+  double tp = l4 == 0 ? d : 0.0;
   for (int o = 16; o > 0; o >>= 1) tp += __shfl_xor_sync(0xffffffffu, tp, o);
-  if (lane == 0) rv[wid] = tp;
+  if (lane == 0 && warp < nw) s_tr[warp] = tp;
   __syncthreads();
   if (tid == 0) {
     double t = 0;
-    for (int k = 0; k < nw; ++k) t += rv[k];
+    for (int k = 0; k < nw; ++k) t += s_tr[k];
     post_tr = t;
   }
-  cluster.sync();
+  barrier();
   double tr = 0.0;
-  for (int q = 0; q < S; ++q) tr += *cluster.map_shared_rank(&post_tr, q);
-  int r = 0;
+  for (int q = 0; q < S; ++q) tr += *remote(&post_tr, q);
+  const double thr = tol * tr;
+  // the best remaining diagonal of all rows: this CTA's into every CTA's slot, the barrier (after
+  // which rows of L written before it are visible too), and the best of the posts
+  auto pivot = [&](int par, int& p) {
+    long long bv = own ? __double_as_longlong(d) : -1;
+    int bi = own ? i : 0x7fffffff;
+    warp_best(bv, bi);
+    if (lane == 0 && warp < nw) {
+      s_v[par][warp] = bv;
+      s_i[par][warp] = bi;
+    }
+    __syncthreads();
+    if (!CLUSTER || warp == 0) {
+      bv = lane < nw ? s_v[par][lane] : -1;
+      bi = lane < nw ? s_i[par][lane] : 0x7fffffff;
+      warp_best(bv, bi);
+    }
+    if constexpr (CLUSTER) {
+      if (warp == 0 && lane < S) {
+        cluster.map_shared_rank(&post_v[par][0], lane)[c] = bv;
+        cluster.map_shared_rank(&post_i[par][0], lane)[c] = bi;
+      }
+      cluster.sync();
+      bv = lane < S ? post_v[par][lane] : -1;
+      bi = lane < S ? post_i[par][lane] : 0x7fffffff;
+      warp_best(bv, bi);
+    }
+    p = bi;
+    return bv < 0 ? -1.0 : __longlong_as_double(bv);
+  };
+  int r = 0, p = -1;
   double last = 0.0;
   for (int j = 0; j < rmax; ++j) {
-    const int par = j & 1;
-    double bv = -1.0;
-    int bi = -1;
-    for (int li = tid; li < nloc; li += blockDim.x)
-      if (d[li] > bv) { bv = d[li]; bi = c + li * S; }
-    for (int o = 16; o > 0; o >>= 1) {
-      double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ov > bv || (ov == bv && oi >= 0 && (bi < 0 || oi < bi))) { bv = ov; bi = oi; }
-    }
-    if (lane == 0) { rv[wid] = bv; ri[wid] = bi; }
-    __syncthreads();
-    if (tid == 0) {
-      double b = -1.0;
-      int p = -1;
-      for (int k = 0; k < nw; ++k)
-        if (rv[k] > b || (rv[k] == b && ri[k] >= 0 && (p < 0 || ri[k] < p))) { b = rv[k]; p = ri[k]; }
-      post_v[par] = b;
-      post_i[par] = p;
-    }
-    cluster.sync();   // posts of column j complete; columns < j of L visible
-    double dp = -1.0;
-    int p = -1;
-    for (int q = 0; q < S; ++q) {
-      const double v = cluster.map_shared_rank(post_v, q)[par];
-      const int i = cluster.map_shared_rank(post_i, q)[par];
-      if (v > dp || (v == dp && i >= 0 && (p < 0 || i < p))) { dp = v; p = i; }
-    }
+    const double dp = pivot(j & 1, p);
     last = dp;
-    if (!(dp > tol * tr) || p < 0) break;
-    for (int k = tid; k < j; k += blockDim.x) lp[k] = __ldcg(&L[(long)p * lr + k]);
-    __syncthreads();
-    const R inv = (R)(1.0 / sqrt(dp));
-    for (int li = tid; li < nloc; li += blockDim.x) {
-      const int i = c + li * S;
-      T acc = w[(long)i * n + p];
-      const T* lrow = L + (long)i * lr;
-      for (int k = 0; k < j; ++k) {
-        T a = lrow[k], b = lp[k];
-        // acc -= a * conj(b)
-        acc.x -= a.x * b.x + a.y * b.y;
-        acc.y -= a.y * b.x - a.x * b.y;
+    if (!(dp > thr)) break;
+    if (piv && c == 0 && tid == 0) piv[j] = p;
+    const T* prow = remote(Ls, p % S) + (size_t)(p / S) * rmax;
+    T wip = mkc<R>(0, 0), acc = mkc<R>(0, 0);
+    if (own) wip = w_rows ? Ws[(size_t)li * n + p] : w[(long)i * n + p];
+    if constexpr (CLUSTER) {
+      for (int k = tid; k < j; k += blockDim.x) lp[k] = prow[k];
+      __syncthreads();
+      prow = lp;
+    }
+    if (own) {
+      const T* lrow = Ls + (size_t)li * rmax;
+      T acc2 = mkc<R>(0, 0);
+      for (int k = l4; k < j; k += kPcLanes) {
+        const T a = lrow[k], b = prow[k];
+        // acc + acc2 += a * conj(b)
+        acc.x = fma(a.x, b.x, acc.x);
+        acc.y = fma(a.y, b.x, acc.y);
+        acc2.x = fma(a.y, b.y, acc2.x);
+        acc2.y = fma(-a.x, b.y, acc2.y);
       }
-      T lij = mkc<R>(acc.x * inv, acc.y * inv);
-      if (i == p) lij = mkc<R>((R)sqrt(dp), R(0));
-      L[(long)i * lr + j] = lij;
-      double nd = (i == p) ? 0.0 : d[li] - ((double)lij.x * lij.x + (double)lij.y * lij.y);
-      d[li] = nd > 0 ? nd : 0.0;
+      acc = cadd(acc, acc2);
+    }
+    if (warp < nw) {
+      for (int o = kPcLanes / 2; o > 0; o >>= 1) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+      }
+      acc = csub(wip, acc);
+    } else {
+      const double inv = rsqrt(dp);
+      if (lane == 0) {
+        s_dp = dp * inv;
+        s_inv = inv;
+        s_inv2 = inv * inv;
+      }
     }
     __syncthreads();
+    if (own) {
+      const R inv = (R)s_inv;
+      T lij = mkc<R>(acc.x * inv, acc.y * inv);
+      if (i == p) lij = mkc<R>((R)s_dp, R(0));
+      if (l4 == 0) Ls[(size_t)li * rmax + j] = lij;
+      const double nd = fma(-((double)acc.x * acc.x + (double)acc.y * acc.y), s_inv2, d);
+      d = (i == p || __double2hiint(nd) < 0) ? 0.0 : nd;
+    }
     r = j + 1;
     last = 0.0;
   }
-  if (r == rmax) {
-    // largest remaining diagonal over the cluster (posted in the free slot)
-    double b = 0.0;
-    for (int li = tid; li < nloc; li += blockDim.x) b = fmax(b, d[li]);
-    for (int o = 16; o > 0; o >>= 1) b = fmax(b, __shfl_xor_sync(0xffffffffu, b, o));
-    if (lane == 0) rv[wid] = b;
-    __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      for (int k = 0; k < nw; ++k) t = fmax(t, rv[k]);
-      post_v[rmax & 1] = t;
-    }
-    cluster.sync();
-    last = 0.0;
-    for (int q = 0; q < S; ++q) last = fmax(last, cluster.map_shared_rank(post_v, q)[rmax & 1]);
-  }
+  if (r == rmax) last = pivot(rmax & 1, p);   // largest remaining diagonal, in the free slot
   if (c == 0 && tid == 0) {
     *rout = r;
-    *resid = tr > 0 ? last / tr : 0.0;
+    *resid = tr > 0 && last > 0.0 ? last / tr : 0.0;
   }
-  cluster.sync();   // no CTA leaves while another may still read its shared memory
+  // L to global memory only now: a store before a cluster barrier holds the barrier up until the
+  // store has landed
+  __syncthreads();
+  for (int e = tid; e < nlm * r; e += blockDim.x) {
+    const int row = e / r, k = e - row * r;
+    if (c + row * S < n) L[(long)(c + row * S) * lr + k] = Ls[(size_t)row * rmax + k];
+  }
+  barrier();   // no CTA leaves while another may still read its shared memory
 }
 
 // zs[i][c] = z[i][c] / sqrt(s_c) (0 where s_c <= 0): eigenvectors of L L^+ from those of L^+ L
@@ -964,15 +1016,39 @@ cudaError_t dual_rows(cudaStream_t st, int kk, int cols, const cx<R>* y, long ld
 
 template <typename R>
 cudaError_t pchol(cudaStream_t st, int n, const cx<R>* w, int rmax, double tol, cx<R>* L, int lr,
-                  int* rout, double* resid) {
+                  int* rout, double* resid, int* piv) {
   if (n < 1 || n > 1024 || rmax < 1 || rmax > kGradedMax) return cudaErrorInvalidValue;
-  // cluster of S CTAs, at least 32 rows each, at most 8 (portable cluster size)
-  const int S = std::min(8, std::max(1, n / 32));
+  // CTAs of the cluster: 64 rows each at most (the warps of a CTA).  One CTA needs no cluster
+  // barriers, which is worth more than the FP64 pipes of others up to 64 rows.
+  const int S = n > 128 ? kPcCtas : n > 64 ? 8 : 1;
   const int rows = (n + S - 1) / S;
-  const int threads = std::min(1024, std::max(64, (rows + 31) / 32 * 32));
+  const int threads = (rows * kPcLanes + 31) / 32 * 32 + 32;   // and the warp of the root
+  rmax = std::min(rmax, n);
+  const size_t lb = (size_t)rows * rmax * sizeof(cx<R>), wb = (size_t)rows * n * sizeof(cx<R>);
+  constexpr size_t kMax = 222 * 1024;   // leaves the static arrays their place
+  const int w_rows = lb + wb <= kMax ? 1 : 0;
+  static const cudaError_t attr = [] {
+    cudaError_t e = cudaFuncSetAttribute(pchol_kernel<R, true>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMax);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(pchol_kernel<R, true>,
+                               cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(pchol_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kMax);
+    return e;
+  }();
+  MPDO_CUDA_TRY(attr);
+  const size_t sm = w_rows ? lb + wb : lb;
+  count_launch();
+  if (S == 1) {
+    pchol_kernel<R, false><<<1, threads, sm, st>>>(n, w, rmax, tol, L, lr, rout, resid, piv, w_rows);
+    return cudaGetLastError();
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(S);
   cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = sm;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -981,13 +1057,13 @@ cudaError_t pchol(cudaStream_t st, int n, const cx<R>* w, int rmax, double tol, 
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  count_launch();
-  return cudaLaunchKernelEx(&cfg, pchol_kernel<R>, n, w, rmax, tol, L, lr, rout, resid);
+  return cudaLaunchKernelEx(&cfg, pchol_kernel<R, true>, n, w, rmax, tol, L, lr, rout, resid, piv,
+                            w_rows);
 }
 template cudaError_t pchol<float>(cudaStream_t, int, const float2*, int, double, float2*, int,
-                                  int*, double*);
+                                  int*, double*, int*);
 template cudaError_t pchol<double>(cudaStream_t, int, const double2*, int, double, double2*, int,
-                                   int*, double*);
+                                   int*, double*, int*);
 template <typename R>
 cudaError_t lift(cudaStream_t st, int r, const cx<R>* z, const double* s, cx<R>* zs) {
   count_launch();

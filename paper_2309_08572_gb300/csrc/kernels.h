@@ -48,10 +48,11 @@ cudaError_t kraus_select(cudaStream_t st, int n, const double* w, const cx<R>* w
 template <typename R>
 cudaError_t trace_pre(cudaStream_t st, int dm, const cx<R>* gi, const cx<R>* gj, StepScalars* sc);
 // Pivoted Cholesky W ~ L L^+ of a Hermitian PSD matrix (n <= 1024, rmax <= kGradedMax); device
-// outputs: L (n x r, row stride lr), *rout = r, *resid = remaining diag max / tr W.
+// outputs: L (n x r, row stride lr), *rout = r, *resid = remaining diag max / tr W, and (not
+// NULL) piv[0..r) = the pivots.
 template <typename R>
 cudaError_t pchol(cudaStream_t st, int n, const cx<R>* w, int rmax, double tol, cx<R>* L, int lr,
-                  int* rout, double* resid);
+                  int* rout, double* resid, int* piv = nullptr);
 // zs = z diag(s^-1/2) (r x r)
 template <typename R>
 cudaError_t lift(cudaStream_t st, int r, const cx<R>* z, const double* s, cx<R>* zs);
