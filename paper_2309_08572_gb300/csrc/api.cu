@@ -120,6 +120,7 @@ struct mpdo_ctx {
   void *wGs = nullptr, *wZ = nullptr, *wLg = nullptr;
   struct PcOut { int r; int pad; double resid; };
   PcOut* dpc = nullptr;
+  int* dpiv = nullptr;        // pivots of the left Gram's factor
   PcOut* hpc = nullptr;       // pinned
   MixWork mixw;              // mixed-precision eigensolver workspace (mixed only)
   void* mixmem = nullptr;
@@ -403,62 +404,85 @@ constexpr double kInnerTolMixed = 1e-10;
 constexpr int kInnerRmax = kGradedMax;   // columns of a factor (FP64)
 constexpr int kInnerRmaxF32 = 128;         // and of the FP32 factor
 
-// Eigenpairs of the PSD Gram g (n x n) through a pivoted Cholesky factor g ~ L L^+
-// (stopping at tol * tr g, at most rmax columns; FP64 factor for FP64 Grams, FP32 for
-// FP32 Grams) and the eigenpairs of the r x r matrix L^+ L, lifted as u = L z / sqrt(s):
-// eigenvectors to v (row stride ldv), eigenvalues to w, descending.  *nvals = r, or 0 when
-// the factor needs more than rmax columns (the caller solves the full problem).  zero_tail:
-// columns r..n-1 of v and w[r..n) zeroed.
+// Pivoted Cholesky factor g ~ L L^+ (n x n, into wLg) stopping at tol * tr g, its pivots to piv:
+// *rank columns, or 0 when it needs more than rmax of them.  One host synchronisation.
+template <typename RM>
+int factor(mpdo_ctx* h, int n, const cx<RM>* g, double tol, int rmax, int* piv, int* rank,
+           bool* zero) {
+  *rank = 0;
+  *zero = false;
+  rmax = std::min(rmax, n);
+  if (n < 1 || n > 1024 || rmax < 1) return MPDO_OK;
+  int pi = prof_begin(h, 2);
+  CK(pchol<RM>(h->st, n, g, rmax, tol, static_cast<cx<RM>*>(h->wLg), kInnerRmax, &h->dpc->r,
+               &h->dpc->resid, piv));
+  prof_end(h, 2, pi, 0.0);
+  CK(cudaMemcpyAsync(h->hpc, h->dpc, sizeof(mpdo_ctx::PcOut), cudaMemcpyDeviceToHost, h->st));
+  CK(sync_stream(h));
+  prof_drain(h);
+  const int r = h->hpc->r;
+  *zero = r < 1;
+  if (r >= 1 && !(r >= rmax && r < n && h->hpc->resid > tol)) *rank = r;
+  return MPDO_OK;
+}
+
+// Eigenpairs of the PSD Gram g (n x n) through its pivoted Cholesky factor (stopping at
+// tol * tr g, at most rmax columns; FP64 factor for FP64 Grams, FP32 for FP32 Grams): the
+// eigenvalues of L^+ L to w, descending, and its eigenvectors times w^-1/2 to wGs, which
+// lift_cols turns into eigenvectors of g, u = L z / sqrt(s), for the columns that the caller
+// keeps.  *nvals = r (w[r..n) zeroed), or 0 when the factor does not fit and the caller solves
+// the full problem.
 // FP64 Grams: L's columns fall off by decades, so L^+ L is graded and one graded solve
 // (heig_graded) resolves all of its pairs.  The levels of the mixed solver that it replaced took
 // 5 rounds of ~9 launches for such a matrix, and the FP64 form's one-sided Jacobi sweeps on L
 // 3.6 ms on one SM (n = 180, r = 40).
 template <typename RM>
-int lift_eig(mpdo_ctx* h, int n, const cx<RM>* g, cx<RM>* v, long ldv, double* w, double tol,
-             int rmax, bool zero_tail, int* nvals) {
+int lift_eig(mpdo_ctx* h, int n, const cx<RM>* g, double* w, double tol, int rmax, int* nvals) {
   using TM = cx<RM>;
   cudaStream_t st = h->st;
-  *nvals = 0;
-  rmax = std::min(rmax, n);
-  if (n < 1 || n > 1024 || rmax < 1) return MPDO_OK;
-  TM* L = static_cast<TM*>(h->wLg);
-  int pi = prof_begin(h, 2);
-  CK(pchol<RM>(st, n, g, rmax, tol, L, kInnerRmax, &h->dpc->r, &h->dpc->resid));
-  prof_end(h, 2, pi, 0.0);
-  CK(cudaMemcpyAsync(h->hpc, h->dpc, sizeof(mpdo_ctx::PcOut), cudaMemcpyDeviceToHost, st));
-  CK(sync_stream(h));
-  prof_drain(h);
-  const int r = h->hpc->r;
-  if (r < 1 || (r >= rmax && r < n && h->hpc->resid > tol)) return MPDO_OK;
+  bool zero;
+  int r = 0;
+  int rc = factor<RM>(h, n, g, tol, rmax, nullptr, &r, &zero);
+  if (rc) return rc;
+  *nvals = r;
+  if (r == 0) return MPDO_OK;
+  const TM* L = static_cast<const TM*>(h->wLg);
   TM* Gs = static_cast<TM*>(h->wGs);
   TM* Z = static_cast<TM*>(h->wZ);
-  CK((pgram<RM, RM>(h, 0, r, n, L, kInnerRmax, Gs, r)));
   if constexpr (std::is_same<RM, double>::value) {
+    CK((pgram<RM, RM>(h, 0, r, n, L, kInnerRmax, Z, r)));
     int pe = prof_begin(h, 1);
     double fl = 0.0;
-    CK(heig_graded(st, r, Gs, r, Z, r, w, h->mixw, &fl));
+    CK(heig_graded(st, r, Z, r, Gs, r, w, h->mixw, true, &fl));
     prof_end(h, 1, pe, fl);
   } else {
+    CK((pgram<RM, RM>(h, 0, r, n, L, kInnerRmax, Gs, r)));
     CK(peig<RM>(h, r, Gs, r, Z, r, w, 0.0));
+    PO(lift<RM>(st, r, Z, w, Gs));
   }
-  PO(lift<RM>(st, r, Z, w, Gs));
-  CK(pgemm<RM>(h, OP_N, OP_N, n, r, r, L, kInnerRmax, 0, Gs, r, 0, v, ldv, 0, 1));
-  if (zero_tail && r < n) {
-    CK(cudaMemset2DAsync(v + r, ldv * sizeof(TM), 0, (n - r) * sizeof(TM), n, st));
-    CK(cudaMemsetAsync(w + r, 0, (n - r) * sizeof(double), st));
-  }
-  *nvals = r;
+  if (r < n) CK(cudaMemsetAsync(w + r, 0, (n - r) * sizeof(double), st));
   return MPDO_OK;
 }
 
+// v (n x cols, row stride ldv) = the first cols eigenvectors of the Gram last factored by
+// lift_eig with rank r.
 template <typename RM>
-int inner_eig(mpdo_ctx* h, int nin, int* nvals) {
+int lift_cols(mpdo_ctx* h, int n, int r, int cols, cx<RM>* v, long ldv) {
+  CK(pgemm<RM>(h, OP_N, OP_N, n, cols, r, static_cast<const cx<RM>*>(h->wLg), kInnerRmax, 0,
+               static_cast<const cx<RM>*>(h->wGs), r, 0, v, ldv, 0, 1));
+  return MPDO_OK;
+}
+
+// *lifted: the eigenvectors wait for lift_cols; else they are in wVk.
+template <typename RM>
+int inner_eig(mpdo_ctx* h, int nin, int* nvals, bool* lifted) {
   cx<RM>* W = static_cast<cx<RM>*>(h->wWK);
   cx<RM>* V = static_cast<cx<RM>*>(h->wVk);
   const bool fp64 = std::is_same<RM, double>::value;
+  *lifted = false;
+  *nvals = nin;
   if (!fp64 && nin <= kInnerDirect) {
     CK(peig<RM>(h, nin, W, nin, V, nin, h->wWv, 1e-10));
-    *nvals = nin;
     return MPDO_OK;
   }
   // FP64 Grams: FP64 factor; C64: FP32 factor down to its floor.  (An FP32 factor of the FP64
@@ -468,15 +492,15 @@ int inner_eig(mpdo_ctx* h, int nin, int* nvals) {
                      : h->mixed                                ? kInnerTolMixed
                                                                : kInnerTol;
   int nv = 0;
-  int rc = lift_eig<RM>(h, nin, W, V, nin, h->wWv, tol, fp64 ? kInnerRmax : kInnerRmaxF32, false,
-                        &nv);
+  int rc = lift_eig<RM>(h, nin, W, h->wWv, tol, fp64 ? kInnerRmax : kInnerRmaxF32, &nv);
   if (rc) return rc;
-  if (nv == 0) {
-    // at most k_max pairs are kept; the PPT's sum of squares comes from ||W||_F
-    CK(peig<RM>(h, nin, W, nin, V, nin, h->wWv, 1e-10, h->kmax + 1));
-    nv = nin;
+  if (nv > 0) {
+    *lifted = true;
+    *nvals = nv;
+    return MPDO_OK;
   }
-  *nvals = nv;
+  // at most k_max pairs are kept; the PPT's sum of squares comes from ||W||_F
+  CK(peig<RM>(h, nin, W, nin, V, nin, h->wWv, 1e-10, h->kmax + 1));
   return MPDO_OK;
 }
 
@@ -528,43 +552,72 @@ int update_lr(mpdo_ctx* h, int i, const DevOp& op, bool mirrored, int chi, int k
   CK((pgram<RS, RM>(h, 0, n3, dl * ki, wM, n3, wGi, n3)));
   CK((pgram<RS, RM>(h, 1, n3, kj * dr, aj, (long)kj * dr, wGj, n3)));
   PO(trace_pre<RM>(st, dm, wGi, wGj, h->dsc));
-  // a3: left factor from the eigendecomposition of G_i (numerical rank by gtol)
-  {
-    int nv = 0;
-    // FP64 Grams: FP64 factor and the graded solver on L^+ L (rank r instead of 3D; rotating
-    // an FP32 copy of the factor instead loses the small eigenvalues: its rounding is relative
-    // to whole columns, not to eigendirections).  C64: the FP32 Jacobi solver.
-    if (h->eltm == 16) {
-      rc = lift_eig<RM>(h, n3, wGi, wVg, n3, h->wSig, pc_tol(h, h->gtol), kInnerRmax, true, &nv);
-      if (rc) return rc;
-    }
-    if (nv == 0) CK(peig<RM>(h, n3, wGi, n3, wVg, n3, h->wSig, 0.1 * h->gtol));
+  // a3: left factor R with G_i = R^+ R.  FP64 Grams: the pivoted Cholesky factor, R = L^+ of rank
+  // rg (its pivots stop at a tenth of the rank cut gtol, since what is left below them sums over
+  // many), whose right inverse has only the pivot rows,
+  // R^-1 = P L1^-+.  The factor need not be the spectral one -- H has the same spectrum for any R
+  // -- so no eigenproblem of G_i is solved, and H shrinks from 9 D to 3 rg rows (40 atoms, two
+  // layers in FP64, D = 20: 180 to ~95).  Beyond its column cap, and in C64: the
+  // eigendecomposition of G_i, rank-cut by gtol.
+  int rg = 0;
+  if constexpr (std::is_same<RM, double>::value) {
+    bool zero;
+    rc = factor<RM>(h, n3, wGi, 0.1 * h->gtol, kInnerRmax, h->dpiv, &rg, &zero);
+    if (rc) return rc;
+    if (zero) return fail(h, MPDO_ERR_NUMERIC, "zero or non-finite state in update");
   }
-  PO(gram_mask<RM>(st, n3, h->wSig, h->gtol, wRs, wIrs, h->dsc));
-  PO(gram_factor<RM>(st, n3, wVg, wRs, wIrs, wR, wVs, wVr));
+  const bool chol = rg > 0;
+  const int nr = chol ? rg : n3, nh = 3 * nr;   // rows of R, of H
+  TM* L = static_cast<TM*>(h->wLg);
+  if (!chol) {
+    CK(peig<RM>(h, n3, wGi, n3, wVg, n3, h->wSig, 0.1 * h->gtol));
+    PO(gram_mask<RM>(st, n3, h->wSig, h->gtol, wRs, wIrs, h->dsc));
+    PO(gram_factor<RM>(st, n3, wVg, wRs, wIrs, wR, wVs, wVr));
+  }
   // a4/a5: Phi from the channel and G_j, then H = (I x R) Phi (I x R)^+
   PO(build_phi<RM>(st, dm, Ct, wGj, wPhi));
-  CK(pgemm<RM>(h, OP_N, OP_N, n3, n9, n3, wR, n3, 0, wPhi, n9, (long)n3 * n9, wX, n9,
-               (long)n3 * n9, 3));
-  CK(pgemm<RM>(h, OP_N, OP_C, n9, n3, n3, wX, n9, n3, wR, n3, 0, wH, n9, n3, 3));
-  // a6: bond eigenpairs and cut
-  {
-    int nv = 0;
-    if (h->eltm == 16) {
-      rc = lift_eig<RM>(h, n9, wH, wU, n9, h->wLam, pc_tol(h, h->htol), kInnerRmax, true, &nv);
-      if (rc) return rc;
-    }
-    // at most chi pairs are kept: the (chi+1)-th decides nothing more (the discarded weight
-    // comes from tr H)
-    if (nv == 0) CK(peig<RM>(h, n9, wH, n9, wU, n9, h->wLam, 0.1 * h->htol, chi + 1));
+  if (chol) {
+    if constexpr (std::is_same<RM, double>::value)
+      PO(pchol_inverse(st, rg, L, kInnerRmax, h->dpiv, wVr));
+    CK(pgemm<RM>(h, OP_C, OP_N, nr, n9, n3, L, kInnerRmax, 0, wPhi, n9, (long)n3 * n9, wX, n9,
+                 (long)nr * n9, 3));
+    CK(pgemm<RM>(h, OP_N, OP_N, nh, nr, n3, wX, n9, n3, L, kInnerRmax, 0, wH, nh, nr, 3));
+  } else {
+    CK(pgemm<RM>(h, OP_N, OP_N, n3, n9, n3, wR, n3, 0, wPhi, n9, (long)n3 * n9, wX, n9,
+                 (long)n3 * n9, 3));
+    CK(pgemm<RM>(h, OP_N, OP_C, n9, n3, n3, wX, n9, n3, wR, n3, 0, wH, n9, n3, 3));
   }
-  PO(bond_select<RM>(st, n9, h->wLam, wH, n9, h->htol, chi, h->dsc, h->dstats));
+  // a6: bond eigenpairs and cut
+  int rh = 0;
+  if (h->eltm == 16) {
+    rc = lift_eig<RM>(h, nh, wH, h->wLam, pc_tol(h, h->htol), kInnerRmax, &rh);
+    if (rc) return rc;
+  }
+  // at most chi pairs are kept: the (chi+1)-th decides nothing more (the discarded weight
+  // comes from tr H)
+  if (rh == 0) CK(peig<RM>(h, nh, wH, nh, wU, nh, h->wLam, 0.1 * h->htol, chi + 1));
+  PO(bond_select<RM>(st, nh, h->wLam, wH, nh, h->htol, chi, h->dsc, h->dstats));
   rc = read_scalars(h);
   if (rc) return rc;
   const int keep = h->hsc->keep;
-  // a7: split.  Vgen = (I x V sigma^-1/2) U_keep
-  CK(pgemm<RM>(h, OP_N, OP_N, n3, keep, n3, wVs, n3, 0, wU, n9, (long)n3 * n9, wVgen, keep,
-               (long)n3 * keep, 3));
+  long ldu = nh;
+  if (rh > 0) {
+    ldu = keep;
+    rc = lift_cols<RM>(h, nh, rh, keep, wU, ldu);
+    if (rc) return rc;
+  }
+  // a7: split.  A = (M_i x I) Vgen with Vgen = (I x R^-1) U_keep: V sigma^-1/2 U_keep of the
+  // spectral factor, or L1^-+ U_keep on the pivot columns of M_i alone
+  const T* am = wM;
+  if (chol) {
+    CK(pgemm<RM>(h, OP_C, OP_N, nr, keep, nr, wVr, nr, 0, wU, ldu, (long)nr * ldu, wVgen, keep,
+                 (long)nr * keep, 3));
+    PO(gather_cols<T>(st, (long)dl * ki, nr, wM, n3, h->dpiv, wWB));
+    am = wWB;
+  } else {
+    CK(pgemm<RM>(h, OP_N, OP_N, n3, keep, n3, wVs, n3, 0, wU, ldu, (long)n3 * ldu, wVgen, keep,
+                 (long)n3 * keep, 3));
+  }
   // The left factor A = (M_i x I)(I x V sigma^-1/2) U_keep is an isometry only up to the
   // error of the small-sigma eigenvectors of G_i, amplified by sigma^-1/2.  One
   // Newton-Schulz polar step (Higham) restores it: A <- A (3I - A^+A)/2.  The centre
@@ -581,7 +634,7 @@ int update_lr(mpdo_ctx* h, int i, const DevOp& op, bool mirrored, int chi, int k
     TM* gaM = static_cast<TM*>(h->wGa);
     TM* polM = static_cast<TM*>(h->wPol);
     TM* qolM = static_cast<TM*>(h->wQol);
-    CK(pwide<RM>(h, OP_N, OP_N, dl * ki, keep, n3, wM, n3, 0, wVgen, keep, (long)n3 * keep, aM,
+    CK(pwide<RM>(h, OP_N, OP_N, dl * ki, keep, nr, am, nr, 0, wVgen, keep, (long)nr * keep, aM,
                  3L * keep, keep, 3));
     CK((pgram<RM, RM>(h, 0, keep, rows, aM, keep, gaM, keep)));
     PO(polar_factors<RM>(st, keep, gaM, polM, qolM));
@@ -595,7 +648,7 @@ int update_lr(mpdo_ctx* h, int i, const DevOp& op, bool mirrored, int chi, int k
     T* wGa = static_cast<T*>(h->wGa);
     T* wPol = static_cast<T*>(h->wPol);
     T* wQol = static_cast<T*>(h->wQol);
-    CK(pgemm<RS>(h, OP_N, OP_N, dl * ki, keep, n3, wM, n3, 0, wVgen, keep, (long)n3 * keep,
+    CK(pgemm<RS>(h, OP_N, OP_N, dl * ki, keep, nr, am, nr, 0, wVgen, keep, (long)nr * keep,
                  wTmp, 3L * keep, keep, 3));
     CK((pgram<RS, RS>(h, 0, keep, rows, wTmp, keep, wGa, keep)));
     PO(polar_factors<RS>(st, keep, wGa, wPol, wQol));
@@ -617,7 +670,8 @@ int update_lr(mpdo_ctx* h, int i, const DevOp& op, bool mirrored, int chi, int k
     const int nc = (int)colsB;
     CK((pgram<RS, RM>(h, 0, nc, KM, wBp, colsB, wWK, nc)));
     int nv;
-    rc = inner_eig<RM>(h, nc, &nv);
+    bool lifted;
+    rc = inner_eig<RM>(h, nc, &nv, &lifted);
     if (rc) return rc;
     // a9: cut + PPT (FP64 scalars); tr(B^+B) = tr(B B^+)
     PO(kraus_select<RM>(st, nv, h->wWv, wWK, nc, h->kcut, kmax, use_ppt, h->wF, h->dsc,
@@ -626,11 +680,13 @@ int update_lr(mpdo_ctx* h, int i, const DevOp& op, bool mirrored, int chi, int k
     if (rc) return rc;
     kk = h->hsc->kkeep;
     // a10: kept rows f_k sqrt(w_k) y_k^+
-    PO((dual_rows<RM, RS>(st, kk, nc, wVk, nc, h->wF, h->wWv, wCn)));
+    if (lifted && (rc = lift_cols<RM>(h, nc, nv, kk, wVk, kk))) return rc;
+    PO((dual_rows<RM, RS>(st, kk, nc, wVk, lifted ? kk : nc, h->wF, h->wWv, wCn)));
   } else {
     CK((pgram<RS, RM>(h, 1, KM, (int)colsB, wBp, colsB, wWK, KM)));
     int nv;
-    rc = inner_eig<RM>(h, KM, &nv);
+    bool lifted;
+    rc = inner_eig<RM>(h, KM, &nv, &lifted);
     if (rc) return rc;
     // a9: cut + PPT (FP64 scalars)
     PO(kraus_select<RM>(st, nv, h->wWv, wWK, KM, h->kcut, kmax, use_ppt, h->wF, h->dsc,
@@ -639,7 +695,8 @@ int update_lr(mpdo_ctx* h, int i, const DevOp& op, bool mirrored, int chi, int k
     if (rc) return rc;
     kk = h->hsc->kkeep;
     // a10: apply the inner isometry with the PPT scales
-    PO((scale_vk<RM, RS>(st, KM, kk, wVk, KM, h->wF, wVks)));
+    if (lifted && (rc = lift_cols<RM>(h, KM, nv, kk, wVk, kk))) return rc;
+    PO((scale_vk<RM, RS>(st, KM, kk, wVk, lifted ? kk : KM, h->wF, wVks)));
     CK(pgemm<RS>(h, OP_C, OP_N, kk, colsB, KM, wVks, kk, 0, wBp, colsB, 0, wCn, colsB, 0, 1));
   }
   PO(swap12<T>(st, 1, kk, (long)keep * 3, dr, wCn, aj));
@@ -1374,7 +1431,8 @@ int mpdo_create(const mpdo_config* cfg, const double* init_site_vec, mpdo_t* out
   if ((rc = alloc_dev(hp, &h->wLg, (size_t)std::max(n9, KM) * kInnerRmax * em)) ||
       (rc = B(&h->wGs, (size_t)kInnerRmax * kInnerRmax)) ||
       (rc = B(&h->wZ, (size_t)kInnerRmax * kInnerRmax)) ||
-      (rc = alloc_dev(hp, (void**)&h->dpc, sizeof(mpdo_ctx::PcOut))))
+      (rc = alloc_dev(hp, (void**)&h->dpc, sizeof(mpdo_ctx::PcOut))) ||
+      (rc = alloc_dev(hp, (void**)&h->dpiv, kGradedMax * sizeof(int))))
     return rc;
   if (cudaEventCreateWithFlags(&h->bev, cudaEventBlockingSync | cudaEventDisableTiming) !=
       cudaSuccess) {
@@ -1863,7 +1921,7 @@ int mpdo_kernel_heig_graded(int n, const void* a, void* v, double* w, void* stre
   // the solver's CTA ticket starts at zero
   cudaError_t e = cudaMemsetAsync(mm, 0, mix_work_bytes(n), st);
   if (e == cudaSuccess)
-    e = heig_graded(st, n, (const double2*)a, n, (double2*)v, n, w, mw);
+    e = heig_graded(st, n, (const double2*)a, n, (double2*)v, n, w, mw, false);
   cudaError_t es = cudaStreamSynchronize(st);
   mix_work_release(mw);
   cudaFree(mm);

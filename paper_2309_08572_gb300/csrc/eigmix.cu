@@ -519,12 +519,29 @@ __global__ void __launch_bounds__(RT * RT) refine_kernel(int m, int n, const dou
 // part of I + E: 120 CTAs at m = 60, where a 16 x 16 tiling would use 30 SMs and leave the
 // elementwise step to one.  In the final pass the last CTA to finish (a ticket; nobody waits)
 // settles runs of unseparated neighbours by Rayleigh-Ritz, 16 at a time.
+//
+// scaled: column j of I + E, and so eigenvector j, comes out times lam_j^-1/2 (0 for lam_j <= 0),
+// the factor that lifts an eigenvector of L^+ L to one of L L^+.
 constexpr int GT = 4;
 constexpr int kSgeThreads = 128;
+__device__ __forceinline__ double col_scale(double lam, int scaled) {
+  return !scaled ? 1.0 : lam > 0.0 ? rsqrt(lam) : 0.0;
+}
+// columns [c0, c0 + c) of IE times lam^-1/2, or (undo) divided by it; all threads of the CTA
+__device__ void scale_cols(int m, int c0, int c, const double* lam, double2* IE, bool undo) {
+  for (int e = threadIdx.x; e < m * c; e += blockDim.x) {
+    const int col = c0 + e % c;
+    const double l = __ldcg(&lam[col]), f = undo ? sqrt(fmax(l, 0.0)) : col_scale(l, 1);
+    double2* x = &IE[(long)(e / c) * m + col];
+    *x = cscale(__ldcg(x), f);
+  }
+  __syncthreads();
+}
 __global__ void __launch_bounds__(kSgeThreads) sge_kernel(int m, const double2* __restrict__ TZ,
                                                           double2* SG, int final_pass,
                                                           double emax, double* lam, double2* IE,
-                                                          unsigned char* sep, unsigned int* ticket) {
+                                                          unsigned char* sep, unsigned int* ticket,
+                                                          int scaled) {
   extern __shared__ double2 sge_col[];   // [k][16]: Z_I, Z_J, T_I, T_J
   __shared__ double2 part[48];
   __shared__ double2 val[48];            // S, G (16 each), then S_ii, G_ii, S_jj, G_jj (4 each)
@@ -570,9 +587,10 @@ __global__ void __launch_bounds__(kSgeThreads) sge_kernel(int m, const double2* 
     const double gi = val[36 + a].x, gj = val[44 + b].x;
     const double li = gi > 0 ? val[32 + a].x / gi : 0.0, lj = gj > 0 ? val[40 + b].x / gj : 0.0;
     const double2 s = val[tid], g = val[16 + tid];
+    const double ci = col_scale(li, scaled), cj = col_scale(lj, scaled);
     if (i == j && i < m) {
       lam[i] = li;
-      IE[(long)i * m + i] = make_double2(1.0 + 0.5 * (1.0 - gi), 0.0);
+      IE[(long)i * m + i] = make_double2(ci * (1.0 + 0.5 * (1.0 - gi)), 0.0);
       SG[i * ld + i] = s;
       SG[i * ld + m + i] = g;
     } else if (i < j && j < m) {
@@ -588,11 +606,11 @@ __global__ void __launch_bounds__(kSgeThreads) sge_kernel(int m, const double2* 
                           cabs2(nij) * mx < lim && cabs2(nji) * mx < lim;
       if (newton) {
         const double r = 1.0 / d;
-        IE[(long)i * m + j] = cscale(nij, r);
-        IE[(long)j * m + i] = cscale(nji, -r);
+        IE[(long)i * m + j] = cscale(nij, r * cj);
+        IE[(long)j * m + i] = cscale(nji, -r * ci);
       } else {
-        IE[(long)i * m + j] = cscale(g, -0.5);
-        IE[(long)j * m + i] = cscale(cconj(g), -0.5);
+        IE[(long)i * m + j] = cscale(g, -0.5 * cj);
+        IE[(long)j * m + i] = cscale(cconj(g), -0.5 * ci);
       }
       if (j == i + 1) sep[i] = newton;
     }
@@ -615,7 +633,12 @@ __global__ void __launch_bounds__(kSgeThreads) sge_kernel(int m, const double2* 
   for (int i = 0; i + 1 < m;) {
     int j = i;
     while (j + 1 < m && !flags[j] && j - i + 1 < kRitzMax) ++j;   // run [i, j]
-    if (j > i) ritz_cluster(m, SG, i, j - i + 1, lam, IE);
+    if (j > i) {
+      // the Ritz step works on unscaled columns and sets the run's eigenvalues
+      if (scaled) scale_cols(m, i, j - i + 1, lam, IE, true);
+      ritz_cluster(m, SG, i, j - i + 1, lam, IE);
+      if (scaled) scale_cols(m, i, j - i + 1, lam, IE, false);
+    }
     i = j + 1;
   }
 }
@@ -1013,7 +1036,7 @@ cudaError_t heig_mixed(cudaStream_t st, int n, const double2* a, long lda, doubl
 // place of the levels of heig_mixed and of FP64 sweeps, whose time went into a chain of small
 // launches per two decades of the spectrum (mixed form) or into one SM's FP64 pipe (FP64 form).
 cudaError_t heig_graded(cudaStream_t st, int n, const double2* a, long lda, double2* z, long ldz,
-                        double* w, MixWork& wk, double* flops_out) {
+                        double* w, MixWork& wk, bool scaled, double* flops_out) {
   if (n <= 0) return cudaSuccess;
   if (n > kGradedMax || n > wk.n_cap) return cudaErrorInvalidValue;
   const long l2 = 2L * n;
@@ -1038,7 +1061,8 @@ cudaError_t heig_graded(cudaStream_t st, int n, const double2* a, long lda, doub
     const int fin = pass == 1;
     count_launch();
     sge_kernel<<<grid, kSgeThreads, sm, st>>>(n, cur, wk.s, fin, fin ? kNewtonFinal : kNewtonMax,
-                                              fin ? w : wk.lam, wk.ie, wk.sepf, wk.ticket);
+                                              fin ? w : wk.lam, wk.ie, wk.sepf, wk.ticket,
+                                              fin && scaled ? 1 : 0);
     MPDO_CUDA_TRY(cudaGetLastError());
     if (fin) {
       MPDO_CUDA_TRY(mul(cur + n, l2, 0, wk.ie, n, z, ldz, 0, 1));

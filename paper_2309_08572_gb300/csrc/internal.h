@@ -113,8 +113,9 @@ cudaError_t heig_mixed(cudaStream_t st, int n, const double2* a, long lda, doubl
 
 // Eigenpairs of a graded Hermitian PSD matrix (L^+ L of a pivoted Cholesky factor, n <=
 // kGradedMax): z (n x n, row stride ldz) and w, descending up to the order of pairs that agree
-// to FP32 rounding, each resolved relative to its own size.  No host synchronisation.
+// to FP32 rounding, each resolved relative to its own size.  scaled: the columns of z are the
+// eigenvectors times w^-1/2.  No host synchronisation.
 cudaError_t heig_graded(cudaStream_t st, int n, const double2* a, long lda, double2* z, long ldz,
-                        double* w, MixWork& wk, double* flops_out = nullptr);
+                        double* w, MixWork& wk, bool scaled, double* flops_out = nullptr);
 
 }  // namespace mpdo

@@ -111,8 +111,7 @@ __global__ void gram_mask_kernel(int n, const double* __restrict__ sig, double g
   __syncthreads();
   if (threadIdx.x == 0) {
     sc->rank_g = cnt;
-    // first flag write of an update: starts the update's flags afresh
-    sc->flags = bad ? 1 : 0;
+    if (bad) sc->flags |= 1;
   }
 }
 
@@ -379,7 +378,10 @@ __global__ void trace_pre_kernel(int dm, const cx<R>* __restrict__ gi, const cx<
     if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
     __syncthreads();
   }
-  if (threadIdx.x == 0) sc->trpre = red[0];
+  if (threadIdx.x == 0) {
+    sc->trpre = red[0];
+    sc->flags = 0;   // the update's flags start afresh
+  }
 }
 
 // out = sum |a_e|^2 over n complex entries, in FP64 (one CTA; the norm of the centre site).
@@ -817,6 +819,60 @@ __global__ void __launch_bounds__(32 * (kPcWarps + 1)) pchol_kernel(
   barrier();   // no CTA leaves while another may still read its shared memory
 }
 
+// x = L1^-1 (r x r, lower triangular, row-major), L1[a][b] = L[piv[a]][b] the pivot rows of a
+// pivoted Cholesky factor.  A warp per column of x, by columns of L1: once x_b is known every
+// lane takes L1[a][b] x_b off its rows a > b.  Bound by the latency of the r dependent steps.
+constexpr int kInvWarps = 4;
+__global__ void __launch_bounds__(32 * kInvWarps) pchol_inverse_kernel(int r,
+                                                                      const double2* __restrict__ L,
+                                                                      int lr,
+                                                                      const int* __restrict__ piv,
+                                                                      double2* x) {
+  constexpr int RL = (kGradedMax + 31) / 32;   // rows of a lane: a = lane + 32 t
+  const int lane = threadIdx.x & 31, j = blockIdx.x * kInvWarps + (threadIdx.x >> 5);
+  if (j >= r) return;
+  const double2* row[RL];
+  double inv[RL];
+  double2 s[RL];
+#pragma unroll
+  for (int t = 0; t < RL; ++t) {
+    const int a = lane + 32 * t;
+    row[t] = L + (long)piv[a < r ? a : 0] * lr;
+    inv[t] = a < r ? 1.0 / row[t][a].x : 0.0;
+    s[t] = make_double2(a == j ? 1.0 : 0.0, 0.0);
+  }
+  for (int b = j; b < r; ++b) {
+    // x_b from its lane: every lane selects its own candidate, the broadcast takes the right one
+    double2 xb = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int t = 0; t < RL; ++t)
+      if (t == b >> 5) xb = cscale(s[t], inv[t]);
+    xb.x = __shfl_sync(0xffffffffu, xb.x, b & 31);
+    xb.y = __shfl_sync(0xffffffffu, xb.y, b & 31);
+#pragma unroll
+    for (int t = 0; t < RL; ++t) {
+      const int a = lane + 32 * t;
+      if (a == b) s[t] = xb;
+      else if (a > b && a < r) s[t] = csub(s[t], cmul(row[t][b], xb));
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < RL; ++t) {
+    const int a = lane + 32 * t;
+    if (a < r) x[(long)a * r + j] = a >= j ? s[t] : make_double2(0.0, 0.0);
+  }
+}
+
+// out (rows x r) = the columns piv[0..r) of in (row stride ldi)
+template <typename T>
+__global__ void gather_cols_kernel(long rows, int r, const T* __restrict__ in, long ldi,
+                                   const int* __restrict__ piv, T* __restrict__ out) {
+  const long total = rows * r;
+  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total;
+       e += (long)gridDim.x * blockDim.x)
+    out[e] = in[(e / r) * ldi + piv[e % r]];
+}
+
 // zs[i][c] = z[i][c] / sqrt(s_c) (0 where s_c <= 0): eigenvectors of L L^+ from those of L^+ L
 template <typename R>
 __global__ void lift_kernel(int r, const cx<R>* __restrict__ z, const double* __restrict__ s,
@@ -1064,6 +1120,24 @@ template cudaError_t pchol<float>(cudaStream_t, int, const float2*, int, double,
                                   int*, double*, int*);
 template cudaError_t pchol<double>(cudaStream_t, int, const double2*, int, double, double2*, int,
                                    int*, double*, int*);
+cudaError_t pchol_inverse(cudaStream_t st, int r, const double2* L, int lr, const int* piv,
+                          double2* x) {
+  if (r < 1 || r > kGradedMax) return cudaErrorInvalidValue;
+  count_launch();
+  pchol_inverse_kernel<<<(r + kInvWarps - 1) / kInvWarps, 32 * kInvWarps, 0, st>>>(r, L, lr, piv, x);
+  return cudaGetLastError();
+}
+template <typename T>
+cudaError_t gather_cols(cudaStream_t st, long rows, int r, const T* in, long ldi, const int* piv,
+                        T* out) {
+  count_launch();
+  gather_cols_kernel<T><<<nblocks(rows * r), 256, 0, st>>>(rows, r, in, ldi, piv, out);
+  return cudaGetLastError();
+}
+template cudaError_t gather_cols<float2>(cudaStream_t, long, int, const float2*, long, const int*,
+                                         float2*);
+template cudaError_t gather_cols<double2>(cudaStream_t, long, int, const double2*, long, const int*,
+                                          double2*);
 template <typename R>
 cudaError_t lift(cudaStream_t st, int r, const cx<R>* z, const double* s, cx<R>* zs) {
   count_launch();

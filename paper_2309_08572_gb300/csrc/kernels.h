@@ -53,6 +53,13 @@ cudaError_t trace_pre(cudaStream_t st, int dm, const cx<R>* gi, const cx<R>* gj,
 template <typename R>
 cudaError_t pchol(cudaStream_t st, int n, const cx<R>* w, int rmax, double tol, cx<R>* L, int lr,
                   int* rout, double* resid, int* piv = nullptr);
+// x = L1^-1 (r x r), L1 the pivot rows of such a factor (r <= kGradedMax)
+cudaError_t pchol_inverse(cudaStream_t st, int r, const double2* L, int lr, const int* piv,
+                          double2* x);
+// out (rows x r) = the columns piv[0..r) of in (row stride ldi)
+template <typename T>
+cudaError_t gather_cols(cudaStream_t st, long rows, int r, const T* in, long ldi, const int* piv,
+                        T* out);
 // zs = z diag(s^-1/2) (r x r)
 template <typename R>
 cudaError_t lift(cudaStream_t st, int r, const cx<R>* z, const double* s, cx<R>* zs);
