@@ -279,9 +279,12 @@ constexpr int kTcMinSide = 16;
 
 // Products with FP64 outputs in the tensor-core forms with FP64 Grams (mixed form): the
 // error-free slice products on the BF16 tensor cores (tc_cgemm_exact) when large enough.
-inline bool tc_exact_route(const mpdo_ctx* h, int m, int n, int k, int batch) {
+// Of those above the threshold the ones that are estimated faster there than on the FP64 CUDA
+// cores (a threshold from the environment is taken as it is).
+inline bool tc_exact_route(const mpdo_ctx* h, int m, int n, int k, int batch, bool gram = false) {
   return h->tcmode >= 0 && h->mixed && (double)m * n * k * batch >= h->tc_min_macs &&
-         m >= kTcMinSide && n >= kTcMinSide && k >= 1;
+         m >= kTcMinSide && n >= kTcMinSide && k >= 1 &&
+         (h->tc_min_macs < kTcMinMacs || tc_exact_faster(m, n, k, batch, gram));
 }
 template <typename TA, typename TB>
 cudaError_t pexact(mpdo_ctx* h, int opa, int opb, int m, int n, int k, const TA* A, long lda,
@@ -359,7 +362,7 @@ cudaError_t pgram(mpdo_ctx* h, int side, int n, int k, const cx<RS>* A, long lda
   if constexpr (std::is_same<RM, float>::value) {
     return pgemm<RS>(h, opa, opb, n, n, k, A, lda, 0, A, lda, 0, C, ldc, 0, 1);
   } else {
-    if (tc_exact_route(h, n, n, k, 1))
+    if (tc_exact_route(h, n, n, k, 1, true))
       return pexact<cx<RS>, cx<RS>>(h, opa, opb, n, n, k, A, lda, 0, A, lda, 0, C, ldc, 0, 1);
     int pi = prof_begin(h, 0);
     cudaError_t e = cgemm_gram<RS>(h->st, side, n, k, A, lda, C, ldc);

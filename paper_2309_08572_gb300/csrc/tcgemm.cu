@@ -31,6 +31,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -405,60 +406,117 @@ __global__ void __launch_bounds__(PT * 8)
 // six slices of integers in [-128, 128] (exact in BF16):
 //   x 2^-e_r = 2^-7 (q_1 + 2^-8 q_2 + ... + 2^-40 q_6) + O(2^-48).
 // The product of slice t of A and slice u of B is a sum of integer products of at most
-// 2^14 each; over a chunk of 1024 real K terms it stays below 2^24 and is therefore exact in
-// the FP32 accumulator.  Each chunk's accumulator is drained into FP64 registers with the
-// weight 2^-(14 + 8(t+u)) (t, u from 0) and, at the end, scaled by 2^(e_r + e_q).  The slice
-// pairs with t + u <= 5 are computed (21 of 36): a dropped pair contributes terms below
-// 2^-48 of the two rows' largest entries.  The result carries the FP32 inputs' product to
+// 2^14 each; 1024 of them stay below 2^24 and are therefore exact in the FP32 accumulator.  The
+// accumulators are taken out in time and added with the weight 2^-(14 + 8(t+u)) (t, u from 0),
+// and the sum is scaled by 2^(e_r + e_q).  The slice pairs with t + u <= 5 are computed (21 of
+// 36): a dropped pair contributes terms below 2^-48 of the two rows' largest entries.  The result carries the FP32 inputs' product to
 // ~2^-48 of the rows' largest entries, enough for the eigenvalues of a Gram matrix of FP32
 // data down to ~1e-14 of the largest (the floor of FP64 sums of the same products).
+//
+// The kernel's tile is 128 rows by 64 real columns.  A stage holds 32 K terms of all six slices
+// of both operands (72 KB, three stages), so the 21 pairs run on operands that were loaded once:
+// 36 bytes per clock and SM from L2, where loading every pair's operands took 128.  The pairs
+// (t, u) of one weight t + u add into one accumulator, six of 64 TMEM columns; a sum stays
+// below 2^24 for 1024 / (t + u + 1) terms, so every XDRAIN = 5 stages (at most 6 x 160 terms) eight
+// warps take the accumulators out, group after group, while the MMAs of the other groups run.
+// They add them as integers -- weights 0..2 and 3..5 shifted into two 64-bit sums, exact -- since
+// the FP64 pipe, at 2 operations per clock and SM, bound the earlier FP64 drain to an eighth of the
+// MMA rate.  The K loop of a product with few tiles is split over CTAs; their integer sums are
+// added by exact_finish_kernel.  Gram matrices compute the tiles that reach the upper half, from
+// one packed operand: the rows of A are the even rows of the packed B.  Bound by the tensor pipe
+// (N = 64: by its operand reads from shared memory).  Kernel times: inner Gram 400 x 400 x 5043 601
+// -> 74 us, 768 x 768 x 4096 Gram 1150 -> 187 us.
 constexpr int XS = 6;          // slices per operand
-constexpr int XPAIRS = 21;     // slice pairs (t, u) with t + u <= XS - 1
 constexpr int XBN = 64;        // output tile width (real columns)
-constexpr int XSTAGES = 8;
-constexpr int XCHUNK = 16;     // k-blocks of 64 BF16 per exact chunk (1024 real terms)
-constexpr int XTHREADS = 192;  // warp 0 TMA, warp 1 MMA, warps 2-5 drain
+constexpr int XKB = 32;        // K terms of a stage
+constexpr int XSTAGES = 3;
+constexpr int XDRAIN = 5;      // stages between drains
+constexpr int XTHREADS = 320;  // warp 0 TMA, warp 1 MMA, warps 2-9 drain
+constexpr int XA_SLICE = BM * XKB * 2, XB_SLICE = XBN * XKB * 2;
+constexpr int XSTAGE_BYTES = XS * (XA_SLICE + XB_SLICE);
+constexpr int kNonFinite = 0x7fffffff;   // exponent of a row with a non-finite entry
+constexpr int kZeroRow = -1000000;       // and of a zero row (any smaller value)
 
-// pair index -> (t, u), enumerating t = 0.., u = 0..XS-1-t
-__device__ __forceinline__ void pair_tu(int p, int& t, int& u) {
-  t = 0;
-  while (p >= XS - t) {
-    p -= XS - t;
-    ++t;
+// As sdesc, for rows of 64 bytes with 64-byte swizzle (8-row groups 512 bytes apart).
+__device__ __forceinline__ uint64_t sdesc64(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(512 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;
+  return d;
+}
+
+// 2^(e_r + e_q) (2^-30 hi + 2^-54 lo), NaN when either row had a non-finite entry.  The power of
+// two goes straight into the exponent field where the result stays normal: three FP64
+// operations an element, where ldexp's multiplications took a third of a short product's time.
+__device__ __forceinline__ double exact_value(long long hi, long long lo, int er, int eq) {
+  if (er == kNonFinite || eq == kNonFinite) return NAN;
+  if (er <= kZeroRow || eq <= kZeroRow || (hi | lo) == 0) return 0.0;
+  const double v = fma((double)lo, 0x1p-24, (double)hi);
+  const int s = er + eq - 30, h = __double2hiint(v), ex = ((h >> 20) & 2047) + s;
+  if (v == 0.0 || ex <= 0 || ex >= 2047) return ldexp(v, s);
+  return __hiloint2double(h + (s << 20), __double2loint(v));
+}
+
+// Output of one complex element (i, q), with its mirror image for a Gram matrix.
+__device__ __forceinline__ void exact_store(double2* C, long ldc, int i, int q, double re, double im,
+                                            int gram, int accumulate) {
+  if (gram && q < i) return;
+  if (gram && q == i) im = 0.0;
+  double2* p = C + (long)i * ldc + q;
+  double2 v = make_double2(re, im);
+  if (accumulate) v = cadd(v, *p);
+  *p = v;
+  if (gram && q > i) C[(long)q * ldc + i] = cconj(v);
+}
+
+// tile index -> (row tile, column tile); a Gram's row tile mt starts at column tile mt * 128 / 32
+__device__ __forceinline__ void exact_tile(int tile, int nt, int gram, int& mt, int& ct) {
+  mt = 0;
+  if (!gram) {
+    mt = tile / nt;
+    ct = tile - mt * nt;
+    return;
   }
-  u = p;
+  constexpr int step = BM / (XBN / 2);
+  while (tile >= nt - mt * step) {
+    tile -= nt - mt * step;
+    ++mt;
+  }
+  ct = mt * step + tile;
 }
 
 __global__ void __launch_bounds__(XTHREADS, 1)
     tc_exact_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb,
-                    int M, int N, int kr, int ldk, const int* __restrict__ ea,
-                    const int* __restrict__ eb, double* C, long ldc, long sc, int accumulate,
-                    int* err) {
-  constexpr uint32_t A_BYTES = BM * 128, B_BYTES = XBN * 128;
-  constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
+                    int M, int N, int ldk, int nst, int per, int gram, const int* __restrict__ ea,
+                    const int* __restrict__ eb, double2* C, long ldc, long sc, int accumulate,
+                    longlong2* part, int* err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024 - (su32(smem_raw) & 1023)) & 1023);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + XSTAGES * STAGE_BYTES);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + XSTAGES * XSTAGE_BYTES);
   uint64_t* empty = full + XSTAGES;
-  uint64_t* tfull = empty + XSTAGES;   // [2] accumulator buffer ready for the drain
-  uint64_t* tempty = tfull + 2;        // [2] accumulator buffer drained
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(tempty + 2);
+  uint64_t* gfull = empty + XSTAGES;   // [XS] accumulator of a weight ready for the drain
+  uint64_t* gempty = gfull + XS;       // [XS] drained
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(gempty + XS);
   int* abort_flag = reinterpret_cast<int*>(tslot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n0 = blockIdx.x * XBN, m0 = blockIdx.y * BM, bz = blockIdx.z;
-  const int nkb = (kr + 63) / 64;                  // k-blocks per slice pair
-  const int nch = (nkb + XCHUNK - 1) / XCHUNK;     // exact chunks per slice pair
-  const int total_chunks = XPAIRS * nch;
+  const int nt = (N + XBN - 1) / XBN, bz = blockIdx.z;
+  int mt, ct;
+  exact_tile(blockIdx.x, nt, gram, mt, ct);
+  const int n0 = ct * XBN, m0 = mt * BM;
+  const int st0 = blockIdx.y * per, stages = min(nst, st0 + per) - st0;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < XSTAGES; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&tfull[b], 1);
-      mbar_init(&tempty[b], 4);
+    for (int g = 0; g < XS; ++g) {
+      mbar_init(&gfull[g], 1);
+      mbar_init(&gempty[g], 8);
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -467,7 +525,7 @@ __global__ void __launch_bounds__(XTHREADS, 1)
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      su32(tslot)),
-                 "r"(2 * XBN)
+                 "r"(512)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -478,23 +536,19 @@ __global__ void __launch_bounds__(XTHREADS, 1)
 
   if (warp == 0) {
     if (lane == 0) {
-      int it = 0;
-      for (int ch = 0; ch < total_chunks && !*(volatile int*)abort_flag; ++ch) {
-        const int pair = ch / nch, c = ch % nch;
-        int t, u;
-        pair_tu(pair, t, u);
-        const int kb1 = min(nkb, (c + 1) * XCHUNK);
-        for (int kb = c * XCHUNK; kb < kb1; ++kb, ++it) {
-          const int s = it % XSTAGES;
-          if (it >= XSTAGES && !mbar_wait(&empty[s], ((it / XSTAGES) - 1) & 1)) {
-            atomicExch(abort_flag, 1);
-            atomicExch(err, 11);
-            break;
-          }
-          uint8_t* sa = smem + s * STAGE_BYTES;
-          mbar_expect_tx(&full[s], STAGE_BYTES);
-          tma_load_3d(sa, &ma, &full[s], t * ldk + kb * 64, m0, bz);
-          tma_load_3d(sa + A_BYTES, &mb, &full[s], u * ldk + kb * 64, n0, bz);
+      for (int it = 0; it < stages && !*(volatile int*)abort_flag; ++it) {
+        const int s = it % XSTAGES;
+        if (it >= XSTAGES && !mbar_wait(&empty[s], ((it / XSTAGES) - 1) & 1)) {
+          atomicExch(abort_flag, 1);
+          atomicExch(err, 11);
+          break;
+        }
+        uint8_t* sa = smem + s * XSTAGE_BYTES;
+        mbar_expect_tx(&full[s], XSTAGE_BYTES);
+        const int c0 = (st0 + it) * XKB;
+        for (int t = 0; t < XS; ++t) {
+          tma_load_3d(sa + t * XA_SLICE, &ma, &full[s], t * ldk + c0, m0, bz);
+          tma_load_3d(sa + XS * XA_SLICE + t * XB_SLICE, &mb, &full[s], t * ldk + c0, n0, bz);
         }
       }
     }
@@ -502,84 +556,95 @@ __global__ void __launch_bounds__(XTHREADS, 1)
   } else if (warp == 1) {
     if (lane == 0) {
       constexpr uint32_t id = idesc<2>(XBN);
-      int it = 0;
-      for (int ch = 0; ch < total_chunks; ++ch) {
-        const int c = ch % nch, buf = ch & 1;
-        // the drain of chunk ch - 2 must have emptied this accumulator buffer
-        if (ch >= 2 && !mbar_wait(&tempty[buf], ((ch >> 1) - 1) & 1)) {
+      bool ok = true;
+      for (int it = 0; it < stages && ok; ++it) {
+        const int s = it % XSTAGES, d = it / XDRAIN;
+        const bool first = it % XDRAIN == 0, last = it % XDRAIN == XDRAIN - 1 || it == stages - 1;
+        if (!mbar_wait(&full[s], (it / XSTAGES) & 1)) {
           atomicExch(abort_flag, 1);
           atomicExch(err, 12);
           break;
         }
         tc_fence_after();
-        const uint32_t td = tmem + buf * XBN;
-        const int kb1 = min(nkb, (c + 1) * XCHUNK);
-        bool ok = true;
-        for (int kb = c * XCHUNK; kb < kb1; ++kb, ++it) {
-          const int s = it % XSTAGES;
-          if (!mbar_wait(&full[s], (it / XSTAGES) & 1)) {
-            atomicExch(abort_flag, 1);
-            atomicExch(err, 13);
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t sa = su32(smem + s * STAGE_BYTES);
-          const uint64_t ad = sdesc(sa), bd = sdesc(sa + A_BYTES);
+        const uint32_t sa = su32(smem + s * XSTAGE_BYTES);
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            umma<2>(td, ad + 2 * kk, bd + 2 * kk, id, (kb > c * XCHUNK || kk) ? 1u : 0u);
-          umma_commit(&empty[s]);
+        for (int g = 0; g < XS; ++g) {
+          // the drain of the period before must have emptied this weight's accumulator
+          if (first && d > 0) {
+            if (!mbar_wait(&gempty[g], (d - 1) & 1)) {
+              atomicExch(abort_flag, 1);
+              atomicExch(err, 13);
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+          }
+#pragma unroll
+          for (int t = 0; t <= g; ++t) {
+            const uint64_t ad = sdesc64(sa + t * XA_SLICE),
+                           bd = sdesc64(sa + XS * XA_SLICE + (g - t) * XB_SLICE);
+#pragma unroll
+            for (int kk = 0; kk < 2; ++kk)
+              umma<2>(tmem + g * XBN, ad + 2 * kk, bd + 2 * kk, id,
+                      (first && t == 0 && kk == 0) ? 0u : 1u);
+          }
+          if (last) umma_commit(&gfull[g]);
         }
-        if (!ok) break;
-        umma_commit(&tfull[buf]);
+        if (ok) umma_commit(&empty[s]);
       }
     }
     __syncwarp();
   } else {
-    // drain warps: TMEM lanes 32 (warp % 4) .. +31 are tile rows
-    const int q = warp & 3;
+    // drain warps: TMEM lanes 32 (warp % 4) .. +31 are tile rows, columns 32 hf .. +31
+    const int q = warp & 3, hf = (warp - 2) >> 2;
     const int row = m0 + q * 32 + lane;
-    double acc[XBN];
+    long long hi[32], lo[32];
 #pragma unroll
-    for (int j = 0; j < XBN; ++j) acc[j] = 0.0;
+    for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
     bool ok = true;
-    for (int ch = 0; ch < total_chunks; ++ch) {
-      const int pair = ch / nch, buf = ch & 1;
-      int t, u;
-      pair_tu(pair, t, u);
-      bool ready = true;
-      if (lane == 0) ready = mbar_wait(&tfull[buf], (ch >> 1) & 1);
-      ready = __shfl_sync(0xffffffffu, ready ? 1 : 0, 0) != 0;
-      if (!ready || *(volatile int*)abort_flag) {
-        if (lane == 0 && !ready) atomicExch(err, 14);
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      const double w = ldexp(1.0, -(14 + 8 * (t + u)));
-      const uint32_t tw = tmem + ((uint32_t)(q * 32) << 16) + buf * XBN;
+    const int periods = (stages + XDRAIN - 1) / XDRAIN;
+    for (int d = 0; d < periods && ok; ++d) {
 #pragma unroll
-      for (int cb = 0; cb < XBN; cb += 32) {
+      for (int g = 0; g < XS; ++g) {
+        bool ready = true;
+        if (lane == 0) ready = mbar_wait(&gfull[g], d & 1);
+        ready = __shfl_sync(0xffffffffu, ready ? 1 : 0, 0) != 0;
+        if (!ready || *(volatile int*)abort_flag) {
+          if (lane == 0 && !ready) atomicExch(err, 14);
+          ok = false;
+          break;
+        }
+        tc_fence_after();
         float v[32];
-        tmem_ld32(tw + cb, v);
+        tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + g * XBN + hf * 32, v);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&gempty[g])) : "memory");
 #pragma unroll
-        for (int j = 0; j < 32; ++j) acc[cb + j] = fma(w, (double)v[j], acc[cb + j]);
+        for (int j = 0; j < 32; ++j) {
+          const long long x = (long long)__float2int_rn(v[j]) * (1 << (8 * (2 - g % 3)));
+          if (g < 3) hi[j] += x; else lo[j] += x;
+        }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&tempty[buf])) : "memory");
     }
     if (ok && row < M) {
-      const int er = ea[(long)bz * M + row];
-      double* cp = C + (long)bz * sc + (long)row * ldc;
+      const int c0 = n0 + hf * 32;
+      if (part) {
+        longlong2* pp = part + (((long)blockIdx.y * gridDim.z + bz) * M + row) * N;
 #pragma unroll
-      for (int j = 0; j < XBN; ++j) {
-        const int col = n0 + j;
-        if (col < N) {
-          const double v = ldexp(acc[j], er + eb[(long)bz * (N / 2) + col / 2]);
-          cp[col] = accumulate ? cp[col] + v : v;
-        }
+        for (int j = 0; j < 32; ++j)
+          if (c0 + j < N) pp[c0 + j] = make_longlong2(hi[j], lo[j]);
+      } else {
+        const int er = ea[(long)bz * M + row];
+        double2* cp = C + (long)bz * sc;
+#pragma unroll
+        for (int j = 0; j < 32; j += 2)
+          if (c0 + j < N) {
+            const int qc = (c0 + j) >> 1, eq = eb[(long)bz * (N / 2) + qc];
+            exact_store(cp, ldc, row, qc, exact_value(hi[j], lo[j], er, eq),
+                        exact_value(hi[j + 1], lo[j + 1], er, eq), gram, accumulate);
+          }
       }
     }
   }
@@ -587,60 +652,117 @@ __global__ void __launch_bounds__(XTHREADS, 1)
   __syncthreads();
   if (warp == 0) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                 "r"(2 * XBN)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512)
                  : "memory");
   }
 }
 
-// e[b][r] = exponent of the largest |Re|, |Im| of row r of X (X[r][c] = src[b*sb + r*s_r +
-// c*s_c], c < kc): max = f 2^e with f in [0.5, 1); 0 for an all-zero row.
-template <typename TIN>
-__global__ void __launch_bounds__(256) row_exp_kernel(int rows, int kc, const TIN* __restrict__ src,
-                                                     long s_r, long s_c, long sb, int* e) {
-  __shared__ double red[256];
-  const int r = blockIdx.x, b = blockIdx.y;
-  const TIN* x = src + (long)b * sb + (long)r * s_r;
-  double mx = 0.0;
-  for (int c = threadIdx.x; c < kc; c += blockDim.x) {
-    const TIN v = x[(long)c * s_c];
-    mx = fmax(mx, fmax(fabs((double)v.x), fabs((double)v.y)));
-  }
-  red[threadIdx.x] = mx;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + s]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    int ex = 0;
-    if (red[0] > 0.0) frexp(red[0], &ex);
-    e[(long)b * rows + r] = ex;
+// Sum of the K slices' integer parts (exact, so in any order) and the output.
+__global__ void __launch_bounds__(256) exact_finish_kernel(int M, int n, int batch, int splits,
+                                                           int gram, const longlong2* part,
+                                                           const int* __restrict__ ea,
+                                                           const int* __restrict__ eb, double2* C,
+                                                           long ldc, long sc, int accumulate) {
+  const long total = (long)batch * M * n;
+  for (long e = blockIdx.x * 256L + threadIdx.x; e < total; e += 256L * gridDim.x) {
+    const int q = (int)(e % n), i = (int)((e / n) % M), b = (int)(e / ((long)n * M));
+    if (gram && q < i) continue;
+    long long rh = 0, rl = 0, ih = 0, il = 0;
+    for (int s = 0; s < splits; ++s) {
+      const longlong2* p = part + (((long)s * batch + b) * M + i) * 2 * n + 2 * q;
+      const longlong2 x = p[0], y = p[1];
+      rh += x.x;
+      rl += x.y;
+      ih += y.x;
+      il += y.y;
+    }
+    const int er = ea[(long)b * M + i], eq = eb[(long)b * n + q];
+    exact_store(C + (long)b * sc, ldc, i, q, exact_value(rh, rl, er, eq), exact_value(ih, il, er, eq),
+                gram, accumulate);
   }
 }
 
-// XS integer slices of x in (-1, 1): x = 2^-7 sum_t 2^-8t q_(t+1) + r, |q| <= 128,
-// |r| <= 2^-(8 XS) (every step is exact in FP32: y - rint(y) is a multiple of y's last bit).
-template <typename F>
-__device__ __forceinline__ void slice_all(F x, float* q) {
-  F y = x * (F)128;
-#pragma unroll
-  for (int t = 0; t < XS; ++t) {
-    const F r = rint(y);
-    q[t] = (float)r;
-    y = (y - r) * (F)256;
+// e[b][r] = exponent of the largest |Re|, |Im| of row r of X (X[r][c] = src[b*sb + r*s_r +
+// c*s_c], c < kc): max = f 2^e with f in [0.5, 1); kNonFinite for a row with an infinity or a NaN.
+// e is set to a value below kZeroRow before.  Reads are coalesced whichever index is
+// contiguous: a warp per row (8 rows of a CTA), or the 32 rows of a CTA across the lanes; the
+// columns are shared out over grid.y.
+template <typename TIN>
+__global__ void __launch_bounds__(256) row_exp_kernel(int rows, int kc, const TIN* __restrict__ src,
+                                                     long s_r, long s_c, long sb, int cols, int* e) {
+  using F = decltype(TIN().x);
+  __shared__ F red[8][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool c_fast = s_c == 1;
+  const int c0 = blockIdx.y * cols, c1 = min(kc, c0 + cols);
+  const int r = c_fast ? blockIdx.x * 8 + warp : blockIdx.x * 32 + lane;
+  F mx = 0, bad = 0;
+  if (r < rows) {
+    const TIN* x = src + (long)blockIdx.z * sb + (long)r * s_r;
+    for (int c = c0 + (c_fast ? lane : warp); c < c1; c += c_fast ? 32 : 8) {
+      const TIN v = x[(long)c * s_c];
+      bad += (v.x - v.x) + (v.y - v.y);     // 0, or NaN for a non-finite entry
+      const F a = fabs(v.x), b = fabs(v.y);
+      mx = a > mx ? a : mx;
+      mx = b > mx ? b : mx;
+    }
   }
+  if (!(bad == 0)) mx = INFINITY;
+  if (c_fast) {
+    for (int o = 16; o > 0; o >>= 1) {
+      const F y = __shfl_xor_sync(0xffffffffu, mx, o);
+      mx = y > mx ? y : mx;
+    }
+    if (lane > 0) return;
+  } else {
+    red[warp][lane] = mx;
+    __syncthreads();
+    if (warp > 0) return;
+    for (int k = 1; k < 8; ++k) mx = red[k][lane] > mx ? red[k][lane] : mx;
+  }
+  if (r < rows && mx > 0) {
+    int ex = kNonFinite;
+    if (!isinf(mx)) frexp(mx, &ex);
+    atomicMax(&e[(long)blockIdx.z * rows + r], ex);
+  }
+}
+
+// x 2^(47 - e) rounded to an integer, for |x| < 2^e: shifts of the significand.
+__device__ __forceinline__ long long shift_round(long long m, int s) {
+  return s >= 0 ? m << s : s < -62 ? 0 : (m + (1LL << (-s - 1))) >> -s;
+}
+__device__ __forceinline__ long long to_fixed(float x, int e) {
+  const int b = __float_as_int(x), ex = (b >> 23) & 255;
+  const long long q = shift_round((b & 0x7fffff) | (ex ? 0x800000 : 0), (ex ? ex : 1) - 150 + 47 - e);
+  return b < 0 ? -q : q;
+}
+__device__ __forceinline__ long long to_fixed(double x, int e) {
+  const long long b = __double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 2047);
+  const long long q = shift_round((b & 0xfffffffffffffLL) | (ex ? 1LL << 52 : 0),
+                                  (ex ? ex : 1) - 1075 + 47 - e);
+  return b < 0 ? -q : q;
+}
+// The XS slices of x: q = sum_t 2^(8 (XS - 1 - t)) d[t], d[t] in [-128, 127] for t > 0 and the
+// first in [-128, 128], so x = 2^-7 sum_t 2^-8t d[t] 2^e to 2^-48 2^e.
+__device__ __forceinline__ void slice_all(long long q, float* d) {
+#pragma unroll
+  for (int t = XS - 1; t > 0; --t) {
+    const int x = (int)((q + 128) & 255) - 128;
+    d[t] = (float)x;
+    q = (q - x) >> 8;
+  }
+  d[0] = (float)(int)q;
 }
 
 // Sliced packing (layout as pack_kernel, with XS K-segments of ldk elements, one per slice;
-// the segment tails up to ldk are written as zeros): row scale 2^-e[b][r] (A side) or the
-// column scale of the complex column (B side, rows 2r and 2r+1).
+// the segment tails up to ldk are zeros): row scale 2^-e[b][r] (A side) or the column scale of
+// the complex column (B side, rows 2r and 2r+1).
 template <typename TIN>
 __global__ void __launch_bounds__(PT * 8)
     pack_exact_kernel(int rows, int kc, const TIN* __restrict__ src, long s_r, long s_c, long sb,
                       int conj, int side, const int* __restrict__ e, __nv_bfloat16* __restrict__ out,
                       long ldo, long so, int ldk) {
-  using F = decltype(TIN().x);
   __shared__ TIN tile[PT][PT + 1];
   const int r0 = blockIdx.y * PT, c0 = blockIdx.x * PT, b = blockIdx.z;
   const int tx = threadIdx.x, ty = threadIdx.y;
@@ -661,43 +783,142 @@ __global__ void __launch_bounds__(PT * 8)
   __syncthreads();
   for (int qq = ty; qq < PT; qq += 8) {
     const int r = r0 + qq, c = c0 + tx;
-    if (r >= rows || c >= kc) continue;
+    if (r >= rows || 2 * c >= ldk) continue;
     const int er = e[(long)b * rows + r];
     const TIN v = tile[qq][tx];
     float qr[XS], qi[XS];
-    slice_all<F>(ldexp(v.x, -er), qr);
-    slice_all<F>(ldexp(v.y, -er), qi);
-    if (side == 0) {
-      __nv_bfloat16* o = out + (long)b * so + (long)r * ldo + 2L * c;
+    const bool live = er != kNonFinite && er > kZeroRow;
+    slice_all(live ? to_fixed(v.x, er) : 0, qr);
+    slice_all(live ? to_fixed(v.y, er) : 0, qi);
+    __nv_bfloat162* o0 = reinterpret_cast<__nv_bfloat162*>(
+        out + (long)b * so + (side == 0 ? (long)r : 2L * r) * ldo + 2L * c);
+    __nv_bfloat162* o1 = o0 + ldo / 2;
 #pragma unroll
-      for (int t = 0; t < XS; ++t) {
-        o[t * ldk] = __float2bfloat16_rn(qr[t]);
-        o[t * ldk + 1] = __float2bfloat16_rn(qi[t]);
-      }
-    } else {
-      __nv_bfloat16* o0 = out + (long)b * so + (2L * r) * ldo + 2L * c;
-      __nv_bfloat16* o1 = o0 + ldo;
-#pragma unroll
-      for (int t = 0; t < XS; ++t) {
-        o0[t * ldk] = __float2bfloat16_rn(qr[t]);
-        o0[t * ldk + 1] = __float2bfloat16_rn(-qi[t]);
-        o1[t * ldk] = __float2bfloat16_rn(qi[t]);
-        o1[t * ldk + 1] = __float2bfloat16_rn(qr[t]);
+    for (int t = 0; t < XS; ++t) {
+      if (side == 0) {
+        o0[t * (ldk / 2)] = __floats2bfloat162_rn(qr[t], qi[t]);
+      } else {
+        o0[t * (ldk / 2)] = __floats2bfloat162_rn(qr[t], -qi[t]);
+        o1[t * (ldk / 2)] = __floats2bfloat162_rn(qi[t], qr[t]);
       }
     }
   }
 }
 
-// Zero the K-segment tails [kr, ldk) of every slice of every packed row (rows_out rows).
-__global__ void zero_tails_kernel(long rows_out, int kr, int ldk, __nv_bfloat16* out, long ldo) {
-  const int w = ldk - kr;
-  const long total = rows_out * XS * w;
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total;
-       e += (long)gridDim.x * blockDim.x) {
-    const long r = e / (XS * w);
-    const int t = (int)((e / w) % XS), j = (int)(e % w);
-    out[r * ldo + (long)t * ldk + kr + j] = __float2bfloat16_rn(0.f);
+// Exponents and sliced packing of both operands of a product in one launch (blockIdx.z = operand
+// x batch + b), for K short enough that one CTA takes PR rows whole: a pass for the exponents,
+// then PW columns at a time through shared memory.  Two launches each, row_exp_kernel and
+// pack_exact_kernel share long rows out over more CTAs.
+constexpr int PR = 16, PW = 128;
+constexpr int kFusedPackK = 256;
+struct PackOp {
+  const void* src;
+  __nv_bfloat16* out;
+  int* e;
+  long s_r, s_c, sb, so;
+  int rows, conj, side;
+};
+template <typename TIN>
+__device__ void pack_rows(const PackOp& op, int b, int kc, int ldk, unsigned char* raw) {
+  using F = decltype(TIN().x);
+  TIN(*tile)[PW + 1] = reinterpret_cast<TIN(*)[PW + 1]>(raw);
+  __shared__ F red[16][PR];
+  __shared__ int s_e[PR];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int r0 = blockIdx.x * PR;
+  if (r0 >= op.rows) return;
+  const TIN* src = static_cast<const TIN*>(op.src) + (long)b * op.sb;
+  const bool c_fast = op.s_c == 1;
+  // largest |Re|, |Im| of a row, INFINITY for one with a non-finite entry
+  auto take = [](const TIN v, F& mx, F& bad) {
+    bad += (v.x - v.x) + (v.y - v.y);
+    const F a = fabs(v.x), c = fabs(v.y);
+    mx = a > mx ? a : mx;
+    mx = c > mx ? c : mx;
+  };
+  if (c_fast) {
+#pragma unroll
+    for (int k = 0; k < PR / 8; ++k) {
+      const int r = r0 + warp + 8 * k;
+      F mx = 0, bad = 0;
+      if (r < op.rows) {
+        const TIN* x = src + (long)r * op.s_r;
+#pragma unroll 4
+        for (int c = lane; c < kc; c += 32) take(x[c], mx, bad);
+      }
+      if (!(bad == 0)) mx = INFINITY;
+      for (int o = 16; o > 0; o >>= 1) {
+        const F y = __shfl_xor_sync(0xffffffffu, mx, o);
+        mx = y > mx ? y : mx;
+      }
+      if (lane == 0) red[0][warp + 8 * k] = mx;
+    }
+    __syncthreads();
+  } else {
+    const int r = r0 + tid % PR;
+    F mx = 0, bad = 0;
+    if (r < op.rows) {
+#pragma unroll 4
+      for (int c = tid / PR; c < kc; c += 16) take(src[(long)r * op.s_r + (long)c * op.s_c], mx, bad);
+    }
+    if (!(bad == 0)) mx = INFINITY;
+    red[tid / PR][tid % PR] = mx;
+    __syncthreads();
+    if (tid < PR) {
+      for (int k = 1; k < 16; ++k) mx = red[k][tid] > mx ? red[k][tid] : mx;
+      red[0][tid] = mx;
+    }
+    __syncthreads();
   }
+  if (tid < PR && r0 + tid < op.rows) {
+    const F mx = red[0][tid];
+    int ex = 2 * kZeroRow;
+    if (isinf(mx)) ex = kNonFinite;
+    else if (mx > 0) frexp(mx, &ex);
+    s_e[tid] = ex;
+    op.e[(long)b * op.rows + r0 + tid] = ex;
+  }
+  for (int c0 = 0; 2 * c0 < ldk; c0 += PW) {
+    __syncthreads();
+    for (int i = tid; i < PR * PW; i += 256) {
+      const int r = c_fast ? i / PW : i % PR, c = c_fast ? i % PW : i / PR;
+      TIN v;
+      v.x = 0;
+      v.y = 0;
+      if (r0 + r < op.rows && c0 + c < kc) {
+        v = src[(long)(r0 + r) * op.s_r + (long)(c0 + c) * op.s_c];
+        if (op.conj) v.y = -v.y;
+      }
+      tile[r][c] = v;
+    }
+    __syncthreads();
+    for (int i = tid; i < PR * PW; i += 256) {
+      const int r = i / PW, c = c0 + i % PW;
+      if (r0 + r >= op.rows || 2 * c >= ldk) continue;
+      const int er = s_e[r];
+      const TIN v = tile[r][i % PW];
+      float qr[XS], qi[XS];
+      const bool live = er != kNonFinite && er > kZeroRow;
+      slice_all(live ? to_fixed(v.x, er) : 0, qr);
+      slice_all(live ? to_fixed(v.y, er) : 0, qi);
+      const long ldo = (long)XS * ldk;
+      __nv_bfloat162* o0 = reinterpret_cast<__nv_bfloat162*>(
+          op.out + (long)b * op.so + (long)(r0 + r) * (op.side ? 2 : 1) * ldo + 2L * c);
+      __nv_bfloat162* o1 = o0 + ldo / 2;
+#pragma unroll
+      for (int t = 0; t < XS; ++t) {
+        o0[t * (ldk / 2)] = __floats2bfloat162_rn(qr[t], op.side ? -qi[t] : qi[t]);
+        if (op.side) o1[t * (ldk / 2)] = __floats2bfloat162_rn(qi[t], qr[t]);
+      }
+    }
+  }
+}
+template <typename TA, typename TB>
+__global__ void __launch_bounds__(256) pack_both_kernel(const PackOp a, const PackOp b, int batch,
+                                                        int kc, int ldk) {
+  __shared__ __align__(16) unsigned char raw[PR * (PW + 1) * sizeof(double2)];
+  if ((int)blockIdx.z < batch) pack_rows<TB>(b, blockIdx.z, kc, ldk, raw);
+  else pack_rows<TA>(a, blockIdx.z - batch, kc, ldk, raw);
 }
 
 // Real operand packing for the BF16 core: out[r][c] = bf16(src[r*s_r + c*s_c]), r < rows,
@@ -740,19 +961,21 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-// 3-D K-major map: dims {K, rows, batch}, box {128 bytes of K, box_rows, 1}.
+// 3-D K-major map: dims {K, rows, batch}, box {row_bytes of K, box_rows, 1}, swizzled over the
+// row's 128 or 64 bytes.
 bool make_map(CUtensorMap* map, int elt, const void* base, long k, long rows, long ld, long sb,
-              int batch, int box_rows) {
+              int batch, int box_rows, int row_bytes = 128) {
   auto fn = encode_fn();
   if (!fn) return false;
   const cuuint64_t dims[3] = {(cuuint64_t)k, (cuuint64_t)rows, (cuuint64_t)batch};
   const cuuint64_t strides[2] = {(cuuint64_t)ld * elt,
                                  (cuuint64_t)(batch > 1 ? sb : rows * ld) * elt};
-  const cuuint32_t box[3] = {(cuuint32_t)(128 / elt), (cuuint32_t)box_rows, 1};
+  const cuuint32_t box[3] = {(cuuint32_t)(row_bytes / elt), (cuuint32_t)box_rows, 1};
   const cuuint32_t es[3] = {1, 1, 1};
   CUresult r = fn(map, elt == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
                   3, const_cast<void*>(base), dims, strides, box, es,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
@@ -899,22 +1122,77 @@ cudaError_t tc_cgemm(cudaStream_t st, int mode, int opa, int opb, int m, int n, 
   return cudaSuccess;
 }
 
-// ---- exact products: C (complex FP64) = op(A) op(B), FP32 complex A and B
-static size_t exact_bytes(long m, long n, long kc, int batch) {
-  const long ldk = (2 * kc + 63) / 64 * 64;
-  const size_t a = ((size_t)batch * m * XS * ldk * 2 + 255) & ~(size_t)255;
+// ---- exact products: C (complex FP64) = op(A) op(B), FP32 or FP64 complex A and B
+namespace {
+struct ExactPlan {
+  int tiles, nst, per, splits;
+};
+// Tiles of the output and the K split: the number of slices (at least 4 stages each) with the
+// fewest stages on the busiest of the 152 SMs, fewer slices where it makes no difference.
+ExactPlan exact_plan(long m, long n, long kc, int batch, bool gram) {
+  ExactPlan p;
+  const long mt = (m + BM - 1) / BM, nt = (2 * n + XBN - 1) / XBN;
+  long tiles = mt * nt;
+  if (gram) {
+    tiles = 0;
+    for (long i = 0; i < mt; ++i) tiles += nt - i * (BM / (XBN / 2));
+  }
+  p.tiles = (int)tiles;
+  p.nst = (int)((2 * kc + XKB - 1) / XKB);
+  p.per = p.nst;
+  p.splits = 1;
+  long best = -1;
+  for (int s = 1; s <= 16 && (s == 1 || p.nst >= 4 * s); ++s) {
+    const int per = (p.nst + s - 1) / s, used = (p.nst + per - 1) / per;
+    // 4: prologue and drain of a CTA; 8: the launch that adds the slices
+    const long cost = ((tiles * batch * used + 151) / 152) * (per + 4) + (used > 1 ? 8 : 0);
+    if (best < 0 || cost < best) {
+      best = cost;
+      p.per = per;
+      p.splits = used;
+    }
+  }
+  return p;
+}
+// op(B) = op(A)^+ of the same data: the product is Hermitian
+template <typename TA, typename TB>
+bool is_gram(int opa, int opb, int m, int n, const TA* A, long lda, long sa, const TB* B, long ldb,
+             long sb) {
+  return std::is_same<TA, TB>::value && (const void*)A == (const void*)B && lda == ldb && sa == sb &&
+         m == n && ((opa == OP_C && opb == OP_N) || (opa == OP_N && opb == OP_C));
+}
+size_t exact_bytes(long m, long n, long kc, int batch, bool gram) {
+  const long ldk = (2 * kc + XKB - 1) / XKB * XKB;
+  const size_t a = gram ? 0 : ((size_t)batch * m * XS * ldk * 2 + 255) & ~(size_t)255;
   const size_t b = ((size_t)batch * 2 * n * XS * ldk * 2 + 255) & ~(size_t)255;
-  return a + b + ((size_t)batch * (m + n) * sizeof(int) + 256);
+  const ExactPlan p = exact_plan(m, n, kc, batch, gram);
+  const size_t part = p.splits > 1 ? (size_t)p.splits * batch * m * 2 * n * sizeof(longlong2) : 0;
+  return a + b + part + (((size_t)batch * (m + n) * sizeof(int) + 255) & ~(size_t)255) + 256;
+}
+}  // namespace
+
+// Time of an exact product against the same product on the FP64 CUDA cores.  The slice kernel
+// costs a fixed part (exponents, packing, output) and its stages on the busiest SM, 1.05 us each;
+// FP64 runs at 304 FMA per clock over the chip.  Both sides as measured: the Gram 41 x 41 x 1968 takes
+// 25 us in FP64 and 36 us plus its packing in slices, the Gram 400 x 400 x 5043 2.6 ms and 74 us.
+bool tc_exact_faster(long m, long n, long k, int batch, bool gram) {
+  const ExactPlan p = exact_plan(m, n, k, batch, gram);
+  const double waves = (double)((p.tiles * (long)batch * p.splits + 151) / 152);
+  const double elems = (double)batch * k * ((gram ? 0 : m) + 2.0 * n);   // packed complex entries
+  const double tc = (k <= kFusedPackK ? 12.0 : 24.0) + (p.splits > 1 ? 8.0 : 0.0) +
+                    1.05 * waves * (p.per + 4) + elems * 24.0 / 3.0e6;
+  const double fp64 = 8.0 + 1.2 * 4.0 * m * n * (double)k * batch * (gram ? 0.5 : 1.0) / (304.0 * 2.0e3);
+  return tc < fp64;
 }
 
 size_t tc_exact_ws_bytes(long m, long n, long k, int batch) {
-  return exact_bytes(m, n, std::min<long>(k, 4096), batch);
+  return exact_bytes(m, n, std::min<long>(k, 4096), batch, false);
 }
 
 cudaError_t tc_exact_init() {
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      tc_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-      (int)(XSTAGES * (BM + XBN) * 128 + 1024 + 256));
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(tc_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(XSTAGES * XSTAGE_BYTES + 1024 + 256));
   return attr;
 }
 
@@ -922,12 +1200,13 @@ template <typename TA, typename TB>
 cudaError_t tc_cgemm_exact(cudaStream_t st, int opa, int opb, int m, int n, int k, const TA* A,
                            long lda, long sa, const TB* B, long ldb, long sb, double2* C, long ldc,
                            long sc, int batch, void* ws, size_t ws_bytes, int* err) {
+  const bool gram = is_gram(opa, opb, m, n, A, lda, sa, B, ldb, sb);
   if (m <= 0 || n <= 0 || batch <= 0) return cudaSuccess;
   if (k <= 0) return cudaErrorInvalidValue;
   long kc = k;
-  while (kc > 64 && exact_bytes(m, n, kc, batch) > ws_bytes) kc = (kc + 1) / 2;
+  while (kc > 64 && exact_bytes(m, n, kc, batch, gram) > ws_bytes) kc = (kc + 1) / 2;
   if (kc < k) kc = std::max(64L, kc / 64 * 64);
-  if (exact_bytes(m, n, kc, batch) > ws_bytes) return cudaErrorMemoryAllocation;
+  if (exact_bytes(m, n, kc, batch, gram) > ws_bytes) return cudaErrorMemoryAllocation;
   long sra, sca, srb, scb;
   int cja, cjb;
   op_strides(0, opa, lda, &sra, &sca, &cja);
@@ -935,44 +1214,72 @@ cudaError_t tc_cgemm_exact(cudaStream_t st, int opa, int opb, int m, int n, int 
   MPDO_CUDA_TRY(tc_exact_init());
   for (long k0 = 0; k0 < k; k0 += kc) {
     const int kn = (int)std::min<long>(kc, k - k0);
-    const int kr = 2 * kn;
-    const int ldk = (kr + 63) / 64 * 64;
+    const ExactPlan pl = exact_plan(m, n, kn, batch, gram);
+    const int ldk = (2 * kn + XKB - 1) / XKB * XKB;
     const long ldo = (long)XS * ldk;
     char* p = static_cast<char*>(ws);
     __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(p);
-    p += ((size_t)batch * m * ldo * 2 + 255) & ~(size_t)255;
+    if (!gram) p += ((size_t)batch * m * ldo * 2 + 255) & ~(size_t)255;
     __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(p);
     p += ((size_t)batch * 2 * n * ldo * 2 + 255) & ~(size_t)255;
-    int* ea = reinterpret_cast<int*>(p);
-    int* eb = ea + (size_t)batch * m;
+    int* eb = reinterpret_cast<int*>(p);
+    int* ea = gram ? eb : eb + (size_t)batch * n;
+    p += ((size_t)batch * (m + n) * sizeof(int) + 255) & ~(size_t)255;
+    longlong2* part = pl.splits > 1 ? reinterpret_cast<longlong2*>(p) : nullptr;
+    auto exps = [&](auto* x, int rows, long sr, long s_c, long s_b, int* e) {
+      const int rb = s_c == 1 ? (rows + 7) / 8 : (rows + 31) / 32;
+      // enough column slices for about two CTAs per SM, at least 64 columns each
+      int sl = std::max(1, std::min((kn + 63) / 64, 304 / std::max(1, rb * batch)));
+      const int cols = (kn + sl - 1) / sl;
+      sl = (kn + cols - 1) / cols;
+      row_exp_kernel<<<dim3(rb, sl, batch), 256, 0, st>>>(rows, kn, x, sr, s_c, s_b, cols, e);
+    };
+    // exponents and packing as launches of their own, over column slices and tiles
+    auto pack = [&](auto* x, int rows, long sr, long s_c, long s_b, int cj, int side, const int* e,
+                    __nv_bfloat16* o) {
+      pack_exact_kernel<<<dim3((ldk / 2 + PT - 1) / PT, (rows + PT - 1) / PT, batch), dim3(PT, 8), 0,
+                          st>>>(rows, kn, x, sr, s_c, s_b, cj, side, e, o, ldo,
+                                (side ? 2L : 1L) * rows * ldo, ldk);
+    };
     const TA* a0 = A + k0 * sca;
     const TB* b0 = B + k0 * scb;
-    row_exp_kernel<TA><<<dim3(m, batch), 256, 0, st>>>(m, kn, a0, sra, sca, sa, ea);
-    row_exp_kernel<TB><<<dim3(n, batch), 256, 0, st>>>(n, kn, b0, srb, scb, sb, eb);
-    dim3 blk(PT, 8);
-    pack_exact_kernel<TA><<<dim3((kn + PT - 1) / PT, (m + PT - 1) / PT, batch), blk, 0, st>>>(
-        m, kn, a0, sra, sca, sa, cja, 0, ea, pa, ldo, (long)m * ldo, ldk);
-    pack_exact_kernel<TB><<<dim3((kn + PT - 1) / PT, (n + PT - 1) / PT, batch), blk, 0, st>>>(
-        n, kn, b0, srb, scb, sb, cjb, 1, eb, pb, ldo, 2L * n * ldo, ldk);
-    count_launch(4);
-    if (ldk > kr) {
-      zero_tails_kernel<<<256, 256, 0, st>>>((long)batch * m, kr, ldk, pa, ldo);
-      zero_tails_kernel<<<256, 256, 0, st>>>((long)batch * 2 * n, kr, ldk, pb, ldo);
-      count_launch(2);
+    if (kn <= kFusedPackK) {
+      const PackOp ob{b0, pb, eb, srb, scb, sb, 2L * n * ldo, n, cjb, 1};
+      const PackOp oa{a0, pa, ea, sra, sca, sa, (long)m * ldo, m, cja, 0};
+      pack_both_kernel<TA, TB><<<dim3((std::max(gram ? 0 : m, n) + PR - 1) / PR, 1, gram ? batch : 2 * batch),
+                                 256, 0, st>>>(oa, ob, batch, kn, ldk);
+      count_launch();
+    } else {
+      // exponents below kZeroRow until a row's entries raise them
+      MPDO_CUDA_TRY(cudaMemsetAsync(eb, 0x80, (size_t)batch * (gram ? n : m + n) * sizeof(int), st));
+      exps(b0, n, srb, scb, sb, eb);
+      pack(b0, n, srb, scb, sb, cjb, 1, eb, pb);
+      if (!gram) {
+        exps(a0, m, sra, sca, sa, ea);
+        pack(a0, m, sra, sca, sa, cja, 0, ea, pa);
+      }
+      count_launch(gram ? 2 : 4);
     }
     MPDO_CUDA_TRY(cudaGetLastError());
     CUtensorMap ma, mb;
-    if (!make_map(&ma, 2, pa, ldo, m, ldo, (long)m * ldo, batch, BM) ||
-        !make_map(&mb, 2, pb, ldo, 2L * n, ldo, 2L * n * ldo, batch, XBN))
+    if (!make_map(&ma, 2, pa, ldo, m, gram ? 2 * ldo : ldo, (gram ? 2L * n : m) * ldo, batch, BM,
+                  XKB * 2) ||
+        !make_map(&mb, 2, pb, ldo, 2L * n, ldo, 2L * n * ldo, batch, XBN, XKB * 2))
       return cudaErrorInvalidValue;
-    dim3 grid((2 * n + XBN - 1) / XBN, (m + BM - 1) / BM, batch);
-    const size_t smem = XSTAGES * (BM + XBN) * 128 + 1024 + 256;
-    tc_exact_kernel<<<grid, XTHREADS, smem, st>>>(ma, mb, m, 2 * n, kr, ldk, ea, eb,
-                                                  reinterpret_cast<double*>(C), 2 * ldc, 2 * sc,
-                                                  k0 > 0 ? 1 : 0, err);
+    const size_t smem = XSTAGES * XSTAGE_BYTES + 1024 + 256;
+    const int acc = k0 > 0 ? 1 : 0;
+    tc_exact_kernel<<<dim3(pl.tiles, pl.splits, batch), XTHREADS, smem, st>>>(
+        ma, mb, m, 2 * n, ldk, pl.nst, pl.per, gram ? 1 : 0, ea, eb, C, ldc, sc, acc, part, err);
     count_launch();
     g_tc_launches.fetch_add(1, std::memory_order_relaxed);
     MPDO_CUDA_TRY(cudaGetLastError());
+    if (part) {
+      const long total = (long)batch * m * n;
+      exact_finish_kernel<<<(int)std::min<long>((total + 255) / 256, 4096), 256, 0, st>>>(
+          m, n, batch, pl.splits, gram ? 1 : 0, part, ea, eb, C, ldc, sc, acc);
+      count_launch();
+      MPDO_CUDA_TRY(cudaGetLastError());
+    }
   }
   return cudaSuccess;
 }

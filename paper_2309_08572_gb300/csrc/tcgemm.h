@@ -56,12 +56,15 @@ size_t tc_cgemm_ws_bytes(int mode, long m, long n, long k, int batch);
 // Complex FP64 C[b] = op(A[b]) op(B[b]) of complex FP32 or FP64 operands (TA, TB: float2 or
 // double2), carried to ~2^-48 of each operand row's largest entry and summed in FP64
 // (error-free BF16 slices on the tensor cores; tcgemm.cu).  Long K is processed in pieces
-// that fit ws, added in FP64.
+// that fit ws, added in FP64.  Where op(B) = op(A)^+ of the same data, C is Hermitian and only its
+// upper half is computed (and mirrored).
 template <typename TA, typename TB>
 cudaError_t tc_cgemm_exact(cudaStream_t st, int opa, int opb, int m, int n, int k, const TA* A,
                            long lda, long sa, const TB* B, long ldb, long sb, double2* C, long ldc,
                            long sc, int batch, void* ws, size_t ws_bytes, int* err);
 size_t tc_exact_ws_bytes(long m, long n, long k, int batch);
+// Whether the product is estimated faster there than on the FP64 CUDA cores.
+bool tc_exact_faster(long m, long n, long k, int batch, bool gram);
 // One-time kernel attribute setup of tc_cgemm_exact; call it before capturing a stream that
 // will run the first exact product of the process.
 cudaError_t tc_exact_init();
