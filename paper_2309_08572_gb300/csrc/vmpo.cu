@@ -8,7 +8,7 @@
 // chain, as in the MPDO engine):
 //   theta  = A_i A_j                       ((9 D_l) x (9 D_r), [l][eta_i][eta_j][r])
 //   theta' = S theta on (eta_i, eta_j)     (81 x 81 superoperator, batched over l)
-//   theta' = U Lambda V^+                  (eigenpairs of theta' theta'^+, FP64 Jacobi;
+//   theta' = U Lambda V^+                  (eigenpairs of theta' theta'^+;
 //                                           Lambda = sqrt of the eigenvalues above the cut,
 //                                           V^+ = Lambda^-1 U^+ theta')
 //   T_k    = (L (x) tau)^T U[:, k] * V^+[k, :] (tau (x) R)   (trace environment: L, R the
@@ -241,6 +241,13 @@ struct mpdo_vmpo_s {
   void* eigmem = nullptr;
   // tensor-core form (mpdo_vmpo_set_precision 1): exact-slice products and the mixed solver
   int tc = 0;
+  // factor of the Gram and the graded solver's workspace (see split)
+  double2 *L = nullptr, *Gs = nullptr, *Zs = nullptr;
+  MixWork gradw;
+  void* gradmem = nullptr;
+  struct PcOut { int r; int pad; double resid; };
+  PcOut* dpc = nullptr;
+  PcOut* hpc = nullptr;   // pinned
   MixWork mixw;
   void* mixmem = nullptr;
   void* tcws = nullptr;
@@ -364,6 +371,40 @@ int reverse(mpdo_vmpo h) {
   return MPDO_OK;
 }
 
+// Eigenpairs of the Gram in h->H (n x n): *nval eigenvalues in h->lam, descending, and *nvec
+// eigenvectors in the columns of h->U (row stride *nvec).  Through the pivoted Cholesky factor
+// H ~ L L^+, stopping at a hundredth of the cut, and the graded solver on L^+ L, as in the MPDO
+// update; a rank beyond the solver's size takes the full solve: FP64 Jacobi, or in the
+// tensor-core form the mixed solver, resolved below a tenth of the cut.  (Eight sites at chi 16,
+// n = 144: the FP64 Jacobi took 28 ms a solve.)  One host synchronisation.
+int split(mpdo_vmpo h, int n, int* nval, int* nvec) {
+  cudaStream_t st = h->st;
+  if (n <= 1024) {
+    const int rmax = std::min(n, kGradedMax);
+    const double tol = std::max(0.01 * h->cut2, 1e-16);
+    VK(pchol<double>(st, n, h->H, rmax, tol, h->L, kGradedMax, &h->dpc->r, &h->dpc->resid));
+    VK(cudaMemcpyAsync(h->hpc, h->dpc, sizeof(*h->hpc), cudaMemcpyDeviceToHost, st));
+    VK(cudaStreamSynchronize(st));
+    const int r = h->hpc->r;
+    if (r < 1) return vfail(h, MPDO_ERR_NUMERIC, "vmpo: zero or non-finite state");
+    if (!(r >= rmax && r < n && h->hpc->resid > tol)) {
+      *nval = r;
+      *nvec = h->mode == 1 ? r : std::min(r, h->chi);
+      VK(cgemm_gram<double>(st, 0, r, n, h->L, kGradedMax, h->Zs, r));
+      VK(heig_graded(st, r, h->Zs, r, h->Gs, r, h->lam, h->gradw, true));
+      VK(u64(h, OP_N, OP_N, n, *nvec, r, h->L, kGradedMax, 0, h->Gs, r, 0, h->U, *nvec, 0, 1));
+      return MPDO_OK;
+    }
+  }
+  *nval = *nvec = n;
+  if (h->tc)
+    VK(heig_mixed(st, n, h->H, n, h->U, n, h->lam, 0.1 * h->cut2, h->mixw, nullptr, nullptr,
+                  h->mode == 1 ? 0 : h->chi + 1));
+  else
+    VK(heig<double>(st, n, h->H, n, h->U, n, h->lam, h->eig, 30));
+  return MPDO_OK;
+}
+
 // one update on storage bond (i, i+1), centre at i; the centre moves to i+1
 int update(mpdo_vmpo h, int i, const VOp& op, mpdo_trunc_stats* acc) {
   cudaStream_t st = h->st;
@@ -375,30 +416,33 @@ int update(mpdo_vmpo h, int i, const VOp& op, mpdo_trunc_stats* acc) {
   VK(u64(h, OP_N, OP_N, rows, cols, dm, h->site(i), dm, 0, h->site(i + 1), cols, 0, h->th, cols,
          0, 1));
   VK(u64(h, OP_N, OP_N, 81, dr, 81, h->S, 81, 0, h->th, dr, 81L * dr, h->th2, dr, 81L * dr, dl));
-  // Schmidt decomposition through the Gram theta' theta'^+: FP64 Jacobi, or in the
-  // tensor-core form the mixed solver (FP32 Jacobi levels, FP64 refinement) resolved below
-  // a tenth of the cut -- in naive mode only the chi + 1 leading pairs (PPT needs T and
-  // Lambda of every Schmidt pair)
-  VK(u64(h, OP_N, OP_C, rows, rows, cols, h->th2, cols, 0, h->th2, cols, 0, h->H, rows, 0, 1));
-  if (h->tc)
-    VK(heig_mixed(st, rows, h->H, rows, h->U, rows, h->lam, 0.1 * h->cut2, h->mixw, nullptr,
-                  nullptr, h->mode == 1 ? 0 : h->chi + 1));
-  else
-    VK(heig<double>(st, rows, h->H, rows, h->U, rows, h->lam, h->eig, 30));
+  // Schmidt decomposition through the Gram theta' theta'^+.  PPT needs T and Lambda of every
+  // Schmidt pair, naive mode those that can be kept.
+  int nval = 0, nvec = 0;
+  if (h->tc) {
+    VK(u64(h, OP_N, OP_C, rows, rows, cols, h->th2, cols, 0, h->th2, cols, 0, h->H, rows, 0, 1));
+  } else {
+    VK(cgemm_gram<double>(st, 1, rows, cols, h->th2, cols, h->H, rows));
+  }
+  int rc = split(h, rows, &nval, &nvec);
+  if (rc) return rc;
+  const int ldu = nvec;
   // trace environment: tl = (L (x) tau)^T U ; W = U^+ theta' (row k = Lambda_k V^+_k) ;
   // trw = W (tau (x) R)
+  VK(u64(h, OP_C, OP_N, nvec, cols, rows, h->U, ldu, 0, h->th2, cols, 0, h->th, cols, 0, 1));
+  if (h->mode == 1) {
+    count_launch();
+    trace_vec_kernel<<<nblk(rows), 256, 0, st>>>(dl, h->Lenv + (long)i * h->chi, 0, h->x);
+    VK(cudaGetLastError());
+    VK(g64(st, OP_N, OP_N, 1, nvec, rows, h->x, rows, 0, h->U, ldu, 0, h->tl, nvec, 0, 1));
+    count_launch();
+    trace_vec_kernel<<<nblk(cols), 256, 0, st>>>(dr, h->Renv + (long)(i + 1) * h->chi, 1,
+                                                  h->x + rows);
+    VK(cudaGetLastError());
+    VK(g64(st, OP_N, OP_N, nvec, 1, cols, h->th, cols, 0, h->x + rows, 1, 0, h->tr, 1, 0, 1));
+  }
   count_launch();
-  trace_vec_kernel<<<nblk(rows), 256, 0, st>>>(dl, h->Lenv + (long)i * h->chi, 0, h->x);
-  VK(cudaGetLastError());
-  VK(g64(st, OP_N, OP_N, 1, rows, rows, h->x, rows, 0, h->U, rows, 0, h->tl, rows, 0, 1));
-  VK(u64(h, OP_C, OP_N, rows, cols, rows, h->U, rows, 0, h->th2, cols, 0, h->th, cols, 0, 1));
-  count_launch();
-  trace_vec_kernel<<<nblk(cols), 256, 0, st>>>(dr, h->Renv + (long)(i + 1) * h->chi, 1,
-                                                h->x + rows);
-  VK(cudaGetLastError());
-  VK(g64(st, OP_N, OP_N, rows, 1, cols, h->th, cols, 0, h->x + rows, 1, 0, h->tr, 1, 0, 1));
-  count_launch();
-  vmpo_cut_kernel<<<1, 32, 0, st>>>(rows, h->lam, h->tl, h->tr, h->cut2, h->chi, h->mode, h->sv,
+  vmpo_cut_kernel<<<1, 32, 0, st>>>(nval, h->lam, h->tl, h->tr, h->cut2, h->chi, h->mode, h->sv,
                                     h->lt, h->dsc);
   VK(cudaGetLastError());
   VK(cudaMemcpyAsync(h->hsc, h->dsc, sizeof(VScalars), cudaMemcpyDeviceToHost, st));
@@ -408,14 +452,14 @@ int update(mpdo_vmpo h, int i, const VOp& op, mpdo_trunc_stats* acc) {
   if (h->hsc->flags & 1) return vfail(h, MPDO_ERR_NUMERIC, "vmpo: zero or non-finite state");
   const int keep = h->hsc->keep;
   // A_i <- U_keep ; A_{i+1} <- diag(Lambda~ / Lambda) W_keep
-  VK(cudaMemcpy2DAsync(h->site(i), keep * sizeof(double2), h->U, rows * sizeof(double2),
+  VK(cudaMemcpy2DAsync(h->site(i), keep * sizeof(double2), h->U, ldu * sizeof(double2),
                        keep * sizeof(double2), rows, cudaMemcpyDeviceToDevice, st));
   count_launch();
   scale_rows_kernel<<<nblk((long)keep * cols), 256, 0, st>>>(keep, cols, h->th, cols, h->lt, h->sv,
                                                              h->site(i + 1), cols);
   VK(cudaGetLastError());
   h->bond[i + 1] = keep;
-  int rc = left_env_step(h, i);
+  rc = left_env_step(h, i);
   if (rc) return rc;
   if (acc) {
     acc->disc_bond_w += h->hsc->disc;
@@ -503,12 +547,19 @@ int mpdo_vmpo_create(int n_sites, int chi_max, int use_ppt, double sv_cutoff,
       (rc = valloc(h, (void**)&h->sv, n9 * sizeof(double))) ||
       (rc = valloc(h, (void**)&h->lt, n9 * sizeof(double))) ||
       (rc = valloc(h, (void**)&h->dsc, sizeof(VScalars))) ||
+      (rc = A((void**)&h->L, (size_t)n9 * kGradedMax)) ||
+      (rc = A((void**)&h->Gs, (size_t)kGradedMax * kGradedMax)) ||
+      (rc = A((void**)&h->Zs, (size_t)kGradedMax * kGradedMax)) ||
+      (rc = valloc(h, (void**)&h->dpc, sizeof(*h->dpc))) ||
+      (rc = valloc(h, &h->gradmem, mix_work_bytes((int)std::min<long>(n9, kGradedMax)))) ||
       (rc = valloc(h, &h->eigmem, eig_work_bytes<double>((int)n9)))) {
     mpdo_vmpo_destroy(hp.release());
     return rc;
   }
   eig_work_bind<double>(h->eig, h->eigmem, (int)n9);
-  if (cudaMallocHost((void**)&h->hsc, sizeof(VScalars)) != cudaSuccess) {
+  mix_work_bind(h->gradw, h->gradmem, (int)std::min<long>(n9, kGradedMax));
+  if (cudaMallocHost((void**)&h->hsc, sizeof(VScalars)) != cudaSuccess ||
+      cudaMallocHost((void**)&h->hpc, sizeof(*h->hpc)) != cudaSuccess) {
     cudaGetLastError();
     mpdo_vmpo_destroy(hp.release());
     return vfail(nullptr, MPDO_ERR_OOM, "vmpo: pinned host allocation");
@@ -720,6 +771,7 @@ int mpdo_vmpo_destroy(mpdo_vmpo h) {
   mix_work_release(h->mixw);
   for (void* p : h->allocs) cudaFree(p);
   if (h->hsc) cudaFreeHost(h->hsc);
+  if (h->hpc) cudaFreeHost(h->hpc);
   if (h->htcerr) cudaFreeHost(h->htcerr);
   if (h->own_stream) cudaStreamDestroy(h->st);
   delete h;
