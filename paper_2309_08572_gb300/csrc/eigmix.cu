@@ -511,7 +511,9 @@ __global__ void __launch_bounds__(RT * RT) refine_kernel(int m, int n, const dou
 // sizes: with lam_i > lam_j the FP32 sweeps leave S_ij ~ delta sqrt(lam_i lam_j) and G_ij ~
 // delta sqrt(lam_j / lam_i), so the correction E is graded as well and a pair is separated when
 // |S_ij - lam G_ij| sqrt(lam_i / lam_j) < emax |lam_i - lam_j| and its relative gap exceeds the
-// rounding of the products (100 m eps_64).  No pair is left to another level.
+// rounding of the products (100 m eps_64).  No pair is left to another level.  A corrected pair
+// keeps about the square of its angle, so in the final pass neighbours whose angle is above
+// kGradedRitz (relative gaps below ~1e-3) go to the Ritz step, which is exact within its run.
 //
 // The step is bound by FP64: a pair costs two dot products of length m and one division.  So
 // one CTA takes a 4 x 4 block of pairs above the diagonal, forms its S, G and the diagonal
@@ -524,6 +526,7 @@ __global__ void __launch_bounds__(RT * RT) refine_kernel(int m, int n, const dou
 // the factor that lifts an eigenvector of L^+ L to one of L L^+.
 constexpr int GT = 4;
 constexpr int kSgeThreads = 128;
+constexpr double kGradedRitz = 1e-6;
 __device__ __forceinline__ double col_scale(double lam, int scaled) {
   return !scaled ? 1.0 : lam > 0.0 ? rsqrt(lam) : 0.0;
 }
@@ -601,9 +604,9 @@ __global__ void __launch_bounds__(kSgeThreads) sge_kernel(int m, const double2* 
       const double d = lj - li, mx = fmax(fabs(li), fabs(lj)), mn = fmin(li, lj);
       const double2 nij = make_double2(s.x - lj * g.x, s.y - lj * g.y);
       const double2 nji = make_double2(s.x - li * g.x, -(s.y - li * g.y));
-      const double lim = emax * emax * d * d * mn;
-      const bool newton = mn > 0.0 && fabs(d) > 100.0 * m * 1.1e-16 * mx &&
-                          cabs2(nij) * mx < lim && cabs2(nji) * mx < lim;
+      const double lim = d * d * mn, ang = fmax(cabs2(nij), cabs2(nji)) * mx;   // ang / lim: angle^2
+      const bool apart = mn > 0.0 && fabs(d) > 100.0 * m * 1.1e-16 * mx;
+      const bool newton = apart && ang < emax * emax * lim;
       if (newton) {
         const double r = 1.0 / d;
         IE[(long)i * m + j] = cscale(nij, r * cj);
@@ -612,7 +615,7 @@ __global__ void __launch_bounds__(kSgeThreads) sge_kernel(int m, const double2* 
         IE[(long)i * m + j] = cscale(g, -0.5 * cj);
         IE[(long)j * m + i] = cscale(cconj(g), -0.5 * ci);
       }
-      if (j == i + 1) sep[i] = newton;
+      if (j == i + 1) sep[i] = apart && ang < kGradedRitz * kGradedRitz * lim;
     }
   }
   if (!final_pass) return;
@@ -1049,7 +1052,7 @@ cudaError_t heig_graded(cudaStream_t st, int n, const double2* a, long lda, doub
     return cgemm<double>(st, OP_N, OP_N, n, n, n, x, ldx, sx, y, ldy, 0, c, ldc, sc, batch,
                          make_double2(1, 0), make_double2(0, 0));
   };
-  MPDO_CUDA_TRY(heig_graded_f32(st, n, a, lda, cur + n, l2, wk.glog, nullptr));
+  MPDO_CUDA_TRY(heig_graded_f32(st, n, a, lda, cur + n, l2, wk.glog));
   MPDO_CUDA_TRY(mul(a, lda, 0, cur + n, l2, cur, l2, 0, 1));
   const int nt = (n + GT - 1) / GT, grid = nt * (nt + 1) / 2;
   const size_t sm = 16 * sizeof(double2) * (size_t)n;

@@ -64,13 +64,12 @@ cudaError_t heig_smem_f32(cudaStream_t st, int n, const cx<RI>* a, long lda, cx<
 
 // FP32 sweeps of a graded Hermitian PSD matrix (n <= kGradedMax, FP64, rounded on load): z =
 // its approximate eigenvectors (columns, descending eigenvalues, FP32 accuracy relative to
-// each pair), to be refined.  mem: graded_log_bytes(n) of device scratch; *meta_out (may be
-// NULL): device ints, logged rounds, sweeps, rotations.
-constexpr int kGradedMax = 168;     // np x (np + 1) complex64 fit one SM's shared memory
+// each pair), to be refined.  mem: graded_log_bytes(n) of device scratch.
+constexpr int kGradedMax = 168;     // np x np complex64 fit one SM's shared memory
 constexpr int kGradedSweeps = 15;
 size_t graded_log_bytes(int n);
 cudaError_t heig_graded_f32(cudaStream_t st, int n, const double2* a, long lda, double2* z,
-                            long ldz, void* mem, int** meta_out);
+                            long ldz, void* mem);
 
 // Workspace of the mixed-precision eigensolver (capacity n_cap).
 struct MixGraphs;   // captured level sequences (eigmix.cu)

@@ -489,167 +489,222 @@ __global__ void __launch_bounds__(SJ_THREADS) jacobi_smem_kernel(int n, int np,
 // square is left, which the FP64 refinement removes (L^+ L of the update's Grams, r = 13..73:
 // 3 to 5 sweeps, mixing angles of 1e-6 to 5e-5 left, 1e-10 after one refinement pass).
 //
-// One CTA, bound by the issue slots of one SM: a round touches every 2 x 2 block.  Hence
-// only the blocks above the diagonal are computed (their mirror images are written, not
-// computed), the pair's own block is set by the thread that found its rotation, rounds in
-// which nothing rotates cost one barrier, and the eigenvectors are not accumulated here: the
-// rotations go to a log, which rot_apply_kernel replays on the rows of the identity, one warp
-// per row on as many SMs as there are rows.  Without the accumulator a matrix of 168 fits the
-// shared memory of an SM (118 with it).
+// One CTA; a round touches every 2 x 2 block, so it is bound by shared-memory traffic and issue
+// slots of one SM, and below ~60 rows by the latency of its two phases.  Hence:
+//  - only the blocks above the diagonal exist;
+//  - the matrix is stored by the seats of the round-robin tournament, not by index: pair k sits
+//    on seats T_k and B_k, block (a, b) is the same four words in every round, and after a
+//    rotation each entry is written to its seats of the next round (players move one seat).  A
+//    thread keeps its blocks, whose addresses it computes once; four planes (T or B row, T or B
+//    column) make every access contiguous across lanes;
+//  - the eigenvectors are not accumulated here: the rotations go to a log, which
+//    rot_apply_kernel replays on the rows of the identity on other SMs.  Without the
+//    accumulator a matrix of 168 fits the shared memory of an SM (118 with it).
+// By index, with looked-up pairs and mirrored writes, a round of n = 118 took 1.2 us.  The pairs
+// have warps of their own: a warp with blocks as well made all others wait for its rotations.
 // In place of one-sided FP64 sweeps on the factor (3.6 ms a Gram on one SM's FP64 pipe) and of
 // the levels of the mixed solver (5 rounds of ~9 launches): 40 atoms, two layers in FP64 719 ->
 // 84 ms, 100 atoms, three layers in the mixed tensor-core form 1488 -> 791 ms.
 constexpr float kGradedRel = 2e-6f;
-constexpr float kGradedStop = 3e-3f;
+constexpr float kGradedStop = 1e-3f;
 constexpr int kGradedHalf = kGradedMax / 2;
+constexpr int kGradedThreads = 512;      // block threads, besides the warps of the pairs ...
+constexpr int kGradedFew = 416;          // ... and with more than 4 blocks each (128 registers)
 
-// log: (c, Re s e, Im s e, 0) of pair k of the i-th logged round at log[i * np / 2 + k];
-// rid[i]: its index in the round-robin order; meta: logged rounds, sweeps, rotations;
+// Seats: T_k = (0, k), B_k = (1, k).  T_0 stays; T_k moves to T_{k-1}, T_1 to B_0, B_k to
+// B_{k+1} and the last B to the last T.
+__device__ __forceinline__ void next_seat(int half, int& t, int& k) {
+  if (half == 1 || (t == 0 && k == 0)) return;
+  if (t == 0) {
+    if (k == 1) { t = 1; k = 0; } else { --k; }
+  } else {
+    if (k == half - 1) t = 0; else ++k;
+  }
+}
+// Player on a seat at the start of a sweep (m = 2 half - 1 moving players, player m on T_0).
+__device__ __forceinline__ int seat_player(int m, int t, int k) {
+  return t == 0 ? (k == 0 ? m : k) : (k == 0 ? 0 : m - k);
+}
+// Where the entry of seats (ta, ka), (tb, kb) goes after a round: its word (below 2^15), with bit
+// 15 set when it is stored conjugated.  Words: plane (row seat type, column seat type) of half x
+// half, then the pairs' own entries g_k = (T_k, B_k).
+__device__ __forceinline__ unsigned seat_target(int half, int ta, int ka, int tb, int kb) {
+  next_seat(half, ta, ka);
+  next_seat(half, tb, kb);
+  const unsigned conj = 0x8000u;
+  const int P = half * half;
+  if (ka == kb) return (4 * P + ka) | (ta == 0 ? 0u : conj);
+  if (ka < kb) return (ta * 2 + tb) * P + ka * half + kb;
+  return ((tb * 2 + ta) * P + kb * half + ka) | conj;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ void seat_store(float2* A, unsigned target, float2 z) {
+  z.y = __uint_as_float(__float_as_uint(z.y) ^ ((target << 16) & 0x80000000u));
+  A[target & 0x7fffu] = z;
+}
+
+// log: (c, Re s e, Im s e, rotated) of pair k of round i < *rounds at log[i * np / 2 + k];
 // perm[i]: column of the i-th largest diagonal entry.  A diagonal that is not finite is left
 // for the caller to find in the refined eigenvalues.
-template <int IT>
-__global__ void __launch_bounds__(1024) jacobi_graded_kernel(int n, int np,
-                                                             const double2* __restrict__ a,
-                                                             long lda, float4* log, int* rid,
-                                                             int* meta, int* perm, int max_sweeps) {
-  extern __shared__ float2 gj_a[];   // np x (np + 1): odd row stride, so columns are free of
-  const int ld = np + 1;             // bank conflicts too
+template <int IT>   // blocks of a thread
+__global__ void __launch_bounds__(IT > 4 ? kGradedFew + 96 : kGradedThreads + 96) jacobi_graded_kernel(
+    int n, int np, const double2* __restrict__ a, long lda, float4* log, int* rounds, int* perm,
+    int max_sweeps) {
+  extern __shared__ float2 gj_a[];   // four planes, then g
   __shared__ float4 s_rot[kGradedHalf];
-  __shared__ int2 s_pq[kGradedHalf];
-  __shared__ double s_red[32];
-  __shared__ unsigned s_max[2];
+  __shared__ float s_d[2][kGradedHalf];   // diagonal of T_k, B_k
+  __shared__ double s_red[kGradedThreads / 32 + 3];
+  __shared__ unsigned s_max;
   __shared__ float s_key[kGradedMax];
   const int tid = threadIdx.x, lane = tid & 31, nthr = blockDim.x;
-  const int half = np / 2, m = np - 1;
+  const int half = np / 2, m = np - 1, P = half * half;
   // a power of two brings the largest diagonal entry near 2^30: FP32 then holds the squares
   // of entries 16 decades below it
   double dm = 0.0;
   for (int i = tid; i < n; i += nthr) dm = fmax(dm, a[(long)i * lda + i].x);
   for (int o = 16; o > 0; o >>= 1) dm = fmax(dm, __shfl_xor_sync(0xffffffffu, dm, o));
   if (lane == 0) s_red[tid >> 5] = dm;
-  if (tid < 2) s_max[tid] = 0u;
   __syncthreads();
   for (int k = 0; k < (nthr >> 5); ++k) dm = fmax(dm, s_red[k]);
   const double sc = (dm > 0.0 && isfinite(dm)) ? ldexp(1.0, 30 - ilogb(dm)) : 1.0;
-  for (int e = tid; e < np * np; e += nthr) {
-    const int i = e / np, j = e - i * np;
-    float2 z = make_float2(0.f, 0.f);
-    if (i < n && j < n) {
-      const double2 t = a[(long)i * lda + j];
-      z = make_float2((float)(t.x * sc), (float)(t.y * sc));
-    }
-    gj_a[i * ld + j] = z;
+  auto entry = [&](int i, int j) {
+    if (i >= n || j >= n) return make_float2(0.f, 0.f);
+    const double2 t = a[(long)i * lda + j];
+    return make_float2((float)(t.x * sc), (float)(t.y * sc));
+  };
+  for (int e = tid; e < 4 * P; e += nthr) {
+    const int pl = e / P, ka = (e % P) / half, kb = e % half;
+    if (ka < kb) gj_a[e] = entry(seat_player(m, pl >> 1, ka), seat_player(m, pl & 1, kb));
   }
-  // the blocks (ka < kb) of this thread, the same in every round: row i of the folded
-  // triangle holds the blocks of pair i and then those of pair half - 1 - i
+  // the first warps take a pair a lane and nothing else: the others wait for their rotations
+  const int pt = (half + 31) / 32 * 32;
+  unsigned own_to = 0;                        // where the pair's own entry goes
+  float *al_to = nullptr, *be_to = nullptr;   // and its diagonal entries
+  if (tid < half) {
+    const int p = seat_player(m, 0, tid), q = seat_player(m, 1, tid);
+    gj_a[4 * P + tid] = entry(p, q);
+    s_d[0][tid] = entry(p, p).x;
+    s_d[1][tid] = entry(q, q).x;
+    own_to = seat_target(half, 0, tid, 1, tid);
+    int t = 0, k = tid;
+    next_seat(half, t, k);
+    al_to = &s_d[t][k];
+    t = 1;
+    k = tid;
+    next_seat(half, t, k);
+    be_to = &s_d[t][k];
+  }
+  // the blocks (ka < kb) of this thread: row i of the folded triangle holds the blocks of pair
+  // i and then those of pair half - 1 - i
   const int nb = half * (half - 1) / 2;
-  int bl[IT];
+  int ab[IT];          // ka | kb << 8, -1 for none; word ka half + kb in every plane
+  unsigned to[IT][2];  // targets of the four words, 16 bits each
 #pragma unroll
   for (int t = 0; t < IT; ++t) {
-    const int e = tid + t * nthr;
-    bl[t] = -1;
-    if (e < nb) {
+    const int e = tid - pt + t * (nthr - pt);
+    ab[t] = -1;
+    if (tid >= pt && e < nb) {
       const int i = e / (half - 1), j = e - i * (half - 1);
       const bool lo = j < half - 1 - i;
       const int ka = lo ? i : half - 1 - i, kb = lo ? i + 1 + j : half - i + (j - (half - 1 - i));
-      bl[t] = ka | (kb << 8);
+      ab[t] = ka | (kb << 8);
+      for (int q = 0; q < 2; ++q)
+        to[t][q] = seat_target(half, q, ka, 0, kb) | (seat_target(half, q, ka, 1, kb) << 16);
     }
   }
-  __syncthreads();
-  int logged = 0, rotated = 0, sweep = 0;
+  int sweep = 0;
   for (; sweep < max_sweeps; ++sweep) {
+    float worst = 0.f;   // the sweep's largest |g|^2 / (al be) of this thread's pair
+    if (tid == 0) s_max = 0u;
+    __syncthreads();
     for (int r = 0; r < m; ++r) {
-      int f = 0;
+      // phase 1: the rotation of every pair; the other warps fetch their blocks meanwhile
+      float2 x[IT][4];
       float4 rot = make_float4(1.f, 0.f, 0.f, 0.f);
-      if (tid < half) {
-        int p, q;
-        if (tid == 0) {
-          p = m;
-          q = r;
-        } else {
-          p = r + tid;
-          if (p >= m) p -= m;
-          q = r - tid;
-          if (q < 0) q += m;
+      float al = 0.f, be = 0.f, g2 = 0.f;
+      float2 g = make_float2(0.f, 0.f);
+      if (tid < pt) {
+        if (tid < half) {
+          g = gj_a[4 * P + tid];
+          al = s_d[0][tid];
+          be = s_d[1][tid];
+          g2 = cabs2(g);
+          if (g2 > kGradedRel * kGradedRel * al * be && g2 > 0.f) {
+            // with d = be - al and s = sqrt(d^2 + 4 |g|^2): c^2 = (|d| + s) / 2s and
+            // s e = sign(d) g / (s c).  Approximate roots (a few ulp): their error is that of
+            // the accumulated rotations' rounding, which the refinement removes.
+            const float d = be - al, s2 = fmaf(d, d, 4.f * g2);
+            const float rs = rsqrt_approx(s2), w = fmaf(s2, rs, fabsf(d)), c2 = 0.5f * w * rs;
+            const float ic = rsqrt_approx(c2), k = copysignf(rs * ic, d);
+            rot = make_float4(c2 * ic, k * g.x, k * g.y, 1.f);
+          }
+          s_rot[tid] = rot;
         }
-        if (p > q) { const int t = p; p = q; q = t; }
-        const float2 g = gj_a[p * ld + q];
-        const float al = gj_a[p * ld + p].x, be = gj_a[q * ld + q].x;
-        const float g2 = cabs2(g), ab = al * be;
-        f = g2 > kGradedRel * kGradedRel * ab && g2 > 0.f;
-        if (f) {
-          // approximate reciprocals and roots (a few ulp): their error is that of the
-          // accumulated rotations' rounding, which the refinement removes
-          const float rg = rsqrtf(g2), ag = g2 * rg, d = be - al, h = 2.f * ag;
-          const float s2 = d * d + h * h;
-          const float t = __fdividef(copysignf(h, d), fabsf(d) + s2 * rsqrtf(s2));
-          const float c = rsqrtf(fmaf(t, t, 1.f)), se = t * c * rg;
-          rot = make_float4(c, se * g.x, se * g.y, 1.f);
-          gj_a[p * ld + p] = make_float2(al - t * ag, 0.f);
-          gj_a[q * ld + q] = make_float2(be + t * ag, 0.f);
-          gj_a[p * ld + q] = make_float2(0.f, 0.f);
-          gj_a[q * ld + p] = make_float2(0.f, 0.f);
-        }
-        s_pq[tid] = make_int2(p, q);
-        s_rot[tid] = rot;
-        // the sweep's largest squared ratio (positive floats compare as integers)
-        const float ratio = f ? (ab > 0.f ? __fdividef(g2, ab) : 1.f) : 0.f;
-        const int left = half - (tid & ~31);   // pairs from this warp's first lane on
-        const unsigned mask = left >= 32 ? 0xffffffffu : (1u << left) - 1u;
-        const unsigned mx = __reduce_max_sync(mask, __float_as_uint(ratio));
-        if (lane == 0 && mx > 0u) atomicMax(&s_max[sweep & 1], mx);
+      } else {
+#pragma unroll
+        for (int t = 0; t < IT; ++t)
+          if (ab[t] >= 0) {
+            const float2* w = gj_a + (ab[t] & 255) * half + (ab[t] >> 8);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) x[t][q] = w[q * P];
+          }
       }
-      const int any = __syncthreads_count(f);
-      if (any == 0) continue;
-      rotated += any;
-      if (tid < half) log[(long)logged * half + tid] = rot;
-      if (tid == 0) rid[logged] = r;
-      ++logged;
+      __syncthreads();
+      // phase 2: rotate, and everything to its next seat
+      if (tid < half) {
+        if (rot.w != 0.f) {
+          const float d = be - al, s2 = fmaf(d, d, 4.f * g2);
+          const float dt = copysignf(__fdividef(2.f * g2, fmaf(s2, rsqrt_approx(s2), fabsf(d))), d);
+          const float pr = al * be;
+          worst = fmaxf(worst, pr > 0.f ? __fdividef(g2, pr) : 1.f);
+          al -= dt;
+          be += dt;
+          g = make_float2(0.f, 0.f);
+        }
+        *al_to = al;
+        *be_to = be;
+        seat_store(gj_a, own_to, g);
+        log[(long)(sweep * m + r) * half + tid] = rot;
+      }
 #pragma unroll
       for (int t = 0; t < IT; ++t) {
-        if (bl[t] < 0) continue;
-        const int ka = bl[t] & 255, kb = bl[t] >> 8;
-        const float4 ra = s_rot[ka], rb = s_rot[kb];
-        if (ra.w == 0.f && rb.w == 0.f) continue;
-        const int2 ia = s_pq[ka], ib = s_pq[kb];
-        const float2 sa = make_float2(ra.y, ra.z), sb = make_float2(rb.y, rb.z);
-        float2* rp = gj_a + ia.x * ld;
-        float2* rq = gj_a + ia.y * ld;
-        const float2 x0 = rp[ib.x], x1 = rp[ib.y], y0 = rq[ib.x], y1 = rq[ib.y];
-        // rows (pair a): p' = c x - s e y, q' = s conj(e) x + c y
-        const float2 u0 = csub(cscale(x0, ra.x), cmul(sa, y0));
-        const float2 u1 = csub(cscale(x1, ra.x), cmul(sa, y1));
-        const float2 w0 = cadd(cmulc(x0, sa), cscale(y0, ra.x));
-        const float2 w1 = cadd(cmulc(x1, sa), cscale(y1, ra.x));
-        // columns (pair b): p' = c x - s conj(e) y, q' = s e x + c y
-        const float2 z0 = csub(cscale(u0, rb.x), cmulc(u1, sb));
-        const float2 z1 = cadd(cmul(u0, sb), cscale(u1, rb.x));
-        const float2 z2 = csub(cscale(w0, rb.x), cmulc(w1, sb));
-        const float2 z3 = cadd(cmul(w0, sb), cscale(w1, rb.x));
-        rp[ib.x] = z0;
-        rp[ib.y] = z1;
-        rq[ib.x] = z2;
-        rq[ib.y] = z3;
-        float2* cp = gj_a + ib.x * ld;
-        float2* cq = gj_a + ib.y * ld;
-        cp[ia.x] = cconj(z0);
-        cq[ia.x] = cconj(z1);
-        cp[ia.y] = cconj(z2);
-        cq[ia.y] = cconj(z3);
+        if (ab[t] < 0) continue;
+        const float4 ra = s_rot[ab[t] & 255], rb = s_rot[ab[t] >> 8];
+        if (ra.w != 0.f || rb.w != 0.f) {
+          const float2 sa = make_float2(ra.y, ra.z), sb = make_float2(rb.y, rb.z);
+          // rows (pair a): T' = c T - s e B, B' = s conj(e) T + c B
+          const float2 u0 = csub(cscale(x[t][0], ra.x), cmul(sa, x[t][2]));
+          const float2 u1 = csub(cscale(x[t][1], ra.x), cmul(sa, x[t][3]));
+          const float2 w0 = cadd(cmulc(x[t][0], sa), cscale(x[t][2], ra.x));
+          const float2 w1 = cadd(cmulc(x[t][1], sa), cscale(x[t][3], ra.x));
+          // columns (pair b): T' = c T - s conj(e) B, B' = s e T + c B
+          x[t][0] = csub(cscale(u0, rb.x), cmulc(u1, sb));
+          x[t][1] = cadd(cmul(u0, sb), cscale(u1, rb.x));
+          x[t][2] = csub(cscale(w0, rb.x), cmulc(w1, sb));
+          x[t][3] = cadd(cmul(w0, sb), cscale(w1, rb.x));
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) seat_store(gj_a, to[t][q >> 1] >> (16 * (q & 1)), x[t][q]);
       }
       __syncthreads();
     }
-    // the last round's barrier made the sweep's largest ratio visible; the other slot is
-    // cleared for the sweep after the next, before anyone writes it
-    const float mx = __uint_as_float(s_max[sweep & 1]);
+    if (worst > 0.f) atomicMax(&s_max, __float_as_uint(worst));   // positive floats order as integers
     __syncthreads();
-    if (tid == 0) s_max[sweep & 1] = 0u;
+    const float mx = __uint_as_float(s_max);
+    __syncthreads();
     if (!(mx > kGradedStop * kGradedStop)) { ++sweep; break; }
   }
-  for (int i = tid; i < n; i += nthr) {
-    s_key[i] = gj_a[i * ld + i].x;
-    perm[i] = i;   // a valid index whatever the keys are (ranks collide on NaN)
+  // whole sweeps bring every player back to its first seat
+  if (tid < half) {
+    const int p = seat_player(m, 0, tid), q = seat_player(m, 1, tid);
+    if (p < n) s_key[p] = s_d[0][tid];
+    if (q < n) s_key[q] = s_d[1][tid];
   }
+  for (int i = tid; i < n; i += nthr) perm[i] = i;   // valid whatever the keys (NaN: ranks collide)
   __syncthreads();
   for (int i = tid; i < n; i += nthr) {
     const float key = s_key[i];
@@ -657,11 +712,7 @@ __global__ void __launch_bounds__(1024) jacobi_graded_kernel(int n, int np,
     for (int k = 0; k < n; ++k) rank += s_key[k] > key || (!(s_key[k] < key) && k < i);
     perm[rank < n ? rank : n - 1] = i;
   }
-  if (tid == 0) {
-    meta[0] = logged;
-    meta[1] = sweep;
-    meta[2] = rotated;
-  }
+  if (tid == 0) *rounds = sweep * m;
 }
 
 // Rows of the accumulated rotations, V = J_1 J_2 ... : the log replayed on rows of the identity
@@ -681,18 +732,16 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
 template <int KP>   // pairs of a lane
 __global__ void __launch_bounds__(32 * kRotWarps) rot_apply_kernel(int n, int np,
                                                                    const float4* __restrict__ log,
-                                                                   const int* __restrict__ rid,
-                                                                   const int* __restrict__ meta,
+                                                                   const int* __restrict__ nrounds,
                                                                    const int* __restrict__ perm,
                                                                    double2* z, long ldz) {
   __shared__ float2 rows[kRotWarps][kGradedMax];
   __shared__ __align__(16) float4 buf[2][kRotChunk][32 * KP];
-  __shared__ int ids[2][kRotChunk];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int row = blockIdx.x * kRotWarps + warp;
   const bool live = row < n;
   float2* v = rows[warp];
-  const int half = np / 2, m = np - 1, rounds = meta[0];
+  const int half = np / 2, m = np - 1, rounds = *nrounds;
   for (int c = lane; c < np; c += 32) v[c] = make_float2(c == row ? 1.f : 0.f, 0.f);
   auto fetch = [&](int i0, int b) {
     const int cnt = min(kRotChunk, rounds - i0);
@@ -700,7 +749,6 @@ __global__ void __launch_bounds__(32 * kRotWarps) rot_apply_kernel(int n, int np
       const int i = e / half, k = e - i * half;
       cp_async16(&buf[b][i][k], &log[(long)(i0 + i) * half + k]);
     }
-    if (threadIdx.x < cnt) ids[b][threadIdx.x] = rid[i0 + threadIdx.x];
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   if (rounds > 0) fetch(0, 0);
@@ -713,17 +761,17 @@ __global__ void __launch_bounds__(32 * kRotWarps) rot_apply_kernel(int n, int np
     }
     __syncthreads();
     const int cnt = min(kRotChunk, rounds - i0);
-    for (int i = 0; live && i < cnt; ++i) {
-      const int r = ids[b][i];
+    int r = i0 % m;
+    for (int i = 0; live && i < cnt; ++i, r = r + 1 == m ? 0 : r + 1) {
 #pragma unroll
       for (int t = 0; t < KP; ++t) {
         const int k = lane + 32 * t;
         if (k >= half) continue;
         const float4 rot = buf[b][i][k];
-        int p = k == 0 ? m : r + k, q = k == 0 ? r : r - k;
+        if (rot.w == 0.f) continue;
+        int p = k == 0 ? m : r + k, q = k == 0 ? r : r - k;   // the players of T_k and B_k
         if (k && p >= m) p -= m;
         if (q < 0) q += m;
-        if (p > q) { const int x = p; p = q; q = x; }
         const float2 x = v[p], y = v[q], se = make_float2(rot.y, rot.z);
         v[p] = csub(cscale(x, rot.x), cmulc(y, se));
         v[q] = cadd(cmul(x, se), cscale(y, rot.x));
@@ -783,52 +831,50 @@ template cudaError_t heig_smem_f32<double, float>(cudaStream_t, int, const doubl
 
 size_t graded_log_bytes(int n) {
   const size_t np = n + (n & 1);
-  return kGradedSweeps * (np - 1) * (np / 2 * sizeof(float4) + sizeof(int)) + 256 +
-         (np + 8) * sizeof(int);
+  return kGradedSweeps * (np - 1) * (np / 2) * sizeof(float4) + 256 + (np + 8) * sizeof(int);
 }
 
 cudaError_t heig_graded_f32(cudaStream_t st, int n, const double2* a, long lda, double2* z,
-                            long ldz, void* mem, int** meta_out) {
+                            long ldz, void* mem) {
   if (n < 1 || n > kGradedMax) return cudaErrorInvalidValue;
   const int np = n + (n & 1), half = np / 2, rounds = kGradedSweeps * (np - 1);
   float4* log = static_cast<float4*>(mem);
-  int* rid = reinterpret_cast<int*>(log + (size_t)rounds * half);
-  int* perm = rid + rounds;
-  int* meta = perm + np;
-  const size_t sm = (size_t)np * (np + 1) * sizeof(float2);
+  int* perm = reinterpret_cast<int*>(log + (size_t)rounds * half);
+  int* nrounds = perm + np;
+  const size_t sm = ((size_t)np * np + half) * sizeof(float2);
   const int nb = half * (half - 1) / 2;
-  const int thr = std::min(1024, std::max(96, (nb + 31) / 32 * 32));
-  const int it = (nb + thr - 1) / thr;   // at most 4 (nb <= 3486)
+  const int bthr = nb > 4 * kGradedThreads ? kGradedFew
+                                           : std::min(kGradedThreads, std::max(32, (nb + 31) / 32 * 32));
+  const int it = (nb + bthr - 1) / bthr;   // at most 9 (nb <= 3486)
+  const int thr = bthr + (half + 31) / 32 * 32;
   auto launch = [&](auto kern) -> cudaError_t {
-    kern<<<1, thr, sm, st>>>(n, np, a, lda, log, rid, meta, perm, kGradedSweeps);
+    kern<<<1, thr, sm, st>>>(n, np, a, lda, log, nrounds, perm, kGradedSweeps);
     return cudaGetLastError();
   };
   // opt in to the largest size, once per instantiation
-  constexpr int kMaxSmem = kGradedMax * (kGradedMax + 1) * (int)sizeof(float2);
   static const cudaError_t attr = [] {
-    cudaError_t e = cudaFuncSetAttribute(jacobi_graded_kernel<1>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(jacobi_graded_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kMaxSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(jacobi_graded_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kMaxSmem);
+    constexpr int kMaxSmem = (kGradedMax * kGradedMax + kGradedHalf) * (int)sizeof(float2);
+    auto set = [](auto kern) {
+      return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    };
+    cudaError_t e = set(jacobi_graded_kernel<1>);
+    if (e == cudaSuccess) e = set(jacobi_graded_kernel<2>);
+    if (e == cudaSuccess) e = set(jacobi_graded_kernel<4>);
+    if (e == cudaSuccess) e = set(jacobi_graded_kernel<9>);
     return e;
   }();
   MPDO_CUDA_TRY(attr);
   count_launch(2);
   MPDO_CUDA_TRY(it <= 1   ? launch(jacobi_graded_kernel<1>)
                 : it <= 2 ? launch(jacobi_graded_kernel<2>)
-                          : launch(jacobi_graded_kernel<4>));
+                : it <= 4 ? launch(jacobi_graded_kernel<4>)
+                          : launch(jacobi_graded_kernel<9>));
   auto apply = [&](auto kern) {
-    kern<<<(n + kRotWarps - 1) / kRotWarps, 32 * kRotWarps, 0, st>>>(n, np, log, rid, meta, perm, z,
-                                                                   ldz);
+    kern<<<(n + kRotWarps - 1) / kRotWarps, 32 * kRotWarps, 0, st>>>(n, np, log, nrounds, perm, z, ldz);
   };
   if (half <= 32) apply(rot_apply_kernel<1>);
   else if (half <= 64) apply(rot_apply_kernel<2>);
   else apply(rot_apply_kernel<3>);
-  if (meta_out) *meta_out = meta;
   return cudaGetLastError();
 }
 
