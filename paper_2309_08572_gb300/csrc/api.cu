@@ -128,6 +128,7 @@ struct mpdo_ctx {
   void* wAcM = nullptr;      // polar-corrected left factor in FP64 (mixed only)
   StepScalars* dsc = nullptr;
   StepScalars* hsc = nullptr;  // pinned
+  double* henergy = nullptr;   // pinned: energy()'s results
   double* dtrace = nullptr;    // trace of the state, carried in FP64 across updates
   double htrace0 = 1.0;        // its initial value (host copy, source of the upload)
   DevStats* dstats = nullptr;
@@ -1078,10 +1079,7 @@ int energy(mpdo_ctx* h, double J, double hx, double bz, double out[7]) {
   TD* F = ebuf[1] + 6 * env;
   TD* G = F + 6 * fsz;
   // initial envs (1x1): E0 = 1, EZ = 0, E1 = 0 for both automata
-  TD init[6] = {one<double>(), zero<double>(), zero<double>(),
-                one<double>(), zero<double>(), zero<double>()};
-  for (int a = 0; a < 6; ++a)
-    CK(cudaMemcpyAsync(ebuf[0] + a * env, &init[a], sizeof(TD), cudaMemcpyHostToDevice, st));
+  PO(energy_init(st, env, ebuf[0]));
   int cur = 0;
   for (int s = 0; s < h->n; ++s) {
     const int dl = h->bond[s], k = h->kd[s], dr = h->bond[s + 1];
@@ -1096,16 +1094,14 @@ int energy(mpdo_ctx* h, double J, double hx, double bz, double out[7]) {
                6));
     cur = 1 - cur;
   }
-  TD res[6];
-  for (int a = 0; a < 6; ++a)
-    CK(cudaMemcpyAsync(&res[a], ebuf[cur] + a * env, sizeof(TD), cudaMemcpyDeviceToHost, st));
-  // the trace carried in FP64 by the updates (the norm the truncations keep)
-  double cnorm = 0;
-  CK(cudaMemcpyAsync(&cnorm, h->dtrace, sizeof(double), cudaMemcpyDeviceToHost, st));
+  // the six results and the trace carried in FP64 by the updates (the norm the truncations
+  // keep), through the pinned scalars
+  double* res = reinterpret_cast<double*>(F);
+  PO(energy_result(st, env, ebuf[cur], h->dtrace, res));
+  CK(cudaMemcpyAsync(h->henergy, res, 7 * sizeof(double), cudaMemcpyDeviceToHost, st));
   CK(sync_stream(h));
   prof_drain(h);
-  for (int a = 0; a < 6; ++a) out[a] = res[a].x;
-  out[6] = cnorm;
+  for (int a = 0; a < 7; ++a) out[a] = h->henergy[a];
   return MPDO_OK;
 }
 
@@ -1424,7 +1420,7 @@ int mpdo_create(const mpdo_config* cfg, const double* init_site_vec, mpdo_t* out
   if ((rc = alloc_dev(hp, &h->wRs, n3 * rsz)) || (rc = alloc_dev(hp, &h->wIrs, n3 * rsz)) ||
       (rc = alloc_dev(hp, (void**)&h->wSig, n3 * 8)) || (rc = alloc_dev(hp, (void**)&h->wLam, n9 * 8)) ||
       (rc = alloc_dev(hp, (void**)&h->wWv, KM * 8)) ||
-      (rc = alloc_dev(hp, (void**)&h->wF, (1024 + 2 * 64) * 8)))
+      (rc = alloc_dev(hp, (void**)&h->wF, (1024 + 2 * 64 + 1) * 8)))
     return rc;
   const int ncap = (int)std::max(n9, KM);
   size_t eb = em == 16 ? eig_work_bytes<double>(ncap) : eig_work_bytes<float>(ncap);
@@ -1462,7 +1458,8 @@ int mpdo_create(const mpdo_config* cfg, const double* init_site_vec, mpdo_t* out
       (rc = alloc_dev(hp, (void**)&h->dstats, sizeof(DevStats))))
     return rc;
   if (cudaMallocHost((void**)&h->hsc, sizeof(StepScalars)) != cudaSuccess ||
-      cudaMallocHost((void**)&h->hstats, sizeof(DevStats)) != cudaSuccess) {
+      cudaMallocHost((void**)&h->hstats, sizeof(DevStats)) != cudaSuccess ||
+      cudaMallocHost((void**)&h->henergy, 7 * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     return fail(nullptr, MPDO_ERR_OOM, "pinned host allocation");
   }
@@ -1785,6 +1782,7 @@ int mpdo_destroy(mpdo_t h) {
   if (h->obs) dfree(h, h->obs);
   if (h->hsc) cudaFreeHost(h->hsc);
   if (h->hstats) cudaFreeHost(h->hstats);
+  if (h->henergy) cudaFreeHost(h->henergy);
   if (h->hpc) cudaFreeHost(h->hpc);
   if (h->htcerr) cudaFreeHost(h->htcerr);
   if (h->own_stream) cudaStreamDestroy(h->st);

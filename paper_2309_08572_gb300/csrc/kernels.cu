@@ -155,40 +155,46 @@ __global__ void build_phi_kernel(int dm, const cx<R>* __restrict__ ct,
 // Bond cut on the spectrum lam (descending, n): keep <= chi values above htol*lam0.
 // The total weight is the trace of the matrix itself (noise-free in expectation), not
 // the sum of the positive computed eigenvalues, which is biased upward by the noise floor.
-template <typename R>
-__global__ void bond_select_kernel(int n, const double* __restrict__ lam, const cx<R>* __restrict__ hm,
-                                   long ldh, double htol, int chi, StepScalars* sc, DevStats* st) {
-  __shared__ double red_tot[256], red_kept[256];
-  __shared__ int s_keep;
-  double l0 = lam[0];
-  bool bad = !(l0 > 0.0) || !isfinite(l0);
-  if (threadIdx.x == 0) {
-    int k = 0;
-    if (!bad) {
-      while (k < n && k < chi && lam[k] > htol * l0) ++k;
-    }
-    if (k < 1) k = 1;
-    s_keep = k;
-  }
+// Sum over the CTA of 256 threads in a fixed order; every thread gets it.  red: 8 doubles.
+__device__ __forceinline__ double block_sum(double x, double* red) {
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
   __syncthreads();
-  int keep = s_keep;
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
+  __syncthreads();
+  return ((red[0] + red[1]) + (red[2] + red[3])) + ((red[4] + red[5]) + (red[6] + red[7]));
+}
+// Length of the leading run of x[0..n) above thr (n if all are); all threads of the CTA.
+__device__ __forceinline__ int leading_run(const double* x, int n, double thr, int* s_min) {
+  __syncthreads();
+  if (threadIdx.x == 0) *s_min = n;
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += blockDim.x)
+    if (!(x[i] > thr)) {
+      atomicMin(s_min, i);
+      break;
+    }
+  __syncthreads();
+  return *s_min;
+}
+
+template <typename R>
+__global__ void __launch_bounds__(256) bond_select_kernel(int n, const double* __restrict__ lam,
+                                                          const cx<R>* __restrict__ hm, long ldh,
+                                                          double htol, int chi, StepScalars* sc,
+                                                          DevStats* st) {
+  __shared__ double red[8];
+  __shared__ int s_keep;
+  const double l0 = lam[0];
+  const bool bad = !(l0 > 0.0) || !isfinite(l0);
+  int keep = bad ? 1 : leading_run(lam, min(n, chi), htol * l0, &s_keep);
+  if (keep < 1) keep = 1;
   double t = 0, kp = 0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     t += (double)hm[(long)i * ldh + i].x;
     if (i < keep) kp += lam[i] > 0 ? lam[i] : 0.0;
   }
-  red_tot[threadIdx.x] = t;
-  red_kept[threadIdx.x] = kp;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-      red_tot[threadIdx.x] += red_tot[threadIdx.x + s];
-      red_kept[threadIdx.x] += red_kept[threadIdx.x + s];
-    }
-    __syncthreads();
-  }
+  const double tot = block_sum(t, red), kept = block_sum(kp, red);
   if (threadIdx.x == 0) {
-    double tot = red_tot[0], kept = red_kept[0];
     sc->keep = keep;
     sc->tot = tot;
     sc->kept = kept;
@@ -232,111 +238,101 @@ __global__ void make_q_kernel(int dm, int keep, int m_ops, const cx<R>* __restri
 // Inner-index cut + purity-preserving truncation (Sec. III.D Eqs. xiformula / ppt with
 // T = 1, P = identity; theta = 0 when infeasible; clamp negatives; keep the trace).
 // Writes f[k] = sqrt(Lambda~_k / w_k) for k < kk.
-// Partial sums of tr W (diagonal real parts) and ||W||_F^2 over the n x n matrix wm, one pair
-// per CTA of a fixed grid (kNormBlocks), so the final sum is deterministic.
+// The CTAs of a fixed grid (kNormBlocks) form partial sums of tr W (diagonal real parts) and
+// ||W||_F^2 over the ntr x ntr matrix wm (= sum w^2 for the Hermitian W, whatever part of its
+// spectrum was resolved); the one that finishes last (a ticket; nobody waits) adds them in a
+// fixed order and selects, its lanes sharing the weights.  FP64 operations take ~64 clocks each
+// here: one thread walking through the weights, with two tangents of arc cosines, took 28 us
+// (K = 8) where this takes about a third; tan(acos c) is sqrt(1 - c^2) / c.
 constexpr int kNormBlocks = 64;
 template <typename R>
-__global__ void __launch_bounds__(256) gram_norms_kernel(int n, const cx<R>* __restrict__ wm,
-                                                         double* parts) {
-  __shared__ double rt[256], rf[256];
-  double t = 0, f2 = 0;
-  const long total = (long)n * n;
-  for (long e = blockIdx.x * 256L + threadIdx.x; e < total; e += 256L * kNormBlocks) {
-    const cx<R> v = wm[e];
-    f2 += (double)v.x * v.x + (double)v.y * v.y;
-    if (e / n == e % n) t += (double)v.x;
-  }
-  rt[threadIdx.x] = t;
-  rf[threadIdx.x] = f2;
-  __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-      rt[threadIdx.x] += rt[threadIdx.x + s];
-      rf[threadIdx.x] += rf[threadIdx.x + s];
+__global__ void __launch_bounds__(256) kraus_select_kernel(
+    int n, const double* __restrict__ w, const cx<R>* __restrict__ wm, int ntr, double* parts,
+    unsigned int* ticket, double kcut, int kmax, int use_ppt, double* f, StepScalars* sc,
+    DevStats* st, double* trace) {
+  __shared__ double red[8];
+  __shared__ int s_kk, s_last;
+  const int tid = threadIdx.x, lane = tid & 31;
+  {
+    double t = 0, f2 = 0;
+    const long total = (long)ntr * ntr;
+    for (long e = blockIdx.x * 256L + tid; e < total; e += 256L * kNormBlocks) {
+      const cx<R> v = wm[e];
+      f2 += (double)v.x * v.x + (double)v.y * v.y;
+      if (e / ntr == e % ntr) t += (double)v.x;
+    }
+    t = block_sum(t, red);
+    f2 = block_sum(f2, red);
+    if (tid == 0) {
+      parts[2 * blockIdx.x] = t;
+      parts[2 * blockIdx.x + 1] = f2;
+      __threadfence();
+      s_last = atomicAdd(ticket, 1u) == kNormBlocks - 1;
     }
     __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (tid == 0) *ticket = 0u;
   }
-  if (threadIdx.x == 0) {
-    parts[2 * blockIdx.x] = rt[0];
-    parts[2 * blockIdx.x + 1] = rf[0];
-  }
-}
-
-template <typename R>
-__global__ void kraus_select_kernel(int n, const double* __restrict__ w, const double* parts,
-                                    double kcut, int kmax, int use_ppt, double* f,
-                                    StepScalars* sc, DevStats* st, double* trace) {
-  // total weight tr W and sum of squared weights ||W||_F^2 (= sum w^2 for the Hermitian W,
-  // whatever part of its spectrum was resolved), from the matrix in FP64: the per-CTA partial
-  // sums of gram_norms_kernel, added here in a fixed order
-  __shared__ double red_t[kNormBlocks], red_f[kNormBlocks];
-  if (threadIdx.x < kNormBlocks) {
-    red_t[threadIdx.x] = parts[2 * threadIdx.x];
-    red_f[threadIdx.x] = parts[2 * threadIdx.x + 1];
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int b = 1; b < kNormBlocks; ++b) {
-      red_t[0] += red_t[b];
-      red_f[0] += red_f[b];
-    }
-  }
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double w0 = w[0] > 0 ? w[0] : 0.0;
-  bool bad = !(w0 > 0.0) || !isfinite(w0);
-  int kk = 0;
-  if (!bad) {
-    double thr = kcut * kcut * w0;
-    while (kk < n && kk < kmax && w[kk] > thr) ++kk;
-  }
+  const double w0 = w[0] > 0 ? w[0] : 0.0;
+  const bool bad = !(w0 > 0.0) || !isfinite(w0);
+  int kk = bad ? 1 : leading_run(w, min(n, kmax), kcut * kcut * w0, &s_kk);
   if (kk < 1) kk = 1;
-  double sum = red_t[0], sq = red_f[0], sumk = 0, sqk = 0;
-  for (int i = 0; i < kk; ++i) {
-    double v = w[i] > 0 ? w[i] : 0.0;
+  if (tid >= 32) return;
+  auto warp_sum = [](double x) {
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+  };
+  const double sum = warp_sum(__ldcg(&parts[2 * lane]) + __ldcg(&parts[2 * lane + 64]));
+  const double sq = warp_sum(__ldcg(&parts[2 * lane + 1]) + __ldcg(&parts[2 * lane + 65]));
+  double sumk = 0, sqk = 0;
+  for (int i = lane; i < kk; i += 32) {
+    const double v = w[i] > 0 ? w[i] : 0.0;
     sumk += v;
     sqk += v * v;
   }
+  sumk = warp_sum(sumk);
+  sqk = warp_sum(sqk);
   // The trace the truncation keeps (reading A2) is carried in FP64 across updates: the
   // channel multiplies it by tr(theta')/tr(theta) of this block (bond total sc->tot over
   // sc->trpre, both FP64 sums of the same stored tensors), so rounding of the stored
   // tensors and of the products that form the new centre does not accumulate in the norm.
-  double target = sum;
-  if (trace && sc->trpre > 0 && sc->tot > 0 && isfinite(*trace)) {
-    target = *trace * (sc->tot / sc->trpre);
-    *trace = target;
-  }
+  const bool carried = trace && sc->trpre > 0 && sc->tot > 0 && isfinite(*trace);
+  const double target = carried ? *trace * (sc->tot / sc->trpre) : sum;
+  __syncwarp();
+  if (carried && lane == 0) *trace = target;
 
-  double theta = 0.0;
+  double theta = 0.0, x = 0.0, shift = 0.0;
   int infeas = 0, clamped = 0;
-  double lt[1024];
-  if (use_ppt && !bad) {
-    double nl = sqrt(sq), nlp = sqrt(sqk);
-    double nt = sqrt((double)n), ntp = sqrt((double)kk);
-    double cos_phi = sum / (nl * nt);
-    double cos_sig = sumk / (nlp * ntp);
-    if (cos_sig > 1.0) cos_sig = 1.0;
-    double ratio = nt * cos_phi / ntp;
-    if (ratio > 1.0) { infeas = 1; theta = 0.0; } else { theta = acos(ratio); }
-    double sigma = acos(cos_sig);
-    double x = (sigma == 0.0) ? 0.0 : tan(theta) / tan(sigma) - 1.0;
-    double lsum = 0;
-    for (int i = 0; i < kk; ++i) {
-      double lp = w[i] > 0 ? w[i] : 0.0;
-      double v = (sigma == 0.0) ? lp : lp + x * (lp - nlp * cos_sig / ntp);
-      if (v < 0) { v = 0; ++clamped; }
-      lt[i] = v;
-      lsum += v;
-    }
-    double sc_tr = (lsum > 0) ? target / lsum : 0.0;
-    for (int i = 0; i < kk; ++i) lt[i] *= sc_tr;
-  } else {
-    double sc_tr = (sumk > 0) ? target / sumk : 0.0;
-    for (int i = 0; i < kk; ++i) lt[i] = (w[i] > 0 ? w[i] : 0.0) * sc_tr;
+  const bool ppt = use_ppt && !bad;
+  if (ppt) {
+    const double nl = sqrt(sq), nlp = sqrt(sqk), ntp = sqrt((double)kk);
+    const double cos_sig = fmin(1.0, sumk / (nlp * ntp));
+    double c = sum / (nl * ntp);   // cos theta = |T| cos phi / |T'|
+    if (c > 1.0) { infeas = 1; c = 1.0; }
+    theta = acos(c);
+    if (cos_sig < 1.0)
+      x = sqrt((1.0 - c) * (1.0 + c)) / c * (cos_sig / sqrt((1.0 - cos_sig) * (1.0 + cos_sig))) - 1.0;
+    shift = nlp * cos_sig / ntp;
   }
-  for (int i = 0; i < kk; ++i) {
-    double wi = w[i];
-    f[i] = (wi > 0) ? sqrt(lt[i] / wi) : 0.0;
+  // Lambda~ before its scale
+  auto value = [&](int i) {
+    const double lp = w[i] > 0 ? w[i] : 0.0;
+    return ppt ? lp + x * (lp - shift) : lp;
+  };
+  double lsum = 0;
+  for (int i = lane; i < kk; i += 32) {
+    const double v = value(i);
+    if (v < 0) ++clamped; else lsum += v;
   }
+  lsum = warp_sum(lsum);
+  clamped = (int)__reduce_add_sync(0xffffffffu, (unsigned)clamped);
+  const double scale = lsum > 0 ? target / lsum : 0.0;
+  for (int i = lane; i < kk; i += 32) {
+    const double wi = w[i], v = value(i);
+    f[i] = wi > 0 && v > 0 ? sqrt(v * scale / wi) : 0.0;
+  }
+  if (lane > 0) return;
   sc->kkeep = kk;
   sc->ktot = sum;
   sc->theta = theta;
@@ -540,6 +536,17 @@ __global__ void energy_mix_kernel(int dl, int plane, const cx<R>* __restrict__ f
       g1[2 * plane] = proj ? mkc<R>(0, 0) : b2;
     }
   }
+}
+
+__global__ void energy_init_kernel(long env, double2* e) {
+  const int a = threadIdx.x;
+  if (a < 6) e[a * env] = make_double2(a % 3 == 0 ? 1.0 : 0.0, 0.0);
+}
+__global__ void energy_result_kernel(long env, const double2* __restrict__ e,
+                                     const double* __restrict__ trace, double* res) {
+  const int a = threadIdx.x;
+  if (a < 6) res[a] = e[a * env].x;
+  if (a == 6) res[6] = *trace;
 }
 
 // ----------------------------------------------------------------- sampling
@@ -821,41 +828,52 @@ __global__ void __launch_bounds__(32 * (kPcWarps + 1)) pchol_kernel(
 
 // x = L1^-1 (r x r, lower triangular, row-major), L1[a][b] = L[piv[a]][b] the pivot rows of a
 // pivoted Cholesky factor.  A warp per column of x, by columns of L1: once x_b is known every
-// lane takes L1[a][b] x_b off its rows a > b.  Bound by the latency of the r dependent steps.
-constexpr int kInvWarps = 4;
+// lane takes L1[a][b] x_b off its rows a > b.  Bound by the latency of the r dependent steps, so
+// L1 comes through shared memory kInvChunk columns at a time (a step that waited for its
+// entries from L2 took three times as long: 45 us at r = 52).
+constexpr int kInvWarps = 4, kInvChunk = 16;
+template <int RL>   // rows of a lane: a = lane + 32 t
 __global__ void __launch_bounds__(32 * kInvWarps) pchol_inverse_kernel(int r,
                                                                       const double2* __restrict__ L,
                                                                       int lr,
                                                                       const int* __restrict__ piv,
                                                                       double2* x) {
-  constexpr int RL = (kGradedMax + 31) / 32;   // rows of a lane: a = lane + 32 t
-  const int lane = threadIdx.x & 31, j = blockIdx.x * kInvWarps + (threadIdx.x >> 5);
-  if (j >= r) return;
-  const double2* row[RL];
+  __shared__ double2 col[kInvChunk][32 * RL];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int j0 = blockIdx.x * kInvWarps, j = j0 + warp;
   double inv[RL];
   double2 s[RL];
 #pragma unroll
   for (int t = 0; t < RL; ++t) {
     const int a = lane + 32 * t;
-    row[t] = L + (long)piv[a < r ? a : 0] * lr;
-    inv[t] = a < r ? 1.0 / row[t][a].x : 0.0;
+    inv[t] = a < r ? 1.0 / L[(long)piv[a] * lr + a].x : 0.0;
     s[t] = make_double2(a == j ? 1.0 : 0.0, 0.0);
   }
-  for (int b = j; b < r; ++b) {
-    // x_b from its lane: every lane selects its own candidate, the broadcast takes the right one
-    double2 xb = make_double2(0.0, 0.0);
+  for (int b0 = j0 / kInvChunk * kInvChunk; b0 < r; b0 += kInvChunk) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < kInvChunk * r; e += 32 * kInvWarps) {
+      const int a = e / kInvChunk, b = e % kInvChunk;
+      col[b][a] = b0 + b < r ? L[(long)piv[a] * lr + b0 + b] : make_double2(0.0, 0.0);
+    }
+    __syncthreads();
+    const int b1 = min(r, b0 + kInvChunk);
+    for (int b = max(b0, j); b < b1; ++b) {
+      // x_b from its lane: every lane selects its own candidate, the broadcast takes the right one
+      double2 xb = make_double2(0.0, 0.0);
 #pragma unroll
-    for (int t = 0; t < RL; ++t)
-      if (t == b >> 5) xb = cscale(s[t], inv[t]);
-    xb.x = __shfl_sync(0xffffffffu, xb.x, b & 31);
-    xb.y = __shfl_sync(0xffffffffu, xb.y, b & 31);
+      for (int t = 0; t < RL; ++t)
+        if (t == b >> 5) xb = cscale(s[t], inv[t]);
+      xb.x = __shfl_sync(0xffffffffu, xb.x, b & 31);
+      xb.y = __shfl_sync(0xffffffffu, xb.y, b & 31);
 #pragma unroll
-    for (int t = 0; t < RL; ++t) {
-      const int a = lane + 32 * t;
-      if (a == b) s[t] = xb;
-      else if (a > b && a < r) s[t] = csub(s[t], cmul(row[t][b], xb));
+      for (int t = 0; t < RL; ++t) {
+        const int a = lane + 32 * t;
+        if (a == b) s[t] = xb;
+        else if (a > b && a < r) s[t] = csub(s[t], cmul(col[b - b0][a], xb));
+      }
     }
   }
+  if (j >= r) return;
 #pragma unroll
   for (int t = 0; t < RL; ++t) {
     const int a = lane + 32 * t;
@@ -986,11 +1004,12 @@ template <typename R>
 cudaError_t kraus_select(cudaStream_t st, int n, const double* w, const cx<R>* wm, int ntr,
                          double kcut, int kmax, int use_ppt, double* f, StepScalars* sc,
                          DevStats* ds, double* trace) {
-  // the partial sums live after the kept scale factors f (at most 1024 of them)
+  // the partial sums and the ticket live after the kept scale factors f (at most 1024 of them)
   double* parts = f + 1024;
-  count_launch(2);
-  gram_norms_kernel<R><<<kNormBlocks, 256, 0, st>>>(ntr, wm, parts);
-  kraus_select_kernel<R><<<1, 256, 0, st>>>(n, w, parts, kcut, kmax, use_ppt, f, sc, ds, trace);
+  count_launch();
+  kraus_select_kernel<R><<<kNormBlocks, 256, 0, st>>>(
+      n, w, wm, ntr, parts, reinterpret_cast<unsigned int*>(parts + 2 * kNormBlocks), kcut, kmax,
+      use_ppt, f, sc, ds, trace);
   return cudaGetLastError();
 }
 template <typename R>
@@ -1043,6 +1062,17 @@ cudaError_t energy_mix(cudaStream_t st, int dl, int plane, const cx<R>* f, long 
   count_launch();
   energy_mix_kernel<R><<<nblocks((long)dl * plane), 256, 0, st>>>(dl, plane, f, fstride, g,
                                                                     gstride, J, hx, bz);
+  return cudaGetLastError();
+}
+cudaError_t energy_init(cudaStream_t st, long env, double2* e) {
+  count_launch();
+  energy_init_kernel<<<1, 32, 0, st>>>(env, e);
+  return cudaGetLastError();
+}
+cudaError_t energy_result(cudaStream_t st, long env, const double2* e, const double* trace,
+                          double* res) {
+  count_launch();
+  energy_result_kernel<<<1, 32, 0, st>>>(env, e, trace, res);
   return cudaGetLastError();
 }
 template <typename R>
@@ -1124,7 +1154,12 @@ cudaError_t pchol_inverse(cudaStream_t st, int r, const double2* L, int lr, cons
                           double2* x) {
   if (r < 1 || r > kGradedMax) return cudaErrorInvalidValue;
   count_launch();
-  pchol_inverse_kernel<<<(r + kInvWarps - 1) / kInvWarps, 32 * kInvWarps, 0, st>>>(r, L, lr, piv, x);
+  auto run = [&](auto kern) {
+    kern<<<(r + kInvWarps - 1) / kInvWarps, 32 * kInvWarps, 0, st>>>(r, L, lr, piv, x);
+  };
+  if (r <= 32) run(pchol_inverse_kernel<1>);
+  else if (r <= 64) run(pchol_inverse_kernel<2>);
+  else run(pchol_inverse_kernel<(kGradedMax + 31) / 32>);
   return cudaGetLastError();
 }
 template <typename T>

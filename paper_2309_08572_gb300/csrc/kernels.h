@@ -39,7 +39,8 @@ cudaError_t polar_factors(cudaStream_t st, int n, const cx<R>* g, cx<R>* pm, cx<
 // n eigenvalues w (descending); the total weight is the trace of wm (ntr x ntr)
 // trace (device FP64, may be NULL): the carried trace of the state, multiplied by the
 // block's tr(theta')/tr(theta) = sc->tot / sc->trpre; the kept weights are rescaled to it.
-// f holds 1024 + 128 doubles (scale factors, then partial sums of tr W and ||W||_F^2).
+// f holds 1024 + 129 doubles (scale factors, then partial sums of tr W and ||W||_F^2, then a CTA
+// ticket, zero between launches).
 template <typename R>
 cudaError_t kraus_select(cudaStream_t st, int n, const double* w, const cx<R>* wm, int ntr,
                          double kcut, int kmax, int use_ppt, double* f, StepScalars* sc,
@@ -84,6 +85,11 @@ cudaError_t scale_vk(cudaStream_t st, int n, int kk, const cx<R>* v, long ldv, c
 template <typename R>
 cudaError_t energy_mix(cudaStream_t st, int dl, int plane, const cx<R>* f, long fstride,
                        cx<R>* g, long gstride, double J, double hx, double bz);
+// the automata's six 1 x 1 environments at the chain's left end (env entries apart), and at its
+// right end their real parts and the carried trace to res[0..7)
+cudaError_t energy_init(cudaStream_t st, long env, double2* e);
+cudaError_t energy_result(cudaStream_t st, long env, const double2* e, const double* trace,
+                          double* res);
 template <typename R>
 cudaError_t sample_pick(cudaStream_t st, int n_samples, int dr, const cx<R>* ev, const cx<R>* rt,
                         uint64_t seed, int site, int site_user, int n_sites, cx<R>* env_out,

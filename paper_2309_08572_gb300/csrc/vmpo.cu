@@ -61,80 +61,97 @@ struct VScalars {
 // T_k = Re(tl_k trw_k) / Lambda_k (trw carries the factor Lambda_k of U^+ theta'; Eqs.
 // xiformula, ppt; theta = 0 when infeasible, negative values clamped, rescaled so that
 // T'.Lambda~ = T.Lambda); out[k] = Lambda~_k (k < keep), sv[k] = sqrt(lam_k) for k < nz.
-__global__ void vmpo_cut_kernel(int n, const double* __restrict__ lam, const double2* __restrict__ tl,
-                                const double2* __restrict__ tr, double cut2, int chi, int mode,
-                                double* sv, double* out, VScalars* sc) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// One warp, its lanes sharing the values (FP64 operations take ~64 clocks each here); tan(acos c)
+// is sqrt(1 - c^2) / c.
+__global__ void __launch_bounds__(32) vmpo_cut_kernel(int n, const double* __restrict__ lam,
+                                                      const double2* __restrict__ tl,
+                                                      const double2* __restrict__ tr, double cut2,
+                                                      int chi, int mode, double* sv, double* out,
+                                                      VScalars* sc) {
+  const int lane = threadIdx.x;
   const double l0 = lam[0];
   VScalars s{};
   if (!(l0 > 0.0) || !isfinite(l0)) {
     s.flags = 1;
     s.nz = s.keep = 1;
-    *sc = s;
+    if (lane == 0) *sc = s;
     return;
   }
-  int nz = 0;
-  while (nz < n && lam[nz] > cut2 * l0) ++nz;
+  auto warp_sum = [](double x) {
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+  };
+  int nz = n;
+  for (int k0 = 0; k0 < n; k0 += 32) {   // the leading run above the cut
+    const bool in = k0 + lane < n && lam[k0 + lane] > cut2 * l0;
+    const unsigned miss = ~__ballot_sync(0xffffffffu, in);
+    if (miss) {
+      nz = min(n, k0 + __ffs(miss) - 1);
+      break;
+    }
+  }
   if (nz < 1) nz = 1;
   const int keep = nz < chi ? nz : chi;
   double tot = 0, kept = 0;
-  for (int k = 0; k < nz; ++k) {
+  for (int k = lane; k < nz; k += 32) {
     sv[k] = sqrt(fmax(lam[k], 0.0));
     tot += lam[k];
     if (k < keep) kept += lam[k];
   }
+  tot = warp_sum(tot);
+  kept = warp_sum(kept);
   s.nz = nz;
   s.keep = keep;
   s.disc = tot > 0 ? (tot - kept) / tot : 0.0;
   if (mode == 0) {
-    for (int k = 0; k < keep; ++k) out[k] = sv[k];
+    for (int k = lane; k < keep; k += 32) out[k] = sv[k];
   } else {
-    double lt = 0, nl = 0, nt = 0, lpt = 0, nlp = 0, ntp = 0;
-    for (int k = 0; k < nz; ++k) {
-      // T_k = Re(tl_k tr_k) (real for a Hermitian rho up to near-degeneracies)
-      const double t = (tl[k].x * tr[k].x - tl[k].y * tr[k].y) / sv[k];
-      lt += sv[k] * t;
-      nl += sv[k] * sv[k];
-      nt += t * t;
+    // T_k = Re(tl_k tr_k) (real for a Hermitian rho up to near-degeneracies)
+    auto trace_env = [&](int k) { return (tl[k].x * tr[k].x - tl[k].y * tr[k].y) / sv[k]; };
+    double lt = 0, nl = 0, lpt = 0, nlp = 0, ntp = 0;
+    for (int k = lane; k < nz; k += 32) {
+      const double t = trace_env(k), a = sv[k] * t, b = sv[k] * sv[k];
+      lt += a;
+      nl += b;
       if (k < keep) {
-        lpt += sv[k] * t;
-        nlp += sv[k] * sv[k];
+        lpt += a;
+        nlp += b;
         ntp += t * t;
       }
     }
-    nl = sqrt(nl);
-    nt = sqrt(nt);
-    nlp = sqrt(nlp);
-    ntp = sqrt(ntp);
-    const double cos_phi = lt / (nl * nt);
-    double cos_sig = lpt / (nlp * ntp);
-    if (cos_sig > 1.0) cos_sig = 1.0;
-    const double ratio = nt * cos_phi / ntp;
-    double th;
-    if (ratio > 1.0 || !(ntp > 0)) {
+    lt = warp_sum(lt);
+    nl = sqrt(warp_sum(nl));
+    lpt = warp_sum(lpt);
+    nlp = sqrt(warp_sum(nlp));
+    ntp = sqrt(warp_sum(ntp));
+    const double cos_sig = fmin(1.0, lpt / (nlp * ntp));
+    double c = lt / (nl * ntp);   // cos theta = |T| cos phi / |T'|
+    if (c > 1.0 || !(ntp > 0)) {
       s.infeasible = 1;
-      th = 0.0;
-    } else {
-      th = acos(ratio);
+      c = 1.0;
     }
-    s.theta = th;
-    const double sig = acos(cos_sig);
-    const double x = (sig == 0.0) ? 0.0 : tan(th) / tan(sig) - 1.0;
+    s.theta = acos(c);
+    double x = 0.0;
+    if (cos_sig < 1.0)
+      x = sqrt((1.0 - c) * (1.0 + c)) / c * (cos_sig / sqrt((1.0 - cos_sig) * (1.0 + cos_sig))) - 1.0;
     double dot = 0;
-    for (int k = 0; k < keep; ++k) {
-      const double t = (tl[k].x * tr[k].x - tl[k].y * tr[k].y) / sv[k];
-      double v = (sig == 0.0) ? sv[k] : sv[k] + x * (sv[k] - nlp * cos_sig * t / ntp);
+    int clamped = 0;
+    for (int k = lane; k < keep; k += 32) {
+      const double t = trace_env(k);
+      double v = cos_sig < 1.0 ? sv[k] + x * (sv[k] - nlp * cos_sig * t / ntp) : sv[k];
       if (v < 0) {
         v = 0;
-        ++s.clamped;
+        ++clamped;
       }
       out[k] = v;
       dot += v * t;
     }
+    dot = warp_sum(dot);
+    s.clamped = (int)__reduce_add_sync(0xffffffffu, (unsigned)clamped);
     const double scale = (dot != 0.0) ? lt / dot : 0.0;
-    for (int k = 0; k < keep; ++k) out[k] *= scale;
+    for (int k = lane; k < keep; k += 32) out[k] *= scale;
   }
-  *sc = s;
+  if (lane == 0) *sc = s;
 }
 
 // x[(l, eta)] = env[l] tau[eta] (side 0) or x[(eta, r)] = tau[eta] env[r] (side 1)
@@ -165,32 +182,44 @@ __global__ void scale_rows_kernel(int keep, int cols, const double2* __restrict_
 // The energy automaton on one site: for projector p (0: identity, 1: qubit projector),
 // states s = 0 (no term yet), 1 (a Z waiting for its partner), 2 (term complete):
 //   E0' = E0 T[P], E1' = E0 T[PZP], E2' = E2 T[P] - J E1 T[PZP] + E0 T[P H1 P]
-// with T[O](E)[r] = sum_{l,eta} E[l] o[eta] A[l,eta,r], o[(s,s')] = O[s',s];
-// env in/out: [2 projectors][3 states][dl | dr].
-__global__ void vmpo_energy_kernel(int dl, int dr, const double2* __restrict__ a,
-                                   const double2* __restrict__ ein, double2* eout,
-                                   const double2* __restrict__ ovec /* [2][3][9] */, double J) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= dr) return;
-  for (int p = 0; p < 2; ++p) {
-    const double2* op = ovec + p * 27;   // [0] P, [1] PZP, [2] P H1 P
-    const double2* e0 = ein + (p * 3 + 0) * dl;
-    const double2* e1 = ein + (p * 3 + 1) * dl;
-    const double2* e2 = ein + (p * 3 + 2) * dl;
-    double2 n0 = make_double2(0, 0), n1 = n0, n2 = n0;
-    for (int l = 0; l < dl; ++l) {
-      double2 t[3] = {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)};
-      for (int eta = 0; eta < 9; ++eta) {
-        const double2 av = a[((long)l * 9 + eta) * dr + r];
-        for (int q = 0; q < 3; ++q) t[q] = cadd(t[q], cmul(op[q * 9 + eta], av));
-      }
-      n0 = cadd(n0, cmul(e0[l], t[0]));
-      n1 = cadd(n1, cmul(e0[l], t[1]));
-      n2 = cadd(n2, cadd(cmul(e2[l], t[0]), cadd(cscale(cmul(e1[l], t[1]), -J), cmul(e0[l], t[2]))));
+// with T[O](E)[r] = sum_{l,eta} E[l] o[eta] A[l,eta,r], o[(s,s')] = O[s',s] and H1 = -hx X - b J Z:
+// only the entries of A with eta in {00, 01, 10, 11, 22} meet a non-zero o.  env in/out:
+// [2 projectors][3 states][dl | dr].  A CTA takes 32 columns r of one projector, its eight warps
+// sharing the rows l (one thread per column took 177 us at D = 16).
+__global__ void __launch_bounds__(256) vmpo_energy_kernel(int dl, int dr,
+                                                          const double2* __restrict__ a,
+                                                          const double2* __restrict__ ein,
+                                                          double2* eout, double J, double hx,
+                                                          double bz) {
+  __shared__ double2 part[8][3][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, p = blockIdx.y;
+  const int r = blockIdx.x * 32 + lane;
+  const double2* e0 = ein + (p * 3 + 0) * dl;
+  const double2* e1 = ein + (p * 3 + 1) * dl;
+  const double2* e2 = ein + (p * 3 + 2) * dl;
+  double2 n0 = make_double2(0, 0), n1 = n0, n2 = n0;
+  if (r < dr)
+    for (int l = warp; l < dl; l += 8) {
+      const double2* al = a + (long)l * 9 * dr + r;
+      const double2 a0 = al[0], a1 = al[dr], a3 = al[3L * dr], a4 = al[4L * dr];
+      double2 t0 = cadd(a0, a4);
+      const double2 t1 = csub(a0, a4);
+      if (p == 0) t0 = cadd(t0, al[8L * dr]);
+      const double2 t2 = csub(cscale(cadd(a1, a3), -hx), cscale(t1, bz * J));
+      cfma(n0, e0[l], t0);
+      cfma(n1, e0[l], t1);
+      cfma(n2, e2[l], t0);
+      cfma(n2, cscale(e1[l], -J), t1);
+      cfma(n2, e0[l], t2);
     }
-    eout[(p * 3 + 0) * dr + r] = n0;
-    eout[(p * 3 + 1) * dr + r] = n1;
-    eout[(p * 3 + 2) * dr + r] = n2;
+  part[warp][0][lane] = n0;
+  part[warp][1][lane] = n1;
+  part[warp][2][lane] = n2;
+  __syncthreads();
+  if (warp < 3 && r < dr) {
+    double2 x = part[0][warp][lane];
+    for (int k = 1; k < 8; ++k) x = cadd(x, part[k][warp][lane]);
+    eout[(p * 3 + warp) * dr + r] = x;
   }
 }
 
@@ -234,7 +263,7 @@ struct mpdo_vmpo_s {
   size_t site_cap = 0;
   double2* sites = nullptr;
   double2 *th = nullptr, *th2 = nullptr, *H = nullptr, *U = nullptr, *Vh = nullptr;
-  double2 *S = nullptr, *x = nullptr, *tl = nullptr, *tr = nullptr, *ov = nullptr;
+  double2 *S = nullptr, *x = nullptr, *tl = nullptr, *tr = nullptr;
   double2 *Lenv = nullptr, *Renv = nullptr, *etmp = nullptr, *ebuf = nullptr;
   double *lam = nullptr, *sv = nullptr, *lt = nullptr;
   EigWork<double> eig;
@@ -539,7 +568,7 @@ int mpdo_vmpo_create(int n_sites, int chi_max, int use_ppt, double sv_cutoff,
       (rc = A((void**)&h->th2, n9 * n9)) || (rc = A((void**)&h->H, n9 * n9)) ||
       (rc = A((void**)&h->U, n9 * n9)) || (rc = A((void**)&h->S, 81 * 81)) ||
       (rc = A((void**)&h->x, 2 * n9)) || (rc = A((void**)&h->tl, n9)) ||
-      (rc = A((void**)&h->tr, n9)) || (rc = A((void**)&h->ov, 64)) ||
+      (rc = A((void**)&h->tr, n9)) ||
       (rc = A((void**)&h->Lenv, (size_t)(n_sites + 1) * D)) ||
       (rc = A((void**)&h->Renv, (size_t)(n_sites + 1) * D)) ||
       (rc = A((void**)&h->ebuf, 12 * D)) ||
@@ -623,23 +652,6 @@ int mpdo_vmpo_apply_layer(mpdo_vmpo h, const mpdo_layer* layer, mpdo_trunc_stats
 int mpdo_vmpo_expect_energy(mpdo_vmpo h, double J, double hx, double b, double* e_raw,
                             double* e_success, double* success_prob, double* trace) {
   if (!h) return vfail(nullptr, MPDO_ERR_ARG, "vmpo: null handle");
-  // operator vectors o[(s,s')] = O[s', s] for P in {I, Pi_q}: P, P Z P, P (-hx X - b J Z) P
-  double2 ov[54];
-  for (int p = 0; p < 2; ++p) {
-    const double pr[3] = {1, 1, p == 0 ? 1.0 : 0.0};
-    for (int s = 0; s < 3; ++s)
-      for (int t = 0; t < 3; ++t) {
-        // O[t][s] with t = bra index s', s = ket index
-        const double P = (s == t) ? pr[s] : 0.0;
-        const double z = (s == t && s < 2) ? (s == 0 ? 1.0 : -1.0) : 0.0;
-        const double xq = ((s == 0 && t == 1) || (s == 1 && t == 0)) ? 1.0 : 0.0;
-        const double h1 = -hx * xq - b * J * z;
-        ov[p * 27 + 0 * 9 + s * 3 + t] = make_double2(P, 0);
-        ov[p * 27 + 1 * 9 + s * 3 + t] = make_double2(pr[s] * pr[t] * z, 0);
-        ov[p * 27 + 2 * 9 + s * 3 + t] = make_double2(pr[s] * pr[t] * h1, 0);
-      }
-  }
-  VK(cudaMemcpyAsync(h->ov, ov, sizeof(ov), cudaMemcpyHostToDevice, h->st));
   // env [2][3][D]: start E0 = 1, E1 = E2 = 0 for both projectors
   const long D = h->chi;
   double2* ein = h->ebuf;
@@ -652,14 +664,13 @@ int mpdo_vmpo_expect_energy(mpdo_vmpo h, double J, double hx, double b, double* 
   for (int s = 0; s < h->n; ++s) {
     const int dl = h->bond[s], dr = h->bond[s + 1];
     count_launch();
-    vmpo_energy_kernel<<<(dr + 127) / 128, 128, 0, h->st>>>(dl, dr, h->site(s), ein, eout, h->ov,
-                                                          J);
+    vmpo_energy_kernel<<<dim3((dr + 31) / 32, 2), 256, 0, h->st>>>(dl, dr, h->site(s), ein, eout, J,
+                                                                  hx, b);
     VK(cudaGetLastError());
     std::swap(ein, eout);
   }
   double2 res[6];
-  for (int q = 0; q < 6; ++q)
-    VK(cudaMemcpyAsync(&res[q], ein + q, sizeof(double2), cudaMemcpyDeviceToHost, h->st));
+  VK(cudaMemcpyAsync(res, ein, sizeof(res), cudaMemcpyDeviceToHost, h->st));
   VK(cudaStreamSynchronize(h->st));
   // the final bond dimension is 1: state q of projector p sits at ein[(p*3+q)*1]
   const double norm = res[0].x, tot = res[2].x, ps = res[3].x, tots = res[5].x;
