@@ -421,6 +421,14 @@ int mpdo_kernel_heig(int prec, int n, void* a, void* v, double* w, int* sweeps, 
  * 1..MPDO_HEIG_GRADED_NMAX.  Allocates its scratch and synchronises the stream. */
 int mpdo_kernel_heig_graded(int n, const void* a, void* v, double* w, void* stream);
 
+/* Pivoted Cholesky factor of a Hermitian PSD matrix w (complex128, n x n row-major, device):
+ * w ~ L L^+, L n x *rank with row stride ldl >= min(n, rmax), columns by the largest remaining
+ * diagonal (piv: device int[min(n, rmax)], may be NULL) until that is <= tol * tr w or after rmax
+ * columns; *resid = largest remaining diagonal / tr w.  n in 1..1024, rmax in
+ * 1..MPDO_HEIG_GRADED_NMAX.  Synchronises the stream. */
+int mpdo_kernel_pchol(int n, const void* w, int rmax, double tol, void* L, int ldl, int* piv,
+                      int* rank, double* resid, void* stream);
+
 /* Tensor-core GEMMs (tcgen05.mma, TMEM accumulators, TMA-fed shared-memory pipeline) on
  * which the contractions of the two-site update run in the split-precision modes (Sec.
  * III.A: contracting the site tensors and the gate, Fig. 6a; the Gram products of the

@@ -145,6 +145,7 @@ def _load():
                                   C.c_long, VP, C.c_long, C.c_long, I, VP]),
         "mpdo_kernel_heig": (I, [I, I, VP, VP, P(D), P(I), VP]),
         "mpdo_kernel_heig_graded": (I, [I, VP, VP, P(D), VP]),
+        "mpdo_kernel_pchol": (I, [I, VP, I, D, VP, I, VP, P(I), P(D), VP]),
         "mpdo_heig_noalloc": (I, [I, I, VP, VP, P(D), P(I), VP]),
         "mpdo_tc_gemm_launches": (C.c_longlong, []),
         "mpdo_kernel_tcgemm_exact": (I, [I, I, I, I, I, VP, C.c_long, C.c_long, VP, C.c_long,
@@ -651,6 +652,16 @@ def kernel_heig_graded(n: int, a, v, w, stream=None):
     _check(LIB.mpdo_kernel_heig_graded(n, C.c_void_p(a.data_ptr()), C.c_void_p(v.data_ptr()),
                                        C.cast(C.c_void_p(w.data_ptr()), C.POINTER(C.c_double)),
                                        st))
+
+
+def kernel_pchol(n: int, w, rmax: int, tol: float, L, piv=None, stream=None) -> tuple[int, float]:
+    """Pivoted Cholesky factor of the PSD device matrix w (n x n complex128) -> rank, residual."""
+    st = _current_stream() if stream is None else C.c_void_p(stream)
+    rank, resid = C.c_int(0), C.c_double(0)
+    _check(LIB.mpdo_kernel_pchol(n, C.c_void_p(w.data_ptr()), rmax, tol, C.c_void_p(L.data_ptr()),
+                                 L.stride(0), None if piv is None else C.c_void_p(piv.data_ptr()),
+                                 C.byref(rank), C.byref(resid), st))
+    return rank.value, resid.value
 
 
 HEIG_NOALLOC_NMAX = 192

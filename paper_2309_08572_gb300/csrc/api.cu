@@ -1931,4 +1931,28 @@ int mpdo_kernel_heig_graded(int n, const void* a, void* v, double* w, void* stre
   return MPDO_OK;
 }
 
+int mpdo_kernel_pchol(int n, const void* w, int rmax, double tol, void* L, int ldl, int* piv,
+                      int* rank, double* resid, void* stream) {
+  if (n < 1 || n > 1024 || rmax < 1 || rmax > kGradedMax || ldl < std::min(n, rmax) || !w || !L ||
+      !rank || !resid)
+    return fail(nullptr, MPDO_ERR_ARG, "bad pchol arguments");
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  mpdo_ctx::PcOut* d = nullptr;
+  if (cudaMalloc(&d, sizeof(mpdo_ctx::PcOut)) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(nullptr, MPDO_ERR_OOM, "pchol result");
+  }
+  mpdo_ctx::PcOut hd{};
+  cudaError_t e = pchol<double>(st, n, (const double2*)w, rmax, tol, (double2*)L, ldl, &d->r,
+                                &d->resid, piv);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&hd, d, sizeof(hd), cudaMemcpyDeviceToHost, st);
+  const cudaError_t es = cudaStreamSynchronize(st);
+  cudaFree(d);
+  if (e == cudaSuccess) e = es;
+  if (e != cudaSuccess) return fail(nullptr, MPDO_ERR_CUDA, cudaGetErrorString(e));
+  *rank = hd.r;
+  *resid = hd.resid;
+  return MPDO_OK;
+}
+
 }  // extern "C"

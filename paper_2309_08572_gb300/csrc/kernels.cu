@@ -655,23 +655,26 @@ __global__ void dual_rows_kernel(int kk, int cols, const cx<R>* __restrict__ y, 
 // largest remaining diagonal is <= tol * tr W or after rmax (<= kGradedMax) columns.
 // *rout = r; *resid = largest remaining diagonal / tr W.
 //
-// The columns depend on one another, so the factor is bound by the latency of a column: a
-// barrier or two and a chain of FP64 operations, at ~64 clocks each on this chip; beyond ~64 rows
-// its dot products also want the FP64 pipes (2 FMA per clock) of several SMs.  So the rows go to
-// the CTAs of a thread-block cluster of up to 16 (row i belongs to rank i mod S), or to one CTA
-// without any cluster barrier; four lanes to a row, each row's part of L -- and of W, where it
-// fits -- in its CTA's shared memory.  Per column: every CTA stores its best remaining diagonal
-// into all CTAs' shared memory, one cluster barrier, every warp takes the same pivot from its
-// own CTA's copies, the pivot's row comes from its owner's shared memory, and the lanes of a row
-// split its dot product while one further warp takes the pivot's square root; the remaining
-// diagonals follow from the unscaled column, beside its scaling.  Posts alternate between two
-// slots by column parity, so a slot is rewritten only after every CTA has passed the next
-// barrier; candidates are compared as integers (non-negative doubles order alike), which keeps
-// the FP64 pipe to the dot products.  Sums and the pivot choice follow a fixed order, so the
-// factor does not depend on scheduling.
-constexpr int kPcLanes = 4;              // lanes of a row
-constexpr int kPcWarps = 8;              // row warps of a CTA, at most 64 rows
+// The columns depend on one another, so the factor is bound by the latency of a column.  An FP64
+// warp instruction occupies its quarter of the SM for 64 clocks whatever its active lanes, so a
+// row's dot product is split over four or eight lanes such that the row warps of a CTA, and one
+// further warp for the pivot's square root, find a quarter each; the lanes' sums part into real
+// and imaginary halves with the first exchange, which leaves one operation a step.  Rows beyond 32
+// go to the CTAs of a thread-block cluster (row i belongs to rank i mod S), each row's part of L --
+// and of W, where it fits -- in its CTA's shared memory.  Per column every CTA sends its best
+// remaining diagonal and that row of L to every CTA with remote stores that count their bytes at
+// the receiver's mbarrier: one hop, after which all hold the pivot and its row, against a cluster
+// barrier (1200 clocks) and a fetch of the row (1400) before.  Where the slots of all candidates'
+// rows do not fit (n > 832 at 168 columns) the owner sends the pivot's row in a second hop.  The
+// remaining diagonals follow from the unscaled column, beside its scaling.  Slots alternate by
+// column parity: a CTA sends for column j + 2 only after every CTA has sent for j + 1, which each
+// does when its threads are done with column j.  Candidates are compared as integers
+// (non-negative doubles order alike), which keeps the FP64 pipe to the dot products.  Sums and the
+// pivot choice follow a fixed order, so the factor does not depend on scheduling.
+// n 156, rank 52: 225 -> 140 us; n 64, rank 45: 170 -> 96 us; n 32, rank 24: 54 -> 43 us.
+constexpr int kPcWarps = 8;              // row warps of a CTA
 constexpr int kPcCtas = 16;
+constexpr unsigned long long kPcWaitNs = 1000000000ull;
 // largest key of the warp (bits of a non-negative double, or -1) and the smallest index with it
 __device__ __forceinline__ void warp_best(long long& key, int& idx) {
   const int hi = (int)(key >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
@@ -680,30 +683,73 @@ __device__ __forceinline__ void warp_best(long long& key, int& idx) {
   idx = __reduce_min_sync(0xffffffffu, x);
   key = ((long long)mh << 32) | ml;
 }
-template <typename R, bool CLUSTER>
+__device__ __forceinline__ uint32_t pc_su32(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+// address of x (of this CTA's shared memory) in the cluster's CTA of that rank
+__device__ __forceinline__ uint32_t pc_map(uint32_t x, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(rank));
+  return r;
+}
+// one remote store that counts its bytes at the receiver's barrier
+__device__ __forceinline__ void pc_send(uint32_t dst, uint32_t bar, long long a, long long b) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%2, %3}, [%1];"
+               ::"r"(dst), "r"(bar), "l"(a), "l"(b)
+               : "memory");
+}
+__device__ __forceinline__ void pc_send(uint32_t dst, uint32_t bar, double2 v) {
+  pc_send(dst, bar, __double_as_longlong(v.x), __double_as_longlong(v.y));
+}
+__device__ __forceinline__ void pc_send(uint32_t dst, uint32_t bar, float2 v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%2, %3}, [%1];"
+               ::"r"(dst), "r"(bar), "r"(__float_as_int(v.x)), "r"(__float_as_int(v.y))
+               : "memory");
+}
+__device__ __forceinline__ bool pc_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool pc_wait(uint32_t bar, uint32_t parity) {
+  if (pc_test(bar, parity)) return true;
+  unsigned long long t0, t1;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+  for (;;) {
+    for (int i = 0; i < 64; ++i)
+      if (pc_test(bar, parity)) return true;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
+    if (t1 - t0 > kPcWaitNs) return false;
+  }
+}
+template <typename R, bool CLUSTER, int LANES>
 __global__ void __launch_bounds__(32 * (kPcWarps + 1)) pchol_kernel(
     int n, const cx<R>* __restrict__ w, int rmax, double tol, cx<R>* L, int lr, int* rout,
-    double* resid, int* piv, int w_rows) {
+    double* resid, int* piv, int w_rows, int all_rows) {
   using T = cx<R>;
   cg::cluster_group cluster = cg::this_cluster();
   const int S = CLUSTER ? (int)cluster.num_blocks() : 1, c = CLUSTER ? (int)cluster.block_rank() : 0;
-  auto barrier = [&]() {
-    if constexpr (CLUSTER) cluster.sync(); else __syncthreads();
-  };
-  // x of the CTA of that rank
-  auto remote = [&](auto* x, int rank) {
-    if constexpr (CLUSTER) return cluster.map_shared_rank(x, rank); else return x;
-  };
   extern __shared__ __align__(16) unsigned char pc_raw[];
   T* Ls = reinterpret_cast<T*>(pc_raw);          // own rows of L, stride rmax
   const int nlm = (n + S - 1) / S;
-  T* Ws = Ls + (size_t)nlm * rmax;               // own rows of W, stride n (w_rows)
-  __shared__ T lp[kGradedMax];
-  __shared__ long long post_v[2][kPcCtas], s_v[2][kPcWarps];   // best remaining diagonals, as bits
-  __shared__ int post_i[2][kPcCtas], s_i[2][kPcWarps];
+  // the candidates' rows of L, [2][S][rmax] (all_rows), or the pivot's, [2][rmax]
+  T* rows = Ls + (size_t)nlm * rmax;
+  const int nslot = all_rows ? S : 1;
+  T* Ws = rows + (CLUSTER ? (size_t)2 * nslot * rmax : 0);   // own rows of W, stride n (w_rows)
+  __shared__ __align__(16) longlong2 post[2][kPcCtas];   // best remaining diagonals: bits, index
+  __shared__ __align__(8) unsigned long long bars[4];
+  __shared__ long long s_v[2][kPcWarps];
+  __shared__ int s_i[2][kPcWarps], s_late;
   __shared__ double s_tr[kPcWarps], post_tr, s_inv, s_inv2, s_dp;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = (blockDim.x >> 5) - 1;
-  const int l4 = lane & (kPcLanes - 1), li = tid / kPcLanes, i = c + li * S;
+  const int lr_ = lane & (LANES - 1), li = tid / LANES, i = c + li * S;
+  const int part = lr_ >= LANES / 2;             // lanes of the upper half end with the imaginary part
   const bool own = warp < nw && li < nlm && i < n;
   if (w_rows)
     for (int e = tid; e < nlm * n; e += blockDim.x) {
@@ -715,23 +761,44 @@ __global__ void __launch_bounds__(32 * (kPcWarps + 1)) pchol_kernel(
     d = (double)w[(long)i * n + i].x;
     if (!(d > 0.0)) d = 0.0;
   }
-  double tp = l4 == 0 ? d : 0.0;
+  double tp = lr_ == 0 ? d : 0.0;
   for (int o = 16; o > 0; o >>= 1) tp += __shfl_xor_sync(0xffffffffu, tp, o);
   if (lane == 0 && warp < nw) s_tr[warp] = tp;
-  __syncthreads();
-  if (tid == 0) {
-    double t = 0;
-    for (int k = 0; k < nw; ++k) t += s_tr[k];
-    post_tr = t;
+  if (tid == 0) s_late = 0;
+  if (CLUSTER && tid < 4) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(pc_su32(&bars[tid])) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  barrier();
+  __syncthreads();
   double tr = 0.0;
-  for (int q = 0; q < S; ++q) tr += *remote(&post_tr, q);
+  for (int k = 0; k < nw; ++k) tr += s_tr[k];
+  if constexpr (CLUSTER) {
+    if (tid == 0) post_tr = tr;
+    cluster.sync();
+    tr = 0.0;
+    for (int q = 0; q < S; ++q) tr += *cluster.map_shared_rank(&post_tr, q);
+  }
   const double thr = tol * tr;
-  // the best remaining diagonal of all rows: this CTA's into every CTA's slot, the barrier (after
-  // which rows of L written before it are visible too), and the best of the posts
-  auto pivot = [&](int par, int& p) {
-    long long bv = own ? __double_as_longlong(d) : -1;
+  auto expect = [&](uint32_t bar, int bytes) {
+    if (tid == 0)
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
+                   : "memory");
+  };
+  // the first j entries of row i of L (this CTA's) into a slot of every CTA
+  auto send_row = [&](int j, int i, const T* slot, uint32_t bar) {
+    const T* mine = Ls + (size_t)(i / S) * rmax;
+    const uint32_t s0 = pc_su32(slot);
+    for (int q = warp; q < S; q += nw + 1) {
+      const uint32_t rb = pc_map(bar, q), rs = pc_map(s0, q);
+      for (int k = lane; k < j; k += 32) pc_send(rs + k * (int)sizeof(T), rb, mine[k]);
+    }
+  };
+  // The best remaining diagonal of all rows, as bits: this CTA's (all_rows: with that row of L, up
+  // to column j) into every CTA's slots, and the best of the posts.  A wait that gave up is noted
+  // in s_late, which the CTA's threads look at together, after their next barrier.
+  auto pivot = [&](int j, long long& bv, int& p) {
+    const int par = j & 1;
+    bv = own ? __double_as_longlong(d) : -1;
     int bi = own ? i : 0x7fffffff;
     warp_best(bv, bi);
     if (lane == 0 && warp < nw) {
@@ -739,91 +806,105 @@ __global__ void __launch_bounds__(32 * (kPcWarps + 1)) pchol_kernel(
       s_i[par][warp] = bi;
     }
     __syncthreads();
-    if (!CLUSTER || warp == 0) {
-      bv = lane < nw ? s_v[par][lane] : -1;
-      bi = lane < nw ? s_i[par][lane] : 0x7fffffff;
-      warp_best(bv, bi);
-    }
+    bv = lane < nw ? s_v[par][lane] : -1;
+    bi = lane < nw ? s_i[par][lane] : 0x7fffffff;
+    warp_best(bv, bi);
     if constexpr (CLUSTER) {
-      if (warp == 0 && lane < S) {
-        cluster.map_shared_rank(&post_v[par][0], lane)[c] = bv;
-        cluster.map_shared_rank(&post_i[par][0], lane)[c] = bi;
-      }
-      cluster.sync();
-      bv = lane < S ? post_v[par][lane] : -1;
-      bi = lane < S ? post_i[par][lane] : 0x7fffffff;
+      const uint32_t bar = pc_su32(&bars[par]);
+      expect(bar, S * (16 + (all_rows ? j * (int)sizeof(T) : 0)));
+      if (all_rows) send_row(j, bi, rows + ((size_t)par * S + c) * rmax, bar);
+      if (warp == 0 && lane < S)
+        pc_send(pc_map(pc_su32(&post[par][c]), lane), pc_map(bar, lane), bv, (long long)bi);
+      if (!pc_wait(bar, (uint32_t)(j >> 1) & 1)) s_late = 1;
+      const longlong2 v = post[par][lane & (kPcCtas - 1)];
+      bv = lane < S ? v.x : -1;
+      bi = lane < S ? (int)v.y : 0x7fffffff;
       warp_best(bv, bi);
     }
     p = bi;
-    return bv < 0 ? -1.0 : __longlong_as_double(bv);
   };
+  const long long thrb = __double_as_longlong(thr);
+  constexpr long long kInf = 0x7ff0000000000000ll;   // above: not a number
   int r = 0, p = -1;
-  double last = 0.0;
+  long long last = 0;
   for (int j = 0; j < rmax; ++j) {
-    const double dp = pivot(j & 1, p);
-    last = dp;
-    if (!(dp > thr)) break;
-    if (piv && c == 0 && tid == 0) piv[j] = p;
-    const T* prow = remote(Ls, p % S) + (size_t)(p / S) * rmax;
-    T wip = mkc<R>(0, 0), acc = mkc<R>(0, 0);
-    if (own) wip = w_rows ? Ws[(size_t)li * n + p] : w[(long)i * n + p];
-    if constexpr (CLUSTER) {
-      for (int k = tid; k < j; k += blockDim.x) lp[k] = prow[k];
+    pivot(j, last, p);
+    if (!(last > thrb && last <= kInf)) {
       __syncthreads();
-      prow = lp;
+      break;
     }
-    if (own) {
-      const T* lrow = Ls + (size_t)li * rmax;
-      T acc2 = mkc<R>(0, 0);
-      for (int k = l4; k < j; k += kPcLanes) {
-        const T a = lrow[k], b = prow[k];
-        // acc + acc2 += a * conj(b)
-        acc.x = fma(a.x, b.x, acc.x);
-        acc.y = fma(a.y, b.x, acc.y);
-        acc2.x = fma(a.y, b.y, acc2.x);
-        acc2.y = fma(-a.x, b.y, acc2.y);
+    if (piv && c == 0 && tid == 0) piv[j] = p;
+    const T* prow = Ls + (size_t)p * rmax;
+    if constexpr (CLUSTER) {
+      prow = rows + ((size_t)(j & 1) * nslot + (all_rows ? p % S : 0)) * rmax;
+      if (!all_rows) {
+        const uint32_t bar = pc_su32(&bars[2 + (j & 1)]);
+        expect(bar, j * (int)sizeof(T));
+        if (p % S == c) send_row(j, p, prow, bar);
+        if (!pc_wait(bar, (uint32_t)(j >> 1) & 1)) s_late = 1;
       }
-      acc = cadd(acc, acc2);
+    }
+    R wip = R(0), v = R(0);
+    if (own) {
+      const T* wr = w_rows ? Ws + (size_t)li * n : w + (long)i * n;
+      wip = reinterpret_cast<const R*>(wr + p)[part];
     }
     if (warp < nw) {
-      for (int o = kPcLanes / 2; o > 0; o >>= 1) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+      T acc = mkc<R>(0, 0), acc2 = mkc<R>(0, 0);
+      if (own) {
+        const T* lrow = Ls + (size_t)li * rmax;
+        for (int k = lr_; k < j; k += LANES) {
+          const T a = lrow[k], b = prow[k];
+          // acc + acc2 += a * conj(b)
+          acc.x = fma(a.x, b.x, acc.x);
+          acc.y = fma(a.y, b.x, acc.y);
+          acc2.x = fma(a.y, b.y, acc2.x);
+          acc2.y = fma(-a.x, b.y, acc2.y);
+        }
       }
-      acc = csub(wip, acc);
+      acc = cadd(acc, acc2);
+      // the first exchange leaves one half of the lanes the real part and the other the imaginary
+      const R give = part ? acc.x : acc.y;
+      v = (part ? acc.y : acc.x) + __shfl_xor_sync(0xffffffffu, give, LANES / 2);
+      for (int o = LANES / 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      v = wip - v;
     } else {
-      const double inv = rsqrt(dp);
+      const double dp = __longlong_as_double(last), inv = rsqrt(dp);
       if (lane == 0) {
         s_dp = dp * inv;
         s_inv = inv;
         s_inv2 = inv * inv;
       }
     }
+    double sq = (double)v * v;
+    sq += __shfl_xor_sync(0xffffffffu, sq, LANES / 2);
     __syncthreads();
+    if (CLUSTER && s_late) break;
     if (own) {
-      const R inv = (R)s_inv;
-      T lij = mkc<R>(acc.x * inv, acc.y * inv);
-      if (i == p) lij = mkc<R>((R)s_dp, R(0));
-      if (l4 == 0) Ls[(size_t)li * rmax + j] = lij;
-      const double nd = fma(-((double)acc.x * acc.x + (double)acc.y * acc.y), s_inv2, d);
+      const double nd = fma(-sq, s_inv2, d);
       d = (i == p || __double2hiint(nd) < 0) ? 0.0 : nd;
+      R lij = v * (R)s_inv;
+      if (i == p) lij = part ? R(0) : (R)s_dp;
+      if ((lr_ & (LANES / 2 - 1)) == 0) reinterpret_cast<R*>(Ls + (size_t)li * rmax + j)[part] = lij;
     }
     r = j + 1;
-    last = 0.0;
+    last = 0;
   }
-  if (r == rmax) last = pivot(rmax & 1, p);   // largest remaining diagonal, in the free slot
+  if (r == rmax) {                          // the largest remaining diagonal
+    pivot(rmax, last, p);
+    __syncthreads();
+  }
   if (c == 0 && tid == 0) {
-    *rout = r;
-    *resid = tr > 0 && last > 0.0 ? last / tr : 0.0;
+    const double ld = __longlong_as_double(last);
+    *rout = s_late ? 0 : r;                 // rank 0: no factor, as for a zero matrix
+    *resid = !s_late && tr > 0 && ld > 0.0 ? ld / tr : 0.0;
   }
-  // L to global memory only now: a store before a cluster barrier holds the barrier up until the
-  // store has landed
-  __syncthreads();
+  // L to global memory only now: a store before an exchange holds it up until the store has landed
   for (int e = tid; e < nlm * r; e += blockDim.x) {
     const int row = e / r, k = e - row * r;
     if (c + row * S < n) L[(long)(c + row * S) * lr + k] = Ls[(size_t)row * rmax + k];
   }
-  barrier();   // no CTA leaves while another may still read its shared memory
+  if constexpr (CLUSTER) cluster.sync();   // no CTA leaves before what was sent to it has landed
 }
 
 // x = L1^-1 (r x r, lower triangular, row-major), L1[a][b] = L[piv[a]][b] the pivot rows of a
@@ -1104,37 +1185,39 @@ template <typename R>
 cudaError_t pchol(cudaStream_t st, int n, const cx<R>* w, int rmax, double tol, cx<R>* L, int lr,
                   int* rout, double* resid, int* piv) {
   if (n < 1 || n > 1024 || rmax < 1 || rmax > kGradedMax) return cudaErrorInvalidValue;
-  // CTAs of the cluster: 64 rows each at most (the warps of a CTA).  One CTA needs no cluster
-  // barriers, which is worth more than the FP64 pipes of others up to 64 rows.
-  const int S = n > 128 ? kPcCtas : n > 64 ? 8 : 1;
+  // One CTA needs no exchange, which is worth more than other CTAs' FP64 pipes up to 32 rows (rank
+  // 24: 43 us against 49 us on four); then 16 to 32 rows a CTA (n 64, rank 45: four CTAs 96 us,
+  // eight 104, two 122; n 156, rank 52: eight 136, sixteen 140, four 171).  Eight lanes a row while
+  // the row warps are few (20 rows, rank 52: 2.87 us a column against 3.02; 32 rows: 3.34 against
+  // 3.00).  FP32 keeps four lanes: its sums keep their order.
+  const int S = n > 256 ? kPcCtas : n > 64 ? 8 : n > 32 ? 4 : 1;
   const int rows = (n + S - 1) / S;
-  const int threads = (rows * kPcLanes + 31) / 32 * 32 + 32;   // and the warp of the root
+  const int lanes = S > 1 && rows <= 20 && sizeof(R) == 8 ? 8 : 4;
+  const int threads = (rows * lanes + 31) / 32 * 32 + 32;   // and the warp of the root
   rmax = std::min(rmax, n);
-  const size_t lb = (size_t)rows * rmax * sizeof(cx<R>), wb = (size_t)rows * n * sizeof(cx<R>);
+  const size_t wb = (size_t)rows * n * sizeof(cx<R>);
   constexpr size_t kMax = 222 * 1024;   // leaves the static arrays their place
+  auto l_bytes = [&](int slots) { return ((size_t)rows + slots) * rmax * sizeof(cx<R>); };
+  const int all_rows = S > 1 && l_bytes(2 * S) <= kMax ? 1 : 0;
+  const size_t lb = l_bytes(S == 1 ? 0 : all_rows ? 2 * S : 2);
   const int w_rows = lb + wb <= kMax ? 1 : 0;
+  auto* kern = S == 1 ? pchol_kernel<R, false, 4>
+                      : lanes == 8 ? pchol_kernel<R, true, 8> : pchol_kernel<R, true, 4>;
   static const cudaError_t attr = [] {
-    cudaError_t e = cudaFuncSetAttribute(pchol_kernel<R, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMax);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(pchol_kernel<R, true>,
-                               cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(pchol_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kMax);
+    cudaError_t e = cudaSuccess;
+    for (auto* f : {pchol_kernel<R, false, 4>, pchol_kernel<R, true, 4>, pchol_kernel<R, true, 8>}) {
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMax);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    }
     return e;
   }();
   MPDO_CUDA_TRY(attr);
-  const size_t sm = w_rows ? lb + wb : lb;
-  count_launch();
-  if (S == 1) {
-    pchol_kernel<R, false><<<1, threads, sm, st>>>(n, w, rmax, tol, L, lr, rout, resid, piv, w_rows);
-    return cudaGetLastError();
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(S);
   cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = sm;
+  cfg.dynamicSmemBytes = w_rows ? lb + wb : lb;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1142,9 +1225,9 @@ cudaError_t pchol(cudaStream_t st, int n, const cx<R>* w, int rmax, double tol, 
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, pchol_kernel<R, true>, n, w, rmax, tol, L, lr, rout, resid, piv,
-                            w_rows);
+  cfg.numAttrs = S > 1 ? 1 : 0;
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, kern, n, w, rmax, tol, L, lr, rout, resid, piv, w_rows, all_rows);
 }
 template cudaError_t pchol<float>(cudaStream_t, int, const float2*, int, double, float2*, int,
                                   int*, double*, int*);
