@@ -76,6 +76,19 @@ cudaError_t rho_site(cudaStream_t st, long dl2, long dr2, cx<R>* r, cx<R>* tr, i
 template <typename R>
 cudaError_t env_dot(cudaStream_t st, long n2, const cx<R>* x, const cx<R>* y, int mode,
                     double* parts, double* out);
+// secondorder.cu: the real basis M[mu][dl^2][dr^2] (mu < 9) of a site's rf[(a,s,r)][(b,s',r')]
+template <typename R>
+cudaError_t so_site(cudaStream_t st, int dl, int dr, const cx<R>* rf, R* m);
+// crossed, diagonal and traced environments through that site, from the left or the right; w and
+// p: 12 matrices of dl^2 dr^2, and of the new environments' size
+template <typename R>
+cudaError_t so_step(cudaStream_t st, bool left, int dl, int dr, const R* m, R* cross, R* diag,
+                    const R* e, R* eout, R* w, R* p);
+// out (device, 5): tr rho^2, tr rho_L^2, tr rho_R^2, collision sum, tr rho from the environments of
+// dimension n on both sides of the cut; parts: 320 doubles
+template <typename R>
+cudaError_t so_dots(cudaStream_t st, int n, const R* cl, const R* cr, const R* dl, const R* dr,
+                    const R* el, const R* er, double* parts, double* out);
 // out (device double) = sum of |a|^2 over n complex entries, accumulated in FP64
 template <typename R>
 cudaError_t sumsq(cudaStream_t st, long n, const cx<R>* a, double* out);
