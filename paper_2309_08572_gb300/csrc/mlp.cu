@@ -30,11 +30,14 @@ namespace {
 
 constexpr int SBM = 64, SBN = 64, SBK = 16, SNT = 256;
 
-// C = op(A) op(B), A is M x K after op, B is K x N after op (row-major storage).
+// C = op(A) op(B), A is M x K after op, B is K x N after op (row-major storage); then, where given,
+// + bias per column, tanh (act), and times 1 - a^2 (a like C): passes of their own over the small
+// matrices would each cost a launch.
 __global__ void __launch_bounds__(SNT) sgemm_kernel(int M, int N, int K, const float* __restrict__ A,
                                                     long sam, long sak, const float* __restrict__ B,
                                                     long sbk, long sbn, float* C, long ldc,
-                                                    const float* __restrict__ bias) {
+                                                    const float* __restrict__ bias, int act,
+                                                    const float* __restrict__ a2) {
   __shared__ float As[SBK][SBM + 4];
   __shared__ float Bs[SBK][SBN + 4];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -76,14 +79,15 @@ __global__ void __launch_bounds__(SNT) sgemm_kernel(int M, int N, int K, const f
     for (int j = 0; j < 4; ++j) {
       int gn = n0 + tx + 16 * j;
       if (gn >= N) continue;
-      C[gm * ldc + gn] = acc[i][j] + (bias ? bias[gn] : 0.f);
+      float v = acc[i][j] + (bias ? bias[gn] : 0.f);
+      if (act) v = tanhf(v);
+      if (a2) {
+        const float x = a2[gm * ldc + gn];
+        v *= (1.f - x * x);
+      }
+      C[gm * ldc + gn] = v;
     }
   }
-}
-
-__global__ void tanh_kernel(long n, float* z) {
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n; e += (long)gridDim.x * blockDim.x)
-    z[e] = tanhf(z[e]);
 }
 
 // dz = 2 (y - t) / (B n_out); per-block partial sums of (y - t)^2 into part[]
@@ -105,20 +109,19 @@ __global__ void mse_grad_kernel(long n, float scale, const float* __restrict__ y
   if (threadIdx.x == 0) part[blockIdx.x] = red[0];
 }
 
-// da <- da * (1 - a^2)
-__global__ void tanh_back_kernel(long n, const float* __restrict__ a, float* da) {
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n; e += (long)gridDim.x * blockDim.x) {
-    float v = a[e];
-    da[e] *= (1.f - v * v);
-  }
-}
-
-// db[j] = sum_i dz[i][j]
-__global__ void colsum_kernel(int rows, int cols, const float* __restrict__ dz, float* db) {
-  int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= cols) return;
+// db[j] = sum_i dz[i][j]: 32 columns a block, the rows over eight warps (one thread a column took
+// 31 us at 512 rows), added in a fixed order.
+__global__ void __launch_bounds__(256) colsum_kernel(int rows, int cols, const float* __restrict__ dz,
+                                                     float* db) {
+  __shared__ float part[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = blockIdx.x * 32 + lane;
   float s = 0.f;
-  for (int i = 0; i < rows; ++i) s += dz[(long)i * cols + j];
+  if (j < cols)
+    for (int i = warp; i < rows; i += 8) s += dz[(long)i * cols + j];
+  part[warp][lane] = s;
+  __syncthreads();
+  if (warp || j >= cols) return;
+  for (int w = 1; w < 8; ++w) s += part[w][lane];
   db[j] = s;
 }
 
@@ -162,11 +165,18 @@ struct mpdo_mlp_s {
   int t = 0;
   int maxw = 0;
   std::string err;
-  // BF16 tensor-core products (mpdo_mlp_set_precision): packed operands and the pipeline's
-  // error flag; the parameters, gradients and Adam moments stay FP32
+  // BF16 tensor-core products (mpdo_mlp_set_precision): the operands of every layer, the parts of
+  // the bias gradients and the loss, and the pipeline's error flag in one allocation; the
+  // parameters, gradients and Adam moments stay FP32
   int tc = 0;
-  void *pa = nullptr, *pb = nullptr;
-  int* tcerr = nullptr;
+  void* tcmem = nullptr;
+  std::vector<__nv_bfloat16*> xr, xc, zr, zc;   // activations and dz (index: layer's units), K-major
+  std::vector<__nv_bfloat16*> wr, wt;           // weights as they are and transposed
+  std::vector<float*> csum;
+  double* lpart = nullptr;
+  struct TcOut { double loss; int err, pad; };
+  TcOut* tcout = nullptr;
+  long ldb = 0;                                 // row stride of xc and zc
 };
 
 namespace {
@@ -183,87 +193,139 @@ int mlp_fail(mpdo_mlp m, int code, const std::string& msg) {
     if (_e != cudaSuccess) return mlp_fail(m, MPDO_ERR_CUDA, std::string(#expr) + ": " + cudaGetErrorString(_e)); \
   } while (0)
 
-__global__ void add_bias_kernel(int M, int N, float* C, long ldc, const float* __restrict__ bias) {
-  const long total = (long)M * N;
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total;
-       e += (long)gridDim.x * blockDim.x)
-    C[(e / N) * ldc + e % N] += bias[e % N];
-}
-
-// C = op(A) op(B) (+ bias per column), A is M x K after op, B is K x N after op.  FP32 on the
-// CUDA cores, or (m->tc) BF16 operands on the tensor cores with FP32 accumulation: op(A) and
-// op(B)^T are packed K-major in BF16 and multiplied by the tcgen05 core.
+// C = op(A) op(B), A is M x K after op, B is K x N after op, in FP32 on the CUDA cores, with
+// sgemm_kernel's elementwise work.
 cudaError_t sgemm(mpdo_mlp m, bool ta, bool tb, int M, int N, int K, const float* A, long lda,
-                  const float* B, long ldb, float* C, long ldc, const float* bias) {
-  cudaStream_t st = m->st;
+                  const float* B, long ldb, float* C, long ldc, const float* bias, int act,
+                  const float* a2) {
   long sam = ta ? 1 : lda, sak = ta ? lda : 1;
   long sbk = tb ? 1 : ldb, sbn = tb ? ldb : 1;
-  if (m->tc && M > 0 && N > 0 && K > 0) {
-    const long ldk = (K + 7) / 8 * 8;   // 16-byte rows
-    MPDO_CUDA_TRY(mpdo::tc_pack_real_bf16(st, M, K, A, sam, sak, m->pa, ldk));
-    MPDO_CUDA_TRY(mpdo::tc_pack_real_bf16(st, N, K, B, sbn, sbk, m->pb, ldk));
-    mpdo::TcEpilogue e;
-    e.d = C;
-    e.ldd = ldc;
-    MPDO_CUDA_TRY(mpdo::tc_gemm_real(st, 2, M, N, K, m->pa, ldk, 0, m->pb, ldk, 0, 1, e,
-                                     m->tcerr, 0));
-    if (bias) {
-      mpdo::count_launch();
-      add_bias_kernel<<<nb((long)M * N), 256, 0, st>>>(M, N, C, ldc, bias);
-    }
-    return cudaGetLastError();
-  }
   dim3 grid((N + SBN - 1) / SBN, (M + SBM - 1) / SBM);
   mpdo::count_launch();
-  sgemm_kernel<<<grid, SNT, 0, st>>>(M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, bias);
+  sgemm_kernel<<<grid, SNT, 0, m->st>>>(M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, bias, act, a2);
   return cudaGetLastError();
 }
 
-// forward pass into m->acts (acts[0] must hold x)
-int run_forward(mpdo_mlp m, int batch) {
+// layers [0, n) of the forward pass into m->acts; y: where the output goes if n is all of them
+int run_forward(mpdo_mlp m, int batch, int n, const float* x, float* y) {
   const int L = (int)m->w.size() - 1;
-  for (int l = 0; l < L; ++l) {
-    MK(sgemm(m, false, false, batch, m->w[l + 1], m->w[l], m->acts[l], m->w[l],
-             m->params + m->woff[l], m->w[l + 1], m->acts[l + 1], m->w[l + 1],
-             m->params + m->boff[l]));
-    if (l < L - 1) {
-      long n = (long)batch * m->w[l + 1];
-      mpdo::count_launch();
-      tanh_kernel<<<nb(n), 256, 0, m->st>>>(n, m->acts[l + 1]);
-      MK(cudaGetLastError());
-    }
-  }
+  for (int l = 0; l < n; ++l)
+    MK(sgemm(m, false, false, batch, m->w[l + 1], m->w[l], l ? m->acts[l] : x, m->w[l],
+             m->params + m->woff[l], m->w[l + 1], l == L - 1 ? y : m->acts[l + 1], m->w[l + 1],
+             m->params + m->boff[l], l < L - 1, nullptr));
   return MPDO_OK;
 }
 
-// backward from d(output) in m->da; fills m->grads if want_params; leaves d(input) in m->da
-int run_backward(mpdo_mlp m, int batch, bool want_params) {
+// backward from d(output) in m->da: the gradients of the parameters (x) or of the input (gx)
+int run_backward(mpdo_mlp m, int batch, const float* x, float* gx) {
   const int L = (int)m->w.size() - 1;
   float* cur = m->da;
   float* nxt = m->db2;
   for (int l = L - 1; l >= 0; --l) {
     const int fi = m->w[l], fo = m->w[l + 1];
-    if (l < L - 1) {
-      long n = (long)batch * fo;
-      mpdo::count_launch();
-      tanh_back_kernel<<<nb(n), 256, 0, m->st>>>(n, m->acts[l + 1], cur);
-      MK(cudaGetLastError());
-    }
-    if (want_params) {
+    if (!gx) {
       // dW = a_{l-1}^T dz  (fi x fo), db = colsum(dz)
-      MK(sgemm(m, true, false, fi, fo, batch, m->acts[l], fi, cur, fo, m->grads + m->woff[l],
-               fo, nullptr));
+      MK(sgemm(m, true, false, fi, fo, batch, l ? m->acts[l] : x, fi, cur, fo,
+               m->grads + m->woff[l], fo, nullptr, 0, nullptr));
       mpdo::count_launch();
-      colsum_kernel<<<(fo + 127) / 128, 128, 0, m->st>>>(batch, fo, cur, m->grads + m->boff[l]);
+      colsum_kernel<<<(fo + 31) / 32, 256, 0, m->st>>>(batch, fo, cur, m->grads + m->boff[l]);
       MK(cudaGetLastError());
+      if (l == 0) break;
     }
-    // da_{l-1} = dz W^T  (batch x fi)
-    MK(sgemm(m, false, true, batch, fi, fo, cur, fo, m->params + m->woff[l], fo, nxt, fi,
-             nullptr));
+    // dz_l = (dz_{l+1} W^T) (1 - a_l^2)  (batch x fi)
+    MK(sgemm(m, false, true, batch, fi, fo, cur, fo, m->params + m->woff[l], fo, l ? nxt : gx, fi,
+             nullptr, 0, l ? m->acts[l] : nullptr));
     std::swap(cur, nxt);
   }
-  if (cur != m->da) MK(cudaMemcpyAsync(m->da, cur, sizeof(float) * (size_t)batch * m->w[0],
-                                       cudaMemcpyDeviceToDevice, m->st));
+  return MPDO_OK;
+}
+
+// ---- the same on the tensor cores (mpdo_mlp_set_precision)
+inline long r8(long x) { return (x + 7) / 8 * 8; }   // 16-byte rows
+
+// BF16 operands of the pass: the weights (tr: transposed, for the forward pass; pl: as they are,
+// for the backward one), x, and wout on every row of the output's dz
+int tc_operands(mpdo_mlp m, int batch, const float* x, bool pl, bool xcol, const float* wout) {
+  const int L = (int)m->w.size() - 1;
+  mpdo::MlpPack g;
+  g.count = 0;
+  g.job[g.count++] = {x, m->w[0], batch, m->w[0], 0, m->xr[0], xcol ? m->xc[0] : nullptr,
+                      r8(m->w[0]), m->ldb};
+  for (int l = 0; l < L; ++l)
+    g.job[g.count++] = {m->params + m->woff[l], m->w[l + 1], m->w[l], m->w[l + 1], 0,
+                        pl ? m->wr[l] : nullptr, m->wt[l], r8(m->w[l + 1]), r8(m->w[l])};
+  if (wout)
+    g.job[g.count++] = {wout, 0, batch, m->w[L], 0, m->zr[L], nullptr, r8(m->w[L]), 0};
+  MK(mpdo::mlp_pack(m->st, g));
+  return MPDO_OK;
+}
+
+int tc_product(mpdo_mlp m, const __nv_bfloat16* A, const __nv_bfloat16* B, int M, int N, int K,
+               const mpdo::MlpEpi& e) {
+  mpdo::MlpGroup<1> g = {};
+  mpdo::MlpProd& p = g.p[0];
+  p.A = A; p.B = B; p.lda = p.ldb = r8(K);
+  p.M = M; p.N = N; p.K = K;
+  p.e = e;
+  g.count = 1;
+  MK(mpdo::mlp_products<1>(m->st, g, &m->tcout->err));
+  return MPDO_OK;
+}
+
+// layers [0, n): hidden ones into m->acts and the operands of the next product (and, train, of the
+// weight gradients); the output layer by `out`
+int tc_forward(mpdo_mlp m, int batch, int n, bool train, const mpdo::MlpEpi& out) {
+  const int L = (int)m->w.size() - 1;
+  for (int l = 0; l < n; ++l) {
+    const int fo = m->w[l + 1];
+    mpdo::MlpEpi e = {};
+    if (l < L - 1) {
+      e.act = 1;
+      e.d = m->acts[l + 1]; e.ldd = fo;
+      e.row = m->xr[l + 1]; e.ldr = r8(fo);
+      if (train) { e.col = m->xc[l + 1]; e.ldc = m->ldb; }
+    } else {
+      e = out;
+    }
+    e.bias = m->params + m->boff[l];
+    int rc = tc_product(m, m->xr[l], m->wt[l], batch, fo, m->w[l], e);
+    if (rc) return rc;
+  }
+  return MPDO_OK;
+}
+
+// from the output's dz (zr[L], zc[L], csum[L]): the gradients of the parameters and the loss, or
+// of the input
+int tc_backward(mpdo_mlp m, int batch, float* gx) {
+  const int L = (int)m->w.size() - 1;
+  for (int l = L - 1; l >= (gx ? 0 : 1); --l) {
+    const int fi = m->w[l], fo = m->w[l + 1];
+    mpdo::MlpEpi e = {};
+    if (l) {
+      e.a = m->acts[l]; e.lda = fi;
+      e.row = m->zr[l]; e.ldr = r8(fi);
+      if (!gx) { e.col = m->zc[l]; e.ldc = m->ldb; e.csum = m->csum[l]; }
+    } else {
+      e.d = gx; e.ldd = fi;
+    }
+    int rc = tc_product(m, m->zr[l + 1], m->wr[l], batch, fi, fo, e);
+    if (rc) return rc;
+  }
+  if (gx) return MPDO_OK;
+  mpdo::MlpGroup<mpdo::kMlpMaxLayers> g = {};
+  for (int l = 0; l < L; ++l) {
+    mpdo::MlpProd& p = g.p[l];
+    p.A = m->xc[l]; p.B = m->zc[l + 1]; p.lda = p.ldb = m->ldb;
+    p.M = m->w[l]; p.N = m->w[l + 1]; p.K = batch;
+    p.e.d = m->grads + m->woff[l]; p.e.ldd = m->w[l + 1];
+    p.sum_in = m->csum[l + 1]; p.sum_out = m->grads + m->boff[l];
+  }
+  g.count = L;
+  g.parts = (batch + 31) / 32;
+  g.loss = m->lpart;
+  g.loss_n = (long)g.parts * ((m->w[L] + 31) / 32);
+  g.loss_sum = &m->tcout->loss;
+  MK(mpdo::mlp_products<mpdo::kMlpMaxLayers>(m->st, g, &m->tcout->err));
   return MPDO_OK;
 }
 
@@ -347,35 +409,55 @@ int mpdo_mlp_get_params(mpdo_mlp m, float* host) {
 
 int mpdo_mlp_forward(mpdo_mlp m, int batch, const float* x, float* y) {
   if (!m || !x || !y || batch < 1 || batch > m->max_batch) return mlp_fail(m, MPDO_ERR_ARG, "mlp: bad forward arguments");
-  MK(cudaMemcpyAsync(m->acts[0], x, sizeof(float) * (size_t)batch * m->w[0], cudaMemcpyDeviceToDevice, m->st));
-  int rc = run_forward(m, batch);
-  if (rc) return rc;
   const int L = (int)m->w.size() - 1;
-  MK(cudaMemcpyAsync(y, m->acts[L], sizeof(float) * (size_t)batch * m->w[L], cudaMemcpyDeviceToDevice, m->st));
-  return MPDO_OK;
+  if (!m->tc) {
+    if (L == 1) {   // the one product reads x while it writes y, which may be the same memory
+      MK(cudaMemcpyAsync(m->acts[0], x, sizeof(float) * (size_t)batch * m->w[0],
+                         cudaMemcpyDeviceToDevice, m->st));
+      x = m->acts[0];
+    }
+    return run_forward(m, batch, L, x, y);
+  }
+  int rc = tc_operands(m, batch, x, false, false, nullptr);
+  if (rc) return rc;
+  mpdo::MlpEpi e = {};
+  e.d = y; e.ldd = m->w[L];
+  return tc_forward(m, batch, L, false, e);
 }
 
 int mpdo_mlp_loss_grad(mpdo_mlp m, int batch, const float* x, const float* t, float* loss,
                        float* grad_host) {
   if (!m || !x || !t || batch < 1 || batch > m->max_batch) return mlp_fail(m, MPDO_ERR_ARG, "mlp: bad loss_grad arguments");
-  MK(cudaMemcpyAsync(m->acts[0], x, sizeof(float) * (size_t)batch * m->w[0], cudaMemcpyDeviceToDevice, m->st));
-  int rc = run_forward(m, batch);
-  if (rc) return rc;
   const int L = (int)m->w.size() - 1;
   const long n = (long)batch * m->w[L];
-  const int blocks = nb(n);
-  mpdo::count_launch();
-  mse_grad_kernel<<<blocks, 256, 0, m->st>>>(n, 1.f / (float)n, m->acts[L], t, m->da, m->part);
-  MK(cudaGetLastError());
-  rc = run_backward(m, batch, true);
-  if (rc) return rc;
-  MK(cudaMemcpyAsync(m->hpart, m->part, sizeof(double) * blocks, cudaMemcpyDeviceToHost, m->st));
+  int rc, blocks = 0;
+  if (m->tc) {
+    if ((rc = tc_operands(m, batch, x, true, true, nullptr))) return rc;
+    mpdo::MlpEpi e = {};
+    e.t = t; e.scale = 1.f / (float)n; e.loss = m->lpart;
+    e.row = m->zr[L]; e.ldr = r8(m->w[L]);
+    e.col = m->zc[L]; e.ldc = m->ldb;
+    e.csum = m->csum[L];
+    if ((rc = tc_forward(m, batch, L, true, e))) return rc;
+    if ((rc = tc_backward(m, batch, nullptr))) return rc;
+    MK(cudaMemcpyAsync(m->hpart, m->tcout, sizeof(mpdo_mlp_s::TcOut), cudaMemcpyDeviceToHost, m->st));
+  } else {
+    if ((rc = run_forward(m, batch, L, x, m->acts[L]))) return rc;
+    blocks = nb(n);
+    mpdo::count_launch();
+    mse_grad_kernel<<<blocks, 256, 0, m->st>>>(n, 1.f / (float)n, m->acts[L], t, m->da, m->part);
+    MK(cudaGetLastError());
+    if ((rc = run_backward(m, batch, x, nullptr))) return rc;
+    MK(cudaMemcpyAsync(m->hpart, m->part, sizeof(double) * blocks, cudaMemcpyDeviceToHost, m->st));
+  }
   if (grad_host) MK(cudaMemcpyAsync(grad_host, m->grads, sizeof(float) * m->n_params, cudaMemcpyDeviceToHost, m->st));
-  if (m->tc) MK(cudaMemcpyAsync(m->hpart + 4095, m->tcerr, sizeof(int), cudaMemcpyDeviceToHost, m->st));
   MK(cudaStreamSynchronize(m->st));
-  if (m->tc && *reinterpret_cast<int*>(m->hpart + 4095))
-    return mlp_fail(m, MPDO_ERR_TIMEOUT, "mlp: a tensor-core pipeline wait gave up");
   double s = 0;
+  if (m->tc) {
+    const mpdo_mlp_s::TcOut& o = *reinterpret_cast<const mpdo_mlp_s::TcOut*>(m->hpart);
+    if (o.err) return mlp_fail(m, MPDO_ERR_TIMEOUT, "mlp: a tensor-core pipeline wait gave up");
+    s = o.loss;
+  }
   for (int b = 0; b < blocks; ++b) s += m->hpart[b];
   if (loss) *loss = (float)(s / (double)n);
   return MPDO_OK;
@@ -396,18 +478,21 @@ int mpdo_mlp_adam_step(mpdo_mlp m, float lr) {
 int mpdo_mlp_input_grad(mpdo_mlp m, int batch, const float* x, const float* wout_host, float* gx) {
   if (!m || !x || !wout_host || !gx || batch < 1 || batch > m->max_batch)
     return mlp_fail(m, MPDO_ERR_ARG, "mlp: bad input_grad arguments");
-  MK(cudaMemcpyAsync(m->acts[0], x, sizeof(float) * (size_t)batch * m->w[0], cudaMemcpyDeviceToDevice, m->st));
-  int rc = run_forward(m, batch);
-  if (rc) return rc;
   const int L = (int)m->w.size() - 1;
-  // d(output) = wout broadcast over rows
+  // d(output) = wout broadcast over rows; the output itself is not needed
   MK(cudaMemcpyAsync(m->db2, wout_host, sizeof(float) * m->w[L], cudaMemcpyHostToDevice, m->st));
-  mpdo::count_launch();
-  fill_rows_kernel<<<nb((long)batch * m->w[L]), 256, 0, m->st>>>(batch, m->w[L], m->db2, m->da);
-  MK(cudaGetLastError());
-  rc = run_backward(m, batch, false);
-  if (rc) return rc;
-  MK(cudaMemcpyAsync(gx, m->da, sizeof(float) * (size_t)batch * m->w[0], cudaMemcpyDeviceToDevice, m->st));
+  int rc;
+  if (m->tc) {
+    if ((rc = tc_operands(m, batch, x, true, false, m->db2))) return rc;
+    if ((rc = tc_forward(m, batch, L - 1, false, {}))) return rc;
+    if ((rc = tc_backward(m, batch, gx))) return rc;
+  } else {
+    if ((rc = run_forward(m, batch, L - 1, x, nullptr))) return rc;
+    mpdo::count_launch();
+    fill_rows_kernel<<<nb((long)batch * m->w[L]), 256, 0, m->st>>>(batch, m->w[L], m->db2, m->da);
+    MK(cudaGetLastError());
+    if ((rc = run_backward(m, batch, x, gx))) return rc;
+  }
   MK(cudaStreamSynchronize(m->st));
   return MPDO_OK;
 }
@@ -415,15 +500,49 @@ int mpdo_mlp_input_grad(mpdo_mlp m, int batch, const float* x, const float* wout
 int mpdo_mlp_set_precision(mpdo_mlp m, int mode) {
   if (!m || (mode != 0 && mode != 1)) return mlp_fail(m, MPDO_ERR_ARG, "mlp: precision mode must be 0 or 1");
   MK(cudaStreamSynchronize(m->st));
-  if (mode == 1 && !m->pa) {
-    const long r = std::max(m->max_batch, m->maxw), ldk = (r + 7) / 8 * 8;
-    const size_t bytes = (size_t)r * ldk * 2;
-    if (cudaMalloc(&m->pa, bytes) != cudaSuccess || cudaMalloc(&m->pb, bytes) != cudaSuccess ||
-        cudaMalloc(&m->tcerr, sizeof(int)) != cudaSuccess) {
-      cudaGetLastError();
-      return mlp_fail(m, MPDO_ERR_OOM, "mlp: tensor-core operand buffers");
+  if (mode == 1 && !m->tcmem) {
+    const int L = (int)m->w.size() - 1;
+    const long ldb = r8(m->max_batch), groups = (m->max_batch + 127) / 128 * 4;
+    // twice: the sizes, then the addresses
+    uintptr_t base = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+      size_t off = 0;
+      auto take = [&](size_t bytes) {
+        void* p = reinterpret_cast<void*>(base + off);
+        off += (bytes + 255) / 256 * 256;
+        return p;
+      };
+      m->xr.assign(L + 1, nullptr);
+      m->xc = m->zr = m->zc = m->wr = m->wt = m->xr;
+      m->csum.assign(L + 1, nullptr);
+      auto bf = [&](long rows, long ld) { return static_cast<__nv_bfloat16*>(take(2 * rows * ld)); };
+      for (int l = 0; l <= L; ++l) {
+        const long w = m->w[l];
+        if (l < L) {
+          m->xr[l] = bf(m->max_batch, r8(w));
+          m->xc[l] = bf(w, ldb);
+          m->wr[l] = bf(w, r8(m->w[l + 1]));
+          m->wt[l] = bf(m->w[l + 1], r8(w));
+        }
+        if (l > 0) {
+          m->zr[l] = bf(m->max_batch, r8(w));
+          m->zc[l] = bf(w, ldb);
+          m->csum[l] = static_cast<float*>(take(sizeof(float) * groups * w));
+        }
+      }
+      m->lpart = static_cast<double*>(take(sizeof(double) * groups * ((m->w[L] + 31) / 32)));
+      m->tcout = static_cast<mpdo_mlp_s::TcOut*>(take(sizeof(mpdo_mlp_s::TcOut)));
+      if (pass == 0) {
+        if (cudaMalloc(&m->tcmem, off) != cudaSuccess) {
+          cudaGetLastError();
+          m->tcmem = nullptr;
+          return mlp_fail(m, MPDO_ERR_OOM, "mlp: tensor-core operand buffers");
+        }
+        base = reinterpret_cast<uintptr_t>(m->tcmem);
+      }
     }
-    MK(cudaMemsetAsync(m->tcerr, 0, sizeof(int), m->st));
+    m->ldb = ldb;
+    MK(cudaMemsetAsync(m->tcout, 0, sizeof(mpdo_mlp_s::TcOut), m->st));
   }
   m->tc = mode;
   return MPDO_OK;
@@ -432,9 +551,7 @@ int mpdo_mlp_set_precision(mpdo_mlp m, int mode) {
 int mpdo_mlp_destroy(mpdo_mlp m) {
   if (!m) return MPDO_OK;
   if (m->st) cudaStreamSynchronize(m->st);
-  if (m->pa) cudaFree(m->pa);
-  if (m->pb) cudaFree(m->pb);
-  if (m->tcerr) cudaFree(m->tcerr);
+  if (m->tcmem) cudaFree(m->tcmem);
   for (float* p : m->acts) if (p) cudaFree(p);
   if (m->params) cudaFree(m->params);
   if (m->grads) cudaFree(m->grads);

@@ -167,10 +167,12 @@ struct Epi {
   int mode;       // 0: FP32 (complex alpha/beta), 1: FP64 accumulate
 };
 
-template <int ELT, int BN, int STAGES>
-__global__ void __launch_bounds__(kThreads, 1)
-    tc_gemm_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb,
-                   int M, int N, int K, Epi ep, int* err) {
+// One output tile of the real product: A rows from m0, B rows from n0, batch entry bz.  epi(row,
+// column, v) takes each thread's 32 columns of its row; all lanes call it, also beyond the matrix.
+// DEP: the launch may begin before its predecessor in the stream has ended, and waits for it here.
+template <int ELT, int BN, int STAGES, bool DEP, typename F>
+__device__ __forceinline__ void tc_tile(const CUtensorMap* ma, const CUtensorMap* mb, int m0, int n0,
+                                        int bz, int K, int* err, F&& epi) {
   constexpr int BK = 128 / ELT;                      // elements per 128-byte k-block row
   constexpr uint32_t A_BYTES = BM * 128, B_BYTES = BN * 128;
   constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
@@ -185,7 +187,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   int* abort_flag = reinterpret_cast<int*>(tslot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n0 = blockIdx.x * BN, m0 = blockIdx.y * BM, bz = blockIdx.z;
   const int nk = (K + BK - 1) / BK;
 
   if (threadIdx.x == 0) {
@@ -209,6 +210,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  if constexpr (DEP) asm volatile("griddepcontrol.wait;" ::: "memory");
 
   if (warp == 0) {
     if (lane == 0) {
@@ -223,8 +225,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (*(volatile int*)abort_flag) break;
         uint8_t* sa = smem + s * STAGE_BYTES;
         mbar_expect_tx(&full[s], STAGE_BYTES);
-        tma_load_3d(sa, &ma, &full[s], kb * BK, m0, bz);
-        tma_load_3d(sa + A_BYTES, &mb, &full[s], kb * BK, n0, bz);
+        tma_load_3d(sa, ma, &full[s], kb * BK, m0, bz);
+        tma_load_3d(sa + A_BYTES, mb, &full[s], kb * BK, n0, bz);
       }
     }
     __syncwarp();
@@ -269,30 +271,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int c = 0; c < BN; c += 32) {
       float v[32];
       tmem_ld32(tw + c, v);
-      if (row < M) {
-        const int col0 = n0 + c;
-        if (ep.mode == 0) {
-          float* dp = ep.d + (long)bz * ep.sd + (long)row * ep.ldd + col0;
-#pragma unroll
-          for (int j = 0; j < 32; j += 2) {
-            if (col0 + j >= N) break;
-            const float xr = v[j], xi = v[j + 1];
-            float yr = ep.ar * xr - ep.ai * xi, yi = ep.ar * xi + ep.ai * xr;
-            if (ep.use_beta) {
-              const float cr = dp[j], ci = (col0 + j + 1 < N) ? dp[j + 1] : 0.f;
-              yr += ep.br * cr - ep.bi * ci;
-              yi += ep.br * ci + ep.bi * cr;
-            }
-            dp[j] = yr;
-            if (col0 + j + 1 < N) dp[j + 1] = yi;
-          }
-        } else {
-          double* dp = ep.d64 + (long)bz * ep.sd + (long)row * ep.ldd + col0;
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (col0 + j < N) dp[j] += ep.scale * (double)v[j];
-        }
-      }
+      epi(row, n0 + c, v);
     }
   }
   tc_fence_before();
@@ -303,6 +282,179 @@ __global__ void __launch_bounds__(kThreads, 1)
                  "r"(TMEM_COLS)
                  : "memory");
   }
+}
+
+template <int ELT, int BN, int STAGES>
+__global__ void __launch_bounds__(kThreads, 1)
+    tc_gemm_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb,
+                   int M, int N, int K, Epi ep, int* err) {
+  const int bz = blockIdx.z;
+  auto epi = [&](int row, int col0, const float* v) {
+    if (row < M) {
+      if (ep.mode == 0) {
+        float* dp = ep.d + (long)bz * ep.sd + (long)row * ep.ldd + col0;
+#pragma unroll
+        for (int j = 0; j < 32; j += 2) {
+          if (col0 + j >= N) break;
+          const float xr = v[j], xi = v[j + 1];
+          float yr = ep.ar * xr - ep.ai * xi, yi = ep.ar * xi + ep.ai * xr;
+          if (ep.use_beta) {
+            const float cr = dp[j], ci = (col0 + j + 1 < N) ? dp[j + 1] : 0.f;
+            yr += ep.br * cr - ep.bi * ci;
+            yi += ep.br * ci + ep.bi * cr;
+          }
+          dp[j] = yr;
+          if (col0 + j + 1 < N) dp[j + 1] = yi;
+        }
+      } else {
+        double* dp = ep.d64 + (long)bz * ep.sd + (long)row * ep.ldd + col0;
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+          if (col0 + j < N) dp[j] += ep.scale * (double)v[j];
+      }
+    }
+  };
+  tc_tile<ELT, BN, STAGES, false>(&ma, &mb, blockIdx.y * BM, blockIdx.x * BN, bz, K, err, epi);
+}
+
+// ------------------------------------------------------------------ surrogate's products
+// Products of the fully connected network in BF16 with the elementwise work around them in the
+// epilogue: bias and tanh going forward, the loss, tanh' going back, the operands of the products
+// that follow (BF16, K-major in both orientations) and the column sums of the biases' gradients.
+// The network is small (256 wide, a batch of 512: 2 us of products), so a pass is bound by its
+// launches, each with its drain and fill: packing, bias, tanh and sums of their own made 52 of
+// them a training step, now it takes 10.  A launch runs a group of products (all weight gradients
+// at once, with the sums of the parts in blocks behind the tiles), and its set-up (barriers, TMEM,
+// descriptors) overlaps the end of the launch before it (programmatic dependent launch).
+// A training step at batch 512 (24-256-256-256-2): 363 -> 99 us (136 without the overlap and with
+// tiles of 64 columns at least), an input gradient at batch 64: 193 -> 54 us (82).
+__device__ __forceinline__ void mlp_epilogue(const MlpEpi& e, int M, int N, int row, int col0,
+                                             float* v, int tiles_n) {
+  if (col0 >= N) return;
+  const int lane = threadIdx.x & 31;
+  const bool in = row < M;
+  if (e.bias) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (col0 + j < N) v[j] += e.bias[col0 + j];
+  }
+  if (e.act) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = tanhf(v[j]);
+  }
+  if (e.t) {
+    double s = 0;
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (in && col0 + j < N) {
+        const float d = v[j] - e.t[(long)row * N + col0 + j];
+        v[j] = 2.f * d * e.scale;
+        s += (double)d * d;
+      }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) e.loss[(long)(row / 32) * tiles_n + col0 / 32] = s;
+  }
+  if (e.a && in) {
+    const float* ap = e.a + (long)row * e.lda + col0;
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (col0 + j < N) {
+        const float x = ap[j];
+        v[j] *= (1.f - x * x);
+      }
+  }
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    if (!in || col0 + j >= N) v[j] = 0.f;
+  if (in && e.d) {
+    float* dp = e.d + (long)row * e.ldd + col0;
+    if (col0 + 32 <= N && e.ldd % 4 == 0 && (reinterpret_cast<uintptr_t>(e.d) & 15) == 0) {
+#pragma unroll
+      for (int j = 0; j < 32; j += 4)
+        *reinterpret_cast<float4*>(dp + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        if (col0 + j < N) dp[j] = v[j];
+    }
+  }
+  if (in && e.row) {   // rows of ldr % 8 == 0, zeros behind the last column
+    __nv_bfloat162* rp = reinterpret_cast<__nv_bfloat162*>(e.row + (long)row * e.ldr + col0);
+#pragma unroll
+    for (int j = 0; j < 32; j += 8)
+      if (col0 + j < e.ldr) {
+        __nv_bfloat162 q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) q[i] = __floats2bfloat162_rn(v[j + 2 * i], v[j + 2 * i + 1]);
+        *reinterpret_cast<uint4*>(rp + j / 2) = *reinterpret_cast<const uint4*>(q);
+      }
+  }
+  if (in && e.col) {   // neighbouring lanes, neighbouring rows
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (col0 + j < N) e.col[(long)(col0 + j) * e.ldc + row] = __float2bfloat16_rn(v[j]);
+  }
+  if (e.csum) {
+    // sums over the warp's rows: each exchange hands half of the remaining columns over, and lane
+    // l ends with column l
+    float x[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) x[j] = v[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const bool up = lane & o;
+#pragma unroll
+      for (int j = 0; j < o; ++j) {
+        const float give = up ? x[j] : x[j + o], keep = up ? x[j + o] : x[j];
+        x[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+    }
+    if (col0 + lane < N) e.csum[(long)(row / 32) * N + col0 + lane] = x[0];
+  }
+}
+
+template <int BN, int STAGES, int CAP>
+__global__ void __launch_bounds__(kThreads, 1)
+    mlp_gemm_kernel(const __grid_constant__ MlpGroup<CAP> g, int* err) {
+  const int b = blockIdx.x;
+  // the next launch may be set up while this one runs; its own wait stands before its first read
+  // or write of memory
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (b >= g.tiles) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // sums of the parts: 128 bias gradients a block, and the loss in the last
+    if (b == (int)gridDim.x - 1) {
+      __shared__ double red[kThreads];
+      double s = 0;
+      for (long i = threadIdx.x; i < g.loss_n; i += kThreads) s += g.loss[i];
+      red[threadIdx.x] = s;
+      __syncthreads();
+      for (int k = kThreads / 2; k > 0; k >>= 1) {
+        if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
+        __syncthreads();
+      }
+      if (threadIdx.x == 0) *g.loss_sum = red[0];
+      return;
+    }
+    int q = b - g.tiles, p = 0;
+    while (p < g.count - 1 && q >= (g.p[p].N + kThreads - 1) / kThreads)
+      q -= (g.p[p++].N + kThreads - 1) / kThreads;
+    const int c = q * kThreads + threadIdx.x, N = g.p[p].N;
+    if (c < N) {
+      float s = 0.f;
+      for (int i = 0; i < g.parts; ++i) s += g.p[p].sum_in[(long)i * N + c];
+      g.p[p].sum_out[c] = s;
+    }
+    return;
+  }
+  int p = 0;
+  while (p + 1 < g.count && b >= g.p[p + 1].tile0) ++p;
+  const MlpProd& q = g.p[p];
+  const int t = b - q.tile0, tn = (q.N + BN - 1) / BN, M = q.M, N = q.N;
+  auto epi = [&](int row, int col0, float* v) {
+    mlp_epilogue(q.e, M, N, row, col0, v, (N + 31) / 32);
+  };
+  tc_tile<2, BN, STAGES, true>(&q.a, &q.b, t / tn * BM, t % tn * BN, 0, q.K, err, epi);
 }
 
 // ------------------------------------------------------------------ operand packing
@@ -921,27 +1073,28 @@ __global__ void __launch_bounds__(256) pack_both_kernel(const PackOp a, const Pa
   else pack_rows<TA>(a, blockIdx.z - batch, kc, ldk, raw);
 }
 
-// Real operand packing for the BF16 core: out[r][c] = bf16(src[r*s_r + c*s_c]), r < rows,
-// c < kc (row stride ldo elements); tiled through shared memory so that both the read and
-// the write are coalesced whichever index is contiguous in the source.
-__global__ void __launch_bounds__(PT * 8)
-    pack_real_bf16_kernel(int rows, int kc, const float* __restrict__ src, long s_r, long s_c,
-                          __nv_bfloat16* __restrict__ out, long ldo) {
+// BF16 copies of FP32 matrices (job: src[r*s_r + c], r < rows, c < cols), as they are and/or
+// transposed, all of a pass in one launch; tiled through shared memory so that reads and both
+// writes are coalesced.
+__global__ void __launch_bounds__(PT * 8) mlp_pack_kernel(const __grid_constant__ MlpPack g) {
   __shared__ float tile[PT][PT + 1];
-  const int r0 = blockIdx.y * PT, c0 = blockIdx.x * PT;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const bool c_fast = (s_c == 1);
-  for (int q = ty; q < PT; q += 8) {
-    const int r = c_fast ? r0 + q : r0 + tx;
-    const int c = c_fast ? c0 + tx : c0 + q;
-    const float v = (r < rows && c < kc) ? src[(long)r * s_r + (long)c * s_c] : 0.f;
-    if (c_fast) tile[q][tx] = v; else tile[tx][q] = v;
-  }
-  __syncthreads();
+  int p = 0;
+  while (p + 1 < g.count && (int)blockIdx.x >= g.job[p + 1].tile0) ++p;
+  const MlpPackJob& j = g.job[p];
+  const int t = blockIdx.x - j.tile0, tc = (j.cols + PT - 1) / PT;
+  const int r0 = t / tc * PT, c0 = t % tc * PT, tx = threadIdx.x, ty = threadIdx.y;
   for (int q = ty; q < PT; q += 8) {
     const int r = r0 + q, c = c0 + tx;
-    if (r < rows && c < kc) out[(long)r * ldo + c] = __float2bfloat16_rn(tile[q][tx]);
+    const float v = r < j.rows && c < j.cols ? j.src[(long)r * j.s_r + c] : 0.f;
+    tile[q][tx] = v;
+    if (j.row && r < j.rows && c < j.cols) j.row[(long)r * j.ldr + c] = __float2bfloat16_rn(v);
   }
+  __syncthreads();
+  if (j.col)
+    for (int q = ty; q < PT; q += 8) {
+      const int c = c0 + q, r = r0 + tx;
+      if (r < j.rows && c < j.cols) j.col[(long)c * j.ldc + r] = __float2bfloat16_rn(tile[tx][q]);
+    }
 }
 
 // ------------------------------------------------------------------ host side
@@ -1042,6 +1195,74 @@ cudaError_t tc_gemm_real(cudaStream_t st, int elt, int M, int N, int K, const vo
   if (bn == 128) return launch_bn<2, 128, 6>(st, ma, mb, M, N, K, batch, ep, err);
   return launch_bn<2, 64, 8>(st, ma, mb, M, N, K, batch, ep, err);
 }
+
+cudaError_t mlp_pack(cudaStream_t st, MlpPack& g) {
+  int tiles = 0;
+  for (int i = 0; i < g.count; ++i) {
+    g.job[i].tile0 = tiles;
+    tiles += ((g.job[i].rows + PT - 1) / PT) * ((g.job[i].cols + PT - 1) / PT);
+  }
+  count_launch();
+  mlp_pack_kernel<<<tiles, dim3(PT, 8), 0, st>>>(g);
+  return cudaGetLastError();
+}
+
+namespace {
+template <int BN, int STAGES, int CAP>
+cudaError_t mlp_launch(cudaStream_t st, MlpGroup<CAP>& g, int* err) {
+  constexpr size_t sm = smem_bytes<2, BN, STAGES>();
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(mlp_gemm_kernel<BN, STAGES, CAP>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (attr != cudaSuccess) return attr;
+  g.tiles = 0;
+  int extra = 0;
+  for (int i = 0; i < g.count; ++i) {
+    MlpProd& q = g.p[i];
+    if (!make_map(&q.a, 2, q.A, q.K, q.M, q.lda, 0, 1, BM) ||
+        !make_map(&q.b, 2, q.B, q.K, q.N, q.ldb, 0, 1, BN))
+      return cudaErrorInvalidValue;
+    q.tile0 = g.tiles;
+    g.tiles += ((q.M + BM - 1) / BM) * ((q.N + BN - 1) / BN);
+    extra += (q.N + kThreads - 1) / kThreads;
+  }
+  if (!g.loss_sum) extra = -1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(g.tiles + extra + 1);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  MPDO_CUDA_TRY(cudaLaunchKernelEx(&cfg, mlp_gemm_kernel<BN, STAGES, CAP>, g, err));
+  count_launch();
+  g_tc_launches.fetch_add(g.count, std::memory_order_relaxed);
+  return cudaGetLastError();
+}
+}  // namespace
+// The tile width by the widest product and the tiles that it leaves the chip (tc_pick_bn's rule
+// over the whole group).
+template <int CAP>
+cudaError_t mlp_products(cudaStream_t st, MlpGroup<CAP>& g, int* err) {
+  int maxn = 0;
+  long t256 = 0, t128 = 0, t64 = 0;
+  for (int i = 0; i < g.count; ++i) {
+    const long mt = (g.p[i].M + BM - 1) / BM;
+    maxn = std::max(maxn, g.p[i].N);
+    t256 += mt * ((g.p[i].N + 255) / 256);
+    t128 += mt * ((g.p[i].N + 127) / 128);
+    t64 += mt * ((g.p[i].N + 63) / 64);
+  }
+  if (maxn > 128 && t256 >= 148) return mlp_launch<256, 4, CAP>(st, g, err);
+  if (maxn > 64 && t128 >= 74) return mlp_launch<128, 6, CAP>(st, g, err);
+  if (t64 >= 74) return mlp_launch<64, 8, CAP>(st, g, err);
+  return mlp_launch<32, 8, CAP>(st, g, err);   // half the epilogue per thread
+}
+template cudaError_t mlp_products<1>(cudaStream_t, MlpGroup<1>&, int*);
+template cudaError_t mlp_products<kMlpMaxLayers>(cudaStream_t, MlpGroup<kMlpMaxLayers>&, int*);
 
 size_t tc_pack_bytes(int mode, long rows, long k, int batch) {
   const int elt = tc_mode_elt(mode);
@@ -1282,16 +1503,6 @@ cudaError_t tc_cgemm_exact(cudaStream_t st, int opa, int opb, int m, int n, int 
     }
   }
   return cudaSuccess;
-}
-
-cudaError_t tc_pack_real_bf16(cudaStream_t st, int rows, int kc, const float* src, long s_r,
-                              long s_c, void* out, long ldo) {
-  if (rows <= 0 || kc <= 0) return cudaSuccess;
-  dim3 grid((kc + PT - 1) / PT, (rows + PT - 1) / PT), block(PT, 8);
-  pack_real_bf16_kernel<<<grid, block, 0, st>>>(rows, kc, src, s_r, s_c,
-                                                static_cast<__nv_bfloat16*>(out), ldo);
-  count_launch();
-  return cudaGetLastError();
 }
 
 template cudaError_t tc_cgemm_exact<float2, float2>(cudaStream_t, int, int, int, int, int,

@@ -1,5 +1,7 @@
 // Tensor-core (tcgen05 + TMA) GEMM of tcgemm.cu: internal interface.
 #pragma once
+#include <cuda.h>
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 
@@ -69,9 +71,58 @@ bool tc_exact_faster(long m, long n, long k, int batch, bool gram);
 // will run the first exact product of the process.
 cudaError_t tc_exact_init();
 
-// out[r][c] = bf16(src[r*s_r + c*s_c]) for r < rows, c < kc (row stride ldo elements): the
-// K-major BF16 operands of tc_gemm_real from a real FP32 matrix in either orientation.
-cudaError_t tc_pack_real_bf16(cudaStream_t st, int rows, int kc, const float* src, long s_r,
-                              long s_c, void* out, long ldo);
+// ---- the surrogate's products (BF16 operands, FP32 accumulation and elementwise work)
+constexpr int kMlpMaxLayers = 16;
+// What becomes of a product's entry v at (row, column): in this order v += bias; v = tanh v; with
+// t: v = 2 scale (v - t), loss parts of (v - t)^2 per 32 x 32 entries; v *= 1 - a^2; then FP32 and
+// BF16 copies (row: as it is, col: transposed; both with rows of a multiple of 8 entries) and sums
+// over 32 rows of each column.  NULL members are left out.
+struct MlpEpi {
+  float* d;
+  long ldd;
+  __nv_bfloat16 *row, *col;
+  long ldr, ldc;
+  const float* bias;
+  int act;
+  const float* t;
+  float scale;
+  double* loss;
+  const float* a;
+  long lda;
+  float* csum;
+};
+// A (M x K) B^T (N x K), both K-major with 16-byte rows.
+struct MlpProd {
+  CUtensorMap a, b;   // set by mlp_products
+  const __nv_bfloat16 *A, *B;
+  long lda, ldb;
+  int M, N, K, tile0;
+  MlpEpi e;
+  const float* sum_in;   // parts x N, their sums over the parts go to sum_out (with loss_sum)
+  float* sum_out;
+};
+template <int CAP>
+struct MlpGroup {
+  MlpProd p[CAP];
+  int count, tiles;
+  int parts;
+  long loss_n;
+  const double* loss;
+  double* loss_sum;      // not NULL: the launch also adds the parts
+};
+template <int CAP>
+cudaError_t mlp_products(cudaStream_t st, MlpGroup<CAP>& g, int* err);
+struct MlpPackJob {
+  const float* src;
+  long s_r;
+  int rows, cols, tile0;
+  __nv_bfloat16 *row, *col;
+  long ldr, ldc;
+};
+struct MlpPack {
+  MlpPackJob job[kMlpMaxLayers + 2];
+  int count;
+};
+cudaError_t mlp_pack(cudaStream_t st, MlpPack& g);
 
 }  // namespace mpdo
