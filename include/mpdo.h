@@ -433,7 +433,8 @@ int mpdo_kernel_pchol(int n, const void* w, int rmax, double tol, void* L, int l
  * which the contractions of the two-site update run in the split-precision modes (Sec.
  * III.A: contracting the site tensors and the gate, Fig. 6a; the Gram products of the
  * truncation).  Device pointers; stream = cudaStream_t (NULL = legacy default stream);
- * both calls synchronise the stream and allocate their own scratch (test entry points).
+ * the calls synchronise the stream and take their scratch from a stream-ordered memory pool of
+ * the library's, which keeps at most 512 MB between calls; mpdo_kernel_trim gives it back.
  * mpdo_kernel_tcgemm_real: d (m x n FP32, row stride ldd) = a b^T with a (m x k) and b
  *   (n x k) K-major, elements FP32 read as TF32 (elt 4) or BF16 (elt 2); lda, ldb in
  *   elements, >= k and multiples of 16 bytes.
@@ -444,6 +445,7 @@ int mpdo_kernel_pchol(int n, const void* w, int rmax, double tol, void* L, int l
  * pipeline wait inside the kernel gave up (the output is then undefined). */
 /* Number of tensor-core GEMM kernels (tcgen05) this library has launched in the process. */
 long long mpdo_tc_gemm_launches(void);
+void mpdo_kernel_trim(void);
 int mpdo_kernel_tcgemm_real(int elt, int m, int n, int k, const void* a, long lda, const void* b,
                             long ldb, float* d, long ldd, void* stream);
 int mpdo_kernel_tcgemm(int mode, int opa, int opb, int m, int n, int k, const void* a, long lda,

@@ -148,6 +148,7 @@ def _load():
         "mpdo_kernel_pchol": (I, [I, VP, I, D, VP, I, VP, P(I), P(D), VP]),
         "mpdo_heig_noalloc": (I, [I, I, VP, VP, P(D), P(I), VP]),
         "mpdo_tc_gemm_launches": (C.c_longlong, []),
+        "mpdo_kernel_trim": (None, []),
         "mpdo_kernel_tcgemm_exact": (I, [I, I, I, I, I, VP, C.c_long, C.c_long, VP, C.c_long,
                                          C.c_long, VP, C.c_long, C.c_long, I, VP]),
         "mpdo_kernel_tcgemm_real": (I, [I, I, I, I, VP, C.c_long, VP, C.c_long, VP, C.c_long,
@@ -683,6 +684,11 @@ TC_MODES = {"tf32": 0, "tf32x3": 1, "bf16": 2, "bf16x3": 3}
 def tc_gemm_launches() -> int:
     """Tensor-core (tcgen05) GEMM kernels launched by libmpdo in this process so far."""
     return int(LIB.mpdo_tc_gemm_launches())
+
+
+def kernel_trim() -> None:
+    """Give the pooled scratch of the tensor-core product entry points back to the device."""
+    LIB.mpdo_kernel_trim()
 
 
 def kernel_tcgemm_real(elt: int, m: int, n: int, k: int, a, lda: int, b, ldb: int, d, ldd: int,

@@ -226,7 +226,11 @@ void* dmalloc(mpdo_ctx* h, size_t bytes) {
   void* p = nullptr;
   if (cudaMalloc(&p, bytes) != cudaSuccess) {
     cudaGetLastError();
-    return nullptr;
+    scratch_trim();
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
   }
   return p;
 }

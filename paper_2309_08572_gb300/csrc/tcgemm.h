@@ -8,6 +8,8 @@
 #include "common.cuh"
 
 namespace mpdo {
+// Gives the entry points' pooled scratch (mpdo_kernel_trim) back to the device.
+void scratch_trim();
 
 // Operand modes of the tensor-core path: the MMA element type and the number of K-segments
 // of a packed complex operand (1 = plain, 3 = split hi/lo precision compensation).
