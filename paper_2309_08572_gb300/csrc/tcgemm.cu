@@ -567,17 +567,26 @@ __global__ void __launch_bounds__(PT * 8)
 //
 // The kernel's tile is 128 rows by 64 real columns.  A stage holds 32 K terms of all six slices
 // of both operands (72 KB, three stages), so the 21 pairs run on operands that were loaded once:
-// 36 bytes per clock and SM from L2, where loading every pair's operands took 128.  The pairs
+// 27 bytes per clock and SM from L2, where loading every pair's operands took 128.  The pairs
 // (t, u) of one weight t + u add into one accumulator, six of 64 TMEM columns; a sum stays
-// below 2^24 for 1024 / (t + u + 1) terms, so every XDRAIN = 5 stages (at most 6 x 160 terms) eight
-// warps take the accumulators out, group after group, while the MMAs of the other groups run.
-// They add them as integers -- weights 0..2 and 3..5 shifted into two 64-bit sums, exact -- since
-// the FP64 pipe, at 2 operations per clock and SM, bound the earlier FP64 drain to an eighth of the
-// MMA rate.  The K loop of a product with few tiles is split over CTAs; their integer sums are
-// added by exact_finish_kernel.  Gram matrices compute the tiles that reach the upper half, from
-// one packed operand: the rows of A are the even rows of the packed B.  Bound by the tensor pipe
-// (N = 64: by its operand reads from shared memory).  Kernel times: inner Gram 400 x 400 x 5043 601
-// -> 74 us, 768 x 768 x 4096 Gram 1150 -> 187 us.
+// below 2^24 for 1024 / (t + u + 1) terms.  Slice t of A meets the slices 0 .. 5 - t of B in
+// products of up to 256 columns -- those slices, and the accumulators of the weights t .. 5, lie
+// one behind the other -- because a product of 64 columns took 88 clocks, more than twice its share
+// of the tensor pipe's rate (3600 -> 2700 clocks a stage with the wide ones).  The sums' limit
+// means that every XDRAIN = 5 stages (at most 6 x 160 terms) eight warps take the accumulators
+// out, weight after weight, while the products of the other weights run.  They add them as
+// integers -- weights 0..2 and 3..5 shifted into two 64-bit sums, exact -- since the FP64 pipe, at
+// 2 operations per clock and SM, bound an FP64 drain to an eighth of the MMA rate.
+//
+// The stages of all tiles, one tile after another, are dealt to at most one CTA per SM in equal
+// ranges (a launch of a tile and K slice per CTA left the last wave nearly empty and paid the fill
+// of the ring, the TMEM allocation and the output for every slice, 17 us each); the ring runs on
+// from tile to tile.  A range's first and last tile may be another CTA's as well: their integer
+// sums (exact, so in any order) are added by exact_finish_kernel.  Gram matrices compute the tiles
+// that reach the upper half, from one packed operand: the rows of A are the even rows of the packed
+// B.  Bound by the tensor pipe and the accumulators' turn-around.  768 x 768 x 4096 Gram, this
+// kernel: 1150 us with every pair's operands loaded anew and an FP64 drain, 367 us with slices of K
+// and 64-column products, 313 us in equal ranges, 201 us with wide products.
 constexpr int XS = 6;          // slices per operand
 constexpr int XBN = 64;        // output tile width (real columns)
 constexpr int XKB = 32;        // K terms of a stage
@@ -586,6 +595,7 @@ constexpr int XDRAIN = 5;      // stages between drains
 constexpr int XTHREADS = 320;  // warp 0 TMA, warp 1 MMA, warps 2-9 drain
 constexpr int XA_SLICE = BM * XKB * 2, XB_SLICE = XBN * XKB * 2;
 constexpr int XSTAGE_BYTES = XS * (XA_SLICE + XB_SLICE);
+constexpr long XPART = BM * XBN;   // entries of a CTA's part of a tile: [column of 32][half, row]
 constexpr int kNonFinite = 0x7fffffff;   // exponent of a row with a non-finite entry
 constexpr int kZeroRow = -1000000;       // and of a zero row (any smaller value)
 
@@ -642,7 +652,8 @@ __device__ __forceinline__ void exact_tile(int tile, int nt, int gram, int& mt, 
 
 __global__ void __launch_bounds__(XTHREADS, 1)
     tc_exact_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb,
-                    int M, int N, int ldk, int nst, int per, int gram, const int* __restrict__ ea,
+                    int M, int N, int ldk, int nst, int tiles, long per, long total, int gram,
+                    const int* __restrict__ ea,
                     const int* __restrict__ eb, double2* C, long ldc, long sc, int accumulate,
                     longlong2* part, int* err) {
   extern __shared__ uint8_t smem_raw[];
@@ -655,11 +666,23 @@ __global__ void __launch_bounds__(XTHREADS, 1)
   int* abort_flag = reinterpret_cast<int*>(tslot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nt = (N + XBN - 1) / XBN, bz = blockIdx.z;
-  int mt, ct;
-  exact_tile(blockIdx.x, nt, gram, mt, ct);
-  const int n0 = ct * XBN, m0 = mt * BM;
-  const int st0 = blockIdx.y * per, stages = min(nst, st0 + per) - st0;
+  const int nt = (N + XBN - 1) / XBN;
+  // this CTA's stages: `left` of them from stage s0 of a tile (over the batch)
+  int s0 = (int)(blockIdx.x * per % nst), tile = (int)(blockIdx.x * per / nst);
+  int left = (int)min(per, total - blockIdx.x * per), len, m0, n0, bz;
+  auto locate = [&]() {
+    len = min(nst - s0, left);
+    bz = tile / tiles;
+    int mt, ct;
+    exact_tile(tile - bz * tiles, nt, gram, mt, ct);
+    m0 = mt * BM;
+    n0 = ct * XBN;
+  };
+  auto next = [&]() {
+    left -= len;
+    s0 = 0;
+    ++tile;
+  };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < XSTAGES; ++s) {
@@ -688,107 +711,126 @@ __global__ void __launch_bounds__(XTHREADS, 1)
 
   if (warp == 0) {
     if (lane == 0) {
-      for (int it = 0; it < stages && !*(volatile int*)abort_flag; ++it) {
-        const int s = it % XSTAGES;
-        if (it >= XSTAGES && !mbar_wait(&empty[s], ((it / XSTAGES) - 1) & 1)) {
-          atomicExch(abort_flag, 1);
-          atomicExch(err, 11);
-          break;
-        }
-        uint8_t* sa = smem + s * XSTAGE_BYTES;
-        mbar_expect_tx(&full[s], XSTAGE_BYTES);
-        const int c0 = (st0 + it) * XKB;
-        for (int t = 0; t < XS; ++t) {
-          tma_load_3d(sa + t * XA_SLICE, &ma, &full[s], t * ldk + c0, m0, bz);
-          tma_load_3d(sa + XS * XA_SLICE + t * XB_SLICE, &mb, &full[s], t * ldk + c0, n0, bz);
+      int it = 0;
+      bool ok = true;
+      for (; left > 0 && ok; next()) {
+        locate();
+        for (int j = 0; j < len && ok; ++j, ++it) {
+          const int s = it % XSTAGES;
+          if (it >= XSTAGES && !mbar_wait(&empty[s], ((it / XSTAGES) - 1) & 1)) {
+            atomicExch(abort_flag, 1);
+            atomicExch(err, 11);
+            ok = false;
+          }
+          if (*(volatile int*)abort_flag) ok = false;
+          if (!ok) break;
+          uint8_t* sa = smem + s * XSTAGE_BYTES;
+          mbar_expect_tx(&full[s], XSTAGE_BYTES);
+          const int c0 = (s0 + j) * XKB;
+          for (int t = 0; t < XS; ++t) {
+            tma_load_3d(sa + t * XA_SLICE, &ma, &full[s], t * ldk + c0, m0, bz);
+            tma_load_3d(sa + XS * XA_SLICE + t * XB_SLICE, &mb, &full[s], t * ldk + c0, n0, bz);
+          }
         }
       }
     }
     __syncwarp();
   } else if (warp == 1) {
     if (lane == 0) {
-      constexpr uint32_t id = idesc<2>(XBN);
       bool ok = true;
-      for (int it = 0; it < stages && ok; ++it) {
-        const int s = it % XSTAGES, d = it / XDRAIN;
-        const bool first = it % XDRAIN == 0, last = it % XDRAIN == XDRAIN - 1 || it == stages - 1;
-        if (!mbar_wait(&full[s], (it / XSTAGES) & 1)) {
-          atomicExch(abort_flag, 1);
-          atomicExch(err, 12);
-          break;
-        }
-        tc_fence_after();
-        const uint32_t sa = su32(smem + s * XSTAGE_BYTES);
+      int it = 0, d = -1;   // stages and drain periods so far
+      for (; left > 0 && ok; next()) {
+        locate();
+        for (int j = 0; j < len && ok; ++j, ++it) {
+          const int s = it % XSTAGES;
+          const bool first = j % XDRAIN == 0, last = j % XDRAIN == XDRAIN - 1 || j == len - 1;
+          if (first) ++d;
+          if (!mbar_wait(&full[s], (it / XSTAGES) & 1)) {
+            atomicExch(abort_flag, 1);
+            atomicExch(err, 12);
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t sa = su32(smem + s * XSTAGE_BYTES);
+          // slice t of A against the slices 0 .. 5 - t of B, which lie one behind the other like the
+          // accumulators of the weights t .. 5: products of up to 256 columns
 #pragma unroll
-        for (int g = 0; g < XS; ++g) {
-          // the drain of the period before must have emptied this weight's accumulator
-          if (first && d > 0) {
-            if (!mbar_wait(&gempty[g], (d - 1) & 1)) {
-              atomicExch(abort_flag, 1);
-              atomicExch(err, 13);
-              ok = false;
-              break;
+          for (int t = 0; t < XS; ++t) {
+#pragma unroll
+            for (int u = 0; u < XS - t; u += 4) {
+              constexpr int kMax = 4;
+              const int nu = XS - t - u < kMax ? XS - t - u : kMax;
+              if (first && t == 0 && d > 0) {
+                // the drain of the period before must have emptied these accumulators
+                for (int g = u; g < u + nu && ok; ++g) ok = mbar_wait(&gempty[g], (d - 1) & 1);
+                if (!ok) {
+                  atomicExch(abort_flag, 1);
+                  atomicExch(err, 13);
+                  break;
+                }
+                tc_fence_after();
+              }
+              const uint64_t ad = sdesc64(sa + t * XA_SLICE),
+                             bd = sdesc64(sa + XS * XA_SLICE + u * XB_SLICE);
+#pragma unroll
+              for (int kk = 0; kk < 2; ++kk)
+                umma<2>(tmem + (t + u) * XBN, ad + 2 * kk, bd + 2 * kk, idesc<2>(nu * XBN),
+                        (first && t == 0 && kk == 0) ? 0u : 1u);
             }
-            tc_fence_after();
+            if (!ok) break;
+            if (last) umma_commit(&gfull[t]);   // weight t has its last pair
           }
-#pragma unroll
-          for (int t = 0; t <= g; ++t) {
-            const uint64_t ad = sdesc64(sa + t * XA_SLICE),
-                           bd = sdesc64(sa + XS * XA_SLICE + (g - t) * XB_SLICE);
-#pragma unroll
-            for (int kk = 0; kk < 2; ++kk)
-              umma<2>(tmem + g * XBN, ad + 2 * kk, bd + 2 * kk, id,
-                      (first && t == 0 && kk == 0) ? 0u : 1u);
-          }
-          if (last) umma_commit(&gfull[g]);
+          if (ok) umma_commit(&empty[s]);
         }
-        if (ok) umma_commit(&empty[s]);
       }
     }
     __syncwarp();
   } else {
     // drain warps: TMEM lanes 32 (warp % 4) .. +31 are tile rows, columns 32 hf .. +31
     const int q = warp & 3, hf = (warp - 2) >> 2;
-    const int row = m0 + q * 32 + lane;
-    long long hi[32], lo[32];
-#pragma unroll
-    for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
     bool ok = true;
-    const int periods = (stages + XDRAIN - 1) / XDRAIN;
-    for (int d = 0; d < periods && ok; ++d) {
+    int d = 0, first = 0;   // periods so far; 0: the range's first tile
+    for (; left > 0 && ok; next(), first = 1) {
+      locate();
+      const int row = m0 + q * 32 + lane;
+      long long hi[32], lo[32];
 #pragma unroll
-      for (int g = 0; g < XS; ++g) {
-        bool ready = true;
-        if (lane == 0) ready = mbar_wait(&gfull[g], d & 1);
-        ready = __shfl_sync(0xffffffffu, ready ? 1 : 0, 0) != 0;
-        if (!ready || *(volatile int*)abort_flag) {
-          if (lane == 0 && !ready) atomicExch(err, 14);
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        float v[32];
-        tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + g * XBN + hf * 32, v);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0)
-          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&gempty[g])) : "memory");
+      for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
+      const int end = d + (len + XDRAIN - 1) / XDRAIN;
+      for (; d < end && ok; ++d) {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const long long x = (long long)__float2int_rn(v[j]) * (1 << (8 * (2 - g % 3)));
-          if (g < 3) hi[j] += x; else lo[j] += x;
+        for (int g = 0; g < XS; ++g) {
+          bool ready = true;
+          if (lane == 0) ready = mbar_wait(&gfull[g], d & 1);
+          ready = __shfl_sync(0xffffffffu, ready ? 1 : 0, 0) != 0;
+          if (!ready || *(volatile int*)abort_flag) {
+            if (lane == 0 && !ready) atomicExch(err, 14);
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          float v[32];
+          tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + g * XBN + hf * 32, v);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0)
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&gempty[g])) : "memory");
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const long long x = (long long)__float2int_rn(v[j]) * (1 << (8 * (2 - g % 3)));
+            if (g < 3) hi[j] += x; else lo[j] += x;
+          }
         }
       }
-    }
-    if (ok && row < M) {
-      const int c0 = n0 + hf * 32;
-      if (part) {
-        longlong2* pp = part + (((long)blockIdx.y * gridDim.z + bz) * M + row) * N;
+      if (!ok) break;
+      if (len < nst) {
+        longlong2* pp = part + (long)(2 * blockIdx.x + first) * XPART +
+                        (hf * 4 + q) * 32 + lane;
 #pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (c0 + j < N) pp[c0 + j] = make_longlong2(hi[j], lo[j]);
-      } else {
-        const int er = ea[(long)bz * M + row];
+        for (int j = 0; j < 32; ++j) pp[j * 256] = make_longlong2(hi[j], lo[j]);
+      } else if (row < M) {
+        const int c0 = n0 + hf * 32, er = ea[(long)bz * M + row];
         double2* cp = C + (long)bz * sc;
 #pragma unroll
         for (int j = 0; j < 32; j += 2)
@@ -809,29 +851,39 @@ __global__ void __launch_bounds__(XTHREADS, 1)
   }
 }
 
-// Sum of the K slices' integer parts (exact, so in any order) and the output.
-__global__ void __launch_bounds__(256) exact_finish_kernel(int M, int n, int batch, int splits,
+// The tiles that belong to more than one CTA's range: the sum of their integer parts and the
+// output.  Eight columns of a tile a block, a thread to a row and half as in the drain.
+__global__ void __launch_bounds__(256) exact_finish_kernel(int M, int N, int nst, int tiles, long per,
                                                            int gram, const longlong2* part,
                                                            const int* __restrict__ ea,
                                                            const int* __restrict__ eb, double2* C,
                                                            long ldc, long sc, int accumulate) {
-  const long total = (long)batch * M * n;
-  for (long e = blockIdx.x * 256L + threadIdx.x; e < total; e += 256L * gridDim.x) {
-    const int q = (int)(e % n), i = (int)((e / n) % M), b = (int)(e / ((long)n * M));
-    if (gram && q < i) continue;
-    long long rh = 0, rl = 0, ih = 0, il = 0;
-    for (int s = 0; s < splits; ++s) {
-      const longlong2* p = part + (((long)s * batch + b) * M + i) * 2 * n + 2 * q;
-      const longlong2 x = p[0], y = p[1];
-      rh += x.x;
-      rl += x.y;
-      ih += y.x;
-      il += y.y;
+  const long tile = blockIdx.x;
+  const long c0 = tile * nst / per, c1 = ((tile + 1) * nst - 1) / per;
+  if (c0 == c1) return;
+  const int j0 = blockIdx.y * 8, bz = (int)(tile / tiles), nt = (N + XBN - 1) / XBN;
+  int mt, ct;
+  exact_tile((int)(tile - (long)bz * tiles), nt, gram, mt, ct);
+  const int row = mt * BM + (threadIdx.x & 127), col = ct * XBN + (threadIdx.x >> 7) * 32 + j0;
+  long long hi[8] = {}, lo[8] = {};
+  for (long c = c0; c <= c1; ++c) {
+    const longlong2* p = part + (2 * c + (c * per / nst == tile ? 0 : 1)) * XPART + j0 * 256 + threadIdx.x;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const longlong2 x = p[j * 256];
+      hi[j] += x.x;
+      lo[j] += x.y;
     }
-    const int er = ea[(long)b * M + i], eq = eb[(long)b * n + q];
-    exact_store(C + (long)b * sc, ldc, i, q, exact_value(rh, rl, er, eq), exact_value(ih, il, er, eq),
-                gram, accumulate);
   }
+  if (row >= M) return;
+  const int er = ea[(long)bz * M + row];
+#pragma unroll
+  for (int j = 0; j < 8; j += 2)
+    if (col + j < N) {
+      const int qc = (col + j) >> 1, eq = eb[(long)bz * (N / 2) + qc];
+      exact_store(C + (long)bz * sc, ldc, row, qc, exact_value(hi[j], lo[j], er, eq),
+                  exact_value(hi[j + 1], lo[j + 1], er, eq), gram, accumulate);
+    }
 }
 
 // e[b][r] = exponent of the largest |Re|, |Im| of row r of X (X[r][c] = src[b*sb + r*s_r +
@@ -1346,10 +1398,13 @@ cudaError_t tc_cgemm(cudaStream_t st, int mode, int opa, int opb, int m, int n, 
 // ---- exact products: C (complex FP64) = op(A) op(B), FP32 or FP64 complex A and B
 namespace {
 struct ExactPlan {
-  int tiles, nst, per, splits;
+  int tiles, nst, ctas;
+  long per, total;   // stages of a CTA, of all tiles of the batch
+  bool parts;        // ranges end within tiles
 };
-// Tiles of the output and the K split: the number of slices (at least 4 stages each) with the
-// fewest stages on the busiest of the 152 SMs, fewer slices where it makes no difference.
+// How many stages a CTA takes: whole tiles, or an equal share of the stages (at least four) where
+// that is less on the busiest of the 152 SMs, counting 4 stages' time for a CTA's prologue and last
+// drain, one for a tile's output and 10 for the parts and the launch that adds them.
 ExactPlan exact_plan(long m, long n, long kc, int batch, bool gram) {
   ExactPlan p;
   const long mt = (m + BM - 1) / BM, nt = (2 * n + XBN - 1) / XBN;
@@ -1360,19 +1415,13 @@ ExactPlan exact_plan(long m, long n, long kc, int batch, bool gram) {
   }
   p.tiles = (int)tiles;
   p.nst = (int)((2 * kc + XKB - 1) / XKB);
-  p.per = p.nst;
-  p.splits = 1;
-  long best = -1;
-  for (int s = 1; s <= 16 && (s == 1 || p.nst >= 4 * s); ++s) {
-    const int per = (p.nst + s - 1) / s, used = (p.nst + per - 1) / per;
-    // 4: prologue and drain of a CTA; 8: the launch that adds the slices
-    const long cost = ((tiles * batch * used + 151) / 152) * (per + 4) + (used > 1 ? 8 : 0);
-    if (best < 0 || cost < best) {
-      best = cost;
-      p.per = per;
-      p.splits = used;
-    }
-  }
+  p.total = tiles * batch * p.nst;
+  const long whole = (tiles * batch + 151) / 152;
+  const long ctas = std::min(152L, std::max(1L, p.total / 4));
+  const long share = (p.total + ctas - 1) / ctas;
+  p.parts = share + share / p.nst + 10 < whole * p.nst + whole;
+  p.per = p.parts ? share : whole * p.nst;
+  p.ctas = (int)((p.total + p.per - 1) / p.per);
   return p;
 }
 // op(B) = op(A)^+ of the same data: the product is Hermitian
@@ -1387,21 +1436,20 @@ size_t exact_bytes(long m, long n, long kc, int batch, bool gram) {
   const size_t a = gram ? 0 : ((size_t)batch * m * XS * ldk * 2 + 255) & ~(size_t)255;
   const size_t b = ((size_t)batch * 2 * n * XS * ldk * 2 + 255) & ~(size_t)255;
   const ExactPlan p = exact_plan(m, n, kc, batch, gram);
-  const size_t part = p.splits > 1 ? (size_t)p.splits * batch * m * 2 * n * sizeof(longlong2) : 0;
+  const size_t part = p.parts ? (size_t)p.ctas * 2 * XPART * sizeof(longlong2) : 0;
   return a + b + part + (((size_t)batch * (m + n) * sizeof(int) + 255) & ~(size_t)255) + 256;
 }
 }  // namespace
 
 // Time of an exact product against the same product on the FP64 CUDA cores.  The slice kernel
-// costs a fixed part (exponents, packing, output) and its stages on the busiest SM, 1.05 us each;
+// costs a fixed part (exponents, packing, output) and its stages on the busiest SM, 1.4 us each;
 // FP64 runs at 304 FMA per clock over the chip.  Both sides as measured: the Gram 41 x 41 x 1968 takes
 // 25 us in FP64 and 36 us plus its packing in slices, the Gram 400 x 400 x 5043 2.6 ms and 74 us.
 bool tc_exact_faster(long m, long n, long k, int batch, bool gram) {
   const ExactPlan p = exact_plan(m, n, k, batch, gram);
-  const double waves = (double)((p.tiles * (long)batch * p.splits + 151) / 152);
   const double elems = (double)batch * k * ((gram ? 0 : m) + 2.0 * n);   // packed complex entries
-  const double tc = (k <= kFusedPackK ? 12.0 : 24.0) + (p.splits > 1 ? 8.0 : 0.0) +
-                    1.05 * waves * (p.per + 4) + elems * 24.0 / 3.0e6;
+  const double tc = (k <= kFusedPackK ? 12.0 : 24.0) + (p.parts ? 8.0 : 0.0) +
+                    1.4 * (p.per + 4 + p.per / p.nst) + elems * 24.0 / 3.0e6;
   const double fp64 = 8.0 + 1.2 * 4.0 * m * n * (double)k * batch * (gram ? 0.5 : 1.0) / (304.0 * 2.0e3);
   return tc < fp64;
 }
@@ -1446,7 +1494,7 @@ cudaError_t tc_cgemm_exact(cudaStream_t st, int opa, int opb, int m, int n, int 
     int* eb = reinterpret_cast<int*>(p);
     int* ea = gram ? eb : eb + (size_t)batch * n;
     p += ((size_t)batch * (m + n) * sizeof(int) + 255) & ~(size_t)255;
-    longlong2* part = pl.splits > 1 ? reinterpret_cast<longlong2*>(p) : nullptr;
+    longlong2* part = pl.parts ? reinterpret_cast<longlong2*>(p) : nullptr;
     auto exps = [&](auto* x, int rows, long sr, long s_c, long s_b, int* e) {
       const int rb = s_c == 1 ? (rows + 7) / 8 : (rows + 31) / 32;
       // enough column slices for about two CTAs per SM, at least 64 columns each
@@ -1489,15 +1537,15 @@ cudaError_t tc_cgemm_exact(cudaStream_t st, int opa, int opb, int m, int n, int 
       return cudaErrorInvalidValue;
     const size_t smem = XSTAGES * XSTAGE_BYTES + 1024 + 256;
     const int acc = k0 > 0 ? 1 : 0;
-    tc_exact_kernel<<<dim3(pl.tiles, pl.splits, batch), XTHREADS, smem, st>>>(
-        ma, mb, m, 2 * n, ldk, pl.nst, pl.per, gram ? 1 : 0, ea, eb, C, ldc, sc, acc, part, err);
+    tc_exact_kernel<<<pl.ctas, XTHREADS, smem, st>>>(ma, mb, m, 2 * n, ldk, pl.nst, pl.tiles, pl.per,
+                                                     pl.total, gram ? 1 : 0, ea, eb, C, ldc, sc, acc,
+                                                     part, err);
     count_launch();
     g_tc_launches.fetch_add(1, std::memory_order_relaxed);
     MPDO_CUDA_TRY(cudaGetLastError());
     if (part) {
-      const long total = (long)batch * m * n;
-      exact_finish_kernel<<<(int)std::min<long>((total + 255) / 256, 4096), 256, 0, st>>>(
-          m, n, batch, pl.splits, gram ? 1 : 0, part, ea, eb, C, ldc, sc, acc);
+      exact_finish_kernel<<<dim3((unsigned)((long)pl.tiles * batch), 4), 256, 0, st>>>(
+          m, 2 * n, pl.nst, pl.tiles, pl.per, gram ? 1 : 0, part, ea, eb, C, ldc, sc, acc);
       count_launch();
       MPDO_CUDA_TRY(cudaGetLastError());
     }

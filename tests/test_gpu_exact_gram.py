@@ -25,7 +25,7 @@ def _rand(rng, shape):
 
 @pytest.mark.parametrize("side", [0, 1])
 @pytest.mark.parametrize("n,k", [(1, 1), (31, 7), (33, 80), (128, 81), (129, 160), (160, 1000),
-                                 (257, 513), (400, 5043)])
+                                 (257, 513), (400, 5043), (700, 1500)])
 def test_gram(lib, n, k, side):
     """C = A^+ A (side 0) or A A^+ with rows of A scaled over eight decades, within the bound that
     the exact products are held to (|err| <= 2^-40 sum |a||b|); C is exactly Hermitian."""
@@ -44,9 +44,11 @@ def test_gram(lib, n, k, side):
 
 
 @pytest.mark.parametrize("m,n,k,batch", [(1, 1, 1, 1), (128, 32, 16, 1), (129, 33, 17, 2),
-                                         (64, 64, 2500, 1), (300, 100, 400, 3)])
+                                         (64, 64, 2500, 1), (300, 100, 400, 3),
+                                         (2100, 600, 40, 1), (500, 500, 300, 2)])
 def test_general(lib, m, n, k, batch):
-    """The same bound; K = 2500 with two tiles runs as split slices of integer sums."""
+    """The same bound; K = 2500 with two tiles, and tiles that do not deal out evenly, share
+    tiles between CTAs as integer sums; 2100 x 600 gives each CTA several tiles."""
     rng = np.random.default_rng(m + n + k)
     a, b = _rand(rng, (batch, m, k)), _rand(rng, (batch, k, n))
     c = torch.full((batch, m, n), float("nan"), dtype=torch.complex128, device="cuda")
