@@ -36,14 +36,16 @@ template <typename R>
 struct EigWork {
   int n_cap = 0;
   cx<R>* ap = nullptr;   // padded working matrix
-  cx<R>* vp = nullptr;   // padded eigenvector accumulator
+  cx<R>* vp = nullptr;   // padded eigenvector accumulator, transposed
+  cx<R>* ug = nullptr;   // unitaries of a round's pairs
+  int* act = nullptr;    // which of them are not the identity
   int* counters = nullptr;  // [0..1] rotation counters, [2] sweeps used
 };
 
 template <typename R>
 size_t eig_work_bytes(int n_cap);
 // padded size used by the eigensolver; each active pair-round of the block Jacobi does
-// 3 * 16 * 16 * padded_n complex multiply-adds (rows, columns and eigenvectors)
+// 2 * 16 * 16 * padded_n complex multiply-adds (half of A from both sides and the eigenvectors)
 int eig_padded_n(int n);
 double eig_flops_per_count(int n, bool fp64);
 template <typename R>

@@ -1,14 +1,18 @@
 // Parallel two-sided block Jacobi eigensolver for Hermitian matrices (FP64 / FP32).
 //
 // The columns are split into blocks of JW = 8; every round pairs the blocks by a
-// round-robin tournament and one CTA per pair diagonalises its 16 x 16 principal
-// sub-matrix with scalar cyclic Jacobi rotations in shared memory (GVL sym.schur2 with
-// the complex phase factored out), then applies the accumulated 16 x 16 unitary to its
-// rows (phase A) and, after a grid-wide barrier, to its columns and to the eigenvector
-// accumulator (phase B).  Pairs in one round touch disjoint rows/columns, so phases A
-// and B need only the two barriers of a cooperative launch.  A sweep in which no pair
-// rotated ends the iteration.  Cost per sweep ~6 n^3 complex MACs; the matrix stays in
-// L2 (it is at most a few MB).
+// round-robin tournament.  One CTA per pair diagonalises its 16 x 16 principal sub-matrix
+// with scalar cyclic Jacobi rotations in shared memory (GVL sym.schur2 with the complex
+// phase factored out) and publishes the accumulated 16 x 16 unitary; after a grid-wide
+// barrier the warps of all CTAs apply the unitaries, A[p, q] <- U_p^+ A[p, q] U_q for the 16 x 16
+// tiles of the upper half (mirrored into the lower) and V[:, q] <- V[:, q] U_q, and a second
+// barrier ends the round.  A tile needs no other tile, so A is read and written once a round, and
+// V is kept transposed, so that its rows are contiguous.  A sweep in which no pair rotated ends
+// the iteration.  Cost per sweep ~4 n^3 complex MACs; the matrix stays in L2 (it is at most a few
+// MB... 29 MB with V at n = 1350).  A round there is bound by FP32 issue in the tiles (~12 us) and
+// the serial chain of 15 rotation steps and two grid barriers before them (~8 us); rows and columns
+// in two passes of 16 x np by the pairs' own CTAs, each waiting for its loads, took 92 us.  An FP32
+// solve of n = 1350 takes 52 ms on average over the mixed solver's levels, 231 ms before.
 #include <cooperative_groups.h>
 #include <cuda.h>
 
@@ -27,8 +31,8 @@ namespace {
 
 constexpr int JW = 8;          // block width
 constexpr int JS = 2 * JW;     // sub-problem size
-constexpr int JT = 256;        // threads per CTA
-constexpr int CH = 64;         // staged chunk (columns in phase A, rows in phase B)
+constexpr int JT = 256;        // threads per CTA: one per entry of the sub-problem
+constexpr int JV = 32;         // columns of V^T in a warp's item
 // Sweeps of the 16x16 sub-problem per block-pair visit.  One sweep per visit is the
 // classic one-sided-update choice: the outer rounds keep rotating the pair, so a fully
 // converged sub-problem buys little and costs 15 warp rounds per extra sweep.
@@ -58,22 +62,55 @@ __global__ void pad_copy_kernel(int n, int np, const cx<R>* __restrict__ a, long
   if (blockIdx.x == 0 && threadIdx.x < 4) counters[threadIdx.x] = 0;
 }
 
+// Warp-private products of 16 x 16 tiles: lane (r = lane / 2, h = lane % 2) has the entries
+// (r, 8 h .. 8 h + 7).  Operands read along a row of 16 are aligned vectors that half of the lanes
+// share; a tile read down its rows has a stride of 17.
+template <typename T>
+__device__ __forceinline__ void tile_zero(T* acc) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) acc[i].x = acc[i].y = 0;
+}
+// acc += sum_k x(k) y[k][8 h + i], x(k) from left(k)
+template <typename T, typename F>
+__device__ __forceinline__ void tile_mul(T* acc, const T* y, int h, F&& left) {
+#pragma unroll 4
+  for (int k = 0; k < JS; ++k) {
+    const T x = left(k);
+    T q[8];
+    const float4* p = reinterpret_cast<const float4*>(y + k * JS + 8 * h);
+#pragma unroll
+    for (int i = 0; i < (int)sizeof(T) / 2; ++i) reinterpret_cast<float4*>(q)[i] = p[i];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) cfma(acc[i], x, q[i]);
+  }
+}
+template <typename T>
+__device__ __forceinline__ void copy8(T* dst, const T* src) {
+#pragma unroll
+  for (int i = 0; i < (int)sizeof(T) / 2; ++i)
+    reinterpret_cast<float4*>(dst)[i] = reinterpret_cast<const float4*>(src)[i];
+}
+
 template <typename R>
-__global__ void __launch_bounds__(JT) jacobi_coop_kernel(int np, int nblk, cx<R>* ap,
-                                                         cx<R>* vp, int* counters,
-                                                         int max_sweeps) {
+constexpr size_t coop_smem() {   // per warp: U_p, U_q, a tile of stride 17
+  return (size_t)(JT / 32) * (2 * JS * JS + JS * (JS + 1)) * sizeof(cx<R>);
+}
+
+template <typename R>
+__global__ void __launch_bounds__(JT, 2) jacobi_coop_kernel(int np, int nblk, cx<R>* ap, cx<R>* vt,
+                                                            cx<R>* ug, int* act, int* counters,
+                                                            int max_sweeps) {
   using T = cx<R>;
   cg::grid_group grid = cg::this_grid();
-  __shared__ T S[JS][JS + 1];
-  __shared__ T U[JS][JS + 1];
-  __shared__ T X[JS][CH + 1];
-  __shared__ int idx[JS];
-  __shared__ R rc[JS / 2], rs[JS / 2];
-  __shared__ T re[JS / 2];
-  __shared__ int ra[JS / 2], rb[JS / 2], rflag[JS / 2];
-  __shared__ int any_rot;
+  extern __shared__ __align__(16) unsigned char jc_raw[];
+  __shared__ T S[2][JS][JS + 1];
+  __shared__ T U[2][JS][JS + 1];
+  __shared__ R rc[JS];             // per index: cosine, partner's coefficient, partner
+  __shared__ T ro[JS];
+  __shared__ int rp[JS];
   __shared__ R s_anorm;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int pairs = nblk / 2;
 
   // |A| scale for the absolute rotation floor: sum of |diag|, reduced in a fixed order so
   // that every CTA (and every run) uses the same threshold
@@ -92,160 +129,161 @@ __global__ void __launch_bounds__(JT) jacobi_coop_kernel(int np, int nblk, cx<R>
   }
   __syncthreads();
   const R atol = Tol<R>::abs * s_anorm;
+  const int i = tid / JS, j = tid % JS;
+  // the warp's buffers and its place among all warps
+  T* Up = reinterpret_cast<T*>(jc_raw) + (size_t)warp * (2 * JS * JS + JS * (JS + 1));
+  T* Uq = Up + JS * JS;
+  T* X = Uq + JS * JS;
+  const int r = lane >> 1, h = lane & 1;
+  const int vcols = (np + JV - 1) / JV, vitems = pairs * vcols;
+  const int items = vitems + pairs * (pairs + 1) / 2;
   int sweep = 0;
   for (; sweep < max_sweeps; ++sweep) {
     for (int round = 0; round < nblk - 1; ++round) {
-      int bi, bj;
-      tourney(round, blockIdx.x, nblk, bi, bj);
-      if (tid < JS) idx[tid] = (tid < JW) ? bi * JW + tid : bj * JW + (tid - JW);
-      __syncthreads();
-      // ---- load the 16x16 principal sub-matrix, U = I
-      for (int e = tid; e < JS * JS; e += JT) {
-        int a = e / JS, b = e % JS;
-        S[a][b] = ap[(long)idx[a] * np + idx[b]];
-        U[a][b] = mkc<R>(a == b ? 1 : 0, 0);
-      }
-      __syncthreads();
-      // ---- scalar cyclic Jacobi on S, by warp 0 alone (warp-level barriers only)
-      if (tid < 32) {
-        const int lane = tid;
-        int rot_seen = 0;
+      // ---- the pairs' sub-problems: cyclic Jacobi, one entry of S and U a thread
+      for (int pr = blockIdx.x; pr < pairs; pr += gridDim.x) {
+        int bi, bj;
+        tourney(round, pr, nblk, bi, bj);
+        auto at = [&](int x) { return x < JW ? bi * JW + x : bj * JW + x - JW; };
+        int cur = 0, active = 0;
+        S[0][i][j] = ap[(long)at(i) * np + at(j)];
+        U[0][i][j] = mkc<R>(i == j ? 1 : 0, 0);
+        __syncthreads();
         for (int inner = 0; inner < kInnerSweeps; ++inner) {
-          int any_inner_w = 0;
-          for (int r = 0; r < JS - 1; ++r) {
+          int any_inner = 0;
+          for (int st = 0; st < JS - 1; ++st) {
             int f = 0;
-            if (lane < JS / 2) {
+            if (tid < JS / 2) {
               int a, b;
-              tourney(r, lane, JS, a, b);
+              tourney(st, tid, JS, a, b);
               if (a > b) { int t = a; a = b; b = t; }
-              T g = S[a][b];
-              R ag = sqrt(cabs2(g));
-              R al = S[a][a].x, be = S[b][b].x;
+              const T g = S[cur][a][b];
+              const R ag = sqrt(cabs2(g));
+              const R al = S[cur][a][a].x, be = S[cur][b][b].x;
               f = (ag > Tol<R>::rel * sqrt(fabs(al * be))) && (ag > atol);
-              ra[lane] = a; rb[lane] = b; rflag[lane] = f;
+              R c = 1;
+              T o = mkc<R>(0, 0);
               if (f) {
-                R tau = (be - al) / (2 * ag);
-                R t = (tau >= 0 ? R(1) : R(-1)) / (fabs(tau) + sqrt(R(1) + tau * tau));
-                R c = R(1) / sqrt(R(1) + t * t);
-                rc[lane] = c; rs[lane] = t * c;
-                re[lane] = mkc<R>(g.x / ag, g.y / ag);
+                const R tau = (be - al) / (2 * ag);
+                const R t = (tau >= 0 ? R(1) : R(-1)) / (fabs(tau) + sqrt(R(1) + tau * tau));
+                c = R(1) / sqrt(R(1) + t * t);
+                o = cscale(mkc<R>(g.x / ag, g.y / ag), t * c);
               }
+              // columns: x_a <- c x_a - s conj(e) x_b, x_b <- s e x_a + c x_b
+              rc[a] = rc[b] = c;
+              ro[a] = mkc<R>(-o.x, o.y);
+              ro[b] = o;
+              rp[a] = b;
+              rp[b] = a;
             }
-            const unsigned any_f = __ballot_sync(0xffffffffu, f);
-            __syncwarp();
-            if (!any_f) continue;
-            any_inner_w = 1;
-            // rows: S <- U^+ S on rows (a, b)
-            for (int e = lane; e < (JS / 2) * JS; e += 32) {
-              int p = e / JS, col = e % JS;
-              if (!rflag[p]) continue;
-              int a = ra[p], b = rb[p];
-              R c = rc[p], s = rs[p];
-              T ee = re[p];
-              T x = S[a][col], y = S[b][col];
-              S[a][col] = csub(cscale(x, c), cscale(cmul(ee, y), s));
-              S[b][col] = cadd(cscale(cmulc(x, ee), s), cscale(y, c));
-            }
-            __syncwarp();
-            // cols: S <- S U and U_acc <- U_acc U on cols (a, b)
-            for (int e = lane; e < (JS / 2) * JS * 2; e += 32) {
-              int which = e / ((JS / 2) * JS);
-              int e2 = e % ((JS / 2) * JS);
-              int p = e2 / JS, row = e2 % JS;
-              if (!rflag[p]) continue;
-              int a = ra[p], b = rb[p];
-              R c = rc[p], s = rs[p];
-              T ee = re[p];
-              if (which) {
-                T x = U[row][a], y = U[row][b];
-                U[row][a] = csub(cscale(x, c), cscale(cmulc(y, ee), s));
-                U[row][b] = cadd(cscale(cmul(x, ee), s), cscale(y, c));
-              } else {
-                T x = S[row][a], y = S[row][b];
-                S[row][a] = csub(cscale(x, c), cscale(cmulc(y, ee), s));
-                S[row][b] = cadd(cscale(cmul(x, ee), s), cscale(y, c));
-              }
-            }
-            __syncwarp();
+            if (!__syncthreads_or(f)) continue;
+            any_inner = 1;
+            const int oi = rp[i], oj = rp[j];
+            const R ci = rc[i], cj = rc[j];
+            const T xi = cconj(ro[i]), xj = ro[j];
+            auto col = [&](T u, T v) {
+              T t = cscale(u, cj);
+              cfma(t, v, xj);
+              return t;
+            };
+            T ns = cscale(col(S[cur][i][j], S[cur][i][oj]), ci);
+            cfma(ns, xi, col(S[cur][oi][j], S[cur][oi][oj]));
+            const T nu = col(U[cur][i][j], U[cur][i][oj]);
+            S[cur ^ 1][i][j] = ns;
+            U[cur ^ 1][i][j] = nu;
+            cur ^= 1;
+            __syncthreads();
           }
-          rot_seen |= any_inner_w;
-          if (!any_inner_w) break;
+          active |= any_inner;
+          if (!any_inner) break;
         }
-        if (lane == 0) any_rot = rot_seen;
-      }
-      __syncthreads();
-      const int active = any_rot;
-      // One Newton-Schulz polar step U <- U (3I - U^+U)/2 removes the drift of the
-      // accumulated rotations from unitarity (quadratic in the drift), so repeated
-      // applications do not scale the spectrum.
-      if (active) {
-        for (int e = tid; e < JS * JS; e += JT) {
-          int a = e / JS, b = e % JS;
+        // One Newton-Schulz polar step U <- U (3I - U^+U)/2 removes the drift of the
+        // accumulated rotations from unitarity (quadratic in the drift), so repeated
+        // applications do not scale the spectrum.
+        T nu = U[cur][i][j];
+        if (active) {
           T acc = mkc<R>(0, 0);
-          for (int r = 0; r < JS; ++r) cfma(acc, cconj(U[r][a]), U[r][b]);
-          X[a][b] = acc;                      // G = U^+ U (X used as scratch)
-        }
-        __syncthreads();
-        T nu[JS * JS / JT > 0 ? JS * JS / JT : 1];
-        int q = 0;
-        for (int e = tid; e < JS * JS; e += JT, ++q) {
-          int a = e / JS, b = e % JS;
-          T acc = cscale(U[a][b], R(1.5));
-          for (int r = 0; r < JS; ++r) cfma(acc, cscale(U[a][r], R(-0.5)), X[r][b]);
-          nu[q] = acc;
-        }
-        __syncthreads();
-        q = 0;
-        for (int e = tid; e < JS * JS; e += JT, ++q) U[e / JS][e % JS] = nu[q];
-        __syncthreads();
-      }
-      // ---- phase A: rows idx of A <- U^+ A[idx, :], in column chunks staged in smem
-      if (active) {
-        for (int c0 = 0; c0 < np; c0 += CH) {
-          int cw = min(CH, np - c0);
-          for (int e = tid; e < JS * CH; e += JT) {
-            int a = e / CH, c = e % CH;
-            X[a][c] = (c < cw) ? ap[(long)idx[a] * np + c0 + c] : mkc<R>(0, 0);
-          }
+          for (int k = 0; k < JS; ++k) cfma(acc, cconj(U[cur][k][i]), U[cur][k][j]);
+          U[cur ^ 1][i][j] = acc;               // G = U^+ U
           __syncthreads();
-          for (int e = tid; e < JS * CH; e += JT) {
-            int a = e / CH, c = e % CH;
-            if (c >= cw) continue;
-            T acc = mkc<R>(0, 0);
-            for (int b = 0; b < JS; ++b) cfma(acc, cconj(U[b][a]), X[b][c]);
-            ap[(long)idx[a] * np + c0 + c] = acc;
-          }
-          __syncthreads();
+          nu = cscale(nu, R(1.5));
+          for (int k = 0; k < JS; ++k) cfma(nu, cscale(U[cur][i][k], R(-0.5)), U[cur ^ 1][k][j]);
         }
+        ug[(long)pr * JS * JS + tid] = nu;
+        if (tid == 0) {
+          act[pr] = active;
+          if (active) {
+            atomicAdd(&counters[sweep & 1], 1);
+            atomicAdd(&counters[3], 1);  // active pair-rounds, for the flop count
+          }
+        }
+        __syncthreads();
       }
       grid.sync();
-      // ---- phase B: columns idx of A and V <- (.) U, in row chunks staged in smem
-      if (active) {
-        for (int r0 = 0; r0 < 2 * np; r0 += CH) {
-          int rw = min(CH, 2 * np - r0);
-          for (int e = tid; e < CH * JS; e += JT) {
-            int r = e / JS, b = e % JS;
-            int gr = r0 + r;
-            if (r < rw) {
-              const T* rowp = (gr < np) ? ap + (long)gr * np : vp + (long)(gr - np) * np;
-              X[b][r] = rowp[idx[b]];
-            }
+      // ---- the tiles, an item a warp: 16 x JV of V^T, or a 16 x 16 tile of A's upper half
+      for (int it = blockIdx.x * (JT / 32) + warp; it < items; it += gridDim.x * (JT / 32)) {
+        T acc[8];
+        if (it < vitems) {
+          const int q = it / vcols, c0 = (it - q * vcols) * JV;
+          if (!act[q]) continue;
+          int bi, bj;
+          tourney(round, q, nblk, bi, bj);
+          copy8(Uq + lane * 8, ug + (long)q * JS * JS + lane * 8);
+          T* row = vt + (long)(r < JW ? bi * JW + r : bj * JW + r - JW) * np;
+#pragma unroll
+          for (int c = 0; c < JV; c += JS) {
+            const int col = c0 + c + 8 * h;     // np is a multiple of 16
+            if (c0 + c >= np) break;
+            copy8(X + r * JS + 8 * h, row + col);
+            __syncwarp();
+            tile_zero(acc);
+            tile_mul(acc, X, h, [&](int k) { return Uq[k * JS + r]; });
+            copy8(row + col, acc);
+            __syncwarp();
           }
-          __syncthreads();
-          for (int e = tid; e < CH * JS; e += JT) {
-            int r = e / JS, a = e % JS;
-            int gr = r0 + r;
-            if (r >= rw) continue;
-            T acc = mkc<R>(0, 0);
-            for (int b = 0; b < JS; ++b) cfma(acc, X[b][r], U[b][a]);
-            T* rowp = (gr < np) ? ap + (long)gr * np : vp + (long)(gr - np) * np;
-            rowp[idx[a]] = acc;
+        } else {
+          const int t = it - vitems;
+          int q = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+          while (q * (q + 1) / 2 > t) --q;
+          while ((q + 1) * (q + 2) / 2 <= t) ++q;
+          const int p = t - q * (q + 1) / 2;
+          if (!act[p] && !act[q]) continue;
+          int pi, pj, qi, qj;
+          tourney(round, p, nblk, pi, pj);
+          tourney(round, q, nblk, qi, qj);
+          copy8(Up + lane * 8, ug + (long)p * JS * JS + lane * 8);
+          copy8(Uq + lane * 8, ug + (long)q * JS * JS + lane * 8);
+          const int prow = r < JW ? pi * JW + r : pj * JW + r - JW;
+          const int qrow = r < JW ? qi * JW + r : qj * JW + r - JW;
+          T* dst = ap + (long)prow * np + (h ? qj : qi) * JW;
+          copy8(acc, dst);
+#pragma unroll
+          for (int c = 0; c < 8; ++c) X[r * (JS + 1) + 8 * h + c] = acc[c];
+          __syncwarp();
+          tile_zero(acc);
+          tile_mul(acc, Uq, h, [&](int k) { return X[r * (JS + 1) + k]; });
+          __syncwarp();
+          copy8(X + r * JS + 8 * h, acc);
+          __syncwarp();
+          tile_zero(acc);
+          tile_mul(acc, X, h, [&](int k) { return cconj(Up[k * JS + r]); });
+          __syncwarp();
+#pragma unroll
+          for (int c = 0; c < 8; ++c) X[r * (JS + 1) + 8 * h + c] = acc[c];
+          __syncwarp();
+          T mir[8];
+#pragma unroll
+          for (int c = 0; c < 8; ++c) mir[c] = cconj(X[(8 * h + c) * (JS + 1) + r]);
+          if (p == q) {
+            // its own mirror image: the upper half decides
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+              if (8 * h + c < r) acc[c] = mir[c];
+          } else {
+            copy8(ap + (long)qrow * np + (h ? pj : pi) * JW, mir);
           }
-          __syncthreads();
-        }
-        if (tid == 0) {
-          atomicAdd(&counters[sweep & 1], 1);
-          atomicAdd(&counters[3], 1);  // active pair-rounds, for the flop count
+          copy8(dst, acc);
+          __syncwarp();
         }
       }
       grid.sync();
@@ -257,12 +295,10 @@ __global__ void __launch_bounds__(JT) jacobi_coop_kernel(int np, int nblk, cx<R>
   if (blockIdx.x == 0 && tid == 0) counters[2] = sweep;
 }
 
-// Sort the eigenvalues (diagonal of the converged matrix, positions < n) descending
-// and gather the matching columns of V.  One CTA, bitonic sort on a power of two.
+// Sort the eigenvalues (diagonal of the converged matrix, positions < n) descending into w, their
+// positions into perm, which may be ap's own memory.  One CTA, bitonic sort on a power of two.
 template <typename R>
-__global__ void eig_finalize_kernel(int n, int np, const cx<R>* __restrict__ ap,
-                                    const cx<R>* __restrict__ vp, cx<R>* v, long ldv,
-                                    double* w) {
+__global__ void eig_sort_kernel(int n, int np, const cx<R>* ap, int* perm, double* w) {
   extern __shared__ unsigned char smem_raw[];
   int P = 1;
   while (P < n) P <<= 1;
@@ -299,13 +335,25 @@ __global__ void eig_finalize_kernel(int n, int np, const cx<R>* __restrict__ ap,
     }
   }
   for (int i = threadIdx.x; i < n; i += blockDim.x) w[i] = (s_nan && i == 0) ? NAN : key[i];
-  long total = (long)n * n;
-  for (long e = threadIdx.x; e < total; e += blockDim.x) {
-    int i = (int)(e / n), k = (int)(e % n);
-    int col = val[k];
-    col = (col >= 0 && col < n) ? col : k;
-    v[(long)i * ldv + k] = vp[(long)i * np + col];
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    const int col = val[k];
+    perm[k] = (col >= 0 && col < n) ? col : k;
   }
+}
+
+// v[i][k] = vt[perm[k]][i], through shared memory (one CTA gathering single entries took 650 us at
+// n = 1350).
+template <typename R>
+__global__ void __launch_bounds__(256) eig_gather_kernel(int n, int np, const int* __restrict__ perm,
+                                                         const cx<R>* __restrict__ vt, cx<R>* v,
+                                                         long ldv) {
+  __shared__ cx<R> tile[32][33];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, k0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
+  for (int q = ty; q < 32; q += 8)
+    if (k0 + q < n && i0 + tx < n) tile[q][tx] = vt[(long)perm[k0 + q] * np + i0 + tx];
+  __syncthreads();
+  for (int q = ty; q < 32; q += 8)
+    if (i0 + q < n && k0 + tx < n) v[(long)(i0 + q) * ldv + k0 + tx] = tile[tx][q];
 }
 
 // ---------------------------------------------------------------------------------------
@@ -883,17 +931,17 @@ int eig_padded_n(int n) { return padded_n(n); }
 // Executed rotation flops per unit of counters[3] (8 real flops per complex element update):
 // the one-CTA kernel counts applied rotations (each updates 2 rows and 2 columns of A and 2
 // columns of V, n elements each: 6 n updates); the block kernel counts active pair-rounds
-// (3 x 16 x 16 x n_pad complex multiply-adds).
+// (2 x 16 x 16 x n_pad complex multiply-adds: both sides of half of A, and V).
 double eig_flops_per_count(int n, bool fp64) {
   const int smax = fp64 ? 84 : 118;
   if (n <= smax) return 8.0 * 6.0 * (double)(n + (n & 1));
-  return 8.0 * 3 * 256 * (double)padded_n(n);
+  return 8.0 * 2 * 256 * (double)padded_n(n);
 }
 
 template <typename R>
 size_t eig_work_bytes(int n_cap) {
   size_t np = padded_n(n_cap);
-  return 2 * np * np * sizeof(cx<R>) + 256;
+  return (2 * np * np + np * JS) * sizeof(cx<R>) + 256 + np * sizeof(int);
 }
 
 template <typename R>
@@ -902,7 +950,9 @@ void eig_work_bind(EigWork<R>& w, void* base, int n_cap) {
   w.n_cap = n_cap;
   w.ap = reinterpret_cast<cx<R>*>(base);
   w.vp = w.ap + np * np;
-  w.counters = reinterpret_cast<int*>(w.vp + np * np);
+  w.ug = w.vp + np * np;
+  w.counters = reinterpret_cast<int*>(w.ug + np * JS);
+  w.act = w.counters + 64;
 }
 
 template <typename R>
@@ -917,24 +967,43 @@ cudaError_t heig(cudaStream_t st, int n, const cx<R>* a, long lda, cx<R>* v, lon
   long total = (long)np * np;
   int blocks = (int)((total + 255) / 256);
   if (blocks > 4096) blocks = 4096;
-  count_launch(3);
+  count_launch(4);
   pad_copy_kernel<R><<<blocks, 256, 0, st>>>(n, np, a, lda, work.ap, work.vp, work.counters);
   MPDO_CUDA_TRY(cudaGetLastError());
-  int grid = nblk / 2;
-  void* args[] = {&np, &nblk, &work.ap, &work.vp, &work.counters, &max_sweeps};
-  MPDO_CUDA_TRY(cudaLaunchCooperativeKernel((void*)jacobi_coop_kernel<R>, dim3(grid),
-                                            dim3(JT), args, 0, st));
+  // as many CTAs as the device holds at once, or as there are items for their warps
+  static const int resident = [] {
+    int dev = 0, sms = 0, per = 0;
+    if (cudaFuncSetAttribute(jacobi_coop_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)coop_smem<R>()) != cudaSuccess ||
+        cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, jacobi_coop_kernel<R>, JT,
+                                                      coop_smem<R>()) != cudaSuccess)
+      return 0;
+    return sms * per;
+  }();
+  if (resident < 1) return cudaErrorInvalidConfiguration;
+  const int pairs = nblk / 2;
+  const long items = (long)pairs * ((np + JV - 1) / JV) + (long)pairs * (pairs + 1) / 2;
+  const int grid = (int)std::min<long>(resident, std::max<long>(pairs, (items + JT / 32 - 1) / (JT / 32)));
+  void* args[] = {&np, &nblk, &work.ap, &work.vp, &work.ug, &work.act, &work.counters, &max_sweeps};
+  MPDO_CUDA_TRY(cudaLaunchCooperativeKernel((void*)jacobi_coop_kernel<R>, dim3(grid), dim3(JT), args,
+                                            coop_smem<R>(), st));
   int P = 1;
   while (P < n) P <<= 1;
   size_t sm = (size_t)P * (sizeof(double) + sizeof(int));
   // sort keys beyond n = 2048 exceed the default 48 KB of shared memory (with the kernel's
   // static flag): opt in up to n = 16384, 192 KB (once per instantiation)
   static const cudaError_t fattr = cudaFuncSetAttribute(
-      eig_finalize_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      eig_sort_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
       (int)(16384 * (sizeof(double) + sizeof(int))));
   MPDO_CUDA_TRY(fattr);
   if (P > 16384) return cudaErrorInvalidValue;
-  eig_finalize_kernel<R><<<1, 1024, sm, st>>>(n, np, work.ap, work.vp, v, ldv, w);
+  int* perm = reinterpret_cast<int*>(work.ap);   // the matrix is read before its memory is written
+  eig_sort_kernel<R><<<1, 1024, sm, st>>>(n, np, work.ap, perm, w);
+  MPDO_CUDA_TRY(cudaGetLastError());
+  eig_gather_kernel<R><<<dim3((n + 31) / 32, (n + 31) / 32), 256, 0, st>>>(n, np, perm, work.vp, v,
+                                                                          ldv);
   return cudaGetLastError();
 }
 
@@ -958,7 +1027,8 @@ template cudaError_t heig<float>(cudaStream_t, int, const float2*, long, float2*
 // with that device current) and passed to the kernels.
 namespace {
 constexpr int kNoAllocNMax = MPDO_HEIG_NOALLOC_NMAX;
-constexpr size_t kNoAllocBytes = 2ull * kNoAllocNMax * kNoAllocNMax * sizeof(double2) + 256;
+constexpr size_t kNoAllocBytes =
+    (2ull * kNoAllocNMax + 16) * kNoAllocNMax * sizeof(double2) + 256 + kNoAllocNMax * sizeof(int);
 static_assert(kNoAllocNMax % (2 * mpdo::JW) == 0, "maximum must be a whole number of block pairs");
 static __device__ __align__(256) unsigned char g_heig_scratch[kNoAllocBytes];
 constexpr int kMaxDevices = 64;
