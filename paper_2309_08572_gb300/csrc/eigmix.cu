@@ -74,6 +74,9 @@ __device__ __forceinline__ bool pair_separated(const double2* SG, long ld, int m
 // pass, [4] lam_max of level 0's first pass (lam_0 of the separation floor), [5] Jacobi
 // rotations of the level, [6] 1 when this level is the last, [7] columns it emits.
 constexpr int kScan = 8;
+// device only, behind them: the resolved run and the least gap, for launches of one step
+constexpr int kScanNl = 8, kScanSep = 9, kScanAll = 10;
+constexpr int kOneCtaRefine = 128;   // levels up to this width refine in one CTA
 
 // Largest cluster solved by Rayleigh-Ritz in the final refinement pass, the most clusters
 // one pass settles, and the most columns whose separation flags live in shared memory
@@ -282,11 +285,11 @@ __device__ void ritz_cluster(int m, const double2* SG, int c0, int c, double* la
 // (bound emax) take the first-order correction, the others are orthonormalised; with cid,
 // pairs inside one Ritz cluster get the identity (the Ritz step sets their block).
 __device__ void fill_ie(int m, const double2* SG, const double* lam, double2* IE, int nl,
-                        double fsep, double emax, const int* cid) {
+                        double fsep, double emax, const int* cid, long first, long step) {
   const long ld = 2L * m;
   // one thread per pair i <= j: the pair's separation is decided once, from the entry above
   // the diagonal, and both entries are written
-  for (long e = threadIdx.x; e < (long)m * m; e += blockDim.x) {
+  for (long e = first; e < (long)m * m; e += step) {
     const int i = (int)(e / m), j = (int)(e % m);
     if (j < i) continue;
     if (cid && cid[i] >= 0 && cid[i] == cid[j]) {
@@ -319,6 +322,30 @@ __device__ void fill_ie(int m, const double2* SG, const double* lam, double2* IE
   }
 }
 
+// A level's scalars, from the largest lam and the resolved run [0, nl).
+template <bool FINAL>
+__device__ void refine_scan(int m, int nl, double vf, int level, double floor, const int* rot,
+                            const double* lam, double* scan, double* red) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  double rst = 0.0;
+  for (int i = nl + tid; i < m; i += nt) rst = fmax(rst, lam[i]);
+  const double rest = block_max(rst, red);
+  if (tid == 0) {
+    scan[0] = vf;
+    scan[1] = (double)nl;
+    scan[2] = rest;
+    if constexpr (FINAL) {
+      if (level == 0) scan[3] = vf;
+      const double top = scan[3];
+      const bool last = (nl >= m) || (level + 1 >= kMaxLevels) || !(rest > floor * top) ||
+                        nl == 0;
+      scan[5] = rot ? (double)rot[3] : 0.0;
+      scan[6] = last ? 1.0 : 0.0;
+      scan[7] = last ? (double)m : (double)nl;
+    }
+  }
+}
+
 // One refinement step's scalars and correction, run by one CTA of 256 threads.
 // S = SG[:, 0:m], G = SG[:, m:2m] (row stride 2m), possibly written by other CTAs of the
 // same launch (read through L2).  lam_i = S_ii / G_ii; IE = I + E.  The final pass
@@ -326,7 +353,9 @@ __device__ void fill_ie(int m, const double2* SG, const double* lam, double2* IE
 // clean boundary and decides whether the level is the last one; its scratch (flags and
 // cluster list) exists only in that instantiation.  sepg: workspace for the neighbour
 // separation flags of levels wider than kSepMax.
-template <bool FINAL>
+// SPLIT leaves I + E, the Ritz steps and the level's scalars to the launches behind it
+// (refine_fill_kernel, refine_ritz_kernel, refine_end_kernel), with nl and fsep in scan.
+template <bool FINAL, bool SPLIT = false>
 __device__ void refine_step(int m, int n, const double2* SG, int level0, int level,
                             double floor, const int* rot, double* lam, double* scan, double2* IE,
                             int* cid, double emax, unsigned char* sepg) {
@@ -356,7 +385,7 @@ __device__ void refine_step(int m, int n, const double2* SG, int level0, int lev
     for (int i = tid; i < m; i += nt)
       if (!(lam[i] > kTau * v)) f = min(f, i);
     nl = block_min_int(f, ired);
-    fill_ie(m, SG, lam, IE, nl, fsep, emax, nullptr);
+    if constexpr (!SPLIT) fill_ie(m, SG, lam, IE, nl, fsep, emax, nullptr, tid, nt);
   } else {
     __shared__ unsigned char s_sep[kSepMax];
     __shared__ int s_cl0[kMaxClusters], s_cln[kMaxClusters];
@@ -408,7 +437,14 @@ __device__ void refine_step(int m, int n, const double2* SG, int level0, int lev
       if (clean) best = max(best, k);
     }
     nl = block_max_int(best, ired);
-    fill_ie(m, SG, lam, IE, nl, fsep, emax, cid);
+    if constexpr (SPLIT) {
+      if (tid == 0) {
+        scan[kScanNl] = (double)nl;
+        scan[kScanSep] = fsep;
+      }
+      return;
+    }
+    fill_ie(m, SG, lam, IE, nl, fsep, emax, cid, tid, nt);
     __syncthreads();
     const int ncl = s_ncl;
     for (int q = 0; q < ncl; ++q) ritz_cluster(m, SG, s_cl0[q], s_cln[q], lam, IE);
@@ -416,23 +452,13 @@ __device__ void refine_step(int m, int n, const double2* SG, int level0, int lev
     for (int i = tid; i < m; i += nt) mx2 = fmax(mx2, lam[i]);
     vf = block_max(mx2, red);
   }
-  double rst = 0.0;
-  for (int i = nl + tid; i < m; i += nt) rst = fmax(rst, lam[i]);
-  const double rest = block_max(rst, red);
-  if (tid == 0) {
-    scan[0] = vf;
-    scan[1] = (double)nl;
-    scan[2] = rest;
-    if constexpr (FINAL) {
-      if (level == 0) scan[3] = vf;
-      const double top = scan[3];
-      const bool last = (nl >= m) || (level + 1 >= kMaxLevels) || !(rest > floor * top) ||
-                        nl == 0;
-      scan[5] = rot ? (double)rot[3] : 0.0;
-      scan[6] = last ? 1.0 : 0.0;
-      scan[7] = last ? (double)m : (double)nl;
+  if constexpr (SPLIT) {
+    if (tid == 0) {
+      scan[kScanNl] = (double)nl;
+      scan[kScanSep] = fsep;
     }
   }
+  refine_scan<FINAL>(m, nl, vf, level, floor, rot, lam, scan, red);
 }
 
 constexpr int RT = 16;   // output tile of the fused products (one element per thread)
@@ -503,6 +529,41 @@ __global__ void __launch_bounds__(RT * RT) refine_kernel(int m, int n, const dou
     refine_step<true>(m, n, SG, level0, level, floor, rot, lam, scan, IE, cid, emax, sepg);
   else
     refine_step<false>(m, n, SG, level0, level, floor, rot, lam, scan, IE, cid, emax, sepg);
+}
+
+// The same for wide levels, in launches that use the chip: on one CTA the divisions of m^2 / 2
+// pairs took 4.5 ms at m = 1350, now 0.1 ms.
+template <bool FINAL>
+__global__ void __launch_bounds__(256) refine_head_kernel(int m, int n, const double2* SG, int level0,
+                                                          int level, double floor, const int* rot,
+                                                          double* lam, double* scan, double2* IE,
+                                                          int* cid, double emax, unsigned char* sepg) {
+  refine_step<FINAL, true>(m, n, SG, level0, level, floor, rot, lam, scan, IE, cid, emax, sepg);
+}
+__global__ void __launch_bounds__(256) refine_fill_kernel(int m, const double2* SG, const double* lam,
+                                                          const double* scan, double2* IE,
+                                                          double emax, const int* cid) {
+  fill_ie(m, SG, lam, IE, (int)scan[kScanNl], scan[kScanSep], emax, cid,
+          blockIdx.x * (long)blockDim.x + threadIdx.x, (long)gridDim.x * blockDim.x);
+}
+// CTA i: the Ritz cluster that starts at i, if one does
+__global__ void __launch_bounds__(256) refine_ritz_kernel(int m, const double2* SG, double* lam,
+                                                          double2* IE, const int* cid) {
+  const int c0 = blockIdx.x;
+  if (cid[c0] != c0) return;
+  int c = 1;
+  while (c0 + c < m && cid[c0 + c] == c0) ++c;
+  ritz_cluster(m, SG, c0, c, lam, IE);
+}
+__global__ void __launch_bounds__(256) refine_end_kernel(int m, int level, double floor,
+                                                         const int* rot, const double* lam,
+                                                         double* scan) {
+  __shared__ double red[32];
+  double mx = -1e300;
+  for (int i = threadIdx.x; i < m; i += blockDim.x) mx = fmax(mx, lam[i]);
+  const double vf = block_max(mx, red);
+  __syncthreads();
+  refine_scan<true>(m, (int)scan[kScanNl], vf, level, floor, rot, lam, scan, red);
 }
 
 // ---- graded matrices (heig_graded): one refinement pass.
@@ -817,7 +878,7 @@ void mix_work_bind(MixWork& w, void* base, int n_cap) {
   w.y32 = reinterpret_cast<float2*>(take(sq * 8));
   w.lam = reinterpret_cast<double*>(take((size_t)n_cap * 8));
   w.w32 = reinterpret_cast<double*>(take((size_t)n_cap * 8));
-  w.scan = reinterpret_cast<double*>(take(kScan * sizeof(double)));
+  w.scan = reinterpret_cast<double*>(take(kScanAll * sizeof(double)));
   w.ticket = reinterpret_cast<unsigned int*>(take(64));
   w.cid = reinterpret_cast<int*>(take((size_t)n_cap * sizeof(int)));
   w.sepf = reinterpret_cast<unsigned char*>(take((size_t)n_cap));
@@ -903,9 +964,26 @@ cudaError_t enqueue_level(cudaStream_t st, int n, int m, int level, const double
       MPDO_CUDA_TRY(gemm64(st, wk, OP_C, OP_N, m, 2 * m, n, cur + m, l2, 0, cur, l2, 0, wk.s, l2,
                            0, 1));
       count_launch();
-      refine_kernel<<<1, RT * RT, 0, st>>>(m, n, wk.s, (lev0 && pass == 0) ? 1 : 0, final_pass,
-                                           level, floor, (const int*)wk.ew.counters, wk.lam,
-                                           wk.scan, wk.ie, wk.cid, emax, wk.sepf);
+      const int level0 = (lev0 && pass == 0) ? 1 : 0;
+      const int* rot = wk.ew.counters;
+      if (m <= kOneCtaRefine) {
+        refine_kernel<<<1, RT * RT, 0, st>>>(m, n, wk.s, level0, final_pass, level, floor, rot, wk.lam,
+                                             wk.scan, wk.ie, wk.cid, emax, wk.sepf);
+      } else {
+        const int fill = (int)std::min<long>(((long)m * m + 255) / 256, 152 * 8);
+        count_launch(final_pass ? 3 : 1);
+        if (final_pass) {
+          refine_head_kernel<true><<<1, 256, 0, st>>>(m, n, wk.s, level0, level, floor, rot, wk.lam,
+                                                      wk.scan, wk.ie, wk.cid, emax, wk.sepf);
+          refine_fill_kernel<<<fill, 256, 0, st>>>(m, wk.s, wk.lam, wk.scan, wk.ie, emax, wk.cid);
+          refine_ritz_kernel<<<m, 256, 0, st>>>(m, wk.s, wk.lam, wk.ie, wk.cid);
+          refine_end_kernel<<<1, 256, 0, st>>>(m, level, floor, rot, wk.lam, wk.scan);
+        } else {
+          refine_head_kernel<false><<<1, 256, 0, st>>>(m, n, wk.s, level0, level, floor, rot, wk.lam,
+                                                       wk.scan, wk.ie, wk.cid, emax, wk.sepf);
+          refine_fill_kernel<<<fill, 256, 0, st>>>(m, wk.s, wk.lam, wk.scan, wk.ie, emax, nullptr);
+        }
+      }
       MPDO_CUDA_TRY(cudaGetLastError());
     } else {
       count_launch();
