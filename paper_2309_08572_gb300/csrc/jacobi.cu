@@ -9,10 +9,13 @@
 // barrier ends the round.  A tile needs no other tile, so A is read and written once a round, and
 // V is kept transposed, so that its rows are contiguous.  A sweep in which no pair rotated ends
 // the iteration.  Cost per sweep ~4 n^3 complex MACs; the matrix stays in L2 (it is at most a few
-// MB... 29 MB with V at n = 1350).  A round there is bound by FP32 issue in the tiles (~12 us) and
-// the serial chain of 15 rotation steps and two grid barriers before them (~8 us); rows and columns
-// in two passes of 16 x np by the pairs' own CTAs, each waiting for its loads, took 92 us.  An FP32
-// solve of n = 1350 takes 52 ms on average over the mixed solver's levels, 231 ms before.
+// MB... 29 MB with V at n = 1350).  A round there is bound by FP32 issue in the tiles (~12 us
+// of FMAs) and, before them, the serial chain of 15 rotation steps and the grid barriers; rows and
+// columns in two passes of 16 x np by the pairs' own CTAs, each waiting for its loads, took 92 us.
+// In the late sweeps few pairs have anything left to rotate: a sub-problem looks first, and a round
+// in which none had leaves out its tiles and second barrier.  The mixed solver's six levels at n =
+// 1350 (FP32 solves of 1350 down to 464): 1240 ms with the passes, 250 ms with tiles, 175 ms with
+// approximate rotations, the look ahead and items from a counter; FP64 at n = 400: 277 -> 92 ms.
 #include <cooperative_groups.h>
 #include <cuda.h>
 
@@ -33,6 +36,7 @@ constexpr int JW = 8;          // block width
 constexpr int JS = 2 * JW;     // sub-problem size
 constexpr int JT = 256;        // threads per CTA: one per entry of the sub-problem
 constexpr int JV = 32;         // columns of V^T in a warp's item
+constexpr int kMaxPairs = 1024;   // n <= 16384
 // Sweeps of the 16x16 sub-problem per block-pair visit.  One sweep per visit is the
 // classic one-sided-update choice: the outer rounds keep rotating the pair, so a fully
 // converged sub-problem buys little and costs 15 warp rounds per extra sweep.
@@ -91,6 +95,30 @@ __device__ __forceinline__ void copy8(T* dst, const T* src) {
     reinterpret_cast<float4*>(dst)[i] = reinterpret_cast<const float4*>(src)[i];
 }
 
+// Rotation of the pair (al, be) with coupling g of modulus ag: cosine and s e of the two columns.
+// FP32 from approximate roots and quotients (a chain of ~150 clocks on the sub-problem's critical
+// path, ~600 with the rounded ones): a rotation off by a few eps is one all the same, and the polar
+// step after the sub-problem takes out what it lacks in unitarity.
+__device__ __forceinline__ float modulus(float2 g) {
+  const float q = g.x * g.x + g.y * g.y;
+  return q > 0.f ? q * rsqrtf(q) : 0.f;
+}
+__device__ __forceinline__ double modulus(double2 g) { return sqrt(cabs2(g)); }
+__device__ __forceinline__ void rotation(float2 g, float ag, float al, float be, float& c, float2& o) {
+  const float inv = __fdividef(1.f, ag);
+  const float tau = fminf(fmaxf((be - al) * 0.5f * inv, -1e18f), 1e18f), q = 1.f + tau * tau;
+  const float t = copysignf(__fdividef(1.f, fabsf(tau) + q * rsqrtf(q)), tau);
+  c = rsqrtf(1.f + t * t);
+  o = cscale(g, inv * t * c);
+}
+__device__ __forceinline__ void rotation(double2 g, double ag, double al, double be, double& c,
+                                         double2& o) {
+  const double tau = (be - al) / (2 * ag);
+  const double t = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
+  c = 1.0 / sqrt(1.0 + t * t);
+  o = cscale(mkc<double>(g.x / ag, g.y / ag), t * c);
+}
+
 template <typename R>
 constexpr size_t coop_smem() {   // per warp: U_p, U_q, a tile of stride 17
   return (size_t)(JT / 32) * (2 * JS * JS + JS * (JS + 1)) * sizeof(cx<R>);
@@ -98,8 +126,8 @@ constexpr size_t coop_smem() {   // per warp: U_p, U_q, a tile of stride 17
 
 template <typename R>
 __global__ void __launch_bounds__(JT, 2) jacobi_coop_kernel(int np, int nblk, cx<R>* ap, cx<R>* vt,
-                                                            cx<R>* ug, int* act, int* counters,
-                                                            int max_sweeps) {
+                                                            cx<R>* ug, int* act, int* next,
+                                                            int* counters, int max_sweeps) {
   using T = cx<R>;
   cg::grid_group grid = cg::this_grid();
   extern __shared__ __align__(16) unsigned char jc_raw[];
@@ -108,9 +136,17 @@ __global__ void __launch_bounds__(JT, 2) jacobi_coop_kernel(int np, int nblk, cx
   __shared__ R rc[JS];             // per index: cosine, partner's coefficient, partner
   __shared__ T ro[JS];
   __shared__ int rp[JS];
+  __shared__ unsigned char s_act[kMaxPairs];
+  __shared__ unsigned char sa[JS - 1][JS / 2], sb[JS - 1][JS / 2];   // pairs of a step, a < b
   __shared__ R s_anorm;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int pairs = nblk / 2;
+  if (tid < (JS - 1) * (JS / 2)) {
+    int a, b;
+    tourney(tid / (JS / 2), tid % (JS / 2), JS, a, b);
+    sa[tid / (JS / 2)][tid % (JS / 2)] = (unsigned char)min(a, b);
+    sb[tid / (JS / 2)][tid % (JS / 2)] = (unsigned char)max(a, b);
+  }
 
   // |A| scale for the absolute rotation floor: sum of |diag|, reduced in a fixed order so
   // that every CTA (and every run) uses the same threshold
@@ -137,38 +173,37 @@ __global__ void __launch_bounds__(JT, 2) jacobi_coop_kernel(int np, int nblk, cx
   const int r = lane >> 1, h = lane & 1;
   const int vcols = (np + JV - 1) / JV, vitems = pairs * vcols;
   const int items = vitems + pairs * (pairs + 1) / 2;
-  int sweep = 0;
+  if (blockIdx.x == 0 && tid == 0) next[0] = gridDim.x * (JT / 32);
+  int sweep = 0, tick = 0;   // tick: rounds so far
   for (; sweep < max_sweeps; ++sweep) {
-    for (int round = 0; round < nblk - 1; ++round) {
+    for (int round = 0; round < nblk - 1; ++round, ++tick) {
+      int* flags = act + (tick & 1) * pairs;
       // ---- the pairs' sub-problems: cyclic Jacobi, one entry of S and U a thread
       for (int pr = blockIdx.x; pr < pairs; pr += gridDim.x) {
         int bi, bj;
         tourney(round, pr, nblk, bi, bj);
         auto at = [&](int x) { return x < JW ? bi * JW + x : bj * JW + x - JW; };
+        auto couples = [&](R ag, R al, R be) {
+          return (ag > Tol<R>::rel * sqrt(fabs(al * be))) && (ag > atol);
+        };
         int cur = 0, active = 0;
         S[0][i][j] = ap[(long)at(i) * np + at(j)];
         U[0][i][j] = mkc<R>(i == j ? 1 : 0, 0);
         __syncthreads();
-        for (int inner = 0; inner < kInnerSweeps; ++inner) {
+        // nothing to rotate, as in most pairs of the late sweeps: one look instead of 15 steps
+        const int live = __syncthreads_or(i < j && couples(modulus(S[0][i][j]), S[0][i][i].x, S[0][j][j].x));
+        for (int inner = 0; inner < (live ? kInnerSweeps : 0); ++inner) {
           int any_inner = 0;
           for (int st = 0; st < JS - 1; ++st) {
             int f = 0;
             if (tid < JS / 2) {
-              int a, b;
-              tourney(st, tid, JS, a, b);
-              if (a > b) { int t = a; a = b; b = t; }
+              const int a = sa[st][tid], b = sb[st][tid];
               const T g = S[cur][a][b];
-              const R ag = sqrt(cabs2(g));
-              const R al = S[cur][a][a].x, be = S[cur][b][b].x;
-              f = (ag > Tol<R>::rel * sqrt(fabs(al * be))) && (ag > atol);
+              const R ag = modulus(g), al = S[cur][a][a].x, be = S[cur][b][b].x;
+              f = couples(ag, al, be);
               R c = 1;
               T o = mkc<R>(0, 0);
-              if (f) {
-                const R tau = (be - al) / (2 * ag);
-                const R t = (tau >= 0 ? R(1) : R(-1)) / (fabs(tau) + sqrt(R(1) + tau * tau));
-                c = R(1) / sqrt(R(1) + t * t);
-                o = cscale(mkc<R>(g.x / ag, g.y / ag), t * c);
-              }
+              if (f) rotation(g, ag, al, be, c, o);
               // columns: x_a <- c x_a - s conj(e) x_b, x_b <- s e x_a + c x_b
               rc[a] = rc[b] = c;
               ro[a] = mkc<R>(-o.x, o.y);
@@ -211,7 +246,7 @@ __global__ void __launch_bounds__(JT, 2) jacobi_coop_kernel(int np, int nblk, cx
         }
         ug[(long)pr * JS * JS + tid] = nu;
         if (tid == 0) {
-          act[pr] = active;
+          flags[pr] = active;
           if (active) {
             atomicAdd(&counters[sweep & 1], 1);
             atomicAdd(&counters[3], 1);  // active pair-rounds, for the flop count
@@ -220,45 +255,67 @@ __global__ void __launch_bounds__(JT, 2) jacobi_coop_kernel(int np, int nblk, cx
         __syncthreads();
       }
       grid.sync();
-      // ---- the tiles, an item a warp: 16 x JV of V^T, or a 16 x 16 tile of A's upper half
-      for (int it = blockIdx.x * (JT / 32) + warp; it < items; it += gridDim.x * (JT / 32)) {
+      // ---- the tiles, an item a warp: 16 x JV of V^T, or a 16 x 16 tile of A's upper half; the
+      // first ones by place, further ones from a counter, asked for an item ahead
+      if (blockIdx.x == 0 && tid == 0) {
+        next[(tick + 1) & 1] = gridDim.x * (JT / 32);
+        if (round == 0) counters[(sweep + 1) & 1] = 0;
+      }
+      int any = 0;
+      for (int p = tid; p < pairs; p += JT) any |= s_act[p] = (unsigned char)flags[p];
+      // no pair rotated: every CTA sees that, and the flags of the next round lie elsewhere
+      if (!__syncthreads_or(any)) continue;
+      int ahead = 0;
+      for (int it = blockIdx.x * (JT / 32) + warp; it < items; it = ahead) {
+        if (lane == 0) ahead = atomicAdd(&next[tick & 1], 1);
+        ahead = __shfl_sync(0xffffffffu, ahead, 0);
         T acc[8];
         if (it < vitems) {
           const int q = it / vcols, c0 = (it - q * vcols) * JV;
-          if (!act[q]) continue;
+          if (!s_act[q]) continue;
           int bi, bj;
           tourney(round, q, nblk, bi, bj);
-          copy8(Uq + lane * 8, ug + (long)q * JS * JS + lane * 8);
-          T* row = vt + (long)(r < JW ? bi * JW + r : bj * JW + r - JW) * np;
-#pragma unroll
-          for (int c = 0; c < JV; c += JS) {
-            const int col = c0 + c + 8 * h;     // np is a multiple of 16
-            if (c0 + c >= np) break;
-            copy8(X + r * JS + 8 * h, row + col);
-            __syncwarp();
+          static_assert(JV == 2 * JS, "two tiles an item");
+          T* row = vt + (long)(r < JW ? bi * JW + r : bj * JW + r - JW) * np + c0 + 8 * h;
+          const bool two = c0 + JS < np;          // np is a multiple of 16
+          T x0[8], x1[8], u[8];
+          copy8(x0, row);
+          if (two) copy8(x1, row + JS);
+          copy8(u, ug + (long)q * JS * JS + lane * 8);
+          copy8(Uq + lane * 8, u);
+          copy8(X + r * JS + 8 * h, x0);
+          if (two) copy8(Up + r * JS + 8 * h, x1);
+          __syncwarp();
+          tile_zero(acc);
+          tile_mul(acc, X, h, [&](int k) { return Uq[k * JS + r]; });
+          copy8(row, acc);
+          if (two) {
             tile_zero(acc);
-            tile_mul(acc, X, h, [&](int k) { return Uq[k * JS + r]; });
-            copy8(row + col, acc);
-            __syncwarp();
+            tile_mul(acc, Up, h, [&](int k) { return Uq[k * JS + r]; });
+            copy8(row + JS, acc);
           }
+          __syncwarp();
         } else {
           const int t = it - vitems;
           int q = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
           while (q * (q + 1) / 2 > t) --q;
           while ((q + 1) * (q + 2) / 2 <= t) ++q;
           const int p = t - q * (q + 1) / 2;
-          if (!act[p] && !act[q]) continue;
+          if (!s_act[p] && !s_act[q]) continue;
           int pi, pj, qi, qj;
           tourney(round, p, nblk, pi, pj);
           tourney(round, q, nblk, qi, qj);
-          copy8(Up + lane * 8, ug + (long)p * JS * JS + lane * 8);
-          copy8(Uq + lane * 8, ug + (long)q * JS * JS + lane * 8);
           const int prow = r < JW ? pi * JW + r : pj * JW + r - JW;
           const int qrow = r < JW ? qi * JW + r : qj * JW + r - JW;
           T* dst = ap + (long)prow * np + (h ? qj : qi) * JW;
+          T u[8], w[8];
           copy8(acc, dst);
+          copy8(u, ug + (long)p * JS * JS + lane * 8);
+          copy8(w, ug + (long)q * JS * JS + lane * 8);
 #pragma unroll
           for (int c = 0; c < 8; ++c) X[r * (JS + 1) + 8 * h + c] = acc[c];
+          copy8(Up + lane * 8, u);
+          copy8(Uq + lane * 8, w);
           __syncwarp();
           tile_zero(acc);
           tile_mul(acc, Uq, h, [&](int k) { return X[r * (JS + 1) + k]; });
@@ -287,7 +344,6 @@ __global__ void __launch_bounds__(JT, 2) jacobi_coop_kernel(int np, int nblk, cx
         }
       }
       grid.sync();
-      if (round == 0 && blockIdx.x == 0 && tid == 0) counters[(sweep + 1) & 1] = 0;
     }
     int done = (atomicAdd(&counters[sweep & 1], 0) == 0);
     if (done) { ++sweep; break; }
@@ -982,11 +1038,13 @@ cudaError_t heig(cudaStream_t st, int n, const cx<R>* a, long lda, cx<R>* v, lon
       return 0;
     return sms * per;
   }();
-  if (resident < 1) return cudaErrorInvalidConfiguration;
   const int pairs = nblk / 2;
+  if (resident < 1 || pairs > kMaxPairs) return cudaErrorInvalidConfiguration;
   const long items = (long)pairs * ((np + JV - 1) / JV) + (long)pairs * (pairs + 1) / 2;
   const int grid = (int)std::min<long>(resident, std::max<long>(pairs, (items + JT / 32 - 1) / (JT / 32)));
-  void* args[] = {&np, &nblk, &work.ap, &work.vp, &work.ug, &work.act, &work.counters, &max_sweeps};
+  int* next = work.counters + 8;   // items handed out in even and odd rounds
+  void* args[] = {&np, &nblk, &work.ap, &work.vp, &work.ug, &work.act, &next, &work.counters,
+                  &max_sweeps};
   MPDO_CUDA_TRY(cudaLaunchCooperativeKernel((void*)jacobi_coop_kernel<R>, dim3(grid), dim3(JT), args,
                                             coop_smem<R>(), st));
   int P = 1;
