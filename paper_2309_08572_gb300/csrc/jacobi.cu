@@ -8,8 +8,8 @@
 // tiles of the upper half (mirrored into the lower) and V[:, q] <- V[:, q] U_q, and a second
 // barrier ends the round.  A tile needs no other tile, so A is read and written once a round, and
 // V is kept transposed, so that its rows are contiguous.  A sweep in which no pair rotated ends
-// the iteration.  Cost per sweep ~4 n^3 complex MACs; the matrix stays in L2 (it is at most a few
-// MB... 29 MB with V at n = 1350).  A round there is bound by FP32 issue in the tiles (~12 us
+// the iteration.  Cost per sweep ~4 n^3 complex MACs; the matrix stays in L2 (29 MB
+// with V at n = 1350).  A round there is bound by FP32 issue in the tiles (~12 us
 // of FMAs) and, before them, the serial chain of 15 rotation steps and the grid barriers; rows and
 // columns in two passes of 16 x np by the pairs' own CTAs, each waiting for its loads, took 92 us.
 // In the late sweeps few pairs have anything left to rotate: a sub-problem looks first, and a round
