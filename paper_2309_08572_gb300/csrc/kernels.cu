@@ -662,8 +662,9 @@ __global__ void dual_rows_kernel(int kk, int cols, const cx<R>* __restrict__ y, 
 // and imaginary halves with the first exchange, which leaves one operation a step.  Rows beyond 32
 // go to the CTAs of a thread-block cluster (row i belongs to rank i mod S), each row's part of L --
 // and of W, where it fits -- in its CTA's shared memory.  Per column every CTA sends its best
-// remaining diagonal and that row of L to every CTA with remote stores that count their bytes at
-// the receiver's mbarrier: one hop, after which all hold the pivot and its row, against a cluster
+// remaining diagonal, a remote store, and that row of L, a bulk copy, to every CTA; both count
+// their bytes at the receiver's mbarrier (a remote store for every entry of the row kept the
+// barriers counting for 1200 clocks): one hop, after which all hold the pivot and its row, against a cluster
 // barrier (1200 clocks) and a fetch of the row (1400) before.  Where the slots of all candidates'
 // rows do not fit (n > 832 at 168 columns) the owner sends the pivot's row in a second hop.  The
 // remaining diagonals follow from the unscaled column, beside its scaling.  Slots alternate by
@@ -671,7 +672,8 @@ __global__ void dual_rows_kernel(int kk, int cols, const cx<R>* __restrict__ y, 
 // does when its threads are done with column j.  Candidates are compared as integers
 // (non-negative doubles order alike), which keeps the FP64 pipe to the dot products.  Sums and the
 // pivot choice follow a fixed order, so the factor does not depend on scheduling.
-// n 156, rank 52: 225 -> 140 us; n 64, rank 45: 170 -> 96 us; n 32, rank 24: 54 -> 43 us.
+// n 156, rank 52: 225 -> 122 us; n 400, rank 55: 258 -> 151; n 64, rank 45: 170 -> 88; n 32, rank
+// 24: 54 -> 41 us.
 constexpr int kPcWarps = 8;              // row warps of a CTA
 constexpr int kPcCtas = 16;
 constexpr unsigned long long kPcWaitNs = 1000000000ull;
@@ -698,8 +700,13 @@ __device__ __forceinline__ void pc_send(uint32_t dst, uint32_t bar, long long a,
                ::"r"(dst), "r"(bar), "l"(a), "l"(b)
                : "memory");
 }
-__device__ __forceinline__ void pc_send(uint32_t dst, uint32_t bar, double2 v) {
-  pc_send(dst, bar, __double_as_longlong(v.x), __double_as_longlong(v.y));
+// bytes (a multiple of 16) from this CTA's shared memory, as one count at the receiver's barrier
+__device__ __forceinline__ void pc_copy(uint32_t dst, uint32_t bar, const void* src, int bytes) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%2], %3, [%1];" ::"r"(
+          dst),
+      "r"(bar), "r"(pc_su32(src)), "r"(bytes)
+      : "memory");
 }
 __device__ __forceinline__ void pc_send(uint32_t dst, uint32_t bar, float2 v) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%2, %3}, [%1];"
@@ -748,6 +755,7 @@ __global__ void __launch_bounds__(32 * (kPcWarps + 1)) pchol_kernel(
   __shared__ int s_i[2][kPcWarps], s_late;
   __shared__ double s_tr[kPcWarps], post_tr, s_inv, s_inv2, s_dp;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = (blockDim.x >> 5) - 1;
+  const int lgS = 31 - __clz(S);                 // S is a power of two
   const int lr_ = lane & (LANES - 1), li = tid / LANES, i = c + li * S;
   const int part = lr_ >= LANES / 2;             // lanes of the upper half end with the imaginary part
   const bool own = warp < nw && li < nlm && i < n;
@@ -786,11 +794,17 @@ __global__ void __launch_bounds__(32 * (kPcWarps + 1)) pchol_kernel(
   };
   // the first j entries of row i of L (this CTA's) into a slot of every CTA
   auto send_row = [&](int j, int i, const T* slot, uint32_t bar) {
-    const T* mine = Ls + (size_t)(i / S) * rmax;
+    const T* mine = Ls + (size_t)(i >> lgS) * rmax;
     const uint32_t s0 = pc_su32(slot);
-    for (int q = warp; q < S; q += nw + 1) {
-      const uint32_t rb = pc_map(bar, q), rs = pc_map(s0, q);
-      for (int k = lane; k < j; k += 32) pc_send(rs + k * (int)sizeof(T), rb, mine[k]);
+    if constexpr (sizeof(R) == 8) {
+      // one copy a receiver: FP64 entries are 16 bytes
+      if (j > 0 && warp == nw && lane < S)
+        pc_copy(pc_map(s0, lane), pc_map(bar, lane), mine, j * (int)sizeof(T));
+    } else {
+      for (int q = warp; q < S; q += nw + 1) {
+        const uint32_t rb = pc_map(bar, q), rs = pc_map(s0, q);
+        for (int k = lane; k < j; k += 32) pc_send(rs + k * (int)sizeof(T), rb, mine[k]);
+      }
     }
   };
   // The best remaining diagonal of all rows, as bits: this CTA's (all_rows: with that row of L, up
@@ -836,11 +850,11 @@ __global__ void __launch_bounds__(32 * (kPcWarps + 1)) pchol_kernel(
     if (piv && c == 0 && tid == 0) piv[j] = p;
     const T* prow = Ls + (size_t)p * rmax;
     if constexpr (CLUSTER) {
-      prow = rows + ((size_t)(j & 1) * nslot + (all_rows ? p % S : 0)) * rmax;
+      prow = rows + ((size_t)(j & 1) * nslot + (all_rows ? p & (S - 1) : 0)) * rmax;
       if (!all_rows) {
         const uint32_t bar = pc_su32(&bars[2 + (j & 1)]);
         expect(bar, j * (int)sizeof(T));
-        if (p % S == c) send_row(j, p, prow, bar);
+        if ((p & (S - 1)) == c) send_row(j, p, prow, bar);
         if (!pc_wait(bar, (uint32_t)(j >> 1) & 1)) s_late = 1;
       }
     }
@@ -886,6 +900,8 @@ __global__ void __launch_bounds__(32 * (kPcWarps + 1)) pchol_kernel(
       R lij = v * (R)s_inv;
       if (i == p) lij = part ? R(0) : (R)s_dp;
       if ((lr_ & (LANES / 2 - 1)) == 0) reinterpret_cast<R*>(Ls + (size_t)li * rmax + j)[part] = lij;
+      // the row may go out as a copy, which reads through the asynchronous proxy
+      if constexpr (CLUSTER && sizeof(R) == 8) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     r = j + 1;
     last = 0;
@@ -1186,11 +1202,11 @@ cudaError_t pchol(cudaStream_t st, int n, const cx<R>* w, int rmax, double tol, 
                   int* rout, double* resid, int* piv) {
   if (n < 1 || n > 1024 || rmax < 1 || rmax > kGradedMax) return cudaErrorInvalidValue;
   // One CTA needs no exchange, which is worth more than other CTAs' FP64 pipes up to 32 rows (rank
-  // 24: 43 us against 49 us on four); then 16 to 32 rows a CTA (n 64, rank 45: four CTAs 96 us,
-  // eight 104, two 122; n 156, rank 52: eight 136, sixteen 140, four 171).  Eight lanes a row while
-  // the row warps are few (20 rows, rank 52: 2.87 us a column against 3.02; 32 rows: 3.34 against
-  // 3.00).  FP32 keeps four lanes: its sums keep their order.
-  const int S = n > 256 ? kPcCtas : n > 64 ? 8 : n > 32 ? 4 : 1;
+  // 24: 41 us against 49 us on four); then up to 20 rows a CTA with eight lanes each (n 64, rank 45:
+  // four CTAs 88 us, two 104; n 200, rank 52: sixteen 119, eight 144; 20 rows: 2.35 us a column with
+  // eight lanes, 2.47 with four), beyond 16 CTAs more rows with four lanes (n 400, rank 55: 151 us,
+  // eight lanes 162).  FP32 keeps four lanes: its sums keep their order.
+  const int S = n > 160 ? kPcCtas : n > 64 ? 8 : n > 32 ? 4 : 1;
   const int rows = (n + S - 1) / S;
   const int lanes = S > 1 && rows <= 20 && sizeof(R) == 8 ? 8 : 4;
   const int threads = (rows * lanes + 31) / 32 * 32 + 32;   // and the warp of the root
