@@ -473,10 +473,10 @@ def run_ours(args):
     single = single_circuit(lib, g, dls[0], circs[0]) if not args.no_single else None
     prof = [g.profile_read(k) for k in range(3)]
     g.profile(0)
-    names = {0: "complex GEMMs (cgemm_kernel, cgemm_small_kernel, FP64-product cgemm_wide; "
+    names = {0: "complex GEMMs (cgemm_tile_kernel, cgemm_kernel, cgemm_small_kernel, cgemm_wide; "
                 "tc_gemm_kernel for the tensor-core forms)",
              1: "eigensolvers (pchol_kernel, jacobi_graded_kernel, jacobi_smem_kernel / jacobi_coop_kernel "
-                "FP32 sweeps, FP64 refinement sg_refine_kernel, level_out_kernel)",
+                "FP32 sweeps, FP64 refinement sge_kernel / sg_refine_kernel)",
              2: "other kernels (selection, PPT, phi, layout)"}
 
     # timed region: K steps (each a batch of circuits run concurrently); events around each

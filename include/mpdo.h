@@ -43,7 +43,9 @@ enum {
 };
 
 /* Arithmetic of the hot path.
- *  MPDO_FP64 : complex128 state, FP64 GEMMs and FP64 Jacobi eigensolves.
+ *  MPDO_FP64 : complex128 state, FP64 GEMMs, eigenpairs to FP64 accuracy (pivoted Cholesky
+ *              factors, FP32 sweeps with FP64 refinement; FP64 Jacobi where a factor falls
+ *              short).
  *  MPDO_C64  : complex64 state, FP32 GEMMs (FP32 accumulation), FP32 Jacobi;
  *              cutoff, PPT and trace renormalisation in FP64 scalars.  With
  *              mpdo_config.gram_fp64 = 1 the Grams and the small matrices are FP64.
@@ -332,7 +334,7 @@ int mpdo_build_qaoa_layer_cz(int n_sites, int k, double alpha, double beta, doub
  * rho as an MPS over the doubled index (s, s') (local dimension 9), complex128, mixed-canonical
  * in the Frobenius inner product.  Each two-site op (kind 2, its Kraus set as for mpdo_op) acts
  * as its superoperator on the pair; the pair is split by an SVD (eigenpairs of the Gram of the
- * updated pair, FP64 Jacobi) and cut to at most chi_max values above sv_cutoff (Schmidt values
+ * updated pair, to FP64 accuracy) and cut to at most chi_max values above sv_cutoff (Schmidt values
  * below sqrt(1e-15) of the largest are numerical zeros in any case).  use_ppt = 0 keeps the
  * largest values unchanged ("naive"); 1 replaces them by PPT's values with the trace
  * environment T_k of each Schmidt pair (from the trace contractions of the two sides), which
@@ -354,7 +356,8 @@ int mpdo_vmpo_expect_energy(mpdo_vmpo h, double J, double hx, double b, double* 
 int mpdo_vmpo_purity(mpdo_vmpo h, double* purity);
 int mpdo_vmpo_collision(mpdo_vmpo h, double* collision);
 /* Arithmetic of the vMPO updates.  mode 0 (default): FP64 products on the CUDA cores and
- * the FP64 Jacobi eigensolver.  mode 1 (the tensor-core form): products of at least 2^21
+ * eigenpairs from pivoted Cholesky factors and the graded solver (FP64 Jacobi where a factor
+ * falls short).  mode 1 (the tensor-core form): products of at least 2^21
  * complex multiply-adds as error-free BF16 slice products on the tensor cores summed in
  * FP64 (carried to ~2^-48 of each operand row's largest entry), and the Gram's eigenpairs
  * from the mixed-precision solver (FP32 Jacobi levels with FP64 refinement); its
@@ -372,7 +375,7 @@ int mpdo_vmpo_destroy(mpdo_vmpo h);
  *   recorded on its stream (bit 0: complex GEMMs, bit 1: eigensolver calls, bit 2: all
  *   other kernels); 0 switches timing off.  Resets the accumulators.
  * mpdo_profile_read: accumulated device milliseconds, launch count and algorithmic FLOPs
- *   (8 m n k per complex GEMM; for the eigensolver 8 x 3 x 16 x 16 x padded n per active
+ *   (8 m n k per complex GEMM; for the eigensolver 8 x 2 x 16 x 16 x padded n per active
  *   block-pair rotation round, the multiply-adds its block Jacobi executes; 0 for other
  *   kernels) of class cls since mpdo_profile. */
 long long mpdo_kernel_launches(void);

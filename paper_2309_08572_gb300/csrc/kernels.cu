@@ -1278,7 +1278,6 @@ cudaError_t lift(cudaStream_t st, int r, const cx<R>* z, const double* s, cx<R>*
   lift_kernel<R><<<nblocks((long)r * r), 256, 0, st>>>(r, z, s, zs);
   return cudaGetLastError();
 }
-template cudaError_t lift<double>(cudaStream_t, int, const double2*, const double*, double2*);
 template cudaError_t lift<float>(cudaStream_t, int, const float2*, const double*, float2*);
 
 #define INST(R)                                                                               \
