@@ -176,7 +176,7 @@ __device__ __forceinline__ void tc_tile(const CUtensorMap* ma, const CUtensorMap
   constexpr int BK = 128 / ELT;                      // elements per 128-byte k-block row
   constexpr uint32_t A_BYTES = BM * 128, B_BYTES = BN * 128;
   constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
-  constexpr uint32_t TMEM_COLS = BN < 32 ? 32 : BN;
+  constexpr uint32_t TMEM_COLS = BN <= 32 ? 32 : BN <= 64 ? 64 : BN <= 128 ? 128 : 256;
   extern __shared__ uint8_t smem_raw[];
   // tiles on a 1024-byte boundary (the 128-byte swizzle pattern repeats every 8 rows)
   uint8_t* smem = smem_raw + ((1024 - (su32(smem_raw) & 1023)) & 1023);
@@ -1208,12 +1208,25 @@ cudaError_t launch_bn(cudaStream_t st, const CUtensorMap& ma, const CUtensorMap&
 
 using namespace tc;
 
+// The tile width with the least time on the busiest SM: waves of tiles times a tile's time, which
+// is its columns and a fixed part (fill, narrow products' lower rate, epilogue) worth 64 of them;
+// the narrower of equals.  2304 x 4608 x 4608 (TF32x3 of a bond's new centre): 324 tiles of 256
+// columns need three waves of 152, and so do 432 of 192, each a quarter
+// shorter: the call takes 242 us instead of 290; 1500 x 1500 x 500 104 instead of 118, 297 x 1600 x
+// 200 54 instead of 66; sizes whose width stays take the same.
 int tc_pick_bn(long M, long N, int batch) {
   const long mt = (M + BM - 1) / BM;
-  const long t256 = mt * ((N + 255) / 256) * batch, t128 = mt * ((N + 127) / 128) * batch;
-  if (N > 128 && t256 >= 148) return 256;
-  if (N > 64 && t128 >= 74) return 128;
-  return 64;
+  int best = 64;
+  long cost = -1;
+  for (int bn : {64, 128, 192, 256}) {
+    if (bn > 64 && N <= bn / 2) break;
+    const long c = (mt * ((N + bn - 1) / bn) * batch + 151) / 152 * (bn + 64);
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = bn;
+    }
+  }
+  return best;
 }
 
 cudaError_t tc_gemm_real(cudaStream_t st, int elt, int M, int N, int K, const void* A, long lda,
@@ -1240,10 +1253,12 @@ cudaError_t tc_gemm_real(cudaStream_t st, int elt, int M, int N, int K, const vo
   ep.mode = e.d64 ? 1 : 0;
   if (elt == 4) {
     if (bn == 256) return launch_bn<4, 256, 4>(st, ma, mb, M, N, K, batch, ep, err);
+    if (bn == 192) return launch_bn<4, 192, 5>(st, ma, mb, M, N, K, batch, ep, err);
     if (bn == 128) return launch_bn<4, 128, 6>(st, ma, mb, M, N, K, batch, ep, err);
     return launch_bn<4, 64, 8>(st, ma, mb, M, N, K, batch, ep, err);
   }
   if (bn == 256) return launch_bn<2, 256, 4>(st, ma, mb, M, N, K, batch, ep, err);
+  if (bn == 192) return launch_bn<2, 192, 5>(st, ma, mb, M, N, K, batch, ep, err);
   if (bn == 128) return launch_bn<2, 128, 6>(st, ma, mb, M, N, K, batch, ep, err);
   return launch_bn<2, 64, 8>(st, ma, mb, M, N, K, batch, ep, err);
 }
@@ -1295,8 +1310,8 @@ cudaError_t mlp_launch(cudaStream_t st, MlpGroup<CAP>& g, int* err) {
   return cudaGetLastError();
 }
 }  // namespace
-// The tile width by the widest product and the tiles that it leaves the chip (tc_pick_bn's rule
-// over the whole group).
+// The widest tile that still gives half of the SMs one: a pass's products are short, and their
+// epilogues, which grow with the tile, are most of their time.
 template <int CAP>
 cudaError_t mlp_products(cudaStream_t st, MlpGroup<CAP>& g, int* err) {
   int maxn = 0;

@@ -35,8 +35,8 @@ struct TcEpilogue {
 
 // Real product D[b] = A[b] B[b]^T with A (M x K), B (N x K), both K-major, elements FP32
 // (read as TF32, elt = 4) or BF16 (elt = 2); leading dimensions and batch strides in
-// elements (multiples of 16 bytes; 16-byte aligned bases).  bn: output tile width (64, 128
-// or 256; <= 0 picks by size).  err: device int set non-zero when a pipeline wait gave up.
+// elements (multiples of 16 bytes; 16-byte aligned bases).  bn: output tile width (64, 128,
+// 192 or 256; <= 0 picks by size).  err: device int set non-zero when a pipeline wait gave up.
 cudaError_t tc_gemm_real(cudaStream_t st, int elt, int M, int N, int K, const void* A, long lda,
                          long sa, const void* B, long ldb, long sb, int batch, const TcEpilogue& e,
                          int* err, int bn);
