@@ -34,6 +34,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "exactplan.h"
 #include "internal.h"
 #include "tcgemm.h"
 
@@ -587,15 +588,17 @@ __global__ void __launch_bounds__(PT * 8)
 // B.  Bound by the tensor pipe and the accumulators' turn-around.  768 x 768 x 4096 Gram, this
 // kernel: 1150 us with every pair's operands loaded anew and an FP64 drain, 367 us with slices of K
 // and 64-column products, 313 us in equal ranges, 201 us with wide products.
-constexpr int XS = 6;          // slices per operand
-constexpr int XBN = 64;        // output tile width (real columns)
-constexpr int XKB = 32;        // K terms of a stage
+constexpr int XS = kExactSlices;
+constexpr int XBN = kExactCols;   // output tile width (real columns)
+constexpr int XKB = kExactK;      // K terms of a stage
+static_assert(BM == kExactRows, "the plan's tile");
 constexpr int XSTAGES = 3;
 constexpr int XDRAIN = 5;      // stages between drains
 constexpr int XTHREADS = 320;  // warp 0 TMA, warp 1 MMA, warps 2-9 drain
 constexpr int XA_SLICE = BM * XKB * 2, XB_SLICE = XBN * XKB * 2;
 constexpr int XSTAGE_BYTES = XS * (XA_SLICE + XB_SLICE);
-constexpr long XPART = BM * XBN;   // entries of a CTA's part of a tile: [column of 32][half, row]
+constexpr long XPART = kExactPart;   // a CTA's part of a tile: [column of 32][half, row]
+static_assert(kExactPartBytes == XPART * (long)sizeof(longlong2), "the plan's parts");
 constexpr int kNonFinite = 0x7fffffff;   // exponent of a row with a non-finite entry
 constexpr int kZeroRow = -1000000;       // and of a zero row (any smaller value)
 
@@ -1412,47 +1415,12 @@ cudaError_t tc_cgemm(cudaStream_t st, int mode, int opa, int opb, int m, int n, 
 
 // ---- exact products: C (complex FP64) = op(A) op(B), FP32 or FP64 complex A and B
 namespace {
-struct ExactPlan {
-  int tiles, nst, ctas;
-  long per, total;   // stages of a CTA, of all tiles of the batch
-  bool parts;        // ranges end within tiles
-};
-// How many stages a CTA takes: whole tiles, or an equal share of the stages (at least four) where
-// that is less on the busiest of the 152 SMs, counting 4 stages' time for a CTA's prologue and last
-// drain, one for a tile's output and 10 for the parts and the launch that adds them.
-ExactPlan exact_plan(long m, long n, long kc, int batch, bool gram) {
-  ExactPlan p;
-  const long mt = (m + BM - 1) / BM, nt = (2 * n + XBN - 1) / XBN;
-  long tiles = mt * nt;
-  if (gram) {
-    tiles = 0;
-    for (long i = 0; i < mt; ++i) tiles += nt - i * (BM / (XBN / 2));
-  }
-  p.tiles = (int)tiles;
-  p.nst = (int)((2 * kc + XKB - 1) / XKB);
-  p.total = tiles * batch * p.nst;
-  const long whole = (tiles * batch + 151) / 152;
-  const long ctas = std::min(152L, std::max(1L, p.total / 4));
-  const long share = (p.total + ctas - 1) / ctas;
-  p.parts = share + share / p.nst + 10 < whole * p.nst + whole;
-  p.per = p.parts ? share : whole * p.nst;
-  p.ctas = (int)((p.total + p.per - 1) / p.per);
-  return p;
-}
 // op(B) = op(A)^+ of the same data: the product is Hermitian
 template <typename TA, typename TB>
 bool is_gram(int opa, int opb, int m, int n, const TA* A, long lda, long sa, const TB* B, long ldb,
              long sb) {
   return std::is_same<TA, TB>::value && (const void*)A == (const void*)B && lda == ldb && sa == sb &&
          m == n && ((opa == OP_C && opb == OP_N) || (opa == OP_N && opb == OP_C));
-}
-size_t exact_bytes(long m, long n, long kc, int batch, bool gram) {
-  const long ldk = (2 * kc + XKB - 1) / XKB * XKB;
-  const size_t a = gram ? 0 : ((size_t)batch * m * XS * ldk * 2 + 255) & ~(size_t)255;
-  const size_t b = ((size_t)batch * 2 * n * XS * ldk * 2 + 255) & ~(size_t)255;
-  const ExactPlan p = exact_plan(m, n, kc, batch, gram);
-  const size_t part = p.parts ? (size_t)p.ctas * 2 * XPART * sizeof(longlong2) : 0;
-  return a + b + part + (((size_t)batch * (m + n) * sizeof(int) + 255) & ~(size_t)255) + 256;
 }
 }  // namespace
 
@@ -1470,7 +1438,7 @@ bool tc_exact_faster(long m, long n, long k, int batch, bool gram) {
 }
 
 size_t tc_exact_ws_bytes(long m, long n, long k, int batch) {
-  return exact_bytes(m, n, std::min<long>(k, 4096), batch, false);
+  return exact_ws_bytes(m, n, k, batch, false);
 }
 
 cudaError_t tc_exact_init() {
@@ -1487,10 +1455,8 @@ cudaError_t tc_cgemm_exact(cudaStream_t st, int opa, int opb, int m, int n, int 
   const bool gram = is_gram(opa, opb, m, n, A, lda, sa, B, ldb, sb);
   if (m <= 0 || n <= 0 || batch <= 0) return cudaSuccess;
   if (k <= 0) return cudaErrorInvalidValue;
-  long kc = k;
-  while (kc > 64 && exact_bytes(m, n, kc, batch, gram) > ws_bytes) kc = (kc + 1) / 2;
-  if (kc < k) kc = std::max(64L, kc / 64 * 64);
-  if (exact_bytes(m, n, kc, batch, gram) > ws_bytes) return cudaErrorMemoryAllocation;
+  const long kc = exact_piece(m, n, k, batch, gram, ws_bytes);
+  if (kc == 0) return cudaErrorMemoryAllocation;
   long sra, sca, srb, scb;
   int cja, cjb;
   op_strides(0, opa, lda, &sra, &sca, &cja);
@@ -1498,8 +1464,8 @@ cudaError_t tc_cgemm_exact(cudaStream_t st, int opa, int opb, int m, int n, int 
   MPDO_CUDA_TRY(tc_exact_init());
   for (long k0 = 0; k0 < k; k0 += kc) {
     const int kn = (int)std::min<long>(kc, k - k0);
-    const ExactPlan pl = exact_plan(m, n, kn, batch, gram);
-    const int ldk = (2 * kn + XKB - 1) / XKB * XKB;
+    const ExactPlan pl = exact_piece_plan(m, n, kn, batch, gram, ws_bytes);
+    const int ldk = (int)exact_ldk(kn);
     const long ldo = (long)XS * ldk;
     char* p = static_cast<char*>(ws);
     __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(p);
