@@ -77,11 +77,18 @@ inline long exact_piece(long m, long n, long k, int batch, bool gram, size_t ws)
     if (kc <= 64) return operands <= ws ? kc : 0;
   }
 }
-// Workspace with which a product of up to 4096 terms runs in one piece.
+// Workspace with which a product runs in pieces of up to 4096 terms, each with the parts it wants.
+// gram: as the product will be planned -- a Gram has half of the tiles, which may be too few to go
+// round whole and then takes up to 40 MB of parts where the general product of its size takes none
+// (768 columns, 1024 rows: four pieces in the general product's workspace, one in its own).
 inline size_t exact_ws_bytes(long m, long n, long k, int batch, bool gram) {
-  const long kc = std::min<long>(k, 4096);
-  return exact_operand_bytes(m, n, kc, batch, gram) +
-         exact_part_bytes(exact_plan(m, n, kc, batch, gram));
+  const long pieces = std::max(1L, (k + 4095) / 4096);
+  const long kc = pieces == 1 ? k : (k + 64 * pieces - 1) / (64 * pieces) * 64;
+  size_t ws = 0;
+  for (const long kn : {kc, k - (k - 1) / kc * kc})
+    ws = std::max(ws, exact_operand_bytes(m, n, kn, batch, gram) +
+                          exact_part_bytes(exact_plan(m, n, kn, batch, gram)));
+  return ws;
 }
 
 }  // namespace mpdo

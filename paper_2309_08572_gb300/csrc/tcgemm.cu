@@ -1437,9 +1437,6 @@ bool tc_exact_faster(long m, long n, long k, int batch, bool gram) {
   return tc < fp64;
 }
 
-size_t tc_exact_ws_bytes(long m, long n, long k, int batch) {
-  return exact_ws_bytes(m, n, k, batch, false);
-}
 
 cudaError_t tc_exact_init() {
   static const cudaError_t attr =
@@ -1704,7 +1701,8 @@ int mpdo_kernel_tcgemm_exact(int opa, int opb, int m, int n, int k, const void* 
       !b || !c)
     return tc_fail(MPDO_ERR_ARG, "bad tcgemm_exact arguments");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const size_t ws = mpdo::tc_exact_ws_bytes(m, n, k, batch);
+  const bool gram = mpdo::is_gram(opa, opb, m, n, a, lda, sa, b, ldb, sb);
+  const size_t ws = mpdo::exact_ws_bytes(m, n, k, batch, gram);
   Scratch w(st);
   if (!w.alloc(ws)) return tc_fail(MPDO_ERR_OOM, "tcgemm_exact workspace");
   cudaError_t ce = mpdo::tc_cgemm_exact<float2, float2>(

@@ -70,3 +70,15 @@ def test_pieces_fit(plan):
         rows.append((m, n, k, b, gram, rng.choice([0, 64 * MB, 256 * MB, log(MB // 4, 64 * MB)])))
     bad = [r for r, (ok, _) in zip(rows, plan(rows)) if not ok]
     assert not bad, (len(bad), bad[:10])
+
+
+def test_own_workspace_takes_one_piece(plan):
+    """With the workspace that the entry points ask for, pieces of up to 4096 terms."""
+    rng = random.Random(8)
+    rows = []
+    for _ in range(20000):
+        n, k = rng.randint(1, 900), int(round(10 ** rng.uniform(0, 4.5)))
+        gram = rng.randrange(2)
+        rows.append((n if gram else rng.randint(1, 900), n, k, rng.choice([1, 1, 3]), gram, 0))
+    bad = [r for r, (ok, p) in zip(rows, plan(rows)) if not ok or p > (r[2] + 4095) // 4096]
+    assert not bad, (len(bad), bad[:10])

@@ -40,3 +40,18 @@ def test_long_k(lib, m, n, k, batch, gram):
     a64, b64 = a.astype(np.complex128), b.astype(np.complex128)
     err = np.abs(c.cpu().numpy() - a64 @ b64) / (np.abs(a64) @ np.abs(b64))
     assert err.max() < 2.0 ** -40
+
+
+@pytest.mark.parametrize("n,k", [(768, 1024), (740, 900), (713, 1720), (423, 235)])
+def test_gram_in_one_piece(lib, n, k):
+    """A Gram whose plan wants parts where the general product's does not: exponents, packing (one
+    launch up to K = 256), the product and its parts, once."""
+    rng = np.random.default_rng(n)
+    t = torch.tensor(_rand(rng, (k, n)), device="cuda")
+    c = torch.zeros((n, n), dtype=torch.complex128, device="cuda")
+    before = lib.kernel_launches()
+    lib.kernel_tcgemm_exact(2, 0, n, n, k, t, n, 0, t, n, 0, c, n, 0, 1)
+    assert lib.kernel_launches() - before <= 4
+    a = t.cpu().numpy().astype(np.complex128)
+    err = np.abs(c.cpu().numpy() - a.conj().T @ a) / (np.abs(a).T @ np.abs(a))
+    assert err.max() < 2.0 ** -40
