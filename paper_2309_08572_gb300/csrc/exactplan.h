@@ -39,7 +39,7 @@ inline ExactPlan exact_plan(long m, long n, long kc, int batch, bool gram, bool 
   const long ctas = std::min(kExactSms, std::max(1L, p.total / 4));
   const long share = (p.total + ctas - 1) / ctas;
   p.parts = may_split && share + share / p.nst + 10 < whole * p.nst + whole;
-  p.per = p.parts ? share : whole * p.nst;
+  p.per = std::max(1L, p.parts ? share : whole * p.nst);   // 1: no tiles at all
   p.ctas = (int)((p.total + p.per - 1) / p.per);
   return p;
 }

@@ -28,7 +28,7 @@ int main() {
       const ExactPlan p = exact_piece_plan(m, n, kn, batch, gram, w);
       ok = ok && exact_operand_bytes(m, n, kn, batch, gram) + exact_part_bytes(p) <= w;
       ok = ok && p.ctas <= kExactSms && p.ctas * p.per >= p.total && (p.ctas - 1) * p.per < p.total;
-      ok = ok && (p.parts || p.per % p.nst == 0);
+      ok = ok && (p.parts || p.per % p.nst == 0 || p.total == 0);
     }
     std::printf("%d %ld\n", ok ? 1 : 0, pieces);
   }
@@ -82,3 +82,11 @@ def test_own_workspace_takes_one_piece(plan):
         rows.append((n if gram else rng.randint(1, 900), n, k, rng.choice([1, 1, 3]), gram, 0))
     bad = [r for r, (ok, p) in zip(rows, plan(rows)) if not ok or p > (r[2] + 4095) // 4096]
     assert not bad, (len(bad), bad[:10])
+
+
+def test_empty_products(plan):
+    """No rows, no columns or no batch: nothing to plan, and no division by a plan of nothing."""
+    rows = [(0, 5, 7, 1, 0, 0), (5, 0, 7, 1, 0, 0), (0, 0, 300, 2, 1, 0), (4, 4, 9, 0, 1, 0)]
+    for r in rows:
+        ((ok, _),) = plan([r])
+        assert ok, r
