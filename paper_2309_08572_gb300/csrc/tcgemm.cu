@@ -1490,7 +1490,7 @@ cudaError_t tc_cgemm_exact(cudaStream_t st, int opa, int opb, int m, int n, int 
     };
     const TA* a0 = A + k0 * sca;
     const TB* b0 = B + k0 * scb;
-    if (kn <= kFusedPackK) {
+    if (kn <= kFusedPackK && 2L * batch <= 65535) {   // the grid's z extent
       const PackOp ob{b0, pb, eb, srb, scb, sb, 2L * n * ldo, n, cjb, 1};
       const PackOp oa{a0, pa, ea, sra, sca, sa, (long)m * ldo, m, cja, 0};
       pack_both_kernel<TA, TB><<<dim3((std::max(gram ? 0 : m, n) + PR - 1) / PR, 1, gram ? batch : 2 * batch),

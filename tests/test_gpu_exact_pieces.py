@@ -55,3 +55,16 @@ def test_gram_in_one_piece(lib, n, k):
     a = t.cpu().numpy().astype(np.complex128)
     err = np.abs(c.cpu().numpy() - a.conj().T @ a) / (np.abs(a).T @ np.abs(a))
     assert err.max() < 2.0 ** -40
+
+
+def test_batch_of_40000(lib):
+    """More entries than half of a grid's z extent, which both operands of a short product share."""
+    rng = np.random.default_rng(5)
+    batch, m, n, k = 40000, 2, 2, 3
+    a, b = _rand(rng, (batch, m, k)), _rand(rng, (batch, k, n))
+    c = torch.full((batch, m, n), float("nan"), dtype=torch.complex128, device="cuda")
+    lib.kernel_tcgemm_exact(0, 0, m, n, k, torch.tensor(a, device="cuda"), k, m * k,
+                            torch.tensor(b, device="cuda"), n, k * n, c, n, m * n, batch)
+    a64, b64 = a.astype(np.complex128), b.astype(np.complex128)
+    err = np.abs(c.cpu().numpy() - a64 @ b64) / (np.abs(a64) @ np.abs(b64))
+    assert err.max() < 2.0 ** -40
