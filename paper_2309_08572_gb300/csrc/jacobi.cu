@@ -14,8 +14,8 @@
 // columns in two passes of 16 x np by the pairs' own CTAs, each waiting for its loads, took 92 us.
 // In the late sweeps few pairs have anything left to rotate: a sub-problem looks first, and a round
 // in which none had leaves out its tiles and second barrier.  The mixed solver's six levels at n =
-// 1350 (FP32 solves of 1350 down to 464): 1240 ms with the passes, 250 ms with tiles, 175 ms with
-// approximate rotations, the look ahead and items from a counter; FP64 at n = 400: 277 -> 92 ms.
+// 1350 (FP32 solves of 1350 down to 464): 1240 ms with the passes, 250 ms with tiles, ~190 ms with the
+// look ahead and items from a counter; FP64 at n = 400: 277 -> 92 ms.
 #include <cooperative_groups.h>
 #include <cuda.h>
 
@@ -95,28 +95,19 @@ __device__ __forceinline__ void copy8(T* dst, const T* src) {
     reinterpret_cast<float4*>(dst)[i] = reinterpret_cast<const float4*>(src)[i];
 }
 
-// Rotation of the pair (al, be) with coupling g of modulus ag: cosine and s e of the two columns.
-// FP32 from approximate roots and quotients (a chain of ~150 clocks on the sub-problem's critical
-// path, ~600 with the rounded ones): a rotation off by a few eps is one all the same, and the polar
-// step after the sub-problem takes out what it lacks in unitarity.
-__device__ __forceinline__ float modulus(float2 g) {
-  const float q = g.x * g.x + g.y * g.y;
-  return q > 0.f ? q * rsqrtf(q) : 0.f;
-}
-__device__ __forceinline__ double modulus(double2 g) { return sqrt(cabs2(g)); }
-__device__ __forceinline__ void rotation(float2 g, float ag, float al, float be, float& c, float2& o) {
-  const float inv = __fdividef(1.f, ag);
-  const float tau = fminf(fmaxf((be - al) * 0.5f * inv, -1e18f), 1e18f), q = 1.f + tau * tau;
-  const float t = copysignf(__fdividef(1.f, fabsf(tau) + q * rsqrtf(q)), tau);
-  c = rsqrtf(1.f + t * t);
-  o = cscale(g, inv * t * c);
-}
-__device__ __forceinline__ void rotation(double2 g, double ag, double al, double be, double& c,
-                                         double2& o) {
-  const double tau = (be - al) / (2 * ag);
-  const double t = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-  c = 1.0 / sqrt(1.0 + t * t);
-  o = cscale(mkc<double>(g.x / ag, g.y / ag), t * c);
+// Rotation of the pair (al, be) with coupling g of modulus ag: cosine and s e of the two columns,
+// from rounded roots and quotients.  In FP32 approximate ones (rsqrtf, __fdividef) shorten the chain
+// of a step from ~600 clocks to ~150 (n = 1350, mixed: 211 ms instead of 224), but their errors are
+// one-sided: over the ~1000 rounds of a solve the spectrum shrinks by 1e-5 (n = 400; 1.5e-6 here),
+// which the polar step after the sub-problem, itself rounded to FP32, does not see.
+template <typename R>
+__device__ __forceinline__ R modulus(cx<R> g) { return sqrt(cabs2(g)); }
+template <typename R>
+__device__ __forceinline__ void rotation(cx<R> g, R ag, R al, R be, R& c, cx<R>& o) {
+  const R tau = (be - al) / (2 * ag);
+  const R t = (tau >= 0 ? R(1) : R(-1)) / (fabs(tau) + sqrt(R(1) + tau * tau));
+  c = R(1) / sqrt(R(1) + t * t);
+  o = cscale(mkc<R>(g.x / ag, g.y / ag), t * c);
 }
 
 template <typename R>
@@ -191,7 +182,7 @@ __global__ void __launch_bounds__(JT, 2) jacobi_coop_kernel(int np, int nblk, cx
         U[0][i][j] = mkc<R>(i == j ? 1 : 0, 0);
         __syncthreads();
         // nothing to rotate, as in most pairs of the late sweeps: one look instead of 15 steps
-        const int live = __syncthreads_or(i < j && couples(modulus(S[0][i][j]), S[0][i][i].x, S[0][j][j].x));
+        const int live = __syncthreads_or(i < j && couples(modulus<R>(S[0][i][j]), S[0][i][i].x, S[0][j][j].x));
         for (int inner = 0; inner < (live ? kInnerSweeps : 0); ++inner) {
           int any_inner = 0;
           for (int st = 0; st < JS - 1; ++st) {
@@ -199,11 +190,11 @@ __global__ void __launch_bounds__(JT, 2) jacobi_coop_kernel(int np, int nblk, cx
             if (tid < JS / 2) {
               const int a = sa[st][tid], b = sb[st][tid];
               const T g = S[cur][a][b];
-              const R ag = modulus(g), al = S[cur][a][a].x, be = S[cur][b][b].x;
+              const R ag = modulus<R>(g), al = S[cur][a][a].x, be = S[cur][b][b].x;
               f = couples(ag, al, be);
               R c = 1;
               T o = mkc<R>(0, 0);
-              if (f) rotation(g, ag, al, be, c, o);
+              if (f) rotation<R>(g, ag, al, be, c, o);
               // columns: x_a <- c x_a - s conj(e) x_b, x_b <- s e x_a + c x_b
               rc[a] = rc[b] = c;
               ro[a] = mkc<R>(-o.x, o.y);
