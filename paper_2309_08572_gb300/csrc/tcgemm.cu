@@ -950,14 +950,16 @@ __device__ __forceinline__ long long to_fixed(double x, int e) {
                                   (ex ? ex : 1) - 1075 + 47 - e);
   return b < 0 ? -q : q;
 }
-// The XS slices of x: q = sum_t 2^(8 (XS - 1 - t)) d[t], d[t] in [-128, 127] for t > 0 and the
-// first in [-128, 128], so x = 2^-7 sum_t 2^-8t d[t] 2^e to 2^-48 2^e.
+// The XS slices of x: q = sum_t 2^(8 (XS - 1 - t)) d[t], |d[t]| <= 128, so x = 2^-7 sum_t 2^-8t d[t]
+// 2^e to 2^-48 2^e.  Halves go to the even neighbour: the digits of -x are those of x negated, and
+// what the dropped pairs leave out has no preferred sign (digits in [-128, 127], of mean -1/2, made
+// the error of a Gram of 500 rows 9 % larger).
 __device__ __forceinline__ void slice_all(long long q, float* d) {
 #pragma unroll
   for (int t = XS - 1; t > 0; --t) {
-    const int x = (int)((q + 128) & 255) - 128;
-    d[t] = (float)x;
-    q = (q - x) >> 8;
+    const long long r = (q + 127 + ((q >> 8) & 1)) >> 8;
+    d[t] = (float)(int)(q - r * 256);
+    q = r;
   }
   d[0] = (float)(int)q;
 }
