@@ -110,14 +110,14 @@ __device__ int block_min_int(int x, int* red) {
 __device__ int block_max_int(int x, int* red) { return -block_min_int(-x, red); }
 
 // Rayleigh-Ritz on one cluster C = [c0, c0 + c) of the final pass (all threads of the CTA):
-// its block of [S | G] gives the pencil (S_CC, G_CC); with P = I - (G_CC - I) / 2
-// (G_CC^-1/2 to first order) the Hermitian H = P^+ S_CC P is diagonalised by FP64 Jacobi
-// rotations, H = Q D Q^+.  IE, filled with I + E outside the cluster blocks, becomes
-// (I + E) B on the cluster's columns with B = P Q (its rows outside C carry their
-// corrections along the rotation), and lam[C] the eigenvalues, both in descending order.
-__device__ void ritz_cluster(int m, const double2* SG, int c0, int c, double* lam, double2* IE) {
+// its block of [S | G] gives the pencil (S_CC, G_CC); with P = I - D / 2 + 3 D^2 / 8, D = G_CC - I
+// (G_CC^-1/2 to second order), the Hermitian H = P^+ S_CC P is diagonalised by FP64 Jacobi
+// rotations, H = Q D Q^+.  lam[C] become the eigenvalues, descending, and the result points to B =
+// P Q in that order, in shared memory until the next call.
+typedef double2 RitzBlock[kRitzMax][kRitzMax + 1];
+__device__ RitzBlock* ritz_cluster(int m, const double2* SG, int c0, int c, double* lam) {
   __shared__ double2 Hs[kRitzMax][kRitzMax + 1];
-  __shared__ double2 Ps[kRitzMax][kRitzMax + 1];
+  __shared__ RitzBlock Ps;
   __shared__ double2 Qs[kRitzMax][kRitzMax + 1];
   __shared__ double rc[kRitzMax / 2], rs[kRitzMax / 2];
   __shared__ double2 rz[kRitzMax / 2];
@@ -138,6 +138,20 @@ __device__ void ritz_cluster(int m, const double2* SG, int c0, int c, double* la
     Hs[a][b] = sv;
     Ps[a][b] = pv;
   }
+  __syncthreads();
+  for (int e = tid; e < c * c; e += nt) {   // P1 = I - D / 2, P = P1 + 3 (I - P1)^2 / 2
+    const int a = e / c, b = e % c;
+    double2 acc = make_double2(0.0, 0.0);
+    for (int k = 0; k < c; ++k) {
+      double2 x = Ps[a][k], y = Ps[k][b];
+      if (a == k) x.x -= 1.0;
+      if (k == b) y.x -= 1.0;
+      cfma(acc, x, y);
+    }
+    Qs[a][b] = cadd(Ps[a][b], cscale(acc, 1.5));
+  }
+  __syncthreads();
+  for (int e = tid; e < c * c; e += nt) Ps[e / c][e % c] = Qs[e / c][e % c];
   __syncthreads();
   for (int e = tid; e < c * c; e += nt) {   // Qs = S_CC P
     const int a = e / c, b = e % c;
@@ -263,8 +277,14 @@ __device__ void ritz_cluster(int m, const double2* SG, int c0, int c, double* la
   for (int e = tid; e < c * c; e += nt, ++nb) Ps[e / c][e % c] = bv[nb];
   for (int b = tid; b < c; b += nt) lam[c0 + b] = Hs[s_perm[b]][s_perm[b]].x;
   __syncthreads();
-  // IE[:, C] <- IE[:, C] B: the cluster's own block is the identity there, i.e. B itself
-  for (int i = tid; i < m; i += nt) {
+  return &Ps;
+}
+
+// IE, filled with I + E outside the cluster blocks, becomes (I + E) B on the cluster's columns (its
+// rows outside C carry their corrections along the rotation).
+__device__ void ritz_apply(int m, const double2* SG, int c0, int c, double* lam, double2* IE) {
+  const RitzBlock& Ps = *ritz_cluster(m, SG, c0, c, lam);
+  for (int i = threadIdx.x; i < m; i += blockDim.x) {
     double2* row = IE + (long)i * m + c0;
     if (i >= c0 && i < c0 + c) {
       for (int b = 0; b < c; ++b) row[b] = Ps[i - c0][b];
@@ -447,7 +467,7 @@ __device__ void refine_step(int m, int n, const double2* SG, int level0, int lev
     fill_ie(m, SG, lam, IE, nl, fsep, emax, cid, tid, nt);
     __syncthreads();
     const int ncl = s_ncl;
-    for (int q = 0; q < ncl; ++q) ritz_cluster(m, SG, s_cl0[q], s_cln[q], lam, IE);
+    for (int q = 0; q < ncl; ++q) ritz_apply(m, SG, s_cl0[q], s_cln[q], lam, IE);
     double mx2 = -1e300;
     for (int i = tid; i < m; i += nt) mx2 = fmax(mx2, lam[i]);
     vf = block_max(mx2, red);
@@ -553,7 +573,7 @@ __global__ void __launch_bounds__(256) refine_ritz_kernel(int m, const double2* 
   if (cid[c0] != c0) return;
   int c = 1;
   while (c0 + c < m && cid[c0 + c] == c0) ++c;
-  ritz_cluster(m, SG, c0, c, lam, IE);
+  ritz_apply(m, SG, c0, c, lam, IE);
 }
 __global__ void __launch_bounds__(256) refine_end_kernel(int m, int level, double floor,
                                                          const int* rot, const double* lam,
@@ -570,46 +590,284 @@ __global__ void __launch_bounds__(256) refine_end_kernel(int m, int level, doubl
 //
 // For a graded matrix (see heig_graded_f32) the mixing of a pair is measured relative to its
 // sizes: with lam_i > lam_j the FP32 sweeps leave S_ij ~ delta sqrt(lam_i lam_j) and G_ij ~
-// delta sqrt(lam_j / lam_i), so the correction E is graded as well and a pair is separated when
-// |S_ij - lam G_ij| sqrt(lam_i / lam_j) < emax |lam_i - lam_j| and its relative gap exceeds the
+// delta sqrt(lam_j / lam_i), so the correction E is graded as well and a pair's angle is
+// |S_ij - lam G_ij| sqrt(lam_i / lam_j) / |lam_i - lam_j|, known where its relative gap exceeds the
 // rounding of the products (100 m eps_64).  No pair is left to another level.  A corrected pair
-// keeps about the square of its angle, so in the final pass neighbours whose angle is above
-// kGradedRitz (relative gaps below ~1e-3) go to the Ritz step, which is exact within its run.
+// keeps about the square of its angle, in its coupling and in the columns' norms, so the first pass
+// corrects angles below kGradedNewton only, and in the last pass pairs above kGradedRitz, mostly those
+// left over (relative gaps below ~1e-3), go to a Ritz step over the whole run of columns that such
+// pairs connect, which is exact within the run, however long (settle_runs).  What remains is the square
+// of the last corrections: 1e-12 at the most, 1e-14 as a rule.  (With corrections up to 1e-2,
+// first-order norms and runs cut after 16 columns it was 1e-8, 2e-6 between columns of longer runs.)
 //
 // The step is bound by FP64: a pair costs two dot products of length m and one division.  So
 // one CTA takes a 4 x 4 block of pairs above the diagonal, forms its S, G and the diagonal
 // entries it needs (48 dot products on 96 threads, halves of the sum over k) and writes its
 // part of I + E: 120 CTAs at m = 60, where a 16 x 16 tiling would use 30 SMs and leave the
 // elementwise step to one.  In the final pass the last CTA to finish (a ticket; nobody waits)
-// settles runs of unseparated neighbours by Rayleigh-Ritz, 16 at a time.
+// settles the runs.
 //
 // scaled: column j of I + E, and so eigenvector j, comes out times lam_j^-1/2 (0 for lam_j <= 0),
 // the factor that lifts an eigenvector of L^+ L to one of L L^+.
 constexpr int GT = 4;
 constexpr int kSgeThreads = 128;
+constexpr double kGradedNewton = 1e-3;
 constexpr double kGradedRitz = 1e-6;
 __device__ __forceinline__ double col_scale(double lam, int scaled) {
   return !scaled ? 1.0 : lam > 0.0 ? rsqrt(lam) : 0.0;
 }
-// columns [c0, c0 + c) of IE times lam^-1/2, or (undo) divided by it; all threads of the CTA
-__device__ void scale_cols(int m, int c0, int c, const double* lam, double2* IE, bool undo) {
-  for (int e = threadIdx.x; e < m * c; e += blockDim.x) {
-    const int col = c0 + e % c;
-    const double l = __ldcg(&lam[col]), f = undo ? sqrt(fmax(l, 0.0)) : col_scale(l, 1);
-    double2* x = &IE[(long)(e / c) * m + col];
-    *x = cscale(__ldcg(x), f);
+
+// ritz_cluster for a run of any length up to kGradedMax, its matrices in global memory (P, X and H,
+// m x m each), B into the run's block of IE: spectra with that many values within 1e-3 of one another
+// are rare, and one CTA takes about 3 ms for 40 columns, the FP64 operations of ~8 sweeps on its SM.
+__device__ __noinline__ void ritz_run(int m, const double2* SG, int c0, int c, double* lam,
+                                      double2* IE, double2* P, double2* X, double2* H) {
+  __shared__ double rc[kGradedMax / 2], rs[kGradedMax / 2], s_lam[kGradedMax];
+  __shared__ double2 rz[kGradedMax / 2];
+  __shared__ short rp[kGradedMax / 2], rq[kGradedMax / 2], s_perm[kGradedMax];
+  __shared__ int rf[kGradedMax / 2];
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const long ld = 2L * m;
+  const int cp = c + (c & 1), half = cp / 2;
+  auto sg = [&](int a, int b) { return __ldcg(&SG[(long)(c0 + a) * ld + c0 + b]); };
+  auto dg = [&](int a, int b) {   // G_CC - I
+    double2 g = __ldcg(&SG[(long)(c0 + a) * ld + m + c0 + b]);
+    if (a == b) g.x -= 1.0;
+    return g;
+  };
+  for (int e = tid; e < c * c; e += nt) {   // P = G_CC^-1/2 to second order
+    const int a = e / c, b = e % c;
+    const double2 d = dg(a, b);
+    double2 d2 = make_double2(0.0, 0.0);
+    for (int k = 0; k < c; ++k) cfma(d2, dg(a, k), dg(k, b));
+    P[e] = make_double2((a == b ? 1.0 : 0.0) - 0.5 * d.x + 0.375 * d2.x, -0.5 * d.y + 0.375 * d2.y);
   }
   __syncthreads();
+  for (int e = tid; e < c * c; e += nt) {   // X = S_CC P
+    const int a = e / c, b = e % c;
+    double2 acc = make_double2(0.0, 0.0);
+    for (int k = 0; k < c; ++k) cfma(acc, sg(a, k), P[k * c + b]);
+    X[e] = acc;
+  }
+  __syncthreads();
+  for (int e = tid; e < c * c; e += nt) {   // H = P^+ X, its upper half and the mirror image
+    const int a = e / c, b = e % c;
+    if (a > b) continue;
+    double2 acc = make_double2(0.0, 0.0);
+    for (int k = 0; k < c; ++k) cfma(acc, cconj(P[k * c + a]), X[k * c + b]);
+    if (a == b) acc.y = 0.0;
+    H[a * c + b] = acc;
+    H[b * c + a] = cconj(acc);
+  }
+  __syncthreads();
+  for (int e = tid; e < c * c; e += nt) X[e] = make_double2(e / c == e % c ? 1.0 : 0.0, 0.0);
+  double tr = 0.0;
+  for (int a = 0; a < c; ++a) tr += fabs(H[a * c + a].x);
+  const double atol = 1e-18 * tr;
+  __syncthreads();
+  for (int sweep = 0; sweep < 16; ++sweep) {
+    int any = 0;
+    for (int r = 0; r < cp - 1; ++r) {
+      int f = 0;
+      if (tid < half) {
+        int p, q;
+        tourney(r, tid, cp, p, q);
+        if (p > q) { const int t = p; p = q; q = t; }
+        rp[tid] = (short)p;
+        rq[tid] = (short)q;
+        if (q < c) {   // an odd run's last seat is empty
+          const double2 g = H[p * c + q];
+          const double ag = sqrt(cabs2(g)), al = H[p * c + p].x, be = H[q * c + q].x;
+          f = (ag > atol) && (ag > 1e-15 * sqrt(fabs(al * be)));
+          if (f) {
+            const double tau = (be - al) / (2.0 * ag);
+            const double t = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
+            const double cc = 1.0 / sqrt(1.0 + t * t);
+            rc[tid] = cc;
+            rs[tid] = t * cc;
+            rz[tid] = make_double2(g.x / ag, g.y / ag);
+          }
+        }
+        rf[tid] = f;
+      }
+      if (!__syncthreads_or(f)) continue;
+      any = 1;
+      // 2 x 2 blocks of H' = J^+ H J (rows of pair a, columns of pair b); X's columns with pair b
+      for (int e = tid; e < half * half; e += nt) {
+        const int ka = e / half, kb = e - ka * half;
+        const int fa = rf[ka], fb = rf[kb];
+        if (!fa && !fb) continue;
+        const int pa = rp[ka], qa = rq[ka], pb = rp[kb], qb = rq[kb];
+        const bool ha = qa < c, hb = qb < c;
+        const double ca = fa ? rc[ka] : 1.0, sa = fa ? rs[ka] : 0.0;
+        const double cb = fb ? rc[kb] : 1.0, sb = fb ? rs[kb] : 0.0;
+        const double2 ea = fa ? rz[ka] : make_double2(1.0, 0.0);
+        const double2 eb = fb ? rz[kb] : make_double2(1.0, 0.0);
+        const double2 z = make_double2(0.0, 0.0);
+        const double2 x0 = H[pa * c + pb], x1 = hb ? H[pa * c + qb] : z;
+        const double2 y0 = ha ? H[qa * c + pb] : z, y1 = ha && hb ? H[qa * c + qb] : z;
+        const double2 u0 = csub(cscale(x0, ca), cscale(cmul(ea, y0), sa));
+        const double2 u1 = csub(cscale(x1, ca), cscale(cmul(ea, y1), sa));
+        const double2 w0 = cadd(cscale(cmulc(x0, ea), sa), cscale(y0, ca));
+        const double2 w1 = cadd(cscale(cmulc(x1, ea), sa), cscale(y1, ca));
+        H[pa * c + pb] = csub(cscale(u0, cb), cscale(cmulc(u1, eb), sb));
+        if (hb) H[pa * c + qb] = cadd(cscale(cmul(u0, eb), sb), cscale(u1, cb));
+        if (ha) H[qa * c + pb] = csub(cscale(w0, cb), cscale(cmulc(w1, eb), sb));
+        if (ha && hb) H[qa * c + qb] = cadd(cscale(cmul(w0, eb), sb), cscale(w1, cb));
+      }
+      for (int e = tid; e < c * half; e += nt) {
+        const int i = e / half, kb = e - i * half;
+        if (!rf[kb]) continue;
+        const int p = rp[kb], q = rq[kb];
+        const double cc = rc[kb], sn = rs[kb];
+        const double2 ee = rz[kb], x = X[i * c + p], y = X[i * c + q];
+        X[i * c + p] = csub(cscale(x, cc), cscale(cmulc(y, ee), sn));
+        X[i * c + q] = cadd(cscale(cmul(x, ee), sn), cscale(y, cc));
+      }
+      __syncthreads();
+    }
+    if (!any) break;
+  }
+  for (int a = tid; a < c; a += nt) {
+    s_lam[a] = H[a * c + a].x;
+    s_perm[a] = (short)a;   // valid whatever the values (NaN: ranks collide)
+  }
+  __syncthreads();
+  for (int a = tid; a < c; a += nt) {
+    int rank = 0;
+    for (int k = 0; k < c; ++k) rank += s_lam[k] > s_lam[a] || (!(s_lam[k] < s_lam[a]) && k < a);
+    s_perm[rank < c ? rank : c - 1] = (short)a;
+  }
+  __syncthreads();
+  for (int e = tid; e < c * c; e += nt) {   // B = P X with its columns sorted
+    const int a = e / c, b = e % c, col = s_perm[b];
+    double2 acc = make_double2(0.0, 0.0);
+    for (int k = 0; k < c; ++k) cfma(acc, P[a * c + k], X[k * c + col]);
+    IE[(long)(c0 + a) * m + c0 + b] = acc;
+  }
+  for (int b = tid; b < c; b += nt) lam[c0 + b] = s_lam[s_perm[b]];
+  __syncthreads();
 }
+
+// First-order correction of a pair of columns (E_ij, E_ji) from S_ij, G_ij and their values.
+struct Corr {
+  double2 ij, ji;
+};
+__device__ __forceinline__ double2 pair_residual(double2 s, double2 g, double l, bool conj) {
+  const double2 n = make_double2(s.x - l * g.x, s.y - l * g.y);
+  return conj ? cconj(n) : n;
+}
+// The squared angle is num / den (den not positive: none); kept below emax where apart.
+__device__ __forceinline__ bool pair_correction(int m, double2 s, double2 g, double li, double lj,
+                                                double emax, Corr& e) {
+  const double d = lj - li, mx = fmax(fabs(li), fabs(lj)), mn = fmin(li, lj);
+  const double2 nij = pair_residual(s, g, lj, false), nji = pair_residual(s, g, li, true);
+  const double lim = d * d * mn, ang = fmax(cabs2(nij), cabs2(nji)) * mx;   // ang / lim: angle^2
+  const bool apart = mn > 0.0 && fabs(d) > 100.0 * m * 1.1e-16 * mx;
+  if (apart && ang < emax * emax * lim) {
+    const double r = 1.0 / d;
+    e.ij = cscale(nij, r);
+    e.ji = cscale(nji, -r);
+    return true;
+  }
+  e.ij = cscale(g, -0.5);
+  e.ji = cscale(cconj(g), -0.5);
+  return false;
+}
+
+// The last pass's runs, by one CTA.  A run's columns are rotated to its Ritz vectors first -- B, in the
+// run's block of IE, and the rows and columns of S and G that cross the run -- and the corrections
+// between them and all other columns formed from those: corrections of the unrotated columns, carried
+// along the rotation, would miss the product of the rotation's angle and their own.  With E in that
+// basis, I + E becomes (I + E) on rows outside runs, and B (E, or I in its own block) on a run's rows.
+__device__ void settle_runs(int m, double2* SG, double* lam, double2* IE, const int* s_reach,
+                            int scaled, double2* wp, double2* wxh) {
+  __shared__ double s_cs[kGradedMax];          // columns' scales
+  __shared__ unsigned char s_in[kGradedMax];   // in a run
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const long ld = 2L * m;
+  auto each = [&](auto&& f) {
+    for (int i = 0; i < m;) {
+      int j = s_reach[i];
+      for (int k = i + 1; k <= j; ++k) j = max(j, s_reach[k]);   // run [i, j]
+      if (j > i) f(i, j - i + 1);
+      i = j + 1;
+    }
+  };
+  for (int i = tid; i < m; i += nt) s_in[i] = 0;
+  __syncthreads();
+  each([&](int c0, int c) {
+    for (int i = tid; i < c; i += nt) s_in[c0 + i] = 1;
+    if (c <= kRitzMax) {
+      const RitzBlock& B = *ritz_cluster(m, SG, c0, c, lam);
+      for (int e = tid; e < c * c; e += nt) IE[(long)(c0 + e / c) * m + c0 + e % c] = B[e / c][e % c];
+      __syncthreads();
+    } else {
+      ritz_run(m, SG, c0, c, lam, IE, wp, wxh, wxh + (long)m * m);
+    }
+    // S[j, C] <- S[j, C] B and G likewise, from their mirror images, then these
+    for (int e = tid; e < (m - c) * c; e += nt) {
+      const int b = e % c, o = e / c, j = o < c0 ? o : o + c;
+      double2 sv = make_double2(0.0, 0.0), gv = sv;
+      for (int k = 0; k < c; ++k) {
+        const double2 x = IE[(long)(c0 + k) * m + c0 + b];
+        cfma(sv, cconj(__ldcg(&SG[(c0 + k) * ld + j])), x);
+        cfma(gv, cconj(__ldcg(&SG[(c0 + k) * ld + m + j])), x);
+      }
+      SG[j * ld + c0 + b] = sv;
+      SG[j * ld + m + c0 + b] = gv;
+    }
+    __syncthreads();
+    for (int e = tid; e < (m - c) * c; e += nt) {
+      const int b = e % c, o = e / c, j = o < c0 ? o : o + c;
+      SG[(c0 + b) * ld + j] = cconj(SG[j * ld + c0 + b]);
+      SG[(c0 + b) * ld + m + j] = cconj(SG[j * ld + m + c0 + b]);
+    }
+    __syncthreads();
+  });
+  for (int i = tid; i < m; i += nt) s_cs[i] = col_scale(__ldcg(&lam[i]), scaled);
+  __syncthreads();
+  each([&](int c0, int c) {
+    for (int e = tid; e < (m - c) * c; e += nt) {
+      const int o = e / c, j = o < c0 ? o : o + c, b = c0 + e % c;
+      if (j < c0 && s_in[j]) continue;   // an earlier run wrote the pair
+      Corr x;
+      pair_correction(m, __ldcg(&SG[j * ld + b]), __ldcg(&SG[j * ld + m + b]), __ldcg(&lam[j]),
+                      __ldcg(&lam[b]), kNewtonFinal, x);
+      IE[(long)j * m + b] = s_in[j] ? x.ij : cscale(x.ij, s_cs[b]);
+      IE[(long)b * m + j] = x.ji;
+    }
+  });
+  __syncthreads();
+  each([&](int c0, int c) {   // IE[C, j] <- B IE[C, j], through S
+    for (int e = tid; e < (m - c) * c; e += nt) {
+      const int o = e % (m - c), j = o < c0 ? o : o + c, a = c0 + e / (m - c);
+      double2 acc = make_double2(0.0, 0.0);
+      for (int k = 0; k < c; ++k) cfma(acc, IE[(long)a * m + c0 + k], IE[(long)(c0 + k) * m + j]);
+      SG[a * ld + j] = cscale(acc, s_cs[j]);
+    }
+  });
+  __syncthreads();
+  each([&](int c0, int c) {
+    for (int e = tid; e < m * c; e += nt) {
+      const int j = e % m, a = c0 + e / m;
+      double2* x = &IE[(long)a * m + j];
+      *x = j >= c0 && j < c0 + c ? cscale(*x, s_cs[j]) : SG[a * ld + j];
+    }
+  });
+}
+
+// reach[i]: the last column that pair (i, .) above kGradedRitz reaches (i if none)
 __global__ void __launch_bounds__(kSgeThreads) sge_kernel(int m, const double2* __restrict__ TZ,
-                                                          double2* SG, int final_pass,
-                                                          double emax, double* lam, double2* IE,
-                                                          unsigned char* sep, unsigned int* ticket,
-                                                          int scaled) {
+                                                          double2* SG, int final_pass, double* lam,
+                                                          double2* IE, int* reach,
+                                                          unsigned int* ticket, int scaled,
+                                                          double2* wp, double2* wxh) {
   extern __shared__ double2 sge_col[];   // [k][16]: Z_I, Z_J, T_I, T_J
   __shared__ double2 part[48];
   __shared__ double2 val[48];            // S, G (16 each), then S_ii, G_ii, S_jj, G_jj (4 each)
   __shared__ int s_last;
+  __shared__ int s_reach[kGradedMax];
   const int tid = threadIdx.x;
   const long ld = 2L * m;
   const int nt = (m + GT - 1) / GT;
@@ -654,29 +912,22 @@ __global__ void __launch_bounds__(kSgeThreads) sge_kernel(int m, const double2* 
     const double ci = col_scale(li, scaled), cj = col_scale(lj, scaled);
     if (i == j && i < m) {
       lam[i] = li;
-      IE[(long)i * m + i] = make_double2(ci * (1.0 + 0.5 * (1.0 - gi)), 0.0);
+      const double t = gi - 1.0;   // gi^-1/2 to second order
+      IE[(long)i * m + i] = make_double2(ci * fma(t, fma(0.375, t, -0.5), 1.0), 0.0);
       SG[i * ld + i] = s;
       SG[i * ld + m + i] = g;
+      if (!final_pass) reach[i] = i;
     } else if (i < j && j < m) {
       SG[i * ld + j] = s;
       SG[i * ld + m + j] = g;
       SG[j * ld + i] = cconj(s);
       SG[j * ld + m + i] = cconj(g);
-      const double d = lj - li, mx = fmax(fabs(li), fabs(lj)), mn = fmin(li, lj);
-      const double2 nij = make_double2(s.x - lj * g.x, s.y - lj * g.y);
-      const double2 nji = make_double2(s.x - li * g.x, -(s.y - li * g.y));
-      const double lim = d * d * mn, ang = fmax(cabs2(nij), cabs2(nji)) * mx;   // ang / lim: angle^2
-      const bool apart = mn > 0.0 && fabs(d) > 100.0 * m * 1.1e-16 * mx;
-      const bool newton = apart && ang < emax * emax * lim;
-      if (newton) {
-        const double r = 1.0 / d;
-        IE[(long)i * m + j] = cscale(nij, r * cj);
-        IE[(long)j * m + i] = cscale(nji, -r * ci);
-      } else {
-        IE[(long)i * m + j] = cscale(g, -0.5 * cj);
-        IE[(long)j * m + i] = cscale(cconj(g), -0.5 * ci);
-      }
-      if (j == i + 1) sep[i] = apart && ang < kGradedRitz * kGradedRitz * lim;
+      Corr x;
+      const bool kept = pair_correction(m, s, g, li, lj, final_pass ? kGradedRitz : kGradedNewton, x);
+      IE[(long)i * m + j] = cscale(x.ij, cj);
+      IE[(long)j * m + i] = cscale(x.ji, ci);
+      // a value that is not positive has no angle with the others: neighbours only
+      if (final_pass && !kept && (!(fmin(li, lj) <= 0.0) || j == i + 1)) atomicMax(&reach[i], j);
     }
   }
   if (!final_pass) return;
@@ -687,24 +938,13 @@ __global__ void __launch_bounds__(kSgeThreads) sge_kernel(int m, const double2* 
   if (!s_last) return;
   __threadfence();
   if (tid == 0) *ticket = 0u;
-  unsigned char* flags = reinterpret_cast<unsigned char*>(sge_col);
   int open = 0;
-  for (int i = tid; i + 1 < m; i += kSgeThreads) {
-    flags[i] = __ldcg(&sep[i]);
-    open |= !flags[i];
+  for (int i = tid; i < m; i += kSgeThreads) {
+    s_reach[i] = __ldcg(&reach[i]);
+    open |= s_reach[i] > i;
   }
   if (!__syncthreads_or(open)) return;
-  for (int i = 0; i + 1 < m;) {
-    int j = i;
-    while (j + 1 < m && !flags[j] && j - i + 1 < kRitzMax) ++j;   // run [i, j]
-    if (j > i) {
-      // the Ritz step works on unscaled columns and sets the run's eigenvalues
-      if (scaled) scale_cols(m, i, j - i + 1, lam, IE, true);
-      ritz_cluster(m, SG, i, j - i + 1, lam, IE);
-      if (scaled) scale_cols(m, i, j - i + 1, lam, IE, false);
-    }
-    i = j + 1;
-  }
+  settle_runs(m, SG, lam, IE, s_reach, scaled, wp, wxh);
 }
 
 // K slices of a small FP64 product: enough to bring the CTAs towards one per SM, each
@@ -1142,9 +1382,9 @@ cudaError_t heig_graded(cudaStream_t st, int n, const double2* a, long lda, doub
   for (int pass = 0; pass < 2; ++pass) {
     const int fin = pass == 1;
     count_launch();
-    sge_kernel<<<grid, kSgeThreads, sm, st>>>(n, cur, wk.s, fin, fin ? kNewtonFinal : kNewtonMax,
-                                              fin ? w : wk.lam, wk.ie, wk.sepf, wk.ticket,
-                                              fin && scaled ? 1 : 0);
+    // a long run's matrices: the next basis' place and the levels' one
+    sge_kernel<<<grid, kSgeThreads, sm, st>>>(n, cur, wk.s, fin, fin ? w : wk.lam, wk.ie, wk.cid,
+                                              wk.ticket, fin && scaled ? 1 : 0, wk.x, nxt);
     MPDO_CUDA_TRY(cudaGetLastError());
     if (fin) {
       MPDO_CUDA_TRY(mul(cur + n, l2, 0, wk.ie, n, z, ldz, 0, 1));
