@@ -402,15 +402,18 @@ int reverse(mpdo_vmpo h) {
 
 // Eigenpairs of the Gram in h->H (n x n): *nval eigenvalues in h->lam, descending, and *nvec
 // eigenvectors in the columns of h->U (row stride *nvec).  Through the pivoted Cholesky factor
-// H ~ L L^+, stopping at a hundredth of the cut, and the graded solver on L^+ L, as in the MPDO
-// update; a rank beyond the solver's size takes the full solve: FP64 Jacobi, or in the
-// tensor-core form the mixed solver, resolved below a tenth of the cut.  (Eight sites at chi 16,
-// n = 144: the FP64 Jacobi took 28 ms a solve.)  One host synchronisation.
+// H ~ L L^+ and the graded solver on L^+ L, as in the MPDO update; a rank beyond the solver's size
+// takes the full solve: FP64 Jacobi, or in the tensor-core form the mixed solver, resolved below a
+// tenth of the cut.  (Eight sites at chi 16, n = 144: the FP64 Jacobi took 28 ms a solve.)  The factor
+// goes down to the rounding of H whatever the cut: what it leaves below its last pivot sums over up to
+// n rows and turns the kept pairs, whose values and T_k enter the result one by one (stopping at a
+// hundredth of the cut: energies off by 3e-4 at a cut of 1e-2, 1e-8 at 1e-4).  One host
+// synchronisation.
 int split(mpdo_vmpo h, int n, int* nval, int* nvec) {
   cudaStream_t st = h->st;
   if (n <= 1024) {
     const int rmax = std::min(n, kGradedMax);
-    const double tol = std::max(0.01 * h->cut2, 1e-16);
+    const double tol = h->tc ? 1e-15 : 1e-16;
     VK(pchol<double>(st, n, h->H, rmax, tol, h->L, kGradedMax, &h->dpc->r, &h->dpc->resid));
     VK(cudaMemcpyAsync(h->hpc, h->dpc, sizeof(*h->hpc), cudaMemcpyDeviceToHost, st));
     VK(cudaStreamSynchronize(st));
