@@ -430,7 +430,8 @@ int mpdo_kernel_heig_graded(int n, const void* a, void* v, double* w, void* stre
  * w ~ L L^+, L n x *rank with row stride ldl >= min(n, rmax), columns by the largest remaining
  * diagonal (piv: device int[min(n, rmax)], may be NULL) until that is <= tol * tr w or after rmax
  * columns; *resid = largest remaining diagonal / tr w.  n in 1..1024, rmax in
- * 1..MPDO_HEIG_GRADED_NMAX.  Synchronises the stream. */
+ * 1..MPDO_HEIG_GRADED_NMAX.  Synchronises the stream.  MPDO_ERR_TIMEOUT when a wait inside the
+ * kernel gave up (updates then solve the full problem). */
 int mpdo_kernel_pchol(int n, const void* w, int rmax, double tol, void* L, int ldl, int* piv,
                       int* rank, double* resid, void* stream);
 

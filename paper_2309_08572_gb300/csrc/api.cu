@@ -118,10 +118,9 @@ struct mpdo_ctx {
   bool block_sync = false;
   // eigenproblems through a pivoted Cholesky factor (see lift_eig)
   void *wGs = nullptr, *wZ = nullptr, *wLg = nullptr;
-  struct PcOut { int r; int pad; double resid; };
-  PcOut* dpc = nullptr;
+  PcholOut* dpc = nullptr;
   int* dpiv = nullptr;        // pivots of the left Gram's factor
-  PcOut* hpc = nullptr;       // pinned
+  PcholOut* hpc = nullptr;    // pinned
   MixWork mixw;              // mixed-precision eigensolver workspace (mixed only)
   void* mixmem = nullptr;
   size_t eltm = 16;          // bytes per complex of the Gram-derived matrices
@@ -413,7 +412,8 @@ constexpr int kInnerRmax = kGradedMax;   // columns of a factor (FP64)
 constexpr int kInnerRmaxF32 = 128;         // and of the FP32 factor
 
 // Pivoted Cholesky factor g ~ L L^+ (n x n, into wLg) stopping at tol * tr g, its pivots to piv:
-// *rank columns, or 0 when it needs more than rmax of them.  One host synchronisation.
+// *rank columns, or 0 when it needs more than rmax of them or the kernel gave up waiting.  One host
+// synchronisation.
 template <typename RM>
 int factor(mpdo_ctx* h, int n, const cx<RM>* g, double tol, int rmax, int* piv, int* rank,
            bool* zero) {
@@ -425,12 +425,12 @@ int factor(mpdo_ctx* h, int n, const cx<RM>* g, double tol, int rmax, int* piv, 
   CK(pchol<RM>(h->st, n, g, rmax, tol, static_cast<cx<RM>*>(h->wLg), kInnerRmax, &h->dpc->r,
                &h->dpc->resid, piv));
   prof_end(h, 2, pi, 0.0);
-  CK(cudaMemcpyAsync(h->hpc, h->dpc, sizeof(mpdo_ctx::PcOut), cudaMemcpyDeviceToHost, h->st));
+  CK(cudaMemcpyAsync(h->hpc, h->dpc, sizeof(PcholOut), cudaMemcpyDeviceToHost, h->st));
   CK(sync_stream(h));
   prof_drain(h);
-  const int r = h->hpc->r;
-  *zero = r < 1;
-  if (r >= 1 && !(r >= rmax && r < n && h->hpc->resid > tol)) *rank = r;
+  const PcholFit fit = pchol_fit(*h->hpc, n, rmax, tol);
+  *zero = fit == PcholFit::zero;
+  if (fit == PcholFit::fits) *rank = h->hpc->r;
   return MPDO_OK;
 }
 
@@ -1510,7 +1510,7 @@ int mpdo_create(const mpdo_config* cfg, const double* init_site_vec, mpdo_t* out
   if ((rc = alloc_dev(hp, &h->wLg, (size_t)std::max(n9, KM) * kInnerRmax * em)) ||
       (rc = B(&h->wGs, (size_t)kInnerRmax * kInnerRmax)) ||
       (rc = B(&h->wZ, (size_t)kInnerRmax * kInnerRmax)) ||
-      (rc = alloc_dev(hp, (void**)&h->dpc, sizeof(mpdo_ctx::PcOut))) ||
+      (rc = alloc_dev(hp, (void**)&h->dpc, sizeof(PcholOut))) ||
       (rc = alloc_dev(hp, (void**)&h->dpiv, kGradedMax * sizeof(int))))
     return rc;
   if (cudaEventCreateWithFlags(&h->bev, cudaEventBlockingSync | cudaEventDisableTiming) !=
@@ -1518,7 +1518,7 @@ int mpdo_create(const mpdo_config* cfg, const double* init_site_vec, mpdo_t* out
     cudaGetLastError();
     h->bev = nullptr;
   }
-  if (cudaMallocHost((void**)&h->hpc, sizeof(mpdo_ctx::PcOut)) != cudaSuccess) {
+  if (cudaMallocHost((void**)&h->hpc, sizeof(PcholOut)) != cudaSuccess) {
     cudaGetLastError();
     return fail(nullptr, MPDO_ERR_OOM, "pinned host allocation");
   }
@@ -2017,12 +2017,12 @@ int mpdo_kernel_pchol(int n, const void* w, int rmax, double tol, void* L, int l
       !rank || !resid)
     return fail(nullptr, MPDO_ERR_ARG, "bad pchol arguments");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  mpdo_ctx::PcOut* d = nullptr;
-  if (cudaMalloc(&d, sizeof(mpdo_ctx::PcOut)) != cudaSuccess) {
+  PcholOut* d = nullptr;
+  if (cudaMalloc(&d, sizeof(PcholOut)) != cudaSuccess) {
     cudaGetLastError();
     return fail(nullptr, MPDO_ERR_OOM, "pchol result");
   }
-  mpdo_ctx::PcOut hd{};
+  PcholOut hd{};
   cudaError_t e = pchol<double>(st, n, (const double2*)w, rmax, tol, (double2*)L, ldl, &d->r,
                                 &d->resid, piv);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hd, d, sizeof(hd), cudaMemcpyDeviceToHost, st);
@@ -2030,6 +2030,7 @@ int mpdo_kernel_pchol(int n, const void* w, int rmax, double tol, void* L, int l
   cudaFree(d);
   if (e == cudaSuccess) e = es;
   if (e != cudaSuccess) return fail(nullptr, MPDO_ERR_CUDA, cudaGetErrorString(e));
+  if (hd.r == kPcholGaveUp) return fail(nullptr, MPDO_ERR_TIMEOUT, "pchol: a wait gave up");
   *rank = hd.r;
   *resid = hd.resid;
   return MPDO_OK;

@@ -653,7 +653,8 @@ __global__ void dual_rows_kernel(int kk, int cols, const cx<R>* __restrict__ y, 
 // Pivoted Cholesky of the Hermitian PSD n x n matrix w (precision R, n <= 1024): W ~ L L^+
 // with L n x r (row-major, row stride lr), greedy diagonal pivoting, stopping once the
 // largest remaining diagonal is <= tol * tr W or after rmax (<= kGradedMax) columns.
-// *rout = r; *resid = largest remaining diagonal / tr W.
+// *rout = r, or kPcholGaveUp when a wait for another CTA gave up; *resid = largest remaining diagonal
+// / tr W.
 //
 // The columns depend on one another, so the factor is bound by the latency of a column.  An FP64
 // warp instruction occupies its quarter of the SM for 64 clocks whatever its active lanes, so a
@@ -912,7 +913,7 @@ __global__ void __launch_bounds__(32 * (kPcWarps + 1)) pchol_kernel(
   }
   if (c == 0 && tid == 0) {
     const double ld = __longlong_as_double(last);
-    *rout = s_late ? 0 : r;                 // rank 0: no factor, as for a zero matrix
+    *rout = r;
     *resid = !s_late && tr > 0 && ld > 0.0 ? ld / tr : 0.0;
   }
   // L to global memory only now: a store before an exchange holds it up until the store has landed
@@ -920,7 +921,10 @@ __global__ void __launch_bounds__(32 * (kPcWarps + 1)) pchol_kernel(
     const int row = e / r, k = e - row * r;
     if (c + row * S < n) L[(long)(c + row * S) * lr + k] = Ls[(size_t)row * rmax + k];
   }
-  if constexpr (CLUSTER) cluster.sync();   // no CTA leaves before what was sent to it has landed
+  if constexpr (CLUSTER) {
+    cluster.sync();   // no CTA leaves before what was sent to it has landed
+    if (s_late && tid == 0) *rout = kPcholGaveUp;   // whichever CTA's wait it was
+  }
 }
 
 // x = L1^-1 (r x r, lower triangular, row-major), L1[a][b] = L[piv[a]][b] the pivot rows of a

@@ -3,6 +3,7 @@
 #include <stdint.h>
 
 #include "common.cuh"
+#include "pcholout.h"
 
 namespace mpdo {
 // out (rows x cols, row stride ldo) = in converted from precision Ri to Ro.
@@ -49,8 +50,8 @@ cudaError_t kraus_select(cudaStream_t st, int n, const double* w, const cx<R>* w
 template <typename R>
 cudaError_t trace_pre(cudaStream_t st, int dm, const cx<R>* gi, const cx<R>* gj, StepScalars* sc);
 // Pivoted Cholesky W ~ L L^+ of a Hermitian PSD matrix (n <= 1024, rmax <= kGradedMax); device
-// outputs: L (n x r, row stride lr), *rout = r, *resid = remaining diag max / tr W, and (not
-// NULL) piv[0..r) = the pivots.
+// outputs: L (n x r, row stride lr), *rout = r (kPcholGaveUp: a wait gave up), *resid = remaining
+// diag max / tr W, and (not NULL) piv[0..r) = the pivots.
 template <typename R>
 cudaError_t pchol(cudaStream_t st, int n, const cx<R>* w, int rmax, double tol, cx<R>* L, int lr,
                   int* rout, double* resid, int* piv = nullptr);

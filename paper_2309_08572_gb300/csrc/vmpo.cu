@@ -274,9 +274,8 @@ struct mpdo_vmpo_s {
   double2 *L = nullptr, *Gs = nullptr, *Zs = nullptr;
   MixWork gradw;
   void* gradmem = nullptr;
-  struct PcOut { int r; int pad; double resid; };
-  PcOut* dpc = nullptr;
-  PcOut* hpc = nullptr;   // pinned
+  PcholOut* dpc = nullptr;
+  PcholOut* hpc = nullptr;   // pinned
   MixWork mixw;
   void* mixmem = nullptr;
   void* tcws = nullptr;
@@ -418,8 +417,9 @@ int split(mpdo_vmpo h, int n, int* nval, int* nvec) {
     VK(cudaMemcpyAsync(h->hpc, h->dpc, sizeof(*h->hpc), cudaMemcpyDeviceToHost, st));
     VK(cudaStreamSynchronize(st));
     const int r = h->hpc->r;
-    if (r < 1) return vfail(h, MPDO_ERR_NUMERIC, "vmpo: zero or non-finite state");
-    if (!(r >= rmax && r < n && h->hpc->resid > tol)) {
+    const PcholFit fit = pchol_fit(*h->hpc, n, rmax, tol);
+    if (fit == PcholFit::zero) return vfail(h, MPDO_ERR_NUMERIC, "vmpo: zero or non-finite state");
+    if (fit == PcholFit::fits) {
       *nval = r;
       *nvec = h->mode == 1 ? r : std::min(r, h->chi);
       VK(cgemm_gram<double>(st, 0, r, n, h->L, kGradedMax, h->Zs, r));
