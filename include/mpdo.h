@@ -389,12 +389,13 @@ int mpdo_profile_read(mpdo_t h, int cls, double* ms, long long* launches, double
  * 2), times on `stream` (cudaStream_t; reps runs after one warm-up, minimum taken, CUDA
  * events) the 64 x 64 tile kernel, the 16 x 16 tile kernel and the 16 x 16 kernel with K
  * split over a thread-block cluster of 2, 4 or 8, on a representative shape of the
- * bucket, and makes the fastest the choice for every product of that bucket.  Untuned
+ * bucket, and makes the fastest the choice for every product of that bucket; for FP64 the
+ * built-in size rules are timed beside them and stay unless a kernel is 5 % faster.  Untuned
  * buckets, and all of them after a call with reps <= 0, follow the built-in size rules.
  * The choice changes the summation order of products, not their precision: call it
  * before running circuits, not while another thread runs them.  Allocates ~70 MB of
  * device scratch for the call; synchronises the stream.  *n_tuned (may be NULL) receives
- * the number of buckets set.  MPDO_ERR_ARG for prec outside {0, 1}; MPDO_ERR_OOM;
+ * the number of buckets timed.  MPDO_ERR_ARG for prec outside {0, 1}; MPDO_ERR_OOM;
  * MPDO_ERR_CUDA (the table is then reset to the size rules). */
 int mpdo_autotune_gemm(int prec, void* stream, int reps, int* n_tuned);
 

@@ -404,8 +404,11 @@ cudaError_t launch_tile(cudaStream_t st, int m, int n, int k, const cx<RA>* A, l
 
 // Tile-shape table of the autotuner (mpdo_autotune_gemm): per precision (0: FP64 products,
 // 1: FP32), per bucket of the 16 x 16 output-tile count (log2, 0..10) and of K (log2(K/16),
-// 0..8), the kernel choice: 0 = size rules above (untuned), 1 = 64 x 64 tiles, 2 = 16 x 16
-// tiles, 3/4/5 = 16 x 16 tiles with K split over a cluster of 2/4/8.
+// 0..8), the kernel choice: 0 = size rules above, 1 = 64 x 64 tiles, 2 = 16 x 16 tiles, 3/4/5 =
+// 16 x 16 tiles with K split over a cluster of 2/4/8.  For FP64 the size rules are a candidate like
+// the others (they alone reach the tiles of 8 x 8 and less, and know a product's shape where a
+// bucket knows its tile count), and give way only to a kernel that is kTuneGain faster.
+constexpr float kTuneGain = 0.95f;
 constexpr int kTileBuckets = 11, kKBuckets = 9, kChoices = 5;
 std::atomic<signed char> g_choice[2][kTileBuckets][kKBuckets];
 
@@ -615,7 +618,7 @@ extern "C" int mpdo_autotune_gemm(int prec, void* stream, int reps, int* n_tuned
       const int m = 16 << ((tb + 1) / 2), n = 16 << (tb / 2), k = 16 << kb;
       float best = 1e30f;
       int best_c = 0;
-      for (int ch = 1; ch <= kChoices && err == cudaSuccess; ++ch) {
+      for (int ch = prec == 0 ? 0 : 1; ch <= kChoices && err == cudaSuccess; ++ch) {
         if (ch >= 3 && k < 16 * (1 << (ch - 2))) continue;   // slices shorter than one step
         table[tb][kb].store((signed char)ch, std::memory_order_relaxed);
         auto run = [&]() {
@@ -639,12 +642,12 @@ extern "C" int mpdo_autotune_gemm(int prec, void* stream, int reps, int* n_tuned
           t_min = std::min(t_min, ms);
         }
         if (err == cudaSuccess && t_min < best) {
-          best = t_min;
+          best = ch == 0 ? kTuneGain * t_min : t_min;
           best_c = ch;
         }
       }
       table[tb][kb].store((signed char)best_c, std::memory_order_relaxed);
-      if (best_c) ++tuned;
+      if (err == cudaSuccess) ++tuned;
     }
   release();
   if (err != cudaSuccess) {
