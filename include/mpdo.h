@@ -59,7 +59,9 @@ enum {
  *              matrices) with its FP32 products -- the new centre B_j, the inner isometry,
  *              sampling -- on the tensor cores.
  *              The routing threshold can be changed with the environment variable
- *              MPDO_TC_MIN_MACS (read at create; 0 routes every product). */
+ *              MPDO_TC_MIN_MACS (read at create; 0 routes every product with both sides
+ *              of at least 16).  Where it is not set, FP64 results also stay on the CUDA cores
+ *              where these are estimated faster; the graded eigensolver's do in any case. */
 typedef enum { MPDO_FP64 = 0, MPDO_C64 = 1, MPDO_TF32X3 = 2, MPDO_BF16X3 = 3 } mpdo_prec;
 
 typedef struct mpdo_ctx* mpdo_t;   /* opaque; the handle owns its device memory (allocated

@@ -32,6 +32,7 @@
 
 #include "../../include/mpdo.h"
 #include "common.cuh"
+#include "exactplan.h"
 #include "internal.h"
 #include "kernels.h"
 #include "tcgemm.h"
@@ -111,6 +112,7 @@ struct mpdo_ctx {
   int* tcerr = nullptr;
   int* htcerr = nullptr;   // pinned
   double tc_min_macs = 0;  // routing threshold (kTcMinMacs; MPDO_TC_MIN_MACS overrides)
+  bool tc_forced = false;  // it was given: no estimate beside it
   // Waits for the host read-backs of the update: spinning (cudaStreamSynchronize) for one
   // circuit; blocking on an event (the thread sleeps) while the batch executor runs many
   // circuits, whose spinning host threads would otherwise take every core.
@@ -284,11 +286,10 @@ constexpr int kTcMinSide = 16;
 // Products with FP64 outputs in the tensor-core forms with FP64 Grams (mixed form): the
 // error-free slice products on the BF16 tensor cores (tc_cgemm_exact) when large enough.
 // Of those above the threshold the ones that are estimated faster there than on the FP64 CUDA
-// cores (a threshold from the environment is taken as it is).
+// cores, or all of them where the threshold was given (MPDO_TC_MIN_MACS).
 inline bool tc_exact_route(const mpdo_ctx* h, int m, int n, int k, int batch, bool gram = false) {
-  return h->tcmode >= 0 && h->mixed && (double)m * n * k * batch >= h->tc_min_macs &&
-         m >= kTcMinSide && n >= kTcMinSide && k >= 1 &&
-         (h->tc_min_macs < kTcMinMacs || tc_exact_faster(m, n, k, batch, gram));
+  return h->tcmode >= 0 && h->mixed &&
+         ExactRoute{h->tc_min_macs, h->tc_forced}.takes(m, n, k, batch, gram);
 }
 template <typename TA, typename TB>
 cudaError_t pexact(mpdo_ctx* h, int opa, int opb, int m, int n, int k, const TA* A, long lda,
@@ -1452,7 +1453,10 @@ int mpdo_create(const mpdo_config* cfg, const double* init_site_vec, mpdo_t* out
   h->eltm = (h->dbl || h->mixed) ? 16 : 8;
   h->tcmode = cfg->prec == MPDO_TF32X3 ? TC_TF32X3 : cfg->prec == MPDO_BF16X3 ? TC_BF16X3 : -1;
   h->tc_min_macs = kTcMinMacs;
-  if (const char* tm = std::getenv("MPDO_TC_MIN_MACS")) h->tc_min_macs = std::atof(tm);
+  if (const char* tm = std::getenv("MPDO_TC_MIN_MACS")) {
+    h->tc_min_macs = std::atof(tm);
+    h->tc_forced = true;
+  }
   // Numerical-zero cuts.  Gram eigenvalues resolve only down to ~eps * max, so the cuts
   // are applied there: bond lambda = s^2 > htol*lambda_0, inner w > kcut^2 * w_0.  With
   // FP64 Grams of FP32 tensors the floor is the rounding of the tensors themselves
@@ -1566,6 +1570,7 @@ int mpdo_create(const mpdo_config* cfg, const double* init_site_vec, mpdo_t* out
       h->mixw.tcws_bytes = h->tcws_bytes;
       h->mixw.tcerr = h->tcerr;
       h->mixw.tc_min_macs = h->tc_min_macs;
+      h->mixw.tc_forced = h->tc_forced;
     }
   }
   {

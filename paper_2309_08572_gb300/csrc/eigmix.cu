@@ -25,6 +25,7 @@
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "exactplan.h"
 #include "internal.h"
 #include "kernels.h"
 #include "tcgemm.h"
@@ -1003,8 +1004,7 @@ __global__ void __launch_bounds__(RT * RT) level_out_kernel(
 // cores (carried to ~2^-48 of each operand row's largest entry, summed in FP64) when the
 // caller lent their workspace and the product is large enough; CUDA-core FP64 otherwise.
 bool tc_route(const MixWork& wk, long m, long n, long k, int batch) {
-  return wk.tcws != nullptr && (double)m * n * k * batch >= wk.tc_min_macs && m >= 16 && n >= 16 &&
-         tc_exact_faster(m, n, k, batch, false);
+  return wk.tcws != nullptr && ExactRoute{wk.tc_min_macs, wk.tc_forced}.takes(m, n, k, batch, false);
 }
 
 // Unit norm for the columns a level emits (v[:, off + j], j < the level's take): the last

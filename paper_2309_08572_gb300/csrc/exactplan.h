@@ -15,6 +15,7 @@ constexpr int kExactSlices = 6;   // slices per operand
 constexpr long kExactPart = (long)kExactRows * kExactCols;   // entries of a CTA's part of a tile
 constexpr long kExactPartBytes = kExactPart * 16;            // two 64-bit sums each
 constexpr long kExactSms = 152;
+constexpr int kExactFusedPackK = 256;   // up to here exponents and packing are one launch
 
 struct ExactPlan {
   int tiles, nst, ctas;
@@ -90,5 +91,29 @@ inline size_t exact_ws_bytes(long m, long n, long k, int batch, bool gram) {
                           exact_part_bytes(exact_plan(m, n, kn, batch, gram)));
   return ws;
 }
+
+// Time of an exact product against the same product on the FP64 CUDA cores.  The slice kernel
+// costs a fixed part (exponents, packing, output) and its stages on the busiest SM, 1.4 us each;
+// FP64 runs at 304 FMA per clock over the chip.  Both sides as measured: the Gram 41 x 41 x 1968 takes
+// 25 us in FP64 and 36 us plus its packing in slices, the Gram 400 x 400 x 5043 2.6 ms and 74 us.
+inline bool exact_faster(long m, long n, long k, int batch, bool gram) {
+  const ExactPlan p = exact_plan(m, n, k, batch, gram);
+  const double elems = (double)batch * k * ((gram ? 0 : m) + 2.0 * n);   // packed complex entries
+  const double tc = (k <= kExactFusedPackK ? 12.0 : 24.0) + (p.parts ? 8.0 : 0.0) +
+                    1.4 * (p.per + 4 + p.per / p.nst) + elems * 24.0 / 3.0e6;
+  const double fp64 = 8.0 + 1.2 * 4.0 * m * n * (double)k * batch * (gram ? 0.5 : 1.0) / (304.0 * 2.0e3);
+  return tc < fp64;
+}
+// Which products with FP64 results run as slices: those of min_macs complex multiply-adds with both
+// sides of at least 16, where that is estimated faster, or (forced: the caller has set the threshold)
+// whatever the estimate.
+struct ExactRoute {
+  double min_macs;
+  bool forced;
+  bool takes(long m, long n, long k, int batch, bool gram) const {
+    return m >= 16 && n >= 16 && k >= 1 && (double)m * n * k * batch >= min_macs &&
+           (forced || exact_faster(m, n, k, batch, gram));
+  }
+};
 
 }  // namespace mpdo

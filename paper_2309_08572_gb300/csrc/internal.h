@@ -90,13 +90,14 @@ struct MixWork {
   cudaEvent_t block_ev = nullptr; // when set, level read-backs wait on it (blocking sync)
   double* hpin = nullptr;         // mapped pinned host area of the level scalars (lazy)
   double* hpin_dev = nullptr;     // its device address
-  // Tensor-core workspace lent by the caller: when set, products of at least tc_min_macs
-  // complex multiply-adds run as error-free BF16 slice products (tc_cgemm_exact) instead of
+  // Tensor-core workspace lent by the caller: when set, products that ExactRoute{tc_min_macs,
+  // tc_forced} takes run as error-free BF16 slice products (tc_cgemm_exact) instead of
   // CUDA-core FP64; tcerr is the device flag of their pipeline waits.
   void* tcws = nullptr;
   size_t tcws_bytes = 0;
   int* tcerr = nullptr;
   double tc_min_macs = 0;
+  bool tc_forced = false;
 };
 size_t mix_work_bytes(int n_cap);
 void mix_work_bind(MixWork& w, void* base, int n_cap);

@@ -1019,7 +1019,7 @@ __global__ void __launch_bounds__(PT * 8)
 // then PW columns at a time through shared memory.  Two launches each, row_exp_kernel and
 // pack_exact_kernel share long rows out over more CTAs.
 constexpr int PR = 16, PW = 128;
-constexpr int kFusedPackK = 256;
+constexpr int kFusedPackK = kExactFusedPackK;
 struct PackOp {
   const void* src;
   __nv_bfloat16* out;
@@ -1425,20 +1425,6 @@ bool is_gram(int opa, int opb, int m, int n, const TA* A, long lda, long sa, con
          m == n && ((opa == OP_C && opb == OP_N) || (opa == OP_N && opb == OP_C));
 }
 }  // namespace
-
-// Time of an exact product against the same product on the FP64 CUDA cores.  The slice kernel
-// costs a fixed part (exponents, packing, output) and its stages on the busiest SM, 1.4 us each;
-// FP64 runs at 304 FMA per clock over the chip.  Both sides as measured: the Gram 41 x 41 x 1968 takes
-// 25 us in FP64 and 36 us plus its packing in slices, the Gram 400 x 400 x 5043 2.6 ms and 74 us.
-bool tc_exact_faster(long m, long n, long k, int batch, bool gram) {
-  const ExactPlan p = exact_plan(m, n, k, batch, gram);
-  const double elems = (double)batch * k * ((gram ? 0 : m) + 2.0 * n);   // packed complex entries
-  const double tc = (k <= kFusedPackK ? 12.0 : 24.0) + (p.parts ? 8.0 : 0.0) +
-                    1.4 * (p.per + 4 + p.per / p.nst) + elems * 24.0 / 3.0e6;
-  const double fp64 = 8.0 + 1.2 * 4.0 * m * n * (double)k * batch * (gram ? 0.5 : 1.0) / (304.0 * 2.0e3);
-  return tc < fp64;
-}
-
 
 cudaError_t tc_exact_init() {
   static const cudaError_t attr =

@@ -66,8 +66,6 @@ template <typename TA, typename TB>
 cudaError_t tc_cgemm_exact(cudaStream_t st, int opa, int opb, int m, int n, int k, const TA* A,
                            long lda, long sa, const TB* B, long ldb, long sb, double2* C, long ldc,
                            long sc, int batch, void* ws, size_t ws_bytes, int* err);
-// Whether the product is estimated faster there than on the FP64 CUDA cores.
-bool tc_exact_faster(long m, long n, long k, int batch, bool gram);
 // One-time kernel attribute setup of tc_cgemm_exact; call it before capturing a stream that
 // will run the first exact product of the process.
 cudaError_t tc_exact_init();

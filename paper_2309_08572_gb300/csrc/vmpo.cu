@@ -31,6 +31,7 @@
 
 #include "../../include/mpdo.h"
 #include "common.cuh"
+#include "exactplan.h"
 #include "internal.h"
 #include "kernels.h"
 #include "tcgemm.h"
@@ -330,8 +331,7 @@ cudaError_t g64(cudaStream_t st, int opa, int opb, int m, int n, int k, const do
 cudaError_t u64(mpdo_vmpo h, int opa, int opb, int m, int n, int k, const double2* A, long lda,
                 long sa, const double2* B, long ldb, long sb, double2* C, long ldc, long sc,
                 int batch) {
-  if (h->tc && m >= 16 && n >= 16 && (double)m * n * k * batch >= (double)(1 << 21) &&
-      tc_exact_faster(m, n, k, batch, A == B))
+  if (h->tc && ExactRoute{(double)(1 << 21), false}.takes(m, n, k, batch, A == B))
     return tc_cgemm_exact<double2, double2>(h->st, opa, opb, m, n, k, A, lda, sa, B, ldb, sb, C,
                                             ldc, sc, batch, h->tcws, h->tcws_bytes, h->tcerr);
   return g64(h->st, opa, opb, m, n, k, A, lda, sa, B, ldb, sb, C, ldc, sc, batch);

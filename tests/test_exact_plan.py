@@ -90,3 +90,29 @@ def test_empty_products(plan):
     for r in rows:
         ((ok, _),) = plan([r])
         assert ok, r
+
+
+ROUTES = r"""
+#include <cstdio>
+#include "exactplan.h"
+using namespace mpdo;
+int main() {
+  // threshold given (0, below and above the default) or not; a small product, one that the FP64 cores
+  // do faster, a large one, one with a short side
+  const long size[4][4] = {{20, 20, 20, 0}, {41, 41, 1968, 1}, {400, 400, 5043, 1}, {15, 900, 900, 0}};
+  for (const ExactRoute& r : {ExactRoute{0, true}, ExactRoute{1 << 20, true}, ExactRoute{1 << 24, true},
+                              ExactRoute{1 << 21, false}})
+    for (const auto& s : size) std::printf("%d ", r.takes(s[0], s[1], s[2], 1, s[3] != 0) ? 1 : 0);
+}
+"""
+
+
+def test_given_threshold_forces_the_route(tmp_path):
+    """A threshold from the environment decides alone, in every caller (updates and eigensolver share
+    the rule); otherwise the estimate has a say."""
+    cxx = shutil.which("g++") or pytest.skip("no host compiler")
+    (tmp_path / "r.cpp").write_text(ROUTES)
+    subprocess.run([cxx, "-std=c++17", "-I", CSRC, str(tmp_path / "r.cpp"), "-o",
+                    str(tmp_path / "r")], check=True)
+    out = subprocess.run([str(tmp_path / "r")], capture_output=True, text=True, check=True).stdout
+    assert list(map(int, out.split())) == [1, 1, 1, 0, 0, 1, 1, 0, 0, 0, 1, 0, 0, 0, 1, 0]
