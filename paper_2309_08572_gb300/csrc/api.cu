@@ -225,14 +225,7 @@ EigWork<float>& eigw<float>(mpdo_ctx* h) { return h->eig32; }
 void* dmalloc(mpdo_ctx* h, size_t bytes) {
   if (h->cfg.alloc) return h->cfg.alloc(bytes, h->cfg.alloc_ctx);
   void* p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    scratch_trim();
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-  }
+  if (dev_malloc(&p, bytes) != cudaSuccess) return nullptr;
   return p;
 }
 void dfree(mpdo_ctx* h, void* p) {
@@ -1930,10 +1923,10 @@ int mpdo_kernel_heig(int prec, int n, void* a, void* v, double* w, int* sweeps, 
     // mixed-precision solver on an FP64 matrix (resolved down to 1e-14 of the largest);
     // prec 3: its FP64 products as exact slice products on the tensor cores
     void* mm = nullptr;
-    if (cudaMalloc(&mm, mix_work_bytes(n)) != cudaSuccess) { cudaGetLastError(); return fail(nullptr, MPDO_ERR_OOM, "heig work"); }
+    if (dev_malloc(&mm, mix_work_bytes(n)) != cudaSuccess) { cudaGetLastError(); return fail(nullptr, MPDO_ERR_OOM, "heig work"); }
     void* tw = nullptr;
     const size_t tw_bytes = (size_t)256 << 20;
-    if (prec == 3 && cudaMalloc(&tw, tw_bytes + 256) != cudaSuccess) {
+    if (prec == 3 && dev_malloc(&tw, tw_bytes + 256) != cudaSuccess) {
       cudaGetLastError();
       cudaFree(mm);
       return fail(nullptr, MPDO_ERR_OOM, "heig tensor-core workspace");
@@ -1969,7 +1962,7 @@ int mpdo_kernel_heig(int prec, int n, void* a, void* v, double* w, int* sweeps, 
     return MPDO_OK;
   }
   size_t bytes = prec == 0 ? eig_work_bytes<double>(n) : eig_work_bytes<float>(n);
-  if (cudaMalloc(&mem, bytes) != cudaSuccess) { cudaGetLastError(); return fail(nullptr, MPDO_ERR_OOM, "heig work"); }
+  if (dev_malloc(&mem, bytes) != cudaSuccess) { cudaGetLastError(); return fail(nullptr, MPDO_ERR_OOM, "heig work"); }
   cudaError_t e;
   int* counters;
   if (prec == 0) {
@@ -1998,7 +1991,7 @@ int mpdo_kernel_heig_graded(int n, const void* a, void* v, double* w, void* stre
     return fail(nullptr, MPDO_ERR_ARG, "bad heig_graded arguments");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   void* mm = nullptr;
-  if (cudaMalloc(&mm, mix_work_bytes(n)) != cudaSuccess) {
+  if (dev_malloc(&mm, mix_work_bytes(n)) != cudaSuccess) {
     cudaGetLastError();
     return fail(nullptr, MPDO_ERR_OOM, "heig_graded work");
   }
@@ -2023,7 +2016,7 @@ int mpdo_kernel_pchol(int n, const void* w, int rmax, double tol, void* L, int l
     return fail(nullptr, MPDO_ERR_ARG, "bad pchol arguments");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   PcholOut* d = nullptr;
-  if (cudaMalloc(&d, sizeof(PcholOut)) != cudaSuccess) {
+  if (dev_malloc(&d, sizeof(PcholOut)) != cudaSuccess) {
     cudaGetLastError();
     return fail(nullptr, MPDO_ERR_OOM, "pchol result");
   }

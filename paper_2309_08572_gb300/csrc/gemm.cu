@@ -11,6 +11,7 @@
 #include "../../include/mpdo.h"
 #include "common.cuh"
 #include "internal.h"
+#include "tcgemm.h"
 
 namespace cg = cooperative_groups;
 
@@ -601,8 +602,8 @@ extern "C" int mpdo_autotune_gemm(int prec, void* stream, int reps, int* n_tuned
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
   };
-  if (cudaMalloc(&a, mmax * kmax * elt) != cudaSuccess || cudaMalloc(&b, kmax * mmax * elt) != cudaSuccess ||
-      cudaMalloc(&c, mmax * mmax * elt) != cudaSuccess || cudaEventCreate(&e0) != cudaSuccess ||
+  if (dev_malloc(&a, mmax * kmax * elt) != cudaSuccess || dev_malloc(&b, kmax * mmax * elt) != cudaSuccess ||
+      dev_malloc(&c, mmax * mmax * elt) != cudaSuccess || cudaEventCreate(&e0) != cudaSuccess ||
       cudaEventCreate(&e1) != cudaSuccess) {
     cudaGetLastError();
     release();

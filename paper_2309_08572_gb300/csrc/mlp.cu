@@ -360,17 +360,17 @@ int mpdo_mlp_create(int n_layers, const int* widths, int max_batch, void* stream
     }
     m->own_stream = true;
   }
-  bool ok = cudaMalloc(&m->params, sizeof(float) * off) == cudaSuccess &&
-            cudaMalloc(&m->grads, sizeof(float) * off) == cudaSuccess &&
-            cudaMalloc(&m->m, sizeof(float) * off) == cudaSuccess &&
-            cudaMalloc(&m->v, sizeof(float) * off) == cudaSuccess &&
-            cudaMalloc(&m->da, sizeof(float) * (size_t)max_batch * m->maxw) == cudaSuccess &&
-            cudaMalloc(&m->db2, sizeof(float) * (size_t)max_batch * m->maxw) == cudaSuccess &&
-            cudaMalloc(&m->part, sizeof(double) * 4096) == cudaSuccess &&
+  bool ok = mpdo::dev_malloc(&m->params, sizeof(float) * off) == cudaSuccess &&
+            mpdo::dev_malloc(&m->grads, sizeof(float) * off) == cudaSuccess &&
+            mpdo::dev_malloc(&m->m, sizeof(float) * off) == cudaSuccess &&
+            mpdo::dev_malloc(&m->v, sizeof(float) * off) == cudaSuccess &&
+            mpdo::dev_malloc(&m->da, sizeof(float) * (size_t)max_batch * m->maxw) == cudaSuccess &&
+            mpdo::dev_malloc(&m->db2, sizeof(float) * (size_t)max_batch * m->maxw) == cudaSuccess &&
+            mpdo::dev_malloc(&m->part, sizeof(double) * 4096) == cudaSuccess &&
             cudaMallocHost(&m->hpart, sizeof(double) * 4096) == cudaSuccess;
   for (int l = 0; ok && l <= n_layers; ++l) {
     float* p = nullptr;
-    ok = cudaMalloc(&p, sizeof(float) * (size_t)max_batch * m->w[l]) == cudaSuccess;
+    ok = mpdo::dev_malloc(&p, sizeof(float) * (size_t)max_batch * m->w[l]) == cudaSuccess;
     m->acts.push_back(p);
   }
   if (!ok) {
@@ -533,7 +533,7 @@ int mpdo_mlp_set_precision(mpdo_mlp m, int mode) {
       m->lpart = static_cast<double*>(take(sizeof(double) * groups * ((m->w[L] + 31) / 32)));
       m->tcout = static_cast<mpdo_mlp_s::TcOut*>(take(sizeof(mpdo_mlp_s::TcOut)));
       if (pass == 0) {
-        if (cudaMalloc(&m->tcmem, off) != cudaSuccess) {
+        if (mpdo::dev_malloc(&m->tcmem, off) != cudaSuccess) {
           cudaGetLastError();
           m->tcmem = nullptr;
           return mlp_fail(m, MPDO_ERR_OOM, "mlp: tensor-core operand buffers");

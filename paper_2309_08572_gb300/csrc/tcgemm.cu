@@ -1601,9 +1601,7 @@ struct Scratch {
     bytes = (bytes + 255) / 256 * 256;
     if (cudaMemPool_t pool = scratch_pool())
       pooled = cudaMallocFromPoolAsync(&p, bytes + 256, pool, st) == cudaSuccess;
-    if (!pooled && (cudaGetLastError(), mpdo::scratch_trim(),
-                    cudaMalloc(&p, bytes + 256) != cudaSuccess)) {
-      cudaGetLastError();
+    if (!pooled && (cudaGetLastError(), mpdo::dev_malloc(&p, bytes + 256) != cudaSuccess)) {
       p = nullptr;
       return false;
     }
@@ -1628,6 +1626,16 @@ void scratch_trim() {
   std::lock_guard<std::mutex> lock(g_pool_mu);
   for (cudaMemPool_t p : g_pool)
     if (p) cudaMemPoolTrimTo(p, 0);
+}
+cudaError_t dev_malloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    scratch_trim();
+    e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) cudaGetLastError();
+  }
+  return e;
 }
 }  // namespace mpdo
 

@@ -10,6 +10,12 @@
 namespace mpdo {
 // Gives the entry points' pooled scratch (mpdo_kernel_trim) back to the device.
 void scratch_trim();
+// cudaMalloc that takes the pooled scratch back before it gives up.
+cudaError_t dev_malloc(void** p, size_t bytes);
+template <typename T>
+cudaError_t dev_malloc(T** p, size_t bytes) {
+  return dev_malloc(reinterpret_cast<void**>(p), bytes);
+}
 
 // Operand modes of the tensor-core path: the MMA element type and the number of K-segments
 // of a packed complex operand (1 = plain, 3 = split hi/lo precision compensation).

@@ -306,7 +306,7 @@ int vfail(mpdo_vmpo h, int code, const std::string& msg) {
   } while (0)
 
 int valloc(mpdo_vmpo h, void** p, size_t bytes) {
-  if (cudaMalloc(p, bytes ? bytes : 16) != cudaSuccess) {
+  if (dev_malloc(p, bytes ? bytes : 16) != cudaSuccess) {
     cudaGetLastError();
     return vfail(h, MPDO_ERR_OOM, "vmpo: device allocation of " + std::to_string(bytes) + " bytes");
   }
