@@ -339,7 +339,7 @@ cudaError_t peig(mpdo_ctx* h, int n, const cx<R>* a, long lda, cx<R>* v, long ld
   }
   e = heig<R>(h->st, n, a, lda, v, ldv, w, eigw<R>(h), sweeps);
   if (pi >= 0 && e == cudaSuccess && h->prof_slot < h->prof_nslots) {
-    // executed flops: 8 real flops per complex MAC, 3*16*16*np MACs per active pair-round
+    // executed flops: 8 real flops per complex MAC, 2*16*16*np MACs per active pair-round
     int slot = h->prof_slot++;
     e = cudaMemcpyAsync(&h->prof_counts[slot], eigw<R>(h).counters + 3, sizeof(int),
                         cudaMemcpyDeviceToHost, h->st);

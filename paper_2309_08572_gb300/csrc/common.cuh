@@ -61,7 +61,6 @@ __device__ __forceinline__ void tourney(int round, int k, int players, int& a, i
 struct StepScalars {
   int keep;        // bond values kept
   int kkeep;       // inner values kept
-  int rank_g;      // rank of the left Gram
   int flags;       // bit 0: numeric problem (NaN / zero state)
   double tot;      // sum of all bond eigenvalues (= tr rho before the cut)
   double kept;     // sum of the kept ones
@@ -85,6 +84,9 @@ struct DevStats {
   int n_updates;
   int numeric_error;
 };
+
+// SMs of the device this library is written for: the rules that deal work out count in them.
+constexpr int kSms = 152;
 
 // Count of kernels launched by this library (all handles), for throughput reports.
 #include <atomic>

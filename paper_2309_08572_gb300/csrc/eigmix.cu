@@ -491,8 +491,8 @@ constexpr int RT = 16;   // output tile of the fused products (one element per t
 // CTAs of a thread-block cluster (dims (splits, 1, 1)); the partial sums meet in rank 0
 // through distributed shared memory, added in rank order.
 __global__ void __launch_bounds__(RT * RT) sg_refine_kernel(
-    int m, int n, const double2* __restrict__ TZ, double2* SG, int level0, int final_pass,
-    int level, double floor, const int* rot, double* lam, double* scan, double2* IE,
+    int m, int n, const double2* __restrict__ TZ, double2* SG, int level0, int level,
+    double floor, const int* rot, double* lam, double* scan, double2* IE,
     unsigned int* ticket, int splits, int* cid, double emax, unsigned char* sepg) {
   __shared__ double2 As[RT][RT + 1];   // [k][i]
   __shared__ double2 Bs[RT][RT + 1];   // [k][j]
@@ -952,7 +952,7 @@ __global__ void __launch_bounds__(kSgeThreads) sge_kernel(int m, const double2* 
 // slice at least 16 long (one tile step), at most 8 (portable cluster size).
 inline int split_count(long tiles, int K) {
   int s = 1;
-  while (s < 8 && tiles * (2 * s) <= 152 && K >= 16 * (2 * s)) s *= 2;
+  while (s < 8 && tiles * (2 * s) <= kSms && K >= 16 * (2 * s)) s *= 2;
   return s;
 }
 
@@ -1210,7 +1210,7 @@ cudaError_t enqueue_level(cudaStream_t st, int n, int m, int level, const double
         refine_kernel<<<1, RT * RT, 0, st>>>(m, n, wk.s, level0, final_pass, level, floor, rot, wk.lam,
                                              wk.scan, wk.ie, wk.cid, emax, wk.sepf);
       } else {
-        const int fill = (int)std::min<long>(((long)m * m + 255) / 256, 152 * 8);
+        const int fill = (int)std::min<long>(((long)m * m + 255) / 256, kSms * 8);
         count_launch(final_pass ? 3 : 1);
         if (final_pass) {
           refine_head_kernel<true><<<1, 256, 0, st>>>(m, n, wk.s, level0, level, floor, rot, wk.lam,
@@ -1239,7 +1239,7 @@ cudaError_t enqueue_level(cudaStream_t st, int n, int m, int level, const double
       cfg.attrs = at;
       cfg.numAttrs = 1;
       MPDO_CUDA_TRY(cudaLaunchKernelEx(&cfg, sg_refine_kernel, m, n, (const double2*)cur, wk.s,
-                                       (lev0 && pass == 0) ? 1 : 0, final_pass, level, floor,
+                                       (lev0 && pass == 0) ? 1 : 0, level, floor,
                                        (const int*)wk.ew.counters, wk.lam, wk.scan, wk.ie,
                                        wk.ticket, splits, wk.cid, emax, wk.sepf));
     }

@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(TT) cgemm_tile_kernel(
 }
 
 // Choice of an FP64 product's tile: 0 = 64 x 64, 1 = 16 x 16, 2 = 8 x 8, 3 = 4 x 8, 4 = 4 x 4, by
-// the FP64 time of its busiest SM, ceil(CTAs / 152) x area x 2 K clocks, with a factor for what
+// the FP64 time of its busiest SM, ceil(CTAs / SMs) x area x 2 K clocks, with a factor for what
 // smaller tiles lose to operand traffic (2304 x 256 x 256, all SMs busy either way: 1042, 1078,
 // 1080, 1125 and 1208 us).  *splits: CTAs of a cluster sharing the K loop of tiles 2 to 4, while
 // every CTA keeps at least four chunks and the SMs at most four CTAs.
@@ -361,7 +361,7 @@ inline int pick_tile(int m, int n, int batch, int k, bool herm, int* splits) {
     const long a = (m + tm[c] - 1) / tm[c], b = (n + tn[c] - 1) / tn[c];
     if ((herm && tm[c] != tn[c]) || a > 65535) continue;   // a: the grid's y extent
     const long q = (herm ? a * (a + 1) / 2 : a * b) * batch;
-    const double cost = (double)((q + 151) / 152) * tm[c] * tn[c] * f[c];
+    const double cost = (double)((q + kSms - 1) / kSms) * tm[c] * tn[c] * f[c];
     if (t < 0 || cost < best) {
       best = cost;
       t = c;
@@ -370,7 +370,7 @@ inline int pick_tile(int m, int n, int batch, int k, bool herm, int* splits) {
   }
   *splits = 1;
   if (t >= 2)
-    while (*splits < 8 && ctas * 2 * *splits <= 608 && k >= 4 * TKC * 2 * *splits) *splits *= 2;
+    while (*splits < 8 && ctas * 2 * *splits <= 4 * kSms && k >= 4 * TKC * 2 * *splits) *splits *= 2;
   return t;
 }
 
@@ -439,7 +439,7 @@ cudaError_t cgemm_impl(cudaStream_t st, int opa, int opb, int m, int n, int k, c
   const long tiles16 = (long)((n + ST - 1) / ST) * ((m + ST - 1) / ST) * batch;
   const int choice =
       g_choice[sizeof(R) == 8 ? 0 : 1][tile_bucket(tiles16)][k_bucket(k)].load(std::memory_order_relaxed);
-  const bool small = choice == 0 ? big_tiles < 152 : choice >= 2;
+  const bool small = choice == 0 ? big_tiles < kSms : choice >= 2;
   for (int b0 = 0; b0 < batch; b0 += 4096) {
     int nb = batch - b0 < 4096 ? batch - b0 : 4096;
     count_launch();

@@ -92,9 +92,6 @@ __global__ void product_state_kernel(cx<R> v0, cx<R> v1, cx<R> v2, cx<R>* base, 
 template <typename R>
 __global__ void gram_mask_kernel(int n, const double* __restrict__ sig, double gtol,
                                  R* rs, R* irs, StepScalars* sc) {
-  __shared__ int cnt;
-  if (threadIdx.x == 0) cnt = 0;
-  __syncthreads();
   double s0 = sig[0];
   bool bad = !(s0 > 0.0) || !isfinite(s0);
   for (int c = threadIdx.x; c < n; c += blockDim.x) {
@@ -102,17 +99,12 @@ __global__ void gram_mask_kernel(int n, const double* __restrict__ sig, double g
     if (!bad && s > gtol * s0) {
       rs[c] = (R)sqrt(s);
       irs[c] = (R)(1.0 / sqrt(s));
-      atomicAdd(&cnt, 1);
     } else {
       rs[c] = 0;
       irs[c] = 0;
     }
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    sc->rank_g = cnt;
-    if (bad) sc->flags |= 1;
-  }
+  if (threadIdx.x == 0 && bad) sc->flags |= 1;
 }
 
 // R[c][x] = rs[c] conj(V[x][c]); Vs[x][c] = V[x][c] irs[c]; Vr[x][c] = V[x][c] rs[c]
@@ -152,9 +144,6 @@ __global__ void build_phi_kernel(int dm, const cx<R>* __restrict__ ct,
   }
 }
 
-// Bond cut on the spectrum lam (descending, n): keep <= chi values above htol*lam0.
-// The total weight is the trace of the matrix itself (noise-free in expectation), not
-// the sum of the positive computed eigenvalues, which is biased upward by the noise floor.
 // Sum over the CTA of 256 threads in a fixed order; every thread gets it.  red: 8 doubles.
 __device__ __forceinline__ double block_sum(double x, double* red) {
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
@@ -177,6 +166,9 @@ __device__ __forceinline__ int leading_run(const double* x, int n, double thr, i
   return *s_min;
 }
 
+// Bond cut on the spectrum lam (descending, n): keep <= chi values above htol*lam0.
+// The total weight is the trace of the matrix itself (noise-free in expectation), not
+// the sum of the positive computed eigenvalues, which is biased upward by the noise floor.
 template <typename R>
 __global__ void __launch_bounds__(256) bond_select_kernel(int n, const double* __restrict__ lam,
                                                           const cx<R>* __restrict__ hm, long ldh,

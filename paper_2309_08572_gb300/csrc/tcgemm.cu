@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(PT * 8)
 constexpr int XS = kExactSlices;
 constexpr int XBN = kExactCols;   // output tile width (real columns)
 constexpr int XKB = kExactK;      // K terms of a stage
-static_assert(BM == kExactRows, "the plan's tile");
+static_assert(BM == kExactRows && kSms == kExactSms, "the plan's tile and device");
 constexpr int XSTAGES = 3;
 constexpr int XDRAIN = 5;      // stages between drains
 constexpr int XTHREADS = 320;  // warp 0 TMA, warp 1 MMA, warps 2-9 drain
@@ -1225,7 +1225,7 @@ int tc_pick_bn(long M, long N, int batch) {
   long cost = -1;
   for (int bn : {64, 128, 192, 256}) {
     if (bn > 64 && N <= bn / 2) break;
-    const long c = (mt * ((N + bn - 1) / bn) * batch + 151) / 152 * (bn + 64);
+    const long c = (mt * ((N + bn - 1) / bn) * batch + kSms - 1) / kSms * (bn + 64);
     if (cost < 0 || c < cost) {
       cost = c;
       best = bn;
@@ -1315,8 +1315,8 @@ cudaError_t mlp_launch(cudaStream_t st, MlpGroup<CAP>& g, int* err) {
   return cudaGetLastError();
 }
 }  // namespace
-// The widest tile that still gives half of the SMs one: a pass's products are short, and their
-// epilogues, which grow with the tile, are most of their time.
+// A pass's products are short, and their epilogues, which grow with the tile, are most of their time:
+// 256 columns only where nearly every SM has such a tile, 128 and 64 where half of them have, else 32.
 template <int CAP>
 cudaError_t mlp_products(cudaStream_t st, MlpGroup<CAP>& g, int* err) {
   int maxn = 0;
