@@ -595,11 +595,15 @@ __global__ void __launch_bounds__(256) refine_end_kernel(int m, int level, doubl
 // |S_ij - lam G_ij| sqrt(lam_i / lam_j) / |lam_i - lam_j|, known where its relative gap exceeds the
 // rounding of the products (100 m eps_64).  No pair is left to another level.  A corrected pair
 // keeps about the square of its angle, in its coupling and in the columns' norms, so the first pass
-// corrects angles below kGradedNewton only, and in the last pass pairs above kGradedRitz, mostly those
-// left over (relative gaps below ~1e-3), go to a Ritz step over the whole run of columns that such
-// pairs connect, which is exact within the run, however long (settle_runs).  What remains is the square
-// of the last corrections: 1e-12 at the most, 1e-14 as a rule.  (With corrections up to 1e-2,
-// first-order norms and runs cut after 16 columns it was 1e-8, 2e-6 between columns of longer runs.)
+// corrects angles below kGradedNewton only, and in the last pass pairs above kGradedRitz -- those left
+// over, and the largest of the first pass's -- go to a Ritz step over the whole run of columns that
+// such pairs connect, which is exact within the run, however long (settle_runs).  Pairs further apart
+// than kGradedFar may have ten times that angle: in crowded spectra (160 values over 14 decades) the
+// FP32 vectors of the small ones are poor, and runs across the spectrum would take 20 ms.  What remains
+// is the square of the last corrections: 1e-14 as a rule, 3e-12 between close pairs, 1e-10 in such
+// spectra.  (With corrections up to 1e-2 and 1e-4, first-order norms and runs cut after 16 columns it was
+// 1e-8, 2e-6 between columns of longer runs.  A bound of 1e-3 in the first pass makes more runs, 1 % of
+// a circuit's time, and a third pass where one is needed costs every solve a launch, as much again.)
 //
 // The step is bound by FP64: a pair costs two dot products of length m and one division.  So
 // one CTA takes a 4 x 4 block of pairs above the diagonal, forms its S, G and the diagonal
@@ -612,8 +616,8 @@ __global__ void __launch_bounds__(256) refine_end_kernel(int m, int level, doubl
 // the factor that lifts an eigenvector of L^+ L to one of L L^+.
 constexpr int GT = 4;
 constexpr int kSgeThreads = 128;
-constexpr double kGradedNewton = 1e-3;
-constexpr double kGradedRitz = 1e-6;
+constexpr double kGradedNewton = 3e-3;
+constexpr double kGradedRitz = 1e-6, kGradedFarRitz = 1e-5, kGradedFar = 0.05;
 __device__ __forceinline__ double col_scale(double lam, int scaled) {
   return !scaled ? 1.0 : lam > 0.0 ? rsqrt(lam) : 0.0;
 }
@@ -758,13 +762,15 @@ __device__ __forceinline__ double2 pair_residual(double2 s, double2 g, double l,
   const double2 n = make_double2(s.x - l * g.x, s.y - l * g.y);
   return conj ? cconj(n) : n;
 }
-// The squared angle is num / den (den not positive: none); kept below emax where apart.
+// Taken where the angle is known and below emax (efar between pairs kGradedFar apart); else the pair is
+// orthonormalised only.
 __device__ __forceinline__ bool pair_correction(int m, double2 s, double2 g, double li, double lj,
-                                                double emax, Corr& e) {
+                                                double emax, double efar, Corr& e) {
   const double d = lj - li, mx = fmax(fabs(li), fabs(lj)), mn = fmin(li, lj);
   const double2 nij = pair_residual(s, g, lj, false), nji = pair_residual(s, g, li, true);
   const double lim = d * d * mn, ang = fmax(cabs2(nij), cabs2(nji)) * mx;   // ang / lim: angle^2
   const bool apart = mn > 0.0 && fabs(d) > 100.0 * m * 1.1e-16 * mx;
+  if (fabs(d) > kGradedFar * mx) emax = efar;
   if (apart && ang < emax * emax * lim) {
     const double r = 1.0 / d;
     e.ij = cscale(nij, r);
@@ -834,7 +840,7 @@ __device__ void settle_runs(int m, double2* SG, double* lam, double2* IE, const 
       if (j < c0 && s_in[j]) continue;   // an earlier run wrote the pair
       Corr x;
       pair_correction(m, __ldcg(&SG[j * ld + b]), __ldcg(&SG[j * ld + m + b]), __ldcg(&lam[j]),
-                      __ldcg(&lam[b]), kNewtonFinal, x);
+                      __ldcg(&lam[b]), kNewtonFinal, kNewtonFinal, x);
       IE[(long)j * m + b] = s_in[j] ? x.ij : cscale(x.ij, s_cs[b]);
       IE[(long)b * m + j] = x.ji;
     }
@@ -924,7 +930,8 @@ __global__ void __launch_bounds__(kSgeThreads) sge_kernel(int m, const double2* 
       SG[j * ld + i] = cconj(s);
       SG[j * ld + m + i] = cconj(g);
       Corr x;
-      const bool kept = pair_correction(m, s, g, li, lj, final_pass ? kGradedRitz : kGradedNewton, x);
+      const bool kept = final_pass ? pair_correction(m, s, g, li, lj, kGradedRitz, kGradedFarRitz, x)
+                                   : pair_correction(m, s, g, li, lj, kGradedNewton, kGradedNewton, x);
       IE[(long)i * m + j] = cscale(x.ij, cj);
       IE[(long)j * m + i] = cscale(x.ji, ci);
       // a value that is not positive has no angle with the others: neighbours only
