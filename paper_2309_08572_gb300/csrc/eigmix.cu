@@ -624,7 +624,7 @@ __device__ __forceinline__ double col_scale(double lam, int scaled) {
 
 // ritz_cluster for a run of any length up to kGradedMax, its matrices in global memory (P, X and H,
 // m x m each), B into the run's block of IE: spectra with that many values within 1e-3 of one another
-// are rare, and one CTA takes about 3 ms for 40 columns, the FP64 operations of ~8 sweeps on its SM.
+// are rare, and one CTA takes about 5 ms for 40 columns, the FP64 operations of ~8 sweeps on its SM.
 __device__ __noinline__ void ritz_run(int m, const double2* SG, int c0, int c, double* lam,
                                       double2* IE, double2* P, double2* X, double2* H) {
   __shared__ double rc[kGradedMax / 2], rs[kGradedMax / 2], s_lam[kGradedMax];
