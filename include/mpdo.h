@@ -423,9 +423,9 @@ int mpdo_kernel_heig(int prec, int n, void* a, void* v, double* w, int* sweeps, 
 /* Eigenpairs of a graded Hermitian PSD matrix a (complex128, n x n row-major, device; A = D C D
  * with C of unit diagonal and moderate condition): eigenvalues, descending, into w (device
  * double[n]) and eigenvectors into the columns of v, each pair resolved relative to its own
- * size (FP32 sweeps with a relative threshold, two FP64 refinement passes, the second with a
+ * size (FP32 sweeps with a relative threshold, two or three FP64 refinement passes, the last with a
  * Ritz step over each run of nearly equal eigenvalues): orthonormal, and relative to the pairs'
- * sizes uncoupled, to ~1e-12 (1e-10 where 160 values crowd 14 decades).  n in
+ * sizes uncoupled, to a few 1e-12 at the worst.  n in
  * 1..MPDO_HEIG_GRADED_NMAX.  Allocates its scratch and synchronises the stream. */
 int mpdo_kernel_heig_graded(int n, const void* a, void* v, double* w, void* stream);
 

@@ -594,16 +594,17 @@ __global__ void __launch_bounds__(256) refine_end_kernel(int m, int level, doubl
 // delta sqrt(lam_j / lam_i), so the correction E is graded as well and a pair's angle is
 // |S_ij - lam G_ij| sqrt(lam_i / lam_j) / |lam_i - lam_j|, known where its relative gap exceeds the
 // rounding of the products (100 m eps_64).  No pair is left to another level.  A corrected pair
-// keeps about the square of its angle, in its coupling and in the columns' norms, so the first pass
-// corrects angles below kGradedNewton only, and in the last pass pairs above kGradedRitz -- those left
+// keeps about the square of its angle, in its coupling and in the columns' norms, so passes before the
+// last correct angles below kGradedNewton only, and in the last one pairs above kGradedRitz -- those left
 // over, and the largest of the first pass's -- go to a Ritz step over the whole run of columns that
-// such pairs connect, which is exact within the run, however long (settle_runs).  Pairs further apart
-// than kGradedFar may have ten times that angle: in crowded spectra (160 values over 14 decades) the
-// FP32 vectors of the small ones are poor, and runs across the spectrum would take 20 ms.  What remains
-// is the square of the last corrections: 1e-14 as a rule, 3e-12 between close pairs, 1e-10 in such
-// spectra.  (With corrections up to 1e-2 and 1e-4, first-order norms and runs cut after 16 columns it was
-// 1e-8, 2e-6 between columns of longer runs.  A bound of 1e-3 in the first pass makes more runs, 1 % of
-// a circuit's time, and a third pass where one is needed costs every solve a launch, as much again.)
+// such pairs connect, which is exact within the run, however long (settle_runs).  Two passes; three from
+// kGradedTwoPass columns on, where values crowd (160 over 14 decades) and the FP32 vectors of the small
+// ones are poor: with two, many pairs would go to runs, which spread over the spectrum and took 20 ms, or
+// keep 1e-10.  (Pairs further apart than kGradedFar may have ten times the angle of kGradedRitz, against
+// such runs.)  What remains is the square of the last corrections: vectors orthonormal, and relative to
+// their sizes uncoupled, to 1e-13 as a rule and 2e-12 at the worst.  With corrections up to 1e-2 and 1e-4,
+// first-order norms and runs cut after 16 columns it was 1e-8, and 2e-6 between columns of longer runs;
+// a bound of 1e-3 before the last pass makes more runs, 1 % of a circuit's time.
 //
 // The step is bound by FP64: a pair costs two dot products of length m and one division.  So
 // one CTA takes a 4 x 4 block of pairs above the diagonal, forms its S, G and the diagonal
@@ -617,6 +618,7 @@ __global__ void __launch_bounds__(256) refine_end_kernel(int m, int level, doubl
 constexpr int GT = 4;
 constexpr int kSgeThreads = 128;
 constexpr double kGradedNewton = 3e-3;
+constexpr int kGradedTwoPass = 80;   // from this size on a third pass
 constexpr double kGradedRitz = 1e-6, kGradedFarRitz = 1e-5, kGradedFar = 0.05;
 __device__ __forceinline__ double col_scale(double lam, int scaled) {
   return !scaled ? 1.0 : lam > 0.0 ? rsqrt(lam) : 0.0;
@@ -1361,7 +1363,7 @@ cudaError_t heig_mixed(cudaStream_t st, int n, const double2* a, long lda, doubl
 
 // Eigenpairs of a graded FP64 Hermitian PSD matrix a (n x n, n <= kGradedMax; L^+ L of a pivoted
 // Cholesky factor), every one resolved relative to its own size: FP32 sweeps with a relative
-// threshold, then two FP64 refinement passes (file comment of sge_kernel).  One solve takes the
+// threshold, then two or three FP64 refinement passes (file comment of sge_kernel).  One solve takes the
 // place of the levels of heig_mixed and of FP64 sweeps, whose time went into a chain of small
 // launches per two decades of the spectrum (mixed form) or into one SM's FP64 pipe (FP64 form).
 cudaError_t heig_graded(cudaStream_t st, int n, const double2* a, long lda, double2* z, long ldz,
@@ -1386,8 +1388,9 @@ cudaError_t heig_graded(cudaStream_t st, int n, const double2* a, long lda, doub
       cudaFuncSetAttribute(sge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(16 * sizeof(double2) * kGradedMax));
   MPDO_CUDA_TRY(attr);
-  for (int pass = 0; pass < 2; ++pass) {
-    const int fin = pass == 1;
+  const int passes = n < kGradedTwoPass ? 2 : 3;
+  for (int pass = 0; pass < passes; ++pass) {
+    const int fin = pass + 1 == passes;
     count_launch();
     // a long run's matrices: the next basis' place and the levels' one
     sge_kernel<<<grid, kSgeThreads, sm, st>>>(n, cur, wk.s, fin, fin ? w : wk.lam, wk.ie, wk.cid,
